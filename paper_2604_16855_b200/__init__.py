@@ -1,5 +1,5 @@
 """B200-native COD-TDQ hot path: token-group dual-constraint activation quantizer and W4A4
-linear layer, as a C-ABI CUDA library (``libtdq.so``) with a thin ctypes binding.
+linear layer, as a C-ABI CUDA library (``libtdq.so``) with a thin Python binding.
 
     from paper_2604_16855_b200 import tdq
     codes, scale = tdq.quantize_act(x)                     # x: CUDA tensor [B, N, C], fp32 or bf16

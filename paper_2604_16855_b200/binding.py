@@ -1,5 +1,8 @@
-"""ctypes binding of libtdq.so.  Argument marshalling only: every step runs in the library's
-CUDA kernels.  torch is used to allocate device memory and to name the current stream."""
+"""Python binding of libtdq.so.  Argument marshalling only: every step runs in the library's
+CUDA kernels.  torch is used to allocate device memory and to name the current stream.
+
+The calls of the hot path go through `_tdq_host` (csrc/tdq_host.cpp), which reads the tensors in C++;
+queries, self-tests and the raw C ABI (`lib()`) go through ctypes."""
 from __future__ import annotations
 
 import ctypes
@@ -10,11 +13,12 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libtdq.so")
 
-if not os.path.exists(LIB_PATH):
+if not (os.path.exists(LIB_PATH) and os.path.exists(os.path.join(_HERE, "_tdq_host.so"))):
     raise ImportError(
-        "libtdq.so is missing: build it with `python -m paper_2604_16855_b200.build` "
+        "libtdq.so or _tdq_host.so is missing: build them with `python -m paper_2604_16855_b200.build` "
         "(there is no fallback implementation)")
 _lib = ctypes.CDLL(LIB_PATH)
+from . import _tdq_host as _host  # noqa: E402  (needs torch and libtdq.so in the process)
 
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_ALIGNMENT, ERR_WORKSPACE, ERR_CUDA, ERR_DEVICE_TIMEOUT = range(7)
 F32, BF16, F16 = 0, 1, 2
@@ -82,6 +86,8 @@ class TdqError(RuntimeError):
         super().__init__("%s: %s (status %d)" % (where, status_string(code), code))
 
 
+_host.set_error_class(TdqError)
+
 def lib():
     """The loaded ctypes library (for callers that want the raw C ABI)."""
     return _lib
@@ -110,16 +116,6 @@ def _check(code, where):
         raise TdqError(code, where)
 
 
-def _dtype_id(t: torch.Tensor) -> int:
-    if t.dtype == torch.float32:
-        return F32
-    if t.dtype == torch.bfloat16:
-        return BF16
-    if t.dtype == torch.float16:
-        return F16          # outputs of the linear layer only; the library refuses it elsewhere
-    raise TypeError("tdq takes float32, bfloat16 or (for outputs) float16 tensors, got %s" % t.dtype)
-
-
 def _stream(t: torch.Tensor):
     return ctypes.c_void_p(torch.cuda.current_stream(t.device).cuda_stream)
 
@@ -138,102 +134,22 @@ def quantize_act(x: torch.Tensor, params: ActParams | None = None, *, codes=None
     """tdq_quantize_act on x [..., C] (last dim contiguous, rows equally spaced).
 
     Returns (codes uint8 [M, C_pad/2], scale float32 [M, K])."""
-    _need_cuda(x)
-    p = params or default_act_params()
-    C = x.shape[-1]
-    x2 = x.reshape(-1, C)
-    if x2.stride(-1) != 1:
-        raise ValueError("the channel axis must be contiguous")
-    M = x2.shape[0]
-    g = p.group_size
-    K = (C + g - 1) // g
-    if codes is None:
-        codes = torch.empty((M, K * g // 2), dtype=torch.uint8, device=x.device)
-    if scale is None:
-        scale = torch.empty((M, K), dtype=torch.float32, device=x.device)
-    if M == 0:          # nothing to do; an empty tensor has no device pointer to pass
-        return codes, scale
-    stride = x2.stride(0) if M > 1 else C
-    _check(_lib.tdq_quantize_act(_ptr(x2), _dtype_id(x2), 1, M, C, stride, ctypes.byref(p), _ptr(codes),
-                                 _ptr(scale), _ptr(offset), _stream(x)), "tdq_quantize_act")
-    return codes, scale
+    return _host.quantize_act(x, params, codes, scale, offset)
 
 
 def quantize_act_fixed(x: torch.Tensor, radius: float, g: int = 32, *, codes=None, scale=None, offset=None):
     """tdq_quantize_act_fixed: the same clip radius in every group.  Returns (codes [M, C/2], scale [M, C/g])."""
-    _need_cuda(x, codes, scale, offset)
-    C = x.shape[-1]
-    x2 = x.reshape(-1, C)
-    M = x2.shape[0]
-    if codes is None:
-        codes = torch.empty((M, C // 2), dtype=torch.uint8, device=x.device)
-    if scale is None:
-        scale = torch.empty((M, max(C // g, 1)), dtype=torch.float32, device=x.device)
-    stride = x2.stride(0) if M > 1 else C
-    _check(_lib.tdq_quantize_act_fixed(_ptr(x2), _dtype_id(x2), 1, M, C, stride, g, radius, _ptr(codes), _ptr(scale),
-                                       _ptr(offset), _stream(x)), "tdq_quantize_act_fixed")
-    return codes, scale
+    return _host.quantize_act_fixed(x, radius, g, codes, scale, offset)
 
 
 def quantize_act_nchw(x: torch.Tensor, params: ActParams | None = None, *, codes=None, scale=None, offset=None):
     """tdq_quantize_act_nchw on a contiguous CUDA tensor [B, C, H, W].  Returns (codes [B*H*W, C/2], scale [B*H*W, C/32])."""
-    _need_cuda(x, codes, scale, offset)
-    p = params or default_act_params()
-    if x.dim() != 4 or not x.is_contiguous():
-        raise ValueError("x must be a contiguous [B, C, H, W] tensor")
-    B, C, H, W = x.shape
-    M = B * H * W
-    if codes is None:
-        codes = torch.empty((M, C // 2), dtype=torch.uint8, device=x.device)
-    if scale is None:
-        scale = torch.empty((M, max(C // 32, 1)), dtype=torch.float32, device=x.device)
-    _check(_lib.tdq_quantize_act_nchw(_ptr(x), _dtype_id(x), B, C, H, W, ctypes.byref(p), _ptr(codes), _ptr(scale),
-                                      _ptr(offset), _stream(x)), "tdq_quantize_act_nchw")
-    return codes, scale
+    return _host.quantize_act_nchw(x, params, codes, scale, offset)
 
 
 def quantize_weight(w: torch.Tensor, pad_to: int = 32, *, wcodes=None, wscale=None):
     """tdq_quantize_weight on w [O, I] (contiguous).  Returns (wcodes uint8 [O, I_pad/2], wscale [O])."""
-    _need_cuda(w)
-    w = w.contiguous()
-    O, I = w.shape
-    I_pad = (I + pad_to - 1) // pad_to * pad_to
-    if wcodes is None:
-        wcodes = torch.empty((O, I_pad // 2), dtype=torch.uint8, device=w.device)
-    if wscale is None:
-        wscale = torch.empty((O,), dtype=torch.float32, device=w.device)
-    _check(_lib.tdq_quantize_weight(_ptr(w), _dtype_id(w), O, I, pad_to, _ptr(wcodes), _ptr(wscale), _stream(w)),
-           "tdq_quantize_weight")
-    return wcodes, wscale
-
-
-def _check_operands(named, y=None):
-    """The layout the C ABI assumes but cannot see: dtype, contiguity, one common device; y may have a row pitch
-    but its columns must be adjacent.  `named` is a list of (name, tensor or None, dtype).  Returns the device."""
-    dev = None
-    for name, t, dt in named:
-        if t is None:
-            continue
-        if t.dtype != dt:
-            raise TypeError("%s must be %s, got %s" % (name, dt, t.dtype))
-        if not t.is_contiguous():
-            raise ValueError("%s must be contiguous" % name)
-        if dev is None:
-            dev = t.device
-        elif t.device != dev:
-            raise ValueError("%s is on %s, the other operands on %s" % (name, t.device, dev))
-    if y is not None:
-        if y.dim() != 2 or (y.shape[1] > 1 and y.stride(1) != 1):
-            raise ValueError("y must be a matrix whose columns are adjacent in memory")
-        if dev is not None and y.device != dev:
-            raise ValueError("y is on %s, the operands on %s" % (y.device, dev))
-    return dev
-
-
-def _linear_operands(xcodes, xscale, wcodes, wscale, bias, y, workspace=None, acc_debug=None):
-    return _check_operands([("xcodes", xcodes, torch.uint8), ("xscale", xscale, torch.float32), ("wcodes", wcodes, torch.uint8),
-                            ("wscale", wscale, torch.float32), ("bias", bias, torch.float32),
-                            ("workspace", workspace, torch.uint8), ("acc_debug", acc_debug, torch.int32)], y)
+    return _host.quantize_weight(w, pad_to, wcodes, wscale)
 
 
 def linear_workspace(M, I_pad, O, g, device) -> torch.Tensor:
@@ -244,38 +160,12 @@ def linear_workspace(M, I_pad, O, g, device) -> torch.Tensor:
 def w4a4_linear(xcodes, xscale, wcodes, wscale, bias=None, *, g=32, out_dtype=torch.float32, y=None,
                 acc_debug=None, workspace=None):
     """tdq_w4a4_linear.  Returns y [M, O]."""
-    _need_cuda(xcodes, xscale, wcodes, wscale, bias)
-    M, half = xcodes.shape
-    I_pad = half * 2
-    O = wcodes.shape[0]
-    if y is None:
-        y = torch.empty((M, O), dtype=out_dtype, device=xcodes.device)
-    if workspace is None:
-        workspace = linear_workspace(M, I_pad, O, g, xcodes.device)
-    dev = _linear_operands(xcodes, xscale, wcodes, wscale, bias, y, workspace, acc_debug)
-    with torch.cuda.device(dev):        # the library works on the current device
-        _check(_lib.tdq_w4a4_linear(_ptr(xcodes), _ptr(xscale), _ptr(wcodes), _ptr(wscale), _ptr(bias), M, I_pad, O, g,
-                                    _ptr(y), _dtype_id(y), y.stride(0) if M > 0 else O, _ptr(acc_debug),
-                                    _ptr(workspace), workspace.numel(), _stream(xcodes)), "tdq_w4a4_linear")
-    return y
+    return _host.w4a4_linear(xcodes, xscale, wcodes, wscale, bias, g, out_dtype, y, acc_debug, workspace, False)
 
 
 def w4a4_linear_pow2(xcodes, xscale, wcodes, wscale, bias=None, *, g=32, out_dtype=torch.float32, y=None, workspace=None):
     """tdq_w4a4_linear_pow2: the linear layer for power-of-two activation steps.  Returns y [M, O]."""
-    _need_cuda(xcodes, xscale, wcodes, wscale, bias)
-    M, half = xcodes.shape
-    I_pad = half * 2
-    O = wcodes.shape[0]
-    if y is None:
-        y = torch.empty((M, O), dtype=out_dtype, device=xcodes.device)
-    if workspace is None:
-        workspace = linear_workspace(M, I_pad, O, g, xcodes.device)
-    dev = _linear_operands(xcodes, xscale, wcodes, wscale, bias, y, workspace)
-    with torch.cuda.device(dev):
-        _check(_lib.tdq_w4a4_linear_pow2(_ptr(xcodes), _ptr(xscale), _ptr(wcodes), _ptr(wscale), _ptr(bias), M, I_pad, O, g,
-                                         _ptr(y), _dtype_id(y), y.stride(0) if M > 0 else O, _ptr(workspace),
-                                         workspace.numel(), _stream(xcodes)), "tdq_w4a4_linear_pow2")
-    return y
+    return _host.w4a4_linear(xcodes, xscale, wcodes, wscale, bias, g, out_dtype, y, None, workspace, True)
 
 
 LINEAR_STATIC_BYTES = 8 << 20   # TDQ_LINEAR_STATIC_BYTES of the header
@@ -286,67 +176,20 @@ def w4a4_linear_static(xcodes, xscale, wcodes, wscale, bias=None, *, g=32, y, wa
 
     The scratch space is a fixed array inside the library, so this wrapper allocates nothing
     either: the caller passes the output tensor y [M, O].  Returns y."""
-    _need_cuda(xcodes, xscale, wcodes, wscale, bias, y)
-    M, half = xcodes.shape
-    O = wcodes.shape[0]
-    dev = _linear_operands(xcodes, xscale, wcodes, wscale, bias, y)
-    with torch.cuda.device(dev):        # the scratch array is looked up on the current device
-        _check(_lib.tdq_w4a4_linear_static(_ptr(xcodes), _ptr(xscale), _ptr(wcodes), _ptr(wscale), _ptr(bias), M, half * 2,
-                                           O, g, _ptr(y), _dtype_id(y), y.stride(0) if M > 0 else O, 1 if wait else 0,
-                                           _stream(xcodes)), "tdq_w4a4_linear_static")
-    return y
+    return _host.w4a4_linear_static(xcodes, xscale, wcodes, wscale, bias, g, y, wait)
 
 
 def quant_linear_fused(x, wcodes, wscale, bias=None, params: ActParams | None = None, *,
                        out_dtype=torch.float32, y=None, workspace=None):
     """tdq_quant_linear_fused: quantizer as the linear layer's A-operand producer.  Returns y [M, O]."""
-    _need_cuda(x, wcodes, wscale, bias)
-    p = params or default_act_params()
-    C = x.shape[-1]
-    x2 = x.reshape(-1, C)
-    M = x2.shape[0]
-    O = wcodes.shape[0]
-    if y is None:
-        y = torch.empty((M, O), dtype=out_dtype, device=x.device)
-    if workspace is None:
-        workspace = linear_workspace(M, wcodes.shape[1] * 2, O, p.group_size, x.device)
-    stride = x2.stride(0) if M > 1 else C
-    if x2.dim() != 2 or (C > 1 and x2.stride(1) != 1):
-        raise ValueError("the channels of x must be adjacent in memory")
-    dev = _check_operands([("wcodes", wcodes, torch.uint8), ("wscale", wscale, torch.float32), ("bias", bias, torch.float32),
-                           ("workspace", workspace, torch.uint8)], y)
-    if x2.device != dev:
-        raise ValueError("x is on %s, the weights on %s" % (x2.device, dev))
-    with torch.cuda.device(dev):
-        _check(_lib.tdq_quant_linear_fused(_ptr(x2), _dtype_id(x2), 1, M, C, stride, ctypes.byref(p), _ptr(wcodes),
-                                           _ptr(wscale), _ptr(bias), O, _ptr(y), _dtype_id(y), y.stride(0),
-                                           _ptr(workspace), workspace.numel(), _stream(x)), "tdq_quant_linear_fused")
-    return y
+    return _host.quant_linear_fused(x, wcodes, wscale, bias, params, out_dtype, y, workspace)
 
 
 def quant_linear_host(x_host: torch.Tensor, wcodes, wscale, bias=None, params: ActParams | None = None, *,
                       out_dtype=torch.float32, y_host=None, device="cuda"):
     """tdq_quant_linear_host: x_host [M, C] (CPU, ideally pinned) in, y_host [M, O] (CPU) out.  The device buffers
     the call needs are allocated here.  Returns (y_host, workspace); synchronise the current stream before reading."""
-    _need_cuda(wcodes, wscale, bias)
-    p = params or default_act_params()
-    M, C = x_host.shape
-    O = wcodes.shape[0]
-    g = p.group_size
-    I_pad = (C + g - 1) // g * g
-    dev = wcodes.device
-    x_dev = torch.empty((M, C), dtype=x_host.dtype, device=dev)
-    codes = torch.empty((M, I_pad // 2), dtype=torch.uint8, device=dev)
-    scale = torch.empty((M, I_pad // g), dtype=torch.float32, device=dev)
-    y_dev = torch.empty((M, O), dtype=out_dtype, device=dev)
-    if y_host is None:
-        y_host = torch.empty((M, O), dtype=out_dtype).pin_memory()
-    workspace = linear_workspace(M, I_pad, O, g, dev)
-    _check(_lib.tdq_quant_linear_host(_ptr(x_host), _dtype_id(x_host), 1, M, C, ctypes.byref(p), _ptr(wcodes), _ptr(wscale),
-                                      _ptr(bias), O, _ptr(y_host), _dtype_id(y_host), _ptr(x_dev), _ptr(codes), _ptr(scale),
-                                      _ptr(y_dev), _ptr(workspace), workspace.numel(), _stream(wcodes)),
-           "tdq_quant_linear_host")
-    return y_host, (workspace, x_dev, codes, scale, y_dev)
+    return _host.quant_linear_host(x_host, wcodes, wscale, bias, params, out_dtype, y_host)
 
 
 def workspace_status(workspace: torch.Tensor):
@@ -371,11 +214,27 @@ def selftest_wait_timeout(which: int, limit_cycles: int, workspace: torch.Tensor
            "tdq_selftest_wait_timeout")
 
 
+def _check_operands(named):
+    """float32, contiguous and on one device.  `named` is a list of (name, tensor or None).  Returns the device."""
+    dev = None
+    for name, t in named:
+        if t is None:
+            continue
+        if t.dtype != torch.float32:
+            raise TypeError("%s must be torch.float32, got %s" % (name, t.dtype))
+        if not t.is_contiguous():
+            raise ValueError("%s must be contiguous" % name)
+        if dev is None:
+            dev = t.device
+        elif t.device != dev:
+            raise ValueError("%s is on %s, the other operands on %s" % (name, t.device, dev))
+    return dev
+
+
 def fold_output_affine(wscale, bias, out_mul, out_add=None):
     """tdq_fold_output_affine: (wscale', bias') such that the linear layer computes out_mul * y + out_add."""
     _need_cuda(wscale, bias, out_mul, out_add)
-    dev = _check_operands([("wscale", wscale, torch.float32), ("bias", bias, torch.float32), ("out_mul", out_mul, torch.float32),
-                           ("out_add", out_add, torch.float32)])
+    dev = _check_operands([("wscale", wscale), ("bias", bias), ("out_mul", out_mul), ("out_add", out_add)])
     O = wscale.shape[0]
     ws2, b2 = torch.empty_like(wscale), torch.empty_like(wscale)
     with torch.cuda.device(dev):

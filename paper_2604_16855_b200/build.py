@@ -1,4 +1,5 @@
-"""Builds libtdq.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a.
+"""Builds libtdq.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _tdq_host.so (the Python binding's host
+side, which reads torch tensors in C++) with g++.
 
     python -m paper_2604_16855_b200.build [--force] [--verbose]
 
@@ -16,28 +17,57 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libtdq.so")
+HOST = os.path.join(HERE, "_tdq_host.so")
+HOST_SOURCE = "tdq_host.cpp"
 SOURCES = ["tdq_quantize_act.cu", "tdq_quantize_weight.cu", "tdq_linear.cu", "tdq_linear_g32.cu", "tdq_fused.cu", "tdq_api.cu", "tdq_peak.cu"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC", "--ftz=false", "--prec-div=true", "--prec-sqrt=true"]
 
 
-def _deps_mtime():
+def _deps_mtime(headers_only: bool = False):
+    """When the newest source (or header, which every source may include) was written."""
     newest = 0.0
     for root in (CSRC, os.path.join(os.path.dirname(HERE), "include")):
         for name in os.listdir(root):
-            newest = max(newest, os.path.getmtime(os.path.join(root, name)))
+            if not headers_only or not name.endswith((".cu", ".cpp")):
+                newest = max(newest, os.path.getmtime(os.path.join(root, name)))
     return max(newest, os.path.getmtime(os.path.abspath(__file__)))
 
 
+def _compile_host():
+    """The extension module: torch's headers and libraries, nothing of CUDA but its headers."""
+    import sysconfig
+    import torch
+    tdir = os.path.dirname(torch.__file__)
+    tmp = HOST + ".tmp.%d" % os.getpid()
+    inc = [os.path.join(tdir, "include"), os.path.join(tdir, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include")]
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)]
+    cmd += ["-I" + d for d in inc] + [os.path.join(CSRC, HOST_SOURCE), "-o", tmp, "-L" + HERE, "-l:libtdq.so",
+                                      "-L" + os.path.join(tdir, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python",
+                                      "-ltorch", "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode:
+        sys.stderr.write(r.stdout + r.stderr)
+        raise RuntimeError("g++ failed on %s" % HOST_SOURCE)
+    os.replace(tmp, HOST)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _deps_mtime():
+    newest = _deps_mtime()
+    if not force and all(os.path.exists(f) and os.path.getmtime(f) >= newest for f in (LIB, HOST)):
         return LIB
     os.makedirs(OBJ, exist_ok=True)
     extra = ["-Xptxas", "-v"] if verbose else []
+    headers = _deps_mtime(headers_only=True)
 
     def compile_one(src):
         obj = os.path.join(OBJ, src.replace(".cu", ".o"))
+        if not (force or verbose) and os.path.exists(obj) and \
+                os.path.getmtime(obj) >= max(headers, os.path.getmtime(os.path.join(CSRC, src))):
+            return obj
         cmd = [NVCC] + FLAGS + extra + ["-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if verbose or r.returncode:
@@ -52,6 +82,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     subprocess.check_call([NVCC, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp] + objs +
                           ["-cudart", "static"])
     os.replace(tmp, LIB)
+    _compile_host()
     return LIB
 
 

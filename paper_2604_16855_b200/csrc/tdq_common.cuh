@@ -70,6 +70,16 @@ inline int current_device_sm_count(int* device = nullptr) {
 inline bool device_marked(const std::atomic<uint64_t>& done, int dev) { return (done.load(std::memory_order_acquire) >> dev) & 1u; }
 inline void mark_device(std::atomic<uint64_t>& done, int dev) { done.fetch_or(1ull << dev, std::memory_order_release); }
 
+// The opt-in to `bytes` of dynamic shared memory for `kernel`, made once per kernel and device (it costs about a
+// microsecond of host time, as much as a quarter of a launch).  `done` is a static of the caller, one per kernel.
+template <typename F>
+inline cudaError_t allow_smem(F* kernel, int bytes, std::atomic<uint64_t>& done, int dev) {
+    if (device_marked(done, dev)) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) mark_device(done, dev);
+    return e;
+}
+
 // Programmatic dependent launch.  The hot-path kernels are launched with the attribute that lets a grid start
 // while its predecessor in the stream is still draining; each of them executes pdl_wait() in every thread before its
 // first access to global memory (the wait returns when the preceding grids have completed and their writes are

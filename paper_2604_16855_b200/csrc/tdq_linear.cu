@@ -1088,8 +1088,6 @@ __global__ void __launch_bounds__(kThreads, 1) w4a4_gemm_kernel(const LinArgs a,
 
 using namespace tdq;
 
-static int sm_count() { return current_device_sm_count(); }
-
 extern "C" size_t tdq_linear_workspace_bytes(int64_t M, int64_t I_pad, int64_t O, int32_t group_size) {
     if (M < 0 || I_pad <= 0 || O <= 0 || group_size <= 0 || group_size % 32 || I_pad % group_size)
         return kWorkspaceHeader;
@@ -1141,7 +1139,8 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
         return TDQ_ERR_ALIGNMENT;
     if (M == 0) return TDQ_OK;
     cudaStream_t stream = reinterpret_cast<cudaStream_t>(cuda_stream);
-    const int n_sm = sm_count();
+    int dev = 0;
+    const int n_sm = current_device_sm_count(&dev);
     if (n_sm <= 0) return TDQ_ERR_CUDA;
     // Output strips: 64-byte rows (32 KB in all) for bf16 output, and for fp32 output of wide groups, which is
     // then written in two passes of 16 columns; the ring gets the other 32 KB.  Both need the bulk tensor store.
@@ -1247,8 +1246,9 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
         if (fx->bf16) kernel = ybf ? w4a4_gemm_kernel<false, true, false, 1> : w4a4_gemm_kernel<false, false, false, 1>;
         else kernel = ybf ? w4a4_gemm_kernel<false, true, false, 2> : w4a4_gemm_kernel<false, false, false, 2>;
     }
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess)
-        return TDQ_ERR_CUDA;
+    static std::atomic<uint64_t> smem_done[12];      // one per instance
+    const int inst = fx ? 8 + (fx->bf16 ? 2 : 0) + (ybf ? 1 : 0) : (i8 ? 4 : 0) + (ybf ? 2 : 0) + (dbg ? 1 : 0);
+    if (allow_smem(kernel, kSmemLimit, smem_done[inst], dev) != cudaSuccess) return TDQ_ERR_CUDA;
 
     const unsigned pieces = (unsigned)((e.tiles_m + e.tiles_n) * p.n_chunks);
     if (pow2_steps) {

@@ -515,8 +515,10 @@ tdq_status launch_linear_g32(const LinArgs& a, const CUtensorMap& ymap, uint32_t
     if (ybf && !dbg) kernel = w4a4_g32_kernel<true, false>;
     if (!ybf && dbg) kernel = w4a4_g32_kernel<false, true>;
     if (ybf && dbg) kernel = w4a4_g32_kernel<true, true>;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess)
-        return TDQ_ERR_CUDA;
+    static std::atomic<uint64_t> smem_done[4];
+    int dev = 0;
+    if (current_device_sm_count(&dev) <= 0) return TDQ_ERR_CUDA;
+    if (allow_smem(kernel, kSmemLimit, smem_done[(ybf ? 1 : 0) + (dbg ? 2 : 0)], dev) != cudaSuccess) return TDQ_ERR_CUDA;
     if (launch_pdl(kernel, dim3(grid), dim3(kThreadsG32), smem_bytes, stream, a, ymap) != cudaSuccess) return TDQ_ERR_CUDA;
     g_launch_count.fetch_add(1, std::memory_order_relaxed);
     return TDQ_OK;

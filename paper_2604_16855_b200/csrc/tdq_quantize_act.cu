@@ -322,11 +322,8 @@ cudaError_t launch_ring(const ActArgs& a, cudaStream_t st) {
     int dev = 0;
     const int n_sm = current_device_sm_count(&dev);
     if (n_sm <= 0) return cudaErrorUnknown;
-    if (!device_marked(attr_done, dev)) {
-        cudaError_t e = cudaFuncSetAttribute(act_g32_ring_kernel<BF16, KZR, KB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        mark_device(attr_done, dev);
-    }
+    const cudaError_t e = allow_smem(act_g32_ring_kernel<BF16, KZR, KB>, smem, attr_done, dev);
+    if (e != cudaSuccess) return e;
     const int64_t n_tiles = (a.total_groups + kFastThreads - 1) / kFastThreads;
     const int64_t grid = n_tiles < 2 * n_sm ? n_tiles : 2 * n_sm;
     return launch_pdl(act_g32_ring_kernel<BF16, KZR, KB>, dim3((unsigned)grid), dim3(kRingThreads), smem, st, a, n_tiles);
