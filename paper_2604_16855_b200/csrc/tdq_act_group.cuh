@@ -7,20 +7,39 @@
 #include "tdq_common.cuh"
 
 namespace tdq {
+
+struct ActArgs {
+    const void* x;
+    int64_t M, C, row_stride;  // elements
+    int64_t total_groups;      // M * K
+    int32_t g, K;              // group size, groups per token
+    int32_t k_zr, k_base;      // 1-indexed ranks
+    float seven_tau;
+    uint32_t flags;
+    uint8_t* codes;
+    float* scale;
+    float* offset;
+};
+
+// Groups of any multiple of 8, any row layout (tdq_quantize_act_wide.cu).
+bool act_wide_ok(const ActArgs& a);
+cudaError_t launch_act_wide(const ActArgs& a, bool bf16, cudaStream_t st);
+
 namespace {
 
 // True when the binary32 moments prove that 7 tau sigma exceeds cmin by a safe margin, i.e.
-// the C1 bound cannot be the minimum.  s1 = sum x, s2 = sum x^2 over the 32 elements.
-// The estimate var = s2/32 - mean^2 has relative error below 1e-4 once var >= s2/512, and
+// the C1 bound cannot be the minimum.  s1 = sum x, s2 = sum x^2 over the g elements, inv_g = 1/g.
+// The estimate var = s2/g - mean^2 has relative error below 1e-4 once var >= s2/512, and
 // the test keeps a 1 % margin on the squared radius, so a true result is always right; a
-// false one only means the deviation is recomputed exactly.
-__device__ __forceinline__ bool c1_cannot_bind(float s1, float s2, float seven_tau, float cmin) {
-    const float mean = s1 * (1.0f / 32.0f);
-    const float ex2 = s2 * (1.0f / 32.0f);
+// false one only means the deviation is recomputed exactly.  When the other bounds already put the radius at or below
+// its floor, the floor decides whatever sigma is (the usual case of groups that are mostly zeros or padding).
+__device__ __forceinline__ bool c1_cannot_bind(float s1, float s2, float seven_tau, float cmin, float inv_g = 1.0f / 32.0f) {
+    const float mean = s1 * inv_g;
+    const float ex2 = s2 * inv_g;
     const float var = fmaf(-mean, mean, ex2);
     const float lhs = seven_tau * seven_tau * var * 0.99f;
     const float rhs = cmin * cmin;
-    return (var >= ex2 * (1.0f / 16.0f)) && (lhs > rhs) && (rhs >= 1e-30f) && (s2 < 1e37f) && (lhs < 1e37f);
+    return cmin <= kClipFloor || ((var >= ex2 * (1.0f / 16.0f)) && (lhs > rhs) && (rhs >= 1e-30f) && (s2 < 1e37f) && (lhs < 1e37f));
 }
 
 // sigma = Std(x_k) + 1e-12 in binary64, sequentially over the group, rounded to binary32.
@@ -60,7 +79,7 @@ __device__ __forceinline__ bool c1_cannot_bind_rough(float s1, float s2, float s
     const float var = fmaf(-mean, mean, ex2);
     const float lhs = seven_tau * seven_tau * var * 0.7f;
     const float rhs = cmin * cmin;
-    return (var >= ex2 * 0.5f) && (lhs > rhs) && (rhs >= 1e-30f) && (s2 < 1e37f) && (lhs < 1e37f);
+    return cmin <= kClipFloor || ((var >= ex2 * 0.5f) && (lhs > rhs) && (rhs >= 1e-30f) && (s2 < 1e37f) && (lhs < 1e37f));
 }
 
 // two binary32 lanes in one 64-bit register; each lane rounds exactly like the scalar .rn instruction

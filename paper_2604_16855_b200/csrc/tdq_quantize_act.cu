@@ -1,6 +1,6 @@
 // tdq_quantize_act: token-group dual-constraint activation quantizer (Algorithm S1 steps 1-7).
 //
-// Five kernels:
+// Seven kernels:
 //   * act_g32_ring_kernel   the fast path on dense rows (row stride == C): persistent, two CTAs per
 //     SM; one producer lane streams 16 KB tiles of 256 groups into a shared-memory ring with 1-D
 //     bulk copies and mbarrier transaction counts, eight consumer warps take one group per thread
@@ -12,11 +12,13 @@
 //     registers: max, sums, a pruned sorting network for the rank-k magnitude, the DCRP
 //     projection, an exact quotient, round-half-even, and one 128-bit store of 32 nibbles.
 //     One pass over HBM: 2 (bf16) or 4 (fp32) bytes in, 0.5 + 0.125 bytes out per element.
+//   * act_g32_ragged_kernel   g = 32 on any other rows: staged element by element.
 //   * act_g32_nchw_kernel   channel-major input [B, C, H*W]: a tile of 32 channel rows is staged in
 //     shared memory and each thread gathers one position's 32 channels (tdq_quantize_act_nchw).
 //   * act_fixed_kernel   the fixed-radius control: no reductions, 8 channels per thread
 //     (tdq_quantize_act_fixed).
-//   * act_generic_kernel   any even g <= 4096, any C, any alignment: one warp per group,
+//   * act_wide_kernel   (tdq_quantize_act_wide.cu) groups of a multiple of 8, any C, any alignment.
+//   * act_generic_kernel   the rest, that is groups that are not a multiple of 8: one warp per group,
 //     rank selection by bisection on the bit patterns of |x|, IEEE division.
 //
 // Exactness.  Codes must equal clip(rint(fl(fl(clip(x)) / Delta))) in binary32.  The fast
@@ -37,19 +39,6 @@ namespace tdq {
 std::atomic<uint64_t> g_launch_count{0};
 
 namespace {
-
-struct ActArgs {
-    const void* x;
-    int64_t M, C, row_stride;  // elements
-    int64_t total_groups;      // M * K
-    int32_t g, K;              // group size, groups per token
-    int32_t k_zr, k_base;      // 1-indexed ranks
-    float seven_tau;
-    uint32_t flags;
-    uint8_t* codes;
-    float* scale;
-    float* offset;
-};
 
 // ------------------------------------------------------------------------------------------
 // generic kernel: one warp per group
@@ -373,6 +362,95 @@ cudaError_t launch_fast(const ActArgs& a, cudaStream_t st) {
 }
 
 // ------------------------------------------------------------------------------------------
+// g = 32 on rows that 16-byte loads cannot read (a channel count that is not a multiple of 32, a base or pitch off the
+// 16-byte grid): the same per-group code behind a staging pass that reads element by element.  A warp stages whole
+// groups, lane = channel (or channel pair of bf16), so every load instruction still reads up to 128 contiguous bytes;
+// channels past the end of the row are zeros.  The staging costs about as many instructions as the groups themselves.
+// Measured, 9217 x 147 fp32: 89 us in the bisection kernel that served these rows before, 6.5 us here.
+
+template <bool BF16, int KZR, int KB>
+__global__ void __launch_bounds__(kFastThreads) act_g32_ragged_kernel(ActArgs a, int32_t pairs_ok) {
+    constexpr int kGroupBytes = BF16 ? 64 : 128;
+    constexpr int kChunks = kGroupBytes / 16;
+    constexpr int kSwzMask = kChunks - 1;
+    __shared__ __align__(16) uint4 tile[kFastThreads * kChunks];
+    pdl_wait();
+    pdl_trigger();
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int64_t g0 = (int64_t)blockIdx.x * kFastThreads;
+    uint8_t* tb = reinterpret_cast<uint8_t*>(tile);
+    // channel `e` of local group `l` lands where act_g32_kernel's 16-byte pieces put it
+    auto slot = [&](int l, int e) -> uint8_t* {
+        const int byte = e * (BF16 ? 2 : 4), swz = BF16 ? ((l >> 1) & kSwzMask) : (l & kSwzMask);
+        return tb + (l * kChunks + ((byte >> 4) ^ swz)) * 16 + (byte & 15);
+    };
+    // The warp's first group; the others follow by stepping through the groups of a token, without a division.  A batch
+    // of loads is in flight before the first of them is stored (one dependent load after the other took 21 us instead).
+    int64_t gi = g0 + warp * 32;
+    int64_t m;
+    int32_t k;
+    if (a.total_groups <= 0x7fffffff) {
+        m = (uint32_t)gi / (uint32_t)a.K;
+        k = (int32_t)((uint32_t)gi - (uint32_t)m * (uint32_t)a.K);
+    } else {
+        m = gi / a.K;
+        k = (int32_t)(gi - m * a.K);
+    }
+    const bool pairs = BF16 && pairs_ok;
+    const int e = pairs ? 2 * (lane & 15) : lane;         // this lane's channel; pairs: half-warps take even and odd groups
+    const int per = pairs ? 2 : 1;
+    const uint8_t* row = reinterpret_cast<const uint8_t*>(a.x) + m * a.row_stride * (BF16 ? 2 : 4);
+    const int64_t pitch = a.row_stride * (BF16 ? 2 : 4);
+    auto step = [&]() {
+        ++gi;
+        if (++k == a.K) { k = 0; row += pitch; }
+    };
+    if (pairs && lane >= 16) step();
+    constexpr int kBatch = 8;
+#pragma unroll 1
+    for (int j0 = 0; j0 < 32; j0 += kBatch * per) {
+        uint32_t v[kBatch];
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+            const int left = gi < a.total_groups ? (int)min((int64_t)32, a.C - (int64_t)k * 32) : 0;   // channels that exist
+            const uint8_t* src = row + ((int64_t)k * 32 + e) * (BF16 ? 2 : 4);
+            v[j] = 0u;
+            if (!BF16) { if (e < left) v[j] = __ldg(reinterpret_cast<const uint32_t*>(src)); }
+            else if (pairs && e + 1 < left) v[j] = __ldg(reinterpret_cast<const uint32_t*>(src));
+            else if (e < left) v[j] = __ldg(reinterpret_cast<const uint16_t*>(src));
+            step();
+            if (pairs) step();
+        }
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+            const int l = warp * 32 + j0 + j * per + (pairs ? lane >> 4 : 0);
+            if (BF16 && !pairs) *reinterpret_cast<uint16_t*>(slot(l, e)) = (uint16_t)v[j];
+            else *reinterpret_cast<uint32_t*>(slot(l, e)) = v[j];
+        }
+    }
+    __syncwarp();                                         // a warp reads back only what it staged
+    gi = g0 + t;
+    if (gi >= a.total_groups) return;
+    uint32_t w[kChunks * 4];
+    const int swz = BF16 ? ((t >> 1) & kSwzMask) : (t & kSwzMask);
+#pragma unroll
+    for (int p = 0; p < kChunks; ++p) {
+        const uint4 v = tile[t * kChunks + (p ^ swz)];
+        w[4 * p + 0] = v.x; w[4 * p + 1] = v.y; w[4 * p + 2] = v.z; w[4 * p + 3] = v.w;
+    }
+    process_group<BF16, KZR, KB>(w, a, gi);
+}
+
+template <bool BF16>
+cudaError_t launch_ragged(const ActArgs& a, cudaStream_t st) {
+    const dim3 grid((unsigned)((a.total_groups + kFastThreads - 1) / kFastThreads)), block(kFastThreads);
+    const int32_t pairs_ok = reinterpret_cast<uintptr_t>(a.x) % 4 == 0 && a.row_stride % 2 == 0;
+    // the paper's ranks have an instance of their own, every other pair shares the one with run-time ranks
+    if (a.k_base == 32 && a.k_zr == 7) return launch_pdl(act_g32_ragged_kernel<BF16, 7, 32>, grid, block, 0, st, a, pairs_ok);
+    return launch_pdl(act_g32_ragged_kernel<BF16, 0, 0>, grid, block, 0, st, a, pairs_ok);
+}
+
+// ------------------------------------------------------------------------------------------
 // channel-major input: x is [B][C][H*W] (a convolutional feature map) and is quantized along C
 // without a permuted copy.  A CTA takes one group of 32 channels and 256 consecutive positions of
 // one image: the 32 channel rows are read with coalesced loads into a shared-memory tile, then
@@ -585,10 +663,14 @@ extern "C" tdq_status tdq_quantize_act(const void* x, tdq_dtype x_dtype, int64_t
     cudaStream_t stream = reinterpret_cast<cudaStream_t>(cuda_stream);
     cudaError_t e;
     const bool out_aligned = reinterpret_cast<uintptr_t>(codes) % 16 == 0;
-    if (out_aligned && act_fast_path_ok(x, x_dtype, C, row_stride_elems, p) &&
-        a.total_groups / kFastThreads < INT32_MAX) {
+    if (out_aligned && g == 32 && a.total_groups / kFastThreads < INT32_MAX) {
         if (!(a.flags & TDQ_ENABLE_C2)) a.k_zr = 7;   // rank unused; pick an instantiated kernel
-        e = (x_dtype == TDQ_BF16) ? launch_fast<true>(a, stream) : launch_fast<false>(a, stream);
+        if (act_fast_path_ok(x, x_dtype, C, row_stride_elems, p))
+            e = (x_dtype == TDQ_BF16) ? launch_fast<true>(a, stream) : launch_fast<false>(a, stream);
+        else
+            e = (x_dtype == TDQ_BF16) ? launch_ragged<true>(a, stream) : launch_ragged<false>(a, stream);
+    } else if (act_wide_ok(a)) {
+        e = launch_act_wide(a, x_dtype == TDQ_BF16, stream);
     } else {
         const size_t smem = (size_t)kGenericWarps * g * sizeof(float);
         int64_t blocks = (a.total_groups + kGenericWarps - 1) / kGenericWarps;

@@ -1,0 +1,52 @@
+"""The quantizer kernel for wide groups and unaligned rows at the edges of its instances: every width at which the lanes
+per group or the chunks per lane change, remainders of a row, every load width, both ranks, ties and zeros."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth_inputs as si
+from parity_utils import compare_quantizer, to_cuda
+
+pytestmark = pytest.mark.gpu
+
+
+def _rows(rng, M, C):
+    x = si.token_mixture(rng, 1, M, C, sigma_log_std=0.5, bg_frac=0.1, bg_nu=3.0, bg_amp=20.0).reshape(M, C)
+    x[1::7] += 3.0                                          # the dispersion bound is the minimum
+    x[2::7] = np.maximum(x[2::7] - 0.8, 0.0)                # more zeros than the zero-bin rank
+    x[3::7] = np.round(x[3::7] * 4.0) / 4.0                 # ties
+    x[4] = 0.0
+    x[5] = np.where(np.arange(C) % 3 == 0, 1e-9, -2e-9)     # below the floors
+    x[6, ::5] = 3e4
+    return x
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("g", [8, 24, 32, 40, 64, 72, 96, 104, 128, 136, 192, 200, 256, 264, 384, 392, 512, 520, 768, 776,
+                               1024, 1032, 1536, 1544, 2048, 2056, 3072, 3080, 4096])
+def test_widths_and_remainders(g, bf16):
+    from paper_2604_16855_b200 import tdq
+    rng = np.random.default_rng(g)
+    for C, offset in ((2 * g, 0), (2 * g + 13, 0), (g + 6, 2), (max(g - 3, 5), 1)):   # offset: first channel of a wider matrix
+        full = _rows(rng, 23, C + offset + 3)
+        full = si.f32_to_bf16_bits(full) if bf16 else full
+        x = np.ascontiguousarray(full[:, offset:offset + C])
+        for kw in (dict(), dict(p=0.9, zr=0.5), dict(tau=0.4, zr=0.05, flags=7)):
+            ref = oracle.quantize_act(x, g=g, **kw)
+            params = tdq.act_params(g=g, tau=kw.get("tau", 1.0), zr=kw.get("zr", 0.2), p=kw.get("p", 1.0), flags=kw.get("flags", 3))
+            codes, scale = tdq.quantize_act(to_cuda(full, bf16=bf16)[:, offset:offset + C], params)
+            rep = compare_quantizer(si.bf16_bits_to_f32(x) if bf16 else x, g, ref, codes.cpu().numpy(), scale.cpu().numpy())
+            assert rep["scale_max_rel"] <= 1e-6, (C, offset, kw, rep)
+
+
+def test_many_groups():
+    """More than one wave of blocks, a last warp that is only partly filled, offsets written."""
+    from paper_2604_16855_b200 import tdq
+    rng = np.random.default_rng(5)
+    x = si.f32_to_bf16_bits(_rows(rng, 9001, 192))
+    ref = oracle.quantize_act(x, g=64)
+    off = torch.full((9001, 3), 7.0, device="cuda")
+    codes, scale = tdq.quantize_act(to_cuda(x, bf16=True), tdq.act_params(g=64), offset=off)
+    assert np.array_equal(codes.cpu().numpy(), ref["codes"]) and np.array_equal(scale.cpu().numpy(), ref["scale"])
+    assert float(off.abs().max()) == 0.0
