@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1) w4a4_gemm_kernel(const LinArgs a,
     const uint32_t ibuf_s = sm_s + kCtrlBytes;
     const uint32_t a_in_ibuf = (uint32_t)a.Kg * kScaleBlock;
     const uint32_t ring_s = sm_s + a.ring_off;
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int t = threadIdx.x, warp = uniform_warp(), lane = t & 31;
     const bool resident = a.a_resident != 0;
 
     if (t == 0) {

@@ -38,12 +38,6 @@ constexpr int kPWarps = 8;
 constexpr int kPCols = kBN / (kPWarps / 4);                 // 64 columns of one row per promotion thread
 constexpr int kThreadsG32 = (kCtlWarps + kPWarps) * 32;     // 512
 constexpr int kRegsCtl = 40, kRegsP = 208;                  // 256 * 40 + 256 * 208 <= 65536
-#ifndef TDQ_ACC_SWAP
-#define TDQ_ACC_SWAP 0
-#endif
-// Which accumulator pair takes which column pair of a landing buffer (pair q goes to accumulator q ^ kAccSwap):
-// a packed multiply-add whose accumulator and multiplicand pairs sit in the same register banks issues at half rate.
-constexpr int kAccSwap = TDQ_ACC_SWAP;
 constexpr uint32_t kBoxF32 = 128 * 128, kBoxBF16 = 128 * 64;   // one 32-column box of 128 rows in the staging area
 static_assert(2 * kBN * 4 <= kWsbBytes, "the tile's channel scales and biases outgrew their reservation");
 static_assert(4 * kBoxF32 <= kStagingBytes, "the staged tile outgrew its reservation");
@@ -82,7 +76,7 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
     const uint32_t a_in_ibuf = (uint32_t)a.Kg * kScaleBlock;
     const uint32_t ring_s = sm_s + a.ring_off;
     const uint32_t stage_s = (sm_s + a.staging_off + 1023u) & ~1023u;   // the swizzle patterns repeat every 1024 bytes
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int t = threadIdx.x, warp = uniform_warp(), lane = t & 31;
     const bool resident = a.a_resident != 0;
 
     if (t == 0) {
@@ -191,7 +185,6 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
                     uint32_t a_lo = ares_lo + off_me;   // resident: walks through the item's A blocks
 #pragma unroll 1
                     for (int k0 = 0; k0 < n_steps; k0 += kChunk) {
-                        const uint32_t act = (k0 + (int)me < n_steps) ? lane0 : 0u;
                         wait_hot(full_s + s * 8, ph, c, a.status, 4u);
                         const uint32_t b_lo = ring_lo + s * stage_step + off_me;
                         if (k0 + (int)me < n_steps) {
@@ -199,9 +192,14 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
                             q_me ^= 1u;
                         }
                         tc_fence_after();
-                        mma_issue_if<false>(act, tm_me, resident ? a_lo : b_lo + a_in_stage, b_lo, 0u);
-                        mma_commit_if(act, tfull_me);
-                        mma_commit_if(lane0, empty_s + s * 8);
+                        if (elect_one()) {
+                            if (k0 + (int)me < n_steps) {
+                                mma_f8_fresh(tm_me, desc_of(resident ? a_lo : b_lo + a_in_stage), desc_of(b_lo), kIdescF8);
+                                mma_commit(tfull_me);
+                            }
+                            mma_commit(empty_s + s * 8);
+                        }
+                        __syncwarp();
                         a_lo += kChunk * (kBlock >> 4);
                         if (++s == n_stages) { s = 0; ph ^= 1; }
                     }
@@ -356,8 +354,8 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
                             float o0, o1, o2, o3;
-                            unpack2(yacc[16 * hh + ((2 * j) ^ kAccSwap)], o0, o1);
-                            unpack2(yacc[16 * hh + ((2 * j + 1) ^ kAccSwap)], o2, o3);
+                            unpack2(yacc[16 * hh + (2 * j)], o0, o1);
+                            unpack2(yacc[16 * hh + (2 * j + 1)], o2, o3);
                             o0 = __fmaf_rn(s4[j].x, o0, b4[j].x);
                             o1 = __fmaf_rn(s4[j].y, o1, b4[j].y);
                             o2 = __fmaf_rn(s4[j].z, o2, b4[j].z);
@@ -370,10 +368,10 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {       // eight columns = one 16-byte chunk of bf16
                             float o[8];
-                            unpack2(yacc[16 * hh + ((4 * j) ^ kAccSwap)], o[0], o[1]);
-                            unpack2(yacc[16 * hh + ((4 * j + 1) ^ kAccSwap)], o[2], o[3]);
-                            unpack2(yacc[16 * hh + ((4 * j + 2) ^ kAccSwap)], o[4], o[5]);
-                            unpack2(yacc[16 * hh + ((4 * j + 3) ^ kAccSwap)], o[6], o[7]);
+                            unpack2(yacc[16 * hh + (4 * j)], o[0], o[1]);
+                            unpack2(yacc[16 * hh + (4 * j + 1)], o[2], o[3]);
+                            unpack2(yacc[16 * hh + (4 * j + 2)], o[4], o[5]);
+                            unpack2(yacc[16 * hh + (4 * j + 3)], o[6], o[7]);
                             const float4 sa = s4[2 * j], sb = s4[2 * j + 1], ba = b4[2 * j], bb = b4[2 * j + 1];
                             sts128(row_s + (((uint32_t)j ^ (((uint32_t)lane >> 1) & 3u)) << 4),
                                    pack16(__fmaf_rn(sa.x, o[0], ba.x), __fmaf_rn(sa.y, o[1], ba.y), a.y_f16),
@@ -431,7 +429,7 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
                 if (a.acc_debug && m < a.M) debug_store<false>(a, va, m, n0, k + (int)U);
             }
 #pragma unroll
-            for (int q = 0; q < 16; ++q) fma2(yacc[q ^ kAccSwap], pack2(va[2 * q], va[2 * q + 1]), d2);
+            for (int q = 0; q < 16; ++q) fma2(yacc[q], pack2(va[2 * q], va[2 * q + 1]), d2);
             tmem_ld_wait_on(vb);
             tc_fence_before();                            // the slot is drained
             __syncwarp();
@@ -450,7 +448,7 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
                 if (a.acc_debug && m < a.M) debug_store<false>(a, vb, m, n0 + 32, k + (int)U);
             }
 #pragma unroll
-            for (int q = 0; q < 16; ++q) fma2(yacc[16 + (q ^ kAccSwap)], pack2(vb[2 * q], vb[2 * q + 1]), d2);
+            for (int q = 0; q < 16; ++q) fma2(yacc[16 + q], pack2(vb[2 * q], vb[2 * q + 1]), d2);
         };
         const std::integral_constant<uint32_t, 0> u0{};
         const std::integral_constant<uint32_t, 1> u1{};
