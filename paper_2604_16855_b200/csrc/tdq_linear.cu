@@ -86,6 +86,7 @@ struct ExpandArgs {
     int32_t row_bytes;       // I_pad / 2
     int32_t n_steps, n_chunks, steps_per_grp, Kg;
     int32_t tiles_m, tiles_n;
+    int32_t b_rows;          // rows per block of B: 128, or 64 for narrower tiles
     uint32_t* status;        // the workspace's status words, cleared here for the GEMM that follows
 };
 
@@ -122,7 +123,11 @@ __global__ void __launch_bounds__(kExpandThreads) expand_kernel(ExpandArgs a) {
     expand8<I8>(p.z, c1.x, c1.y);
     expand8<I8>(p.w, c1.z, c1.w);
     uint8_t* dst = (is_a ? a.a_blocks : a.b_blocks) + ((int64_t)tile * a.n_steps + ks) * kBlock;
-    const int off = (r >> 3) * 256 + (r & 7) * 16;
+    int off = (r >> 3) * 256 + (r & 7) * 16;
+    if (!is_a && a.b_rows == 64) {                         // [64 rows][n_steps] blocks of half the size
+        dst = a.b_blocks + ((int64_t)(2 * tile + (r >> 6)) * a.n_steps + ks) * (kBlock / 2);
+        off = ((r & 63) >> 3) * 256 + (r & 7) * 16;
+    }
     *reinterpret_cast<uint4*>(dst + off) = c0;
     *reinterpret_cast<uint4*>(dst + off + 128) = c1;
     if (is_a && ks % a.steps_per_grp == 0) {
@@ -1145,8 +1150,10 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     // Output strips: 64-byte rows (32 KB in all) for bf16 output, and for fp32 output of wide groups, which is
     // then written in two passes of 16 columns; the ring gets the other 32 KB.  Both need the bulk tensor store.
     const int64_t y_esz = y_dtype == TDQ_BF16 ? 2 : 4;
-    const bool y_tma = reinterpret_cast<uintptr_t>(y) % 16 == 0 && (y_row_stride * y_esz) % 16 == 0 && O <= INT32_MAX &&
-                       M <= INT32_MAX;
+    // (The copy engine clips at the edges of y in whole 16-byte pieces: a last column off that grid, in a y with a padded
+    // row pitch, would have zeros written behind it.)
+    const bool y_tma = reinterpret_cast<uintptr_t>(y) % 16 == 0 && (y_row_stride * y_esz) % 16 == 0 && (O * y_esz) % 16 == 0 &&
+                       O <= INT32_MAX && M <= INT32_MAX;
     const bool half_strips = y_tma && y_dtype == TDQ_F32 && !fx && !acc_debug && group_size >= 128;
     const bool narrow_strips = y_tma && (y_dtype == TDQ_BF16 || half_strips);
     // several instructions chain into one slot: keep the integer accumulator (the power-of-two variant
@@ -1193,9 +1200,15 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     // workspace; its promotion warps do that at the start of an item, though, with the tensor core idle,
     // so it only pays when an item carries much more work than its own unpacking.
     const int64_t steps_per_item = (p.tiles_n + p.n_parts - 1) / p.n_parts * (int64_t)p.n_steps;
-    const bool unpack_a = !fx && !pow2_steps && p.a_resident && steps_per_item >= 256;
+    // g = 32 goes to the kernels built for it.  Two blocks per SM with narrow tiles (tdq_linear_g32_pair.cu) win up to about
+    // 1536 channels (16384 x 1024 -> 2048 86.6 against 92.7 us, 2048 channels 158 against 156) and whenever wide tiles would
+    // leave most SMs idle (1152 x 2048 -> 512 13.9 against 16.0 us), and they also take a y that tensor stores cannot write.
+    const bool use_g32 = group_size == 32 && !pow2_steps && !fx && p.tiles_m * p.tiles_n <= INT32_MAX / 4;
+    const bool use_pair = use_g32 && (!y_tma || p.n_steps <= 48 || p.tiles_m * p.tiles_n * 4 <= n_sm);
+    const bool unpack_a = !fx && !pow2_steps && !use_pair && p.a_resident && steps_per_item >= 256;
     e.tiles_m = (fx || unpack_a) ? 0 : (int32_t)p.tiles_m;   // then only the weights are expanded here
     e.tiles_n = (int32_t)p.tiles_n;
+    e.b_rows = use_pair ? 64 : 128;
     e.status = reinterpret_cast<uint32_t*>(workspace);
 
     LinArgs a;
@@ -1215,14 +1228,13 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     CUtensorMap ymap;
     memset(&ymap, 0, sizeof(ymap));
     a.tma_ok = 0;
-    // g = 32 with y that tensor stores can write goes to the kernel built for it (tdq_linear_g32.cu)
-    const bool use_g32 = group_size == 32 && !pow2_steps && !fx && y_tma;
     if (y_tma && encode_y_map(&ymap, y, y_dtype == TDQ_BF16, M, O, y_row_stride,
                               quarter_strips ? (y_dtype == TDQ_BF16 ? kCols / 2 : kCols / 4) : half_strips ? kCols / 2 : kCols,
                               use_g32 ? kBM : 32, y_f16))
         a.tma_ok = 1;
     else if (narrow_strips || quarter_strips)
         return TDQ_ERR_CUDA;   // the plan counted on the tensor store
+    a.y_words = reinterpret_cast<uintptr_t>(y) % 4 == 0 && y_row_stride % 2 == 0 ? 1 : 0;
     a.staging_bytes = (uint32_t)staging_bytes;
     a.half_strips = quarter_strips ? 2 : half_strips ? 1 : 0;
     a.out_scale = i8 ? 0.00390625f : 262144.0f;
@@ -1265,6 +1277,10 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
 
     const int64_t items = p.tiles_m * p.n_parts;
     const unsigned grid = (unsigned)(items < n_sm ? items : n_sm);
+    if (use_pair) {
+        a.tiles_n = (int32_t)((O + 63) / 64);
+        return launch_linear_g32_pair(a, ymap, n_sm, dev, ybf, dbg, stream);
+    }
     if (use_g32 && a.tma_ok) return launch_linear_g32(a, ymap, p.smem_bytes, grid, ybf, dbg, stream);
     if (launch_pdl(kernel, dim3(grid), dim3(kThreads), p.smem_bytes, stream, a, ymap) != cudaSuccess) return TDQ_ERR_CUDA;
     g_launch_count.fetch_add(1, std::memory_order_relaxed);

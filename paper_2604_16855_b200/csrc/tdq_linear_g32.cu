@@ -1,5 +1,6 @@
 // The W4A4 linear layer at the paper's group size g = 32 (Algorithm S1 step 10 with Eq. 9 and Eq. 4
-// substituted), with y that bulk tensor stores can write (16-byte aligned base and row pitch):
+// substituted) for long contractions, with y that bulk tensor stores can write (16-byte aligned base and row pitch); shorter
+// ones go to tdq_linear_g32_pair.cu:
 //
 //   acc[m,o,k] = sum_{i in group k} q_x[m,i] q_w[o,i]      one tcgen05.mma (E4M3 operands, exact) per group
 //   y[m,o]     = s_o * sum_k Delta[m,k] * acc[m,o,k] + b_o  fp32 in registers ("promotion")

@@ -1,0 +1,448 @@
+// The W4A4 linear layer at the paper's group size g = 32 for contractions of up to about 1536 channels (Algorithm S1 step 10
+// with Eq. 9 and Eq. 4 substituted), and of any length where y is not one that bulk tensor stores can write.
+// The arithmetic is tdq_linear_g32.cu's, bit for bit:
+//
+//   acc[m,o,k] = sum_{i in group k} q_x[m,i] q_w[o,i]      one tcgen05.mma (E4M3 operands, exact) per group
+//   y[m,o]     = s_o * sum_k Delta[m,k] * acc[m,o,k] + b_o  fp32 in registers ("promotion")
+//
+// What bounds it.  Every K-step of the tensor core ends an accumulator.  Per 128 x 128 group the SM needs 64 clocks of
+// tensor time, 64 of TMEM reads (1 KB per clock) and about 145 of its FMA pipes (packed multiply-adds at 1.13 clocks an
+// element and scheduler), and TMEM holds four such groups, each of which spends most of its stay in signalling (arrival to
+// MMA warp, issue, commit to barrier, notice, load: about 800 clocks).  One block per SM with all of TMEM
+// (tdq_linear_g32.cu) adds to that, per tile, everything the epilogue takes, because nothing is promoted meanwhile: a
+// third of a 768-channel tile, nearly all of a 64-channel one.
+//
+// So: two thread blocks per SM, each with half of TMEM, that drift against each other: one's loads, waits, epilogue and
+// output run under the other's multiply-adds.  A block is persistent, works on 128 x 64 tiles and takes a tile's groups two
+// at a time, a pair of 64-column slots with one barrier each way, since the handshake and not the data is what costs (a
+// barrier per slot: 7 % slower):
+//
+//   warp 0      producer: operand blocks and steps Delta of 4 groups (16 KB of A, 8 KB of B, 2 KB) through a ring of stages
+//   warps 1-2   MMA issue, one pair of slots each
+//   warp 3      stores: starts a staged tile's bulk tensor stores, hands the area back when the engine has read it,
+//               and fetches the next tile's channel constants meanwhile
+//   warps 4-7   promotion and epilogue: warp = 32 TMEM lanes (rows), all 64 columns: 64 float sums, 128 landing registers
+//
+// Measured against the other kernel (us; with the operand expansion): 73728 x 64 -> 64 fp32 16.2 -> 11.0, 73728 x 64 -> 192
+// 25.0 -> 18.0, 9216 x 64 -> 256 8.4 -> 7.2, 16384 x 512 -> 2048 bf16 63.8 -> 51.4, 16384 x 1024 -> 2048 92.7 -> 86.6,
+// 18464 x 768 -> 3072 fp32 119.7 -> 115.4; from 2048 channels on the other one is 1-9 % faster (narrower tiles read A twice
+// as often and the older of an SM's two blocks runs an eighth faster than the other).
+#include "tdq_tc.cuh"
+
+namespace tdq {
+namespace {
+
+constexpr int kN = 64;                       // columns per tile = one TMEM slot
+constexpr int kBHalf = kN * 32;              // operand bytes of 64 rows of B and one K-step
+constexpr int kPairThreads = 256;
+constexpr int kPairStages = 3;
+constexpr uint32_t kPairScales = kChunk * (kBlock + kBHalf);   // offset of a stage's scales: 4 groups x 128 rows
+constexpr uint32_t kPairStageBytes = kPairScales + kChunk * kScaleBlock;
+constexpr uint32_t kPairCtrl = 512;
+constexpr int kProducerWarp = 0, kFirstMmaWarp = 1, kPairStoreWarp = 3, kFirstPromoWarp = 4, kPairPromoWarps = 4;
+constexpr int kRegsPairCtl = 40, kRegsPairPromo = 216;     // 128 * 40 + 128 * 216 = 256 * 128
+constexpr uint32_t kIdescN64 = (1u << 4) | ((uint32_t)(kN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
+constexpr uint32_t kPairBoxF32 = 128 * 128, kPairBoxBF16 = 128 * 64;   // one 32-column box of 128 rows in the staging area
+
+struct PairCtrl {
+    uint64_t full[kPairStages], empty[kPairStages];
+    uint64_t tfull[2], tempty[2];            // per pair of slots
+    uint64_t sfull, sfree;                   // the staged output tile is complete / has been read by the copy engine
+};
+static_assert(sizeof(Ctrl) + sizeof(PairCtrl) <= kPairCtrl, "control block outgrew its reservation");
+
+__device__ __forceinline__ void tmem_ld_wait_on(uint32_t* v) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                   "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]),
+                   "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
+                   "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
+                 :
+                 : "memory");
+}
+
+__device__ __forceinline__ void wait_cold(uint32_t bar_s, uint32_t parity, Ctrl* c, uint32_t* status, uint32_t code) {
+    uint64_t* bar = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(c) + (bar_s - smem_u32(c)));
+    mbar_wait_slow(bar, parity, c, status, code);
+}
+__device__ __forceinline__ void wait_hot(uint32_t bar_s, uint32_t parity, Ctrl* c, uint32_t* status, uint32_t code) {
+    if (!mbar_test_s(bar_s, parity)) wait_cold(bar_s, parity, c, status, code);
+}
+
+template <bool YBF16, bool DBG>
+__global__ void __launch_bounds__(kPairThreads, 2) w4a4_g32_pair_kernel(const LinArgs a, const __grid_constant__ CUtensorMap ymap) {
+    extern __shared__ __align__(128) uint8_t smem_raw[];
+    Ctrl* c = reinterpret_cast<Ctrl*>(smem_raw);            // its abort flag and TMEM address; the barriers are g's
+    PairCtrl* g = reinterpret_cast<PairCtrl*>(smem_raw + sizeof(Ctrl));
+    const uint32_t sm_s = smem_u32(smem_raw);
+    const uint32_t ring_s = sm_s + kPairCtrl;
+    const uint32_t stage_s = (ring_s + kPairStages * kPairStageBytes + 1023u) & ~1023u;   // the swizzle patterns repeat every 1024 bytes
+    const uint32_t wsb_s = stage_s + (YBF16 ? 2 * kPairBoxBF16 : 2 * kPairBoxF32);   // [64] channel scales, [64] biases of the current tile
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kPairStages; ++i) { mbar_init(&g->full[i], 1); mbar_init(&g->empty[i], 2 + kPairPromoWarps); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&g->tfull[i], 1); mbar_init(&g->tempty[i], kPairPromoWarps); }
+        mbar_init(&g->sfull, kPairPromoWarps);
+        mbar_init(&g->sfree, 1);
+        c->abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == kFirstMmaWarp) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&c->tmem_base)),
+                     "r"(kSlots * kN)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    pdl_wait();          // barrier set-up and the TMEM allocation overlap the tail of the kernel before this one
+    pdl_trigger();
+    const uint32_t tmem_base = c->tmem_base;
+    const int n_tiles = a.tiles_m * a.tiles_n;
+    const int n_steps = a.n_steps;
+
+    if (warp < kFirstPromoWarp) {
+        setmaxnreg_dec<kRegsPairCtl>();
+        if (warp == kProducerWarp) {
+            // ------------------------------------------------------------ operand blocks
+            const uint32_t empty_s = smem_u32(&g->empty[0]);
+            uint32_t s = 0, ph = 1;
+            for (int tile = blockIdx.x; tile < n_tiles && !c->abort_flag; tile += gridDim.x) {
+                const int mt = tile / a.tiles_n, nt = tile - mt * a.tiles_n;
+                const uint8_t* a_src = a.a_blocks + (int64_t)mt * n_steps * kBlock;
+                const uint8_t* b_src = a.b_blocks + (int64_t)nt * n_steps * kBHalf;
+                const uint8_t* s_src = a.s_blocks + (int64_t)mt * n_steps * kScaleBlock;
+#pragma unroll 1
+                for (int k0 = 0; k0 < n_steps; k0 += kChunk) {
+                    const uint32_t nk = (uint32_t)min(kChunk, n_steps - k0);
+                    wait_hot(empty_s + s * 8, ph, c, a.status, 5u);
+                    if (c->abort_flag) break;
+                    if (elect_one()) {
+                        const uint32_t st = ring_s + s * kPairStageBytes;
+                        mbar_expect_tx(&g->full[s], nk * (kBlock + kBHalf + kScaleBlock));
+                        bulk_load(st, a_src, nk * kBlock, &g->full[s]);
+                        bulk_load(st + kChunk * kBlock, b_src, nk * kBHalf, &g->full[s]);
+                        bulk_load(st + kPairScales, s_src, nk * kScaleBlock, &g->full[s]);
+                    }
+                    __syncwarp();
+                    a_src += kChunk * kBlock;
+                    b_src += kChunk * kBHalf;
+                    s_src += kChunk * kScaleBlock;
+                    if (++s == kPairStages) { s = 0; ph ^= 1; }
+                }
+            }
+        } else if (warp < kPairStoreWarp) {
+            // ------------------------------------------------------------ MMA issue
+            // Warp `me` owns slots 2 me and 2 me + 1: of every stage it issues steps 2 me and 2 me + 1 and reports them with
+            // one commit.
+            const uint32_t me = (uint32_t)(warp - kFirstMmaWarp);
+            const uint32_t full_s = smem_u32(&g->full[0]), empty_s = smem_u32(&g->empty[0]);
+            const uint32_t tfull_s = smem_u32(&g->tfull[me]), tempty_s = smem_u32(&g->tempty[me]);
+            const uint32_t tm = tmem_base + 2 * me * kN;
+            const uint32_t a_lo = desc_lo(ring_s) + 2 * me * (kBlock >> 4);
+            const uint32_t b_lo = desc_lo(ring_s + kChunk * kBlock) + 2 * me * (kBHalf >> 4);
+            uint32_t s = 0, ph = 0;
+            uint32_t q = 1;                      // parity to wait for on tempty; a fresh barrier passes parity 1
+            for (int tile = blockIdx.x; tile < n_tiles && !c->abort_flag; tile += gridDim.x) {
+#pragma unroll 1
+                for (int k0 = 0; k0 < n_steps; k0 += kChunk) {
+                    const int mine = n_steps - k0 - 2 * (int)me;         // steps left from this warp's first one on
+                    const uint32_t so = s * (kPairStageBytes >> 4);
+                    const bool rf = mbar_test_s(full_s + s * 8, ph);     // the two tests are in flight together
+                    const bool rt = mbar_test_s(tempty_s, q);
+                    if (!rf) wait_cold(full_s + s * 8, ph, c, a.status, 4u);
+                    if (mine > 0) {
+                        if (!rt) wait_cold(tempty_s, q, c, a.status, 3u);
+                        q ^= 1u;
+                        tc_fence_after();
+                        if (elect_one()) {
+                            mma_f8_fresh(tm, desc_of(a_lo + so), desc_of(b_lo + so), kIdescN64);
+                            if (mine > 1) mma_f8_fresh(tm + kN, desc_of(a_lo + so + (kBlock >> 4)), desc_of(b_lo + so + (kBHalf >> 4)), kIdescN64);
+                            mma_commit(tfull_s);
+                            mma_commit(empty_s + s * 8);
+                        }
+                    } else if (elect_one()) {
+                        mma_commit(empty_s + s * 8);
+                    }
+                    __syncwarp();
+                    if (++s == kPairStages) { s = 0; ph ^= 1; }
+                }
+            }
+        } else {
+            // ------------------------------------------------------------ output stores, channel constants
+            // A staged tile is two boxes of 32 columns x 128 rows; the copy engine clips them at the edges of y.
+            // The staging area goes back to the promotion warps when the engine has read it.  The same hand-over
+            // carries the next tile's channel scales (times the accumulator's power of two) and biases: phase n of
+            // `sfree` says that tile n of this CTA may be staged and that its constants are in place.
+            constexpr uint32_t box_bytes = YBF16 ? kPairBoxBF16 : kPairBoxF32;
+            float* wsb = reinterpret_cast<float*>(smem_raw + (wsb_s - sm_s));
+            auto fetch = [&](int nt) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int64_t col = (int64_t)nt * kN + 32 * i + lane;
+                    wsb[32 * i + lane] = col < a.O ? __fmul_rn(__ldg(a.wscale + col), a.out_scale) : 0.f;
+                    wsb[kN + 32 * i + lane] = (a.bias && col < a.O) ? __ldg(a.bias + col) : 0.f;
+                }
+                __syncwarp();
+            };
+            uint32_t sph = 0;
+            if ((int)blockIdx.x < n_tiles) {
+                fetch((int)blockIdx.x % a.tiles_n);
+                mbar_arrive_lane0(&g->sfree, lane);
+            }
+            for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+                const int mt = tile / a.tiles_n, nt = tile - mt * a.tiles_n;
+                wait_hot(smem_u32(&g->sfull), sph, c, a.status, 8u);
+                if (c->abort_flag) break;
+                sph ^= 1u;
+                if (lane == 0 && a.tma_ok) {
+                    const int64_t n0 = (int64_t)nt * kN;
+#pragma unroll
+                    for (int cb = 0; cb < 2; ++cb)
+                        if (n0 + 32 * cb < a.O)
+                            tma_store_2d(&ymap, stage_s + (uint32_t)cb * box_bytes, (int32_t)n0 + 32 * cb, mt * kBM);
+                    bulk_commit_group();
+                }
+                const int next = tile + (int)gridDim.x;
+                if (next < n_tiles) fetch(next % a.tiles_n);
+                if (lane == 0) bulk_wait_group_read0();
+                __syncwarp();
+                mbar_arrive_lane0(&g->sfree, lane);
+            }
+            if (lane == 0) bulk_wait_group0();   // no store may still be reading this CTA's shared memory at exit
+        }
+    } else {
+        setmaxnreg_inc<kRegsPairPromo>();
+        // ------------------------------------------------------------ promotion + epilogue
+        const int quarter = warp & 3;                 // TMEM lanes 32 * quarter .. + 31
+        const int row = quarter * 32 + lane;
+        uint64_t yacc[kN / 2];                        // 64 floats of one output row, packed in pairs
+        uint32_t va[32], vb[32], vc[32], vd[32];      // landing buffers: columns 0-31 and 32-63 of an even and of an odd slot
+#pragma unroll
+        for (int q = 0; q < 32; ++q) { va[q] = 0u; vb[q] = 0u; vc[q] = 0u; vd[q] = 0u; }
+        uint32_t p_full = 0u;                         // bit p: parity of the completion of tfull[p] to wait for next
+        uint32_t sf_par = 0u;                         // parity to wait for on sfree
+        uint32_t rs = 0, rph = 0;                     // ring stage and its phase
+        int tile = blockIdx.x, mt = 0, nt = 0;
+        uint32_t tfull_s = smem_u32(&g->tfull[0]), tempty_s = smem_u32(&g->tempty[0]);
+        const uint32_t full_s = smem_u32(&g->full[0]), empty_s = smem_u32(&g->empty[0]);
+        uint32_t tmem_row = tmem_base + ((uint32_t)(quarter * 32) << 16);
+        // opaque to the compiler: kept in registers instead of being recomputed from the thread index at every use
+        asm volatile("" : "+r"(tfull_s), "+r"(tempty_s), "+r"(tmem_row));
+
+        auto wait_pair = [&](uint32_t p, bool ready) {
+            if (!ready) wait_cold(tfull_s + p * 8, (p_full >> p) & 1u, c, a.status, 2u);
+            p_full ^= 1u << p;
+            tc_fence_after();
+        };
+        auto load_lo = [&](uint32_t slot) { tmem_ld32(tmem_row + slot * kN, va); tmem_ld32(tmem_row + slot * kN + 32, vb); };
+        auto load_hi = [&](uint32_t slot) { tmem_ld32(tmem_row + slot * kN, vc); tmem_ld32(tmem_row + slot * kN + 32, vd); };
+        auto fold = [&](const uint32_t* x, const uint32_t* z, uint32_t dbits) {
+            const uint64_t d2 = pack2(dbits, dbits);
+#pragma unroll
+            for (int q = 0; q < 16; ++q) fma2(yacc[q], pack2(x[2 * q], x[2 * q + 1]), d2);
+#pragma unroll
+            for (int q = 0; q < 16; ++q) fma2(yacc[16 + q], pack2(z[2 * q], z[2 * q + 1]), d2);
+        };
+        auto debug = [&](const uint32_t* x, const uint32_t* z, int k) {
+            const int64_t m = (int64_t)mt * kBM + row;
+            if (a.acc_debug && m < a.M) {
+                debug_store<false>(a, x, m, (int64_t)nt * kN, k);
+                debug_store<false>(a, z, m, (int64_t)nt * kN + 32, k);
+            }
+        };
+        // The four steps Delta of the current ring stage for this row; then the stage is this warp's no longer.  (The
+        // stage's scales came with its operands, so they are there when the first accumulator of the stage is.)
+        uint32_t d[4];
+        auto take_steps = [&](bool ready) {
+            if (!ready) wait_cold(full_s + rs * 8, rph, c, a.status, 7u);
+            const uint32_t src = ring_s + rs * kPairStageBytes + kPairScales + (uint32_t)row * 4;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) d[j] = lds32(src + j * kScaleBlock);
+        };
+        auto leave_stage = [&]() {
+            // read through the generic proxy, refilled through the async proxy: only a proxy fence orders the two
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            mbar_arrive_lane0_s(empty_s + rs * 8, lane);
+            if (++rs == kPairStages) { rs = 0; rph ^= 1; }
+        };
+
+        // A tile's groups are taken two at a time (a pair of slots): wait for the pair's landing, hand both slots back
+        // with one arrival, fold the first group in, start the next pair's first load into the registers that frees, fold
+        // the second, start the second load.
+        if (tile < n_tiles) {
+            mt = tile / a.tiles_n;
+            nt = tile - mt * a.tiles_n;
+            wait_pair(0, mbar_test_s(tfull_s, p_full & 1u));
+            load_lo(0);
+            if (n_steps > 1) load_hi(1);
+            take_steps(mbar_test_s(full_s, 0u));
+#pragma unroll 1
+            while (!c->abort_flag) {
+                // one tile; the load of its first pair is in flight, its first steps are in d
+#pragma unroll
+                for (int j = 0; j < kN / 2; ++j) yacc[j] = 0ull;
+                const int next = tile + (int)gridDim.x;
+                const bool another = next < n_tiles;
+                int left = n_steps;                       // groups not yet folded in
+#pragma unroll 1
+                for (;;) {
+                    // first pair of the stage: slots 0 and 1
+                    const bool second = left > 2;         // the stage has another pair
+                    bool r1 = true;
+                    if (second) r1 = mbar_test_s(tfull_s + 8, (p_full >> 1) & 1u);
+                    tmem_ld_wait_on(va); tmem_ld_wait_on(vb); tmem_ld_wait_on(vc); tmem_ld_wait_on(vd);
+                    tc_fence_before();
+                    __syncwarp();
+                    mbar_arrive_lane0_s(tempty_s, lane);
+                    if (DBG) { debug(va, vb, n_steps - left); if (left > 1) debug(vc, vd, n_steps - left + 1); }
+                    fold(va, vb, d[0]);
+                    if (second) { wait_pair(1, r1); load_lo(2); }
+                    leave_stage();
+                    if (left > 1) fold(vc, vd, d[1]);
+                    if (!second) break;
+                    if (left > 3) load_hi(3);
+                    // second pair: slots 2 and 3
+                    const bool more = left > 4;
+                    bool r0 = true, rf = true;
+                    if (more) {
+                        r0 = mbar_test_s(tfull_s, p_full & 1u);
+                        rf = mbar_test_s(full_s + rs * 8, rph);
+                    }
+                    tmem_ld_wait_on(va); tmem_ld_wait_on(vb); tmem_ld_wait_on(vc); tmem_ld_wait_on(vd);
+                    tc_fence_before();
+                    __syncwarp();
+                    mbar_arrive_lane0_s(tempty_s + 8, lane);
+                    if (DBG) { debug(va, vb, n_steps - left + 2); if (left > 3) debug(vc, vd, n_steps - left + 3); }
+                    fold(va, vb, d[2]);
+                    if (more) { wait_pair(0, r0); load_lo(0); }
+                    if (left > 3) fold(vc, vd, d[3]);
+                    if (!more) break;
+                    if (left > 5) load_hi(1);
+                    take_steps(rf);
+                    left -= 4;
+                }
+                if (another) {                            // the next tile's first pair lands under the epilogue
+                    wait_pair(0, mbar_test_s(tfull_s, p_full & 1u));
+                    load_lo(0);
+                    if (n_steps > 1) load_hi(1);
+                    take_steps(mbar_test_s(full_s + rs * 8, rph));
+                }
+
+                // y = (s_o * 2^18) * sum + bias, parked as the source of the bulk tensor stores: box cb = columns
+                // 32 cb .. + 31 of all 128 rows, rows of 128 bytes whose 16-byte chunk j sits at j ^ (row & 7) (fp32), or
+                // rows of 64 bytes with chunk j at j ^ ((row >> 1) & 3) (16-bit types).
+                wait_hot(smem_u32(&g->sfree), sf_par, c, a.status, 9u);   // the previous tile's stores have read the area
+                sf_par ^= 1u;
+                const float4* wsb4 = reinterpret_cast<const float4*>(smem_raw + (wsb_s - sm_s));
+#pragma unroll
+                for (int cb = 0; cb < 2; ++cb) {
+                    const uint32_t row_s = stage_s + (uint32_t)cb * (YBF16 ? kPairBoxBF16 : kPairBoxF32) + (uint32_t)row * (YBF16 ? 64u : 128u);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {          // eight columns
+                        const float4 sa = wsb4[8 * cb + 2 * j], sb = wsb4[8 * cb + 2 * j + 1];
+                        const float4 ba = wsb4[kN / 4 + 8 * cb + 2 * j], bb = wsb4[kN / 4 + 8 * cb + 2 * j + 1];
+                        float o[8];
+                        unpack2(yacc[16 * cb + 4 * j], o[0], o[1]);
+                        unpack2(yacc[16 * cb + 4 * j + 1], o[2], o[3]);
+                        unpack2(yacc[16 * cb + 4 * j + 2], o[4], o[5]);
+                        unpack2(yacc[16 * cb + 4 * j + 3], o[6], o[7]);
+                        o[0] = __fmaf_rn(sa.x, o[0], ba.x); o[1] = __fmaf_rn(sa.y, o[1], ba.y);
+                        o[2] = __fmaf_rn(sa.z, o[2], ba.z); o[3] = __fmaf_rn(sa.w, o[3], ba.w);
+                        o[4] = __fmaf_rn(sb.x, o[4], bb.x); o[5] = __fmaf_rn(sb.y, o[5], bb.y);
+                        o[6] = __fmaf_rn(sb.z, o[6], bb.z); o[7] = __fmaf_rn(sb.w, o[7], bb.w);
+                        if (!YBF16) {
+                            const uint32_t x7 = (uint32_t)lane & 7u;
+                            sts128(row_s + (((uint32_t)(2 * j) ^ x7) << 4), __float_as_uint(o[0]), __float_as_uint(o[1]), __float_as_uint(o[2]), __float_as_uint(o[3]));
+                            sts128(row_s + (((uint32_t)(2 * j + 1) ^ x7) << 4), __float_as_uint(o[4]), __float_as_uint(o[5]), __float_as_uint(o[6]), __float_as_uint(o[7]));
+                        } else {
+                            sts128(row_s + (((uint32_t)j ^ (((uint32_t)lane >> 1) & 3u)) << 4), pack16(o[0], o[1], a.y_f16), pack16(o[2], o[3], a.y_f16),
+                                   pack16(o[4], o[5], a.y_f16), pack16(o[6], o[7], a.y_f16));
+                        }
+                    }
+                }
+                if (a.tma_ok) {
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes before the engine's reads
+                    __syncwarp();
+                } else {
+                    // y off the 16-byte grid: the warp writes its own 32 rows, a row's columns side by side (two columns a
+                    // lane where a pair of 16-bit values is one aligned word).  9217 x 160 -> 63 fp32 9.5 -> RAGGED us against
+                    // the general kernel.
+                    __syncwarp();
+                    const int64_t m0 = (int64_t)mt * kBM + quarter * 32, c0 = (int64_t)nt * kN;
+                    const int rows = (int)min((int64_t)32, a.M - m0), cols = (int)min((int64_t)kN, a.O - c0);
+                    uint8_t* out = reinterpret_cast<uint8_t*>(a.y) + (m0 * a.y_stride + c0) * (YBF16 ? 2 : 4);
+                    if (!YBF16 || a.y_words) {
+#pragma unroll 4
+                        for (int r = 0; r < rows; ++r) {
+                            const uint32_t rs_ = stage_s + (uint32_t)(quarter * 32 + r) * (YBF16 ? 64u : 128u);
+                            if (!YBF16) {
+                                const uint32_t at = rs_ + ((((uint32_t)lane >> 2) ^ ((uint32_t)r & 7u)) << 4) + ((uint32_t)lane & 3u) * 4u;
+                                float* dst = reinterpret_cast<float*>(out + r * a.y_stride * 4) + lane;
+                                if (lane < cols) dst[0] = __uint_as_float(lds32(at));
+                                if (lane + 32 < cols) dst[32] = __uint_as_float(lds32(at + kPairBoxF32));
+                            } else {
+                                const uint32_t w = (uint32_t)lane & 15u;
+                                const uint32_t at = rs_ + ((uint32_t)lane >> 4) * kPairBoxBF16 + (((w >> 2) ^ (((uint32_t)r >> 1) & 3u)) << 4) + (w & 3u) * 4u;
+                                uint32_t* dst = reinterpret_cast<uint32_t*>(out + r * a.y_stride * 2) + lane;
+                                if (2 * lane + 1 < cols) *dst = lds32(at);
+                                else if (2 * lane < cols) *reinterpret_cast<uint16_t*>(dst) = (uint16_t)lds32(at);
+                            }
+                        }
+                    } else {
+#pragma unroll 4
+                        for (int r = 0; r < rows; ++r) {
+                            const uint32_t at = stage_s + (uint32_t)(quarter * 32 + r) * 64u + ((((uint32_t)lane >> 3) ^ (((uint32_t)r >> 1) & 3u)) << 4) +
+                                                ((uint32_t)lane & 7u) * 2u;
+                            uint16_t* dst = reinterpret_cast<uint16_t*>(out + r * a.y_stride * 2) + lane;
+                            if (lane < cols) dst[0] = (uint16_t)lds16(at);
+                            if (lane + 32 < cols) dst[32] = (uint16_t)lds16(at + kPairBoxBF16);
+                        }
+                    }
+                    __syncwarp();
+                }
+                mbar_arrive_lane0(&g->sfull, lane);
+                if (!another) break;
+                tile = next;
+                mt = tile / a.tiles_n;
+                nt = tile - mt * a.tiles_n;
+            }
+        }
+        tmem_ld_wait();            // nothing may still be landing when TMEM is released
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == kFirstMmaWarp) {
+        // all MMAs this CTA issued have completed unless a wait gave up; in that case give the
+        // tensor core a moment before the columns are handed back
+        if (c->abort_flag) __nanosleep(1000000);
+        __syncwarp();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kSlots * kN) : "memory");
+    }
+}
+
+}  // namespace
+
+// a.tiles_n and a.b_blocks are in units of 64 columns here (see ExpandArgs::b_rows).
+tdq_status launch_linear_g32_pair(const LinArgs& a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, bool dbg, cudaStream_t stream) {
+    void (*kernel)(LinArgs, CUtensorMap) = nullptr;
+    if (!ybf && !dbg) kernel = w4a4_g32_pair_kernel<false, false>;
+    if (ybf && !dbg) kernel = w4a4_g32_pair_kernel<true, false>;
+    if (!ybf && dbg) kernel = w4a4_g32_pair_kernel<false, true>;
+    if (ybf && dbg) kernel = w4a4_g32_pair_kernel<true, true>;
+    const uint32_t smem = kPairCtrl + kPairStages * kPairStageBytes + 1024 + 2 * (ybf ? kPairBoxBF16 : kPairBoxF32) + 2 * kN * 4;
+    static_assert(kPairCtrl + kPairStages * kPairStageBytes + 1024 + 2 * kPairBoxF32 + 2 * kN * 4 <= 113 * 1024, "two CTAs per SM");
+    static std::atomic<uint64_t> smem_done[4];
+    if (allow_smem(kernel, 113 * 1024, smem_done[(ybf ? 1 : 0) + (dbg ? 2 : 0)], dev) != cudaSuccess) return TDQ_ERR_CUDA;
+    const int64_t tiles = (int64_t)a.tiles_m * a.tiles_n;
+    const unsigned grid = (unsigned)(tiles < 2 * n_sm ? tiles : 2 * n_sm);
+    if (launch_pdl(kernel, dim3(grid), dim3(kPairThreads), smem, stream, a, ymap) != cudaSuccess) return TDQ_ERR_CUDA;
+    g_launch_count.fetch_add(1, std::memory_order_relaxed);
+    return TDQ_OK;
+}
+
+}  // namespace tdq

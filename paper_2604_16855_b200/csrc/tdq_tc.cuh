@@ -66,6 +66,7 @@ struct LinArgs {
     int32_t* acc_debug;
     uint32_t* status;
     int32_t tma_ok;            // y can be written with bulk tensor stores (16-byte aligned base and row pitch)
+    int32_t y_words;           // without tensor stores, 16-bit y: even pitch and 4-byte aligned base, pairs can be stored
     float out_scale;           // 2^18 (E4M3 route) or 2^-8 (int8 route)
     int32_t y_f16;             // 16-bit output is fp16 (else bf16); the kernels' 16-bit instances serve both
     // resident A without the fused producer: the promotion warps unpack the item's codes themselves
@@ -101,6 +102,8 @@ struct Plan {
 };
 
 // The g = 32 kernel (tdq_linear_g32.cu); the caller has run the operand expansion and built the plan and the map.
+tdq_status launch_linear_g32_pair(const LinArgs& a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, bool dbg,
+                                  cudaStream_t stream);   // tiles of 128 x 64, tdq_linear_g32_pair.cu
 tdq_status launch_linear_g32(const LinArgs& a, const CUtensorMap& ymap, uint32_t smem_bytes, unsigned grid, bool ybf,
                              bool dbg, cudaStream_t stream);
 
