@@ -375,31 +375,44 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_g32_pair_kernel(const Li
                     const int64_t m0 = (int64_t)mt * kBM + quarter * 32, c0 = (int64_t)nt * kN;
                     const int rows = (int)min((int64_t)32, a.M - m0), cols = (int)min((int64_t)kN, a.O - c0);
                     uint8_t* out = reinterpret_cast<uint8_t*>(a.y) + (m0 * a.y_stride + c0) * (YBF16 ? 2 : 4);
-                    if (!YBF16 || a.y_words) {
-#pragma unroll 4
-                        for (int r = 0; r < rows; ++r) {
-                            const uint32_t rs_ = stage_s + (uint32_t)(quarter * 32 + r) * (YBF16 ? 64u : 128u);
+                    const uint8_t* tile_sm = smem_raw + (stage_s - sm_s) + (uint32_t)(quarter * 32) * (YBF16 ? 64u : 128u);
+                    // eight rows at a time: all their reads, then all their writes
+                    constexpr int kBatch = 8;
+#pragma unroll 1
+                    for (int r0 = 0; r0 < rows; r0 += kBatch) {
+                        uint32_t lo[kBatch], hi[kBatch];
+#pragma unroll
+                        for (int i = 0; i < kBatch; ++i) {
+                            const uint32_t r = (uint32_t)(r0 + i);
                             if (!YBF16) {
-                                const uint32_t at = rs_ + ((((uint32_t)lane >> 2) ^ ((uint32_t)r & 7u)) << 4) + ((uint32_t)lane & 3u) * 4u;
-                                float* dst = reinterpret_cast<float*>(out + r * a.y_stride * 4) + lane;
-                                if (lane < cols) dst[0] = __uint_as_float(lds32(at));
-                                if (lane + 32 < cols) dst[32] = __uint_as_float(lds32(at + kPairBoxF32));
-                            } else {
+                                const uint8_t* at = tile_sm + r * 128u + ((((uint32_t)lane >> 2) ^ (r & 7u)) << 4) + ((uint32_t)lane & 3u) * 4u;
+                                lo[i] = *reinterpret_cast<const uint32_t*>(at);
+                                hi[i] = *reinterpret_cast<const uint32_t*>(at + kPairBoxF32);
+                            } else if (a.y_words) {
                                 const uint32_t w = (uint32_t)lane & 15u;
-                                const uint32_t at = rs_ + ((uint32_t)lane >> 4) * kPairBoxBF16 + (((w >> 2) ^ (((uint32_t)r >> 1) & 3u)) << 4) + (w & 3u) * 4u;
-                                uint32_t* dst = reinterpret_cast<uint32_t*>(out + r * a.y_stride * 2) + lane;
-                                if (2 * lane + 1 < cols) *dst = lds32(at);
-                                else if (2 * lane < cols) *reinterpret_cast<uint16_t*>(dst) = (uint16_t)lds32(at);
+                                lo[i] = *reinterpret_cast<const uint32_t*>(tile_sm + r * 64u + ((uint32_t)lane >> 4) * kPairBoxBF16 +
+                                                                           (((w >> 2) ^ ((r >> 1) & 3u)) << 4) + (w & 3u) * 4u);
+                                hi[i] = 0u;
+                            } else {
+                                const uint8_t* at = tile_sm + r * 64u + ((((uint32_t)lane >> 3) ^ ((r >> 1) & 3u)) << 4) + ((uint32_t)lane & 7u) * 2u;
+                                lo[i] = *reinterpret_cast<const uint16_t*>(at);
+                                hi[i] = *reinterpret_cast<const uint16_t*>(at + kPairBoxBF16);
                             }
                         }
-                    } else {
-#pragma unroll 4
-                        for (int r = 0; r < rows; ++r) {
-                            const uint32_t at = stage_s + (uint32_t)(quarter * 32 + r) * 64u + ((((uint32_t)lane >> 3) ^ (((uint32_t)r >> 1) & 3u)) << 4) +
-                                                ((uint32_t)lane & 7u) * 2u;
-                            uint16_t* dst = reinterpret_cast<uint16_t*>(out + r * a.y_stride * 2) + lane;
-                            if (lane < cols) dst[0] = (uint16_t)lds16(at);
-                            if (lane + 32 < cols) dst[32] = (uint16_t)lds16(at + kPairBoxBF16);
+#pragma unroll
+                        for (int i = 0; i < kBatch; ++i) {
+                            if (r0 + i >= rows) break;
+                            uint8_t* dst = out + (int64_t)(r0 + i) * a.y_stride * (YBF16 ? 2 : 4);
+                            if (!YBF16) {
+                                if (lane < cols) reinterpret_cast<uint32_t*>(dst)[lane] = lo[i];
+                                if (lane + 32 < cols) reinterpret_cast<uint32_t*>(dst)[lane + 32] = hi[i];
+                            } else if (a.y_words) {
+                                if (2 * lane + 1 < cols) reinterpret_cast<uint32_t*>(dst)[lane] = lo[i];
+                                else if (2 * lane < cols) reinterpret_cast<uint16_t*>(dst)[2 * lane] = (uint16_t)lo[i];
+                            } else {
+                                if (lane < cols) reinterpret_cast<uint16_t*>(dst)[lane] = (uint16_t)lo[i];
+                                if (lane + 32 < cols) reinterpret_cast<uint16_t*>(dst)[lane + 32] = (uint16_t)hi[i];
+                            }
                         }
                     }
                     __syncwarp();
