@@ -1169,7 +1169,11 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     // with 32-byte rows (16 KB in all, written in passes) leave room for more stages.  Taken when that gives the smaller
     // half of the ring another stage without changing whether A stays resident; with several groups per tile only where
     // the operands stream (a long contraction), since the passes cost a short tile more than the stage gives.
-    bool quarter_strips = y_tma && !fx && !acc_debug && (wide || pow2_steps) && p.n_chunks >= 2 &&
+    // One group per token, or power-of-two steps: pairs of CTAs on 256 x 256 tiles (tdq_linear_one.cu), unless there are too
+    // few of those: with 24 (2000 x 768 -> 768) the two kernels are level, with 64 (2048 x 2048 -> 2048) it is 15.7 -> 13.0 us.
+    const int64_t tiles256 = ((p.tiles_m + 1) / 2) * ((p.tiles_n + 1) / 2);
+    const bool use_one = y_tma && !fx && !acc_debug && p.Kg == 1 && (group_size > 32 || pow2_steps) && tiles256 <= INT32_MAX / 4 && tiles256 * 4 >= n_sm;
+    bool quarter_strips = !use_one && y_tma && !fx && !acc_debug && (wide || pow2_steps) && p.n_chunks >= 2 &&
                           ((p.Kg == 1 && p.n_steps % kChunk == 0) ||
                            (wide && (group_size / 32) % kChunk == 0 && p.Kg >= 2 && !p.a_resident));
     if (quarter_strips) {
@@ -1205,7 +1209,7 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     // leave most SMs idle (1152 x 2048 -> 512 13.9 against 16.0 us), and they also take a y that tensor stores cannot write.
     const bool use_g32 = group_size == 32 && !pow2_steps && !fx && p.tiles_m * p.tiles_n <= INT32_MAX / 4;
     const bool use_pair = use_g32 && (!y_tma || p.n_steps <= 48 || p.tiles_m * p.tiles_n * 4 <= n_sm);
-    const bool unpack_a = !fx && !pow2_steps && !use_pair && p.a_resident && steps_per_item >= 256;
+    const bool unpack_a = !fx && !pow2_steps && !use_pair && !use_one && p.a_resident && steps_per_item >= 256;
     e.tiles_m = (fx || unpack_a) ? 0 : (int32_t)p.tiles_m;   // then only the weights are expanded here
     e.tiles_n = (int32_t)p.tiles_n;
     e.b_rows = use_pair ? 64 : 128;
@@ -1229,7 +1233,7 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     memset(&ymap, 0, sizeof(ymap));
     a.tma_ok = 0;
     if (y_tma && encode_y_map(&ymap, y, y_dtype == TDQ_BF16, M, O, y_row_stride,
-                              quarter_strips ? (y_dtype == TDQ_BF16 ? kCols / 2 : kCols / 4) : half_strips ? kCols / 2 : kCols,
+                              use_one ? kCols : quarter_strips ? (y_dtype == TDQ_BF16 ? kCols / 2 : kCols / 4) : half_strips ? kCols / 2 : kCols,
                               use_g32 ? kBM : 32, y_f16))
         a.tma_ok = 1;
     else if (narrow_strips || quarter_strips)
@@ -1277,6 +1281,7 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
 
     const int64_t items = p.tiles_m * p.n_parts;
     const unsigned grid = (unsigned)(items < n_sm ? items : n_sm);
+    if (use_one) return launch_linear_one(a, ymap, n_sm, dev, i8, ybf, stream);
     if (use_pair) {
         a.tiles_n = (int32_t)((O + 63) / 64);
         return launch_linear_g32_pair(a, ymap, n_sm, dev, ybf, dbg, stream);

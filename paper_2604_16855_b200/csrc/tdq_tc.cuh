@@ -102,6 +102,8 @@ struct Plan {
 };
 
 // The g = 32 kernel (tdq_linear_g32.cu); the caller has run the operand expansion and built the plan and the map.
+// One accumulator per output element over the whole contraction (tdq_linear_one.cu).
+tdq_status launch_linear_one(LinArgs a, const CUtensorMap& ymap, int n_sm, int dev, bool i8, bool ybf, cudaStream_t stream);
 tdq_status launch_linear_g32_pair(const LinArgs& a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, bool dbg,
                                   cudaStream_t stream);   // tiles of 128 x 64, tdq_linear_g32_pair.cu
 tdq_status launch_linear_g32(const LinArgs& a, const CUtensorMap& ymap, uint32_t smem_bytes, unsigned grid, bool ybf,
