@@ -10,6 +10,8 @@
 #include <Python.h>
 
 #include <ATen/ATen.h>
+#include <ATen/cuda/EmptyTensor.h>
+#include <c10/cuda/CUDACachingAllocator.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Dtype.h>
@@ -134,9 +136,31 @@ PyObject* tuple2(const at::Tensor& a, const at::Tensor& b) {
     Py_XDECREF(pb);
     return t;
 }
-at::Tensor new_like(const at::Tensor& on, at::IntArrayRef sizes, at::ScalarType s) { return at::empty(sizes, on.options().dtype(s)); }
+// Straight to the caching allocator: the dispatcher's share of at::empty is half of its time, and a small layer whose
+// outputs the calls make allocates four times.
+at::Tensor new_like(const at::Tensor& on, at::IntArrayRef sizes, at::ScalarType s) {
+    return at::Tensor(at::detail::empty_cuda(sizes, s, on.device(), c10::nullopt));
+}
+// The caller's workspace, or one from the caching allocator for the length of the call (given back to the stream's pool, so
+// whatever the stream runs next is ordered behind its use).  Every linear call writes what it reads of the workspace, so
+// nothing has to be cleared.
+struct Workspace {
+    at::DataPtr own;
+    void* ptr;
+    size_t bytes;
+    Workspace(const at::Tensor* given, const at::Tensor& on, int64_t M, int64_t I_pad, int64_t O, int64_t g) {
+        if (given) {
+            ptr = given->data_ptr();
+            bytes = (size_t)given->numel();
+        } else {
+            c10::cuda::CUDAGuard guard(on.device());
+            bytes = tdq_linear_workspace_bytes(M, I_pad, O, (int32_t)g);
+            own = c10::cuda::CUDACachingAllocator::get()->allocate(bytes);
+            ptr = own.get();
+        }
+    }
+};
 at::Tensor workspace_for(const at::Tensor& on, int64_t M, int64_t I_pad, int64_t O, int64_t g) {
-    // every linear call writes what it reads of the workspace, so nothing has to be cleared
     return new_like(on, {(int64_t)tdq_linear_workspace_bytes(M, I_pad, O, (int32_t)g)}, at::kByte);
 }
 
@@ -233,24 +257,24 @@ PyObject* w4a4_linear(PyObject* const* a) {
     if (wc.dim() < 1) throw Bad{PyExc_ValueError, "wcodes must be a matrix"};
     const int64_t M = xc.size(0), I_pad = 2 * xc.size(1), O = wc.size(0);
     const at::Tensor y = oy ? *oy : new_like(xc, {M, O}, dtype_arg(a[6]));
-    const at::Tensor workspace = ow ? *ow : workspace_for(xc, M, I_pad, O, g);
     const at::Tensor* first = nullptr;
     check_operand("xcodes", &xc, at::kByte, first);
     check_operand("xscale", &xs, at::kFloat, first);
     check_operand("wcodes", &wc, at::kByte, first);
     check_operand("wscale", &ws, at::kFloat, first);
     check_operand("bias", bias, at::kFloat, first);
-    check_operand("workspace", &workspace, at::kByte, first);
+    check_operand("workspace", ow, at::kByte, first);
     check_operand("acc_debug", acc, at::kInt, first);
     check_y(y, first);
     const tdq_dtype dt = dtype_id(y);
+    const Workspace workspace(ow, xc, M, I_pad, O, g);
     const int64_t y_stride = M > 0 ? y.stride(0) : O;
     check(call(xc, [&](void* st) {
               if (pow2)
                   return tdq_w4a4_linear_pow2(ptr<uint8_t>(xc), ptr<float>(xs), ptr<uint8_t>(wc), ptr<float>(ws), ptr<float>(bias), M, I_pad,
-                                              O, (int32_t)g, ptr(y), dt, y_stride, ptr(workspace), (size_t)workspace.numel(), st);
+                                              O, (int32_t)g, ptr(y), dt, y_stride, workspace.ptr, workspace.bytes, st);
               return tdq_w4a4_linear(ptr<uint8_t>(xc), ptr<float>(xs), ptr<uint8_t>(wc), ptr<float>(ws), ptr<float>(bias), M, I_pad, O,
-                                     (int32_t)g, ptr(y), dt, y_stride, ptr<int32_t>(acc), ptr(workspace), (size_t)workspace.numel(), st);
+                                     (int32_t)g, ptr(y), dt, y_stride, ptr<int32_t>(acc), workspace.ptr, workspace.bytes, st);
           }), pow2 ? "tdq_w4a4_linear_pow2" : "tdq_w4a4_linear");
     return THPVariable_Wrap(y);
 }
@@ -293,20 +317,20 @@ PyObject* quant_linear_fused(PyObject* const* a) {
     if (wc.dim() != 2) throw Bad{PyExc_ValueError, "wcodes must be a matrix"};
     const int64_t M = x2.size(0), O = wc.size(0);
     const at::Tensor y = oy ? *oy : new_like(x, {M, O}, dtype_arg(a[5]));
-    const at::Tensor workspace = ow ? *ow : workspace_for(x, M, wc.size(1) * 2, O, p.group_size);
     if (C > 1 && x2.stride(1) != 1) throw Bad{PyExc_ValueError, "the channels of x must be adjacent in memory"};
     const at::Tensor* first = nullptr;
     check_operand("wcodes", &wc, at::kByte, first);
     check_operand("wscale", &ws, at::kFloat, first);
     check_operand("bias", bias, at::kFloat, first);
-    check_operand("workspace", &workspace, at::kByte, first);
+    check_operand("workspace", ow, at::kByte, first);
     check_y(y, first);
     if (x2.device() != first->device())
         throw Bad{PyExc_ValueError, "x is on " + x2.device().str() + ", the weights on " + first->device().str()};
     const tdq_dtype xdt = dtype_id(x2), ydt = dtype_id(y);
+    const Workspace workspace(ow, x, M, wc.size(1) * 2, O, p.group_size);
     check(call(x, [&](void* st) {
               return tdq_quant_linear_fused(ptr(x2), xdt, 1, M, C, M > 1 ? x2.stride(0) : C, &p, ptr<uint8_t>(wc), ptr<float>(ws),
-                                            ptr<float>(bias), O, ptr(y), ydt, y.stride(0), ptr(workspace), (size_t)workspace.numel(), st);
+                                            ptr<float>(bias), O, ptr(y), ydt, y.stride(0), workspace.ptr, workspace.bytes, st);
           }), "tdq_quant_linear_fused");
     return THPVariable_Wrap(y);
 }
