@@ -23,7 +23,7 @@ namespace {
 
 // Side streams and events of the host-buffer call, made once per process and device (the call is a
 // convenience for callers who hold host data; it is the one entry point that creates CUDA objects).
-constexpr int kHostChunks = 8;
+constexpr int kHostChunks = 8;   // at most
 struct HostPipe {
     cudaStream_t h2d = nullptr, d2h = nullptr;
     cudaEvent_t start = nullptr, done = nullptr, in[kHostChunks] = {}, out[kHostChunks] = {};
@@ -53,9 +53,12 @@ HostPipe* host_pipe() {
 
 }  // namespace
 
-// Rows go through in up to eight chunks so that the copy-out of one chunk (the long pole: y is eight
-// times the size of x at cfg4) overlaps the copy-in and the kernels of the next; kernels run on the
-// caller's stream, the copies on two side streams tied to it by events.
+// Rows go through in chunks so that the copy-out of one chunk (the long pole: y is eight times the size of x at cfg4)
+// overlaps the copy-in and the kernels of the next; kernels run on the caller's stream, the copies on two side streams tied
+// to it by events.  Bound by the bus (35 MB of y take 636 us in one copy).  Five chunks, small ones first and last: nothing
+// is copied out before the first chunk is through, nothing in while the last one is finished, and every further chunk costs
+// the copy engine a few microseconds.  9216 x 320 -> 960 fp32: 731 -> 709 us against eight equal chunks.  A workspace that
+// holds only an eighth of the rows still gets those.
 extern "C" tdq_status tdq_quant_linear_host(const void* x_host, tdq_dtype x_dtype, int64_t B, int64_t N, int64_t C,
                                             const tdq_act_params* p, const uint8_t* wcodes, const float* wscale,
                                             const float* bias, int64_t O, void* y_host, tdq_dtype y_dtype,
@@ -94,9 +97,13 @@ extern "C" tdq_status tdq_quant_linear_host(const void* x_host, tdq_dtype x_dtyp
     if (cudaEventRecord(hp->start, stream) != cudaSuccess) return TDQ_ERR_CUDA;
     if (cudaStreamWaitEvent(hp->h2d, hp->start, 0) != cudaSuccess || cudaStreamWaitEvent(hp->d2h, hp->start, 0) != cudaSuccess)
         return TDQ_ERR_CUDA;
+    const int64_t half = ((M + 1) / 2 + 127) / 128 * 128;
+    const bool ramp = linear_check_shape(half < M ? half : M, I_pad, O, p->group_size, workspace_bytes) == TDQ_OK;
     int chunk = 0;
-    for (int64_t m0 = 0; m0 < M; m0 += rows_per, ++chunk) {
-        const int64_t rows = M - m0 < rows_per ? M - m0 : rows_per;
+    for (int64_t m0 = 0, rows = 0; m0 < M; m0 += rows, ++chunk) {
+        static const int64_t kSixteenths[5] = {1, 3, 8, 3, 16};
+        const int64_t want = ramp ? ((M * kSixteenths[chunk < 4 ? chunk : 4] + 15) / 16 + 127) / 128 * 128 : rows_per;
+        rows = M - m0 < want ? M - m0 : want;
         const char* xh = reinterpret_cast<const char*>(x_host) + m0 * C * xe;
         char* xd = reinterpret_cast<char*>(x_dev) + m0 * C * xe;
         char* yd = reinterpret_cast<char*>(y_dev) + m0 * O * ye;
