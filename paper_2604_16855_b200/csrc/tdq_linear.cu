@@ -1204,11 +1204,16 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     // workspace; its promotion warps do that at the start of an item, though, with the tensor core idle,
     // so it only pays when an item carries much more work than its own unpacking.
     const int64_t steps_per_item = (p.tiles_n + p.n_parts - 1) / p.n_parts * (int64_t)p.n_steps;
-    // g = 32 goes to the kernels built for it.  Two blocks per SM with narrow tiles (tdq_linear_g32_pair.cu) win up to about
+    // g = 32 goes to the kernels built for it.  Two blocks per SM with narrow tiles (tdq_linear_pair.cu) win up to about
     // 1536 channels (16384 x 1024 -> 2048 86.6 against 92.7 us, 2048 channels 158 against 156) and whenever wide tiles would
     // leave most SMs idle (1152 x 2048 -> 512 13.9 against 16.0 us), and they also take a y that tensor stores cannot write.
     const bool use_g32 = group_size == 32 && !pow2_steps && !fx && p.tiles_m * p.tiles_n <= INT32_MAX / 4;
-    const bool use_pair = use_g32 && (!y_tma || p.n_steps <= 48 || p.tiles_m * p.tiles_n * 4 <= n_sm);
+    // Groups of 64 and 128 too where the general kernel's wide tiles are mostly overhead: contractions of up to 512 channels
+    // (9216 x 128 -> 512 at 64 10.1 -> 8.3 us), at most 64 outputs (30000 x 640 -> 64 at 128 17.7 -> 12.5 us), fewer tiles than
+    // SMs (1000 x 2048 -> 256 at 64 14.9 -> 12.0 us).  4616 x 768 -> 3072 at 128 is level, 18464 rows 87 -> 99 us.
+    const bool use_pair_wide = !pow2_steps && !fx && !use_one && (group_size == 64 || group_size == 128) && p.tiles_m * p.tiles_n <= INT32_MAX / 4 &&
+                               (p.n_steps <= 16 || O <= 64 || p.tiles_m * p.tiles_n <= n_sm);
+    const bool use_pair = use_pair_wide || (use_g32 && (!y_tma || p.n_steps <= 48 || p.tiles_m * p.tiles_n * 4 <= n_sm));
     const bool unpack_a = !fx && !pow2_steps && !use_pair && !use_one && p.a_resident && steps_per_item >= 256;
     e.tiles_m = (fx || unpack_a) ? 0 : (int32_t)p.tiles_m;   // then only the weights are expanded here
     e.tiles_n = (int32_t)p.tiles_n;
@@ -1233,8 +1238,8 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     memset(&ymap, 0, sizeof(ymap));
     a.tma_ok = 0;
     if (y_tma && encode_y_map(&ymap, y, y_dtype == TDQ_BF16, M, O, y_row_stride,
-                              use_one ? kCols : quarter_strips ? (y_dtype == TDQ_BF16 ? kCols / 2 : kCols / 4) : half_strips ? kCols / 2 : kCols,
-                              use_g32 ? kBM : 32, y_f16))
+                              (use_one || use_pair) ? kCols : quarter_strips ? (y_dtype == TDQ_BF16 ? kCols / 2 : kCols / 4) : half_strips ? kCols / 2 : kCols,
+                              (use_g32 || use_pair) ? kBM : 32, y_f16))
         a.tma_ok = 1;
     else if (narrow_strips || quarter_strips)
         return TDQ_ERR_CUDA;   // the plan counted on the tensor store
@@ -1284,7 +1289,7 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     if (use_one) return launch_linear_one(a, ymap, n_sm, dev, i8, ybf, stream);
     if (use_pair) {
         a.tiles_n = (int32_t)((O + 63) / 64);
-        return launch_linear_g32_pair(a, ymap, n_sm, dev, ybf, dbg, stream);
+        return launch_linear_pair(a, ymap, n_sm, dev, ybf, dbg, stream);
     }
     if (use_g32 && a.tma_ok) return launch_linear_g32(a, ymap, p.smem_bytes, grid, ybf, dbg, stream);
     if (launch_pdl(kernel, dim3(grid), dim3(kThreads), p.smem_bytes, stream, a, ymap) != cudaSuccess) return TDQ_ERR_CUDA;

@@ -1,6 +1,6 @@
 // The W4A4 linear layer at the paper's group size g = 32 (Algorithm S1 step 10 with Eq. 9 and Eq. 4
 // substituted) for long contractions, with y that bulk tensor stores can write (16-byte aligned base and row pitch); shorter
-// ones go to tdq_linear_g32_pair.cu:
+// ones go to tdq_linear_pair.cu:
 //
 //   acc[m,o,k] = sum_{i in group k} q_x[m,i] q_w[o,i]      one tcgen05.mma (E4M3 operands, exact) per group
 //   y[m,o]     = s_o * sum_k Delta[m,k] * acc[m,o,k] + b_o  fp32 in registers ("promotion")
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
                         tc_fence_after();
                         if (elect_one()) {
                             if (k0 + (int)me < n_steps) {
-                                mma_f8_fresh(tm_me, desc_of(resident ? a_lo : b_lo + a_in_stage), desc_of(b_lo), kIdescF8);
+                                mma_f8(tm_me, desc_of(resident ? a_lo : b_lo + a_in_stage), desc_of(b_lo), kIdescF8);
                                 mma_commit(tfull_me);
                             }
                             mma_commit(empty_s + s * 8);

@@ -23,6 +23,9 @@
 //               and fetches the next tile's channel constants meanwhile
 //   warps 4-7   promotion and epilogue: warp = 32 TMEM lanes (rows), all 64 columns: 64 float sums, 128 landing registers
 //
+// Groups of 64 and 128 codes take the same kernel (template argument SPG) for short contractions, narrow layers and few
+// tiles; larger ones are bound by the operands' way through shared memory, which the general kernel's wider tiles halve.
+//
 // Measured against the other kernel (us; with the operand expansion): 73728 x 64 -> 64 fp32 16.2 -> 11.0, 73728 x 64 -> 192
 // 25.0 -> 18.0, 9216 x 64 -> 256 8.4 -> 7.2, 16384 x 512 -> 2048 bf16 63.8 -> 51.4, 16384 x 1024 -> 2048 92.7 -> 86.6,
 // 18464 x 768 -> 3072 fp32 119.7 -> 115.4; from 2048 channels on the other one is 1-9 % faster (narrower tiles read A twice
@@ -69,8 +72,10 @@ __device__ __forceinline__ void wait_hot(uint32_t bar_s, uint32_t parity, Ctrl* 
     if (!mbar_test_s(bar_s, parity)) wait_cold(bar_s, parity, c, status, code);
 }
 
-template <bool YBF16, bool DBG>
-__global__ void __launch_bounds__(kPairThreads, 2) w4a4_g32_pair_kernel(const LinArgs a, const __grid_constant__ CUtensorMap ymap) {
+// SPG: K-steps per group (1, 2 or 4).  With one, a stage holds two pairs of groups and their steps; with more, a pair of
+// groups is one stage or two, one MMA warp takes them all, and the row's steps come from global memory a pair ahead.
+template <bool YBF16, bool DBG, int SPG>
+__global__ void __launch_bounds__(kPairThreads, 2) w4a4_pair_kernel(const LinArgs a, const __grid_constant__ CUtensorMap ymap) {
     extern __shared__ __align__(128) uint8_t smem_raw[];
     Ctrl* c = reinterpret_cast<Ctrl*>(smem_raw);            // its abort flag and TMEM address; the barriers are g's
     PairCtrl* g = reinterpret_cast<PairCtrl*>(smem_raw + sizeof(Ctrl));
@@ -81,7 +86,7 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_g32_pair_kernel(const Li
     const int warp = uniform_warp(), lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kPairStages; ++i) { mbar_init(&g->full[i], 1); mbar_init(&g->empty[i], 2 + kPairPromoWarps); }
+        for (int i = 0; i < kPairStages; ++i) { mbar_init(&g->full[i], 1); mbar_init(&g->empty[i], SPG == 1 ? 2 + kPairPromoWarps : 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(&g->tfull[i], 1); mbar_init(&g->tempty[i], kPairPromoWarps); }
         mbar_init(&g->sfull, kPairPromoWarps);
         mbar_init(&g->sfree, 1);
@@ -121,10 +126,10 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_g32_pair_kernel(const Li
                     if (c->abort_flag) break;
                     if (elect_one()) {
                         const uint32_t st = ring_s + s * kPairStageBytes;
-                        mbar_expect_tx(&g->full[s], nk * (kBlock + kBHalf + kScaleBlock));
+                        mbar_expect_tx(&g->full[s], nk * (kBlock + kBHalf + (SPG == 1 ? kScaleBlock : 0)));
                         bulk_load(st, a_src, nk * kBlock, &g->full[s]);
                         bulk_load(st + kChunk * kBlock, b_src, nk * kBHalf, &g->full[s]);
-                        bulk_load(st + kPairScales, s_src, nk * kScaleBlock, &g->full[s]);
+                        if (SPG == 1) bulk_load(st + kPairScales, s_src, nk * kScaleBlock, &g->full[s]);
                     }
                     __syncwarp();
                     a_src += kChunk * kBlock;
@@ -135,17 +140,16 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_g32_pair_kernel(const Li
             }
         } else if (warp < kPairStoreWarp) {
             // ------------------------------------------------------------ MMA issue
-            // Warp `me` owns slots 2 me and 2 me + 1: of every stage it issues steps 2 me and 2 me + 1 and reports them with
-            // one commit.
+            // Warp `me` owns slots 2 me and 2 me + 1, one group each, and reports a pair with one commit.
             const uint32_t me = (uint32_t)(warp - kFirstMmaWarp);
             const uint32_t full_s = smem_u32(&g->full[0]), empty_s = smem_u32(&g->empty[0]);
             const uint32_t tfull_s = smem_u32(&g->tfull[me]), tempty_s = smem_u32(&g->tempty[me]);
             const uint32_t tm = tmem_base + 2 * me * kN;
-            const uint32_t a_lo = desc_lo(ring_s) + 2 * me * (kBlock >> 4);
-            const uint32_t b_lo = desc_lo(ring_s + kChunk * kBlock) + 2 * me * (kBHalf >> 4);
+            const uint32_t a_lo = desc_lo(ring_s) + (SPG == 1 ? 2 * me * (kBlock >> 4) : 0u);
+            const uint32_t b_lo = desc_lo(ring_s + kChunk * kBlock) + (SPG == 1 ? 2 * me * (kBHalf >> 4) : 0u);
             uint32_t s = 0, ph = 0;
             uint32_t q = 1;                      // parity to wait for on tempty; a fresh barrier passes parity 1
-            for (int tile = blockIdx.x; tile < n_tiles && !c->abort_flag; tile += gridDim.x) {
+            for (int tile = blockIdx.x; SPG == 1 && tile < n_tiles && !c->abort_flag; tile += gridDim.x) {   // steps 2 me and 2 me + 1 of every stage
 #pragma unroll 1
                 for (int k0 = 0; k0 < n_steps; k0 += kChunk) {
                     const int mine = n_steps - k0 - 2 * (int)me;         // steps left from this warp's first one on
@@ -158,8 +162,8 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_g32_pair_kernel(const Li
                         q ^= 1u;
                         tc_fence_after();
                         if (elect_one()) {
-                            mma_f8_fresh(tm, desc_of(a_lo + so), desc_of(b_lo + so), kIdescN64);
-                            if (mine > 1) mma_f8_fresh(tm + kN, desc_of(a_lo + so + (kBlock >> 4)), desc_of(b_lo + so + (kBHalf >> 4)), kIdescN64);
+                            mma_f8(tm, desc_of(a_lo + so), desc_of(b_lo + so), kIdescN64);
+                            if (mine > 1) mma_f8(tm + kN, desc_of(a_lo + so + (kBlock >> 4)), desc_of(b_lo + so + (kBHalf >> 4)), kIdescN64);
                             mma_commit(tfull_s);
                             mma_commit(empty_s + s * 8);
                         }
@@ -168,6 +172,40 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_g32_pair_kernel(const Li
                     }
                     __syncwarp();
                     if (++s == kPairStages) { s = 0; ph ^= 1; }
+                }
+            }
+            // SPG > 1: one warp takes all the pairs.  (Two in turn would each skip stages of the ring, and a parity wait cannot
+            // tell the phase a warp means from the one two phases before it that its neighbour has not got to yet.)
+            uint32_t n = 0;                      // pairs of groups so far; pair n uses slots 2 (n & 1) and the next
+            for (int tile = blockIdx.x; SPG > 1 && me == 0 && tile < n_tiles && !c->abort_flag; tile += gridDim.x) {
+#pragma unroll 1
+                for (int g0 = 0; g0 < a.Kg; g0 += 2, ++n) {
+                    const int groups = min(2, a.Kg - g0), stages = SPG == 4 ? groups : 1;
+                    const uint32_t p = n & 1u, d = tmem_base + 2 * p * kN;
+                    const bool rt = mbar_test_s(tempty_s + p * 8, ((n >> 1) & 1u) ^ 1u);
+                    bool rf = mbar_test_s(full_s + s * 8, ph);
+                    if (!rt) wait_cold(tempty_s + p * 8, ((n >> 1) & 1u) ^ 1u, c, a.status, 3u);
+#pragma unroll
+                    for (int j = 0; j < (SPG == 4 ? 2 : 1); ++j) {
+                        if (j >= stages) break;
+                        if (!rf) wait_cold(full_s + s * 8, ph, c, a.status, 4u);
+                        tc_fence_after();
+                        if (elect_one()) {
+                            const uint32_t so = s * (kPairStageBytes >> 4);
+#pragma unroll
+                            for (int k = 0; k < kChunk; ++k) {
+                                const int slot = SPG == 4 ? j : k >> 1;
+                                if (SPG == 4 || slot < groups)
+                                    mma_f8(d + slot * kN, desc_of(a_lo + so + k * (kBlock >> 4)), desc_of(b_lo + so + k * (kBHalf >> 4)), kIdescN64,
+                                           (k & (SPG - 1)) != 0 ? 1u : 0u);
+                            }
+                            if (j == stages - 1) mma_commit(tfull_s + p * 8);
+                            mma_commit(empty_s + s * 8);
+                        }
+                        __syncwarp();
+                        if (++s == kPairStages) { s = 0; ph ^= 1; }
+                        if (j + 1 < stages) rf = mbar_test_s(full_s + s * 8, ph);
+                    }
                 }
             }
         } else {
@@ -270,6 +308,14 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_g32_pair_kernel(const Li
             if (++rs == kPairStages) { rs = 0; rph ^= 1; }
         };
 
+        // SPG > 1: the steps of groups k and k + 1 of row block `block` (zero past the end)
+        auto global_steps = [&](uint32_t (&e)[4], int block, int k) {
+            const uint32_t* src = reinterpret_cast<const uint32_t*>(a.s_blocks) + ((int64_t)block * a.Kg + k) * kBM + row;
+            e[0] = __ldg(src);
+            e[1] = k + 1 < a.Kg ? __ldg(src + kBM) : 0u;
+        };
+        uint32_t n = 0;                               // SPG > 1: pairs of groups so far; pair n uses slots 2 (n & 1) and the next
+
         // A tile's groups are taken two at a time (a pair of slots): wait for the pair's landing, hand both slots back
         // with one arrival, fold the first group in, start the next pair's first load into the registers that frees, fold
         // the second, start the second load.
@@ -278,8 +324,9 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_g32_pair_kernel(const Li
             nt = tile - mt * a.tiles_n;
             wait_pair(0, mbar_test_s(tfull_s, p_full & 1u));
             load_lo(0);
-            if (n_steps > 1) load_hi(1);
-            take_steps(mbar_test_s(full_s, 0u));
+            if (a.Kg > 1) load_hi(1);
+            if (SPG == 1) take_steps(mbar_test_s(full_s, 0u));
+            else global_steps(d, mt, 0);
 #pragma unroll 1
             while (!c->abort_flag) {
                 // one tile; the load of its first pair is in flight, its first steps are in d
@@ -287,9 +334,29 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_g32_pair_kernel(const Li
                 for (int j = 0; j < kN / 2; ++j) yacc[j] = 0ull;
                 const int next = tile + (int)gridDim.x;
                 const bool another = next < n_tiles;
+                const int mt_next = another ? next / a.tiles_n : mt;
+#pragma unroll 1
+                for (int k = 0; SPG > 1 && k < a.Kg; k += 2, ++n) {
+                    const bool tile_end = k + 2 >= a.Kg, more = !tile_end || another;
+                    const uint32_t p = (n + 1) & 1u;      // the next pair's slots
+                    const bool r = more ? mbar_test_s(tfull_s + p * 8, (p_full >> p) & 1u) : true;
+                    uint32_t e[4] = {0u, 0u, 0u, 0u};
+                    if (more) global_steps(e, tile_end ? mt_next : mt, tile_end ? 0 : k + 2);
+                    tmem_ld_wait_on(va); tmem_ld_wait_on(vb); tmem_ld_wait_on(vc); tmem_ld_wait_on(vd);
+                    tc_fence_before();
+                    __syncwarp();
+                    mbar_arrive_lane0_s(tempty_s + (n & 1u) * 8, lane);
+                    if (DBG) { debug(va, vb, k); if (k + 1 < a.Kg) debug(vc, vd, k + 1); }
+                    fold(va, vb, d[0]);
+                    if (more) { wait_pair(p, r); load_lo(2 * p); }
+                    if (k + 1 < a.Kg) fold(vc, vd, d[1]);
+                    if (more && (tile_end ? a.Kg > 1 : k + 3 < a.Kg)) load_hi(2 * p + 1);
+                    d[0] = e[0];
+                    d[1] = e[1];
+                }
                 int left = n_steps;                       // groups not yet folded in
 #pragma unroll 1
-                for (;;) {
+                for (; SPG == 1;) {
                     // first pair of the stage: slots 0 and 1
                     const bool second = left > 2;         // the stage has another pair
                     bool r1 = true;
@@ -325,7 +392,7 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_g32_pair_kernel(const Li
                     take_steps(rf);
                     left -= 4;
                 }
-                if (another) {                            // the next tile's first pair lands under the epilogue
+                if (SPG == 1 && another) {                // the next tile's first pair lands under the epilogue
                     wait_pair(0, mbar_test_s(tfull_s, p_full & 1u));
                     load_lo(0);
                     if (n_steps > 1) load_hi(1);
@@ -420,7 +487,7 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_g32_pair_kernel(const Li
                 mbar_arrive_lane0(&g->sfull, lane);
                 if (!another) break;
                 tile = next;
-                mt = tile / a.tiles_n;
+                mt = mt_next;
                 nt = tile - mt * a.tiles_n;
             }
         }
@@ -441,16 +508,19 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_g32_pair_kernel(const Li
 }  // namespace
 
 // a.tiles_n and a.b_blocks are in units of 64 columns here (see ExpandArgs::b_rows).
-tdq_status launch_linear_g32_pair(const LinArgs& a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, bool dbg, cudaStream_t stream) {
-    void (*kernel)(LinArgs, CUtensorMap) = nullptr;
-    if (!ybf && !dbg) kernel = w4a4_g32_pair_kernel<false, false>;
-    if (ybf && !dbg) kernel = w4a4_g32_pair_kernel<true, false>;
-    if (!ybf && dbg) kernel = w4a4_g32_pair_kernel<false, true>;
-    if (ybf && dbg) kernel = w4a4_g32_pair_kernel<true, true>;
+tdq_status launch_linear_pair(const LinArgs& a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, bool dbg, cudaStream_t stream) {
+    constexpr int kInst = 12;
+    void (*const kernels[kInst])(LinArgs, CUtensorMap) = {
+        w4a4_pair_kernel<false, false, 1>, w4a4_pair_kernel<true, false, 1>, w4a4_pair_kernel<false, true, 1>, w4a4_pair_kernel<true, true, 1>,
+        w4a4_pair_kernel<false, false, 2>, w4a4_pair_kernel<true, false, 2>, w4a4_pair_kernel<false, true, 2>, w4a4_pair_kernel<true, true, 2>,
+        w4a4_pair_kernel<false, false, 4>, w4a4_pair_kernel<true, false, 4>, w4a4_pair_kernel<false, true, 4>, w4a4_pair_kernel<true, true, 4>};
+    const int inst = (ybf ? 1 : 0) + (dbg ? 2 : 0) + 4 * (a.steps_per_grp >> 1);
+    if (inst >= kInst) return TDQ_ERR_UNSUPPORTED;
+    void (*const kernel)(LinArgs, CUtensorMap) = kernels[inst];
     const uint32_t smem = kPairCtrl + kPairStages * kPairStageBytes + 1024 + 2 * (ybf ? kPairBoxBF16 : kPairBoxF32) + 2 * kN * 4;
     static_assert(kPairCtrl + kPairStages * kPairStageBytes + 1024 + 2 * kPairBoxF32 + 2 * kN * 4 <= 113 * 1024, "two CTAs per SM");
-    static std::atomic<uint64_t> smem_done[4];
-    if (allow_smem(kernel, 113 * 1024, smem_done[(ybf ? 1 : 0) + (dbg ? 2 : 0)], dev) != cudaSuccess) return TDQ_ERR_CUDA;
+    static std::atomic<uint64_t> smem_done[kInst];
+    if (allow_smem(kernel, 113 * 1024, smem_done[inst], dev) != cudaSuccess) return TDQ_ERR_CUDA;
     const int64_t tiles = (int64_t)a.tiles_m * a.tiles_n;
     const unsigned grid = (unsigned)(tiles < 2 * n_sm ? tiles : 2 * n_sm);
     if (launch_pdl(kernel, dim3(grid), dim3(kPairThreads), smem, stream, a, ymap) != cudaSuccess) return TDQ_ERR_CUDA;

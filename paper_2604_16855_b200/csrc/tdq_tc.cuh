@@ -104,8 +104,8 @@ struct Plan {
 // The g = 32 kernel (tdq_linear_g32.cu); the caller has run the operand expansion and built the plan and the map.
 // One accumulator per output element over the whole contraction (tdq_linear_one.cu).
 tdq_status launch_linear_one(LinArgs a, const CUtensorMap& ymap, int n_sm, int dev, bool i8, bool ybf, cudaStream_t stream);
-tdq_status launch_linear_g32_pair(const LinArgs& a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, bool dbg,
-                                  cudaStream_t stream);   // tiles of 128 x 64, tdq_linear_g32_pair.cu
+tdq_status launch_linear_pair(const LinArgs& a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, bool dbg,
+                                  cudaStream_t stream);   // tiles of 128 x 64, tdq_linear_pair.cu
 tdq_status launch_linear_g32(const LinArgs& a, const CUtensorMap& ymap, uint32_t smem_bytes, unsigned grid, bool ybf,
                              bool dbg, cudaStream_t stream);
 
@@ -330,11 +330,11 @@ __device__ __forceinline__ bool elect_one() {
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
     return ok != 0;
 }
-// E4M3 tensor-core instruction (no accumulation) and commit for the elected lane, descriptors as 64-bit values
+// E4M3 tensor-core instruction and commit for the elected lane, descriptors as 64-bit values
 __device__ __forceinline__ uint64_t desc_of(uint32_t lo) { return ((uint64_t)kDescHi << 32) | lo; }
-__device__ __forceinline__ void mma_f8_fresh(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc) {
+__device__ __forceinline__ void mma_f8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate = 0u) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
-                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(0u) : "memory");
+                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint32_t bar_s) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar_s) : "memory");
