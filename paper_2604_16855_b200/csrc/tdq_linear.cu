@@ -1248,7 +1248,7 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     a.half_strips = quarter_strips ? 2 : half_strips ? 1 : 0;
     a.out_scale = i8 ? 0.00390625f : 262144.0f;
     a.y_f16 = y_f16 ? 1 : 0;
-    a.xcodes = xcodes; a.xscale = xscale; a.row_bytes = e.row_bytes; a.unpack_a = unpack_a ? 1 : 0;
+    a.xcodes = xcodes; a.wcodes = wcodes; a.xscale = xscale; a.row_bytes = e.row_bytes; a.unpack_a = unpack_a ? 1 : 0;
     a.pair_groups = (wide && a.steps_per_grp % kChunk == 0 && a.Kg >= 2) ? 1 : 0;
     // one group per tile: the group's chunks go to the two MMA warps in turn, each with an accumulator of its own
     if ((wide || pow2_steps) && !fx && a.Kg == 1 && a.steps_per_grp % kChunk == 0 && p.n_chunks >= 2) a.pair_groups = 2;
@@ -1271,6 +1271,15 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     const int inst = fx ? 8 + (fx->bf16 ? 2 : 0) + (ybf ? 1 : 0) : (i8 ? 4 : 0) + (ybf ? 2 : 0) + (dbg ? 1 : 0);
     if (allow_smem(kernel, kSmemLimit, smem_done[inst], dev) != cudaSuccess) return TDQ_ERR_CUDA;
 
+    if (use_pair) {
+        a.tiles_n = (int32_t)((O + 63) / 64);
+        // Few groups and one tile per block: the kernel expands its own operands, and the call is one launch.  Quantizer and
+        // linear layer, us: 256 x 64 -> 64 fp32 9.1 -> 7.2, 9216 x 64 -> 128 10.6 -> 7.4, 18432 x 128 -> 128 13.3 -> 10.6,
+        // 2000 x 192 -> 192 9.25 -> 7.6, 9217 x 147 -> 63 15.7 -> 13.4.  With more tiles than blocks a block would have to
+        // refill its ring with nothing under way (9216 x 320 -> 320, 360 tiles: 16.5 -> 18.5).
+        if (use_g32 && !dbg && p.n_steps <= kPairRing && p.tiles_m * a.tiles_n <= 2 * n_sm)
+            return launch_linear_pair(a, ymap, n_sm, dev, ybf, false, true, stream);
+    }
     const unsigned pieces = (unsigned)((e.tiles_m + e.tiles_n) * p.n_chunks);
     if (pow2_steps) {
         const unsigned pieces2 = (unsigned)((e.tiles_m + e.tiles_n) * ((p.n_chunks + kPow2Chunks - 1) / kPow2Chunks));
@@ -1287,10 +1296,7 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     const int64_t items = p.tiles_m * p.n_parts;
     const unsigned grid = (unsigned)(items < n_sm ? items : n_sm);
     if (use_one) return launch_linear_one(a, ymap, n_sm, dev, i8, ybf, stream);
-    if (use_pair) {
-        a.tiles_n = (int32_t)((O + 63) / 64);
-        return launch_linear_pair(a, ymap, n_sm, dev, ybf, dbg, stream);
-    }
+    if (use_pair) return launch_linear_pair(a, ymap, n_sm, dev, ybf, dbg, false, stream);
     if (use_g32 && a.tma_ok) return launch_linear_g32(a, ymap, p.smem_bytes, grid, ybf, dbg, stream);
     if (launch_pdl(kernel, dim3(grid), dim3(kThreads), p.smem_bytes, stream, a, ymap) != cudaSuccess) return TDQ_ERR_CUDA;
     g_launch_count.fetch_add(1, std::memory_order_relaxed);

@@ -39,6 +39,7 @@ constexpr int kN = 64;                       // columns per tile = one TMEM slot
 constexpr int kBHalf = kN * 32;              // operand bytes of 64 rows of B and one K-step
 constexpr int kPairThreads = 256;
 constexpr int kPairStages = 3;
+static_assert(kPairStages * kChunk == kPairRing);
 constexpr uint32_t kPairScales = kChunk * (kBlock + kBHalf);   // offset of a stage's scales: 4 groups x 128 rows
 constexpr uint32_t kPairStageBytes = kPairScales + kChunk * kScaleBlock;
 constexpr uint32_t kPairCtrl = 512;
@@ -72,9 +73,60 @@ __device__ __forceinline__ void wait_hot(uint32_t bar_s, uint32_t parity, Ctrl* 
     if (!mbar_test_s(bar_s, parity)) wait_cold(bar_s, parity, c, status, code);
 }
 
-// SPG: K-steps per group (1, 2 or 4).  With one, a stage holds two pairs of groups and their steps; with more, a pair of
+// The operands of a block's only tile straight from the packed codes (DIRECT; contractions that the ring holds whole): 128 rows
+// of A, 64 of B and the rows' steps, stage by stage.  A lane takes a row, so that the 16-byte stores of a quarter warp fill a
+// core matrix; the loads of neighbouring K-steps share sectors.  STAGES: how many stages' loads are in flight together.
+template <int STAGES>
+__device__ __forceinline__ void fill_stages(const LinArgs& a, int mt, int nt, uint32_t ring_s) {
+    const int t = threadIdx.x, ra = t & 127, rb = t & 63;
+    const int64_t ma = (int64_t)mt * kBM + ra, ob = (int64_t)nt * kN + rb;
+    const uint4* sa = reinterpret_cast<const uint4*>(a.xcodes + ma * a.row_bytes);
+    const uint4* sb = reinterpret_cast<const uint4*>(a.wcodes + ob * a.row_bytes);
+    const float* sx = a.xscale + ma * a.n_steps;
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    uint4 pa[STAGES][2], pb[STAGES];
+    float d[STAGES][2];
+#pragma unroll
+    for (int i = 0; i < STAGES; ++i) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int ks = kChunk * i + (t >> 7) + 2 * j;
+            const bool on = ks < a.n_steps && ma < a.M;
+            pa[i][j] = on ? __ldg(sa + ks) : zero;
+            d[i][j] = on ? __ldg(sx + ks) : 0.0f;
+        }
+        const int ks = kChunk * i + (t >> 6);
+        pb[i] = (ks < a.n_steps && ob < a.O) ? __ldg(sb + ks) : zero;
+    }
+    auto put = [&](uint32_t dst, const uint4& p) {
+        uint4 c0, c1;
+        expand8<false>(p.x, c0.x, c0.y);
+        expand8<false>(p.y, c0.z, c0.w);
+        expand8<false>(p.z, c1.x, c1.y);
+        expand8<false>(p.w, c1.z, c1.w);
+        sts128(dst, c0.x, c0.y, c0.z, c0.w);
+        sts128(dst + 128, c1.x, c1.y, c1.z, c1.w);
+    };
+#pragma unroll
+    for (int i = 0; i < STAGES; ++i) {
+        const uint32_t st = ring_s + i * kPairStageBytes;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int k = (t >> 7) + 2 * j;
+            if (kChunk * i + k < a.n_steps) {
+                put(st + (uint32_t)k * kBlock + (uint32_t)((ra >> 3) * 256 + (ra & 7) * 16), pa[i][j]);
+                sts32(st + kPairScales + (uint32_t)k * kScaleBlock + (uint32_t)ra * 4, __float_as_uint(d[i][j]));
+            }
+        }
+        const int k = t >> 6;
+        if (kChunk * i + k < a.n_steps) put(st + kChunk * kBlock + (uint32_t)k * kBHalf + (uint32_t)((rb >> 3) * 256 + (rb & 7) * 16), pb[i]);
+    }
+}
+
+// DIRECT: at most 12 groups (the ring holds them all) and one tile per block; the operands come from the packed codes
+// (fill_stages), and the call is one launch instead of an expansion and this.  SPG: K-steps per group (1, 2 or 4).  With one, a stage holds two pairs of groups and their steps; with more, a pair of
 // groups is one stage or two, one MMA warp takes them all, and the row's steps come from global memory a pair ahead.
-template <bool YBF16, bool DBG, int SPG>
+template <bool YBF16, bool DBG, int SPG, bool DIRECT = false>
 __global__ void __launch_bounds__(kPairThreads, 2) w4a4_pair_kernel(const LinArgs a, const __grid_constant__ CUtensorMap ymap) {
     extern __shared__ __align__(128) uint8_t smem_raw[];
     Ctrl* c = reinterpret_cast<Ctrl*>(smem_raw);            // its abort flag and TMEM address; the barriers are g's
@@ -107,6 +159,15 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_pair_kernel(const LinArg
     const uint32_t tmem_base = c->tmem_base;
     const int n_tiles = a.tiles_m * a.tiles_n;
     const int n_steps = a.n_steps;
+    if (DIRECT) {
+        if (blockIdx.x == 0 && threadIdx.x < 4) a.status[threadIdx.x] = 0u;   // the expansion's job otherwise
+        const int mt = (int)blockIdx.x / a.tiles_n;
+        const int nt = (int)blockIdx.x - mt * a.tiles_n;
+        if (n_steps <= kChunk) fill_stages<1>(a, mt, nt, ring_s);
+        else fill_stages<kPairStages>(a, mt, nt, ring_s);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // written through the generic proxy, read by the tensor core
+        __syncthreads();
+    }
 
     if (warp < kFirstPromoWarp) {
         setmaxnreg_dec<kRegsPairCtl>();
@@ -114,7 +175,7 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_pair_kernel(const LinArg
             // ------------------------------------------------------------ operand blocks
             const uint32_t empty_s = smem_u32(&g->empty[0]);
             uint32_t s = 0, ph = 1;
-            for (int tile = blockIdx.x; tile < n_tiles && !c->abort_flag; tile += gridDim.x) {
+            for (int tile = blockIdx.x; !DIRECT && tile < n_tiles && !c->abort_flag; tile += gridDim.x) {
                 const int mt = tile / a.tiles_n, nt = tile - mt * a.tiles_n;
                 const uint8_t* a_src = a.a_blocks + (int64_t)mt * n_steps * kBlock;
                 const uint8_t* b_src = a.b_blocks + (int64_t)nt * n_steps * kBHalf;
@@ -154,7 +215,7 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_pair_kernel(const LinArg
                 for (int k0 = 0; k0 < n_steps; k0 += kChunk) {
                     const int mine = n_steps - k0 - 2 * (int)me;         // steps left from this warp's first one on
                     const uint32_t so = s * (kPairStageBytes >> 4);
-                    const bool rf = mbar_test_s(full_s + s * 8, ph);     // the two tests are in flight together
+                    const bool rf = DIRECT || mbar_test_s(full_s + s * 8, ph);    // the two tests are in flight together
                     const bool rt = mbar_test_s(tempty_s, q);
                     if (!rf) wait_cold(full_s + s * 8, ph, c, a.status, 4u);
                     if (mine > 0) {
@@ -165,9 +226,9 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_pair_kernel(const LinArg
                             mma_f8(tm, desc_of(a_lo + so), desc_of(b_lo + so), kIdescN64);
                             if (mine > 1) mma_f8(tm + kN, desc_of(a_lo + so + (kBlock >> 4)), desc_of(b_lo + so + (kBHalf >> 4)), kIdescN64);
                             mma_commit(tfull_s);
-                            mma_commit(empty_s + s * 8);
+                            if (!DIRECT) mma_commit(empty_s + s * 8);
                         }
-                    } else if (elect_one()) {
+                    } else if (!DIRECT && elect_one()) {
                         mma_commit(empty_s + s * 8);
                     }
                     __syncwarp();
@@ -295,16 +356,18 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_pair_kernel(const LinArg
         // stage's scales came with its operands, so they are there when the first accumulator of the stage is.)
         uint32_t d[4];
         auto take_steps = [&](bool ready) {
-            if (!ready) wait_cold(full_s + rs * 8, rph, c, a.status, 7u);
+            if (!DIRECT && !ready) wait_cold(full_s + rs * 8, rph, c, a.status, 7u);
             const uint32_t src = ring_s + rs * kPairStageBytes + kPairScales + (uint32_t)row * 4;
 #pragma unroll
             for (int j = 0; j < 4; ++j) d[j] = lds32(src + j * kScaleBlock);
         };
         auto leave_stage = [&]() {
-            // read through the generic proxy, refilled through the async proxy: only a proxy fence orders the two
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-            mbar_arrive_lane0_s(empty_s + rs * 8, lane);
+            if (!DIRECT) {
+                // read through the generic proxy, refilled through the async proxy: only a proxy fence orders the two
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                mbar_arrive_lane0_s(empty_s + rs * 8, lane);
+            }
             if (++rs == kPairStages) { rs = 0; rph ^= 1; }
         };
 
@@ -508,13 +571,15 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_pair_kernel(const LinArg
 }  // namespace
 
 // a.tiles_n and a.b_blocks are in units of 64 columns here (see ExpandArgs::b_rows).
-tdq_status launch_linear_pair(const LinArgs& a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, bool dbg, cudaStream_t stream) {
-    constexpr int kInst = 12;
+tdq_status launch_linear_pair(const LinArgs& a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, bool dbg, bool direct,
+                              cudaStream_t stream) {
+    constexpr int kInst = 14;
     void (*const kernels[kInst])(LinArgs, CUtensorMap) = {
         w4a4_pair_kernel<false, false, 1>, w4a4_pair_kernel<true, false, 1>, w4a4_pair_kernel<false, true, 1>, w4a4_pair_kernel<true, true, 1>,
         w4a4_pair_kernel<false, false, 2>, w4a4_pair_kernel<true, false, 2>, w4a4_pair_kernel<false, true, 2>, w4a4_pair_kernel<true, true, 2>,
-        w4a4_pair_kernel<false, false, 4>, w4a4_pair_kernel<true, false, 4>, w4a4_pair_kernel<false, true, 4>, w4a4_pair_kernel<true, true, 4>};
-    const int inst = (ybf ? 1 : 0) + (dbg ? 2 : 0) + 4 * (a.steps_per_grp >> 1);
+        w4a4_pair_kernel<false, false, 4>, w4a4_pair_kernel<true, false, 4>, w4a4_pair_kernel<false, true, 4>, w4a4_pair_kernel<true, true, 4>,
+        w4a4_pair_kernel<false, false, 1, true>, w4a4_pair_kernel<true, false, 1, true>};
+    const int inst = direct ? 12 + (ybf ? 1 : 0) : (ybf ? 1 : 0) + (dbg ? 2 : 0) + 4 * (a.steps_per_grp >> 1);
     if (inst >= kInst) return TDQ_ERR_UNSUPPORTED;
     void (*const kernel)(LinArgs, CUtensorMap) = kernels[inst];
     const uint32_t smem = kPairCtrl + kPairStages * kPairStageBytes + 1024 + 2 * (ybf ? kPairBoxBF16 : kPairBoxF32) + 2 * kN * 4;

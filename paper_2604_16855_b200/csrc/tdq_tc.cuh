@@ -71,6 +71,7 @@ struct LinArgs {
     int32_t y_f16;             // 16-bit output is fp16 (else bf16); the kernels' 16-bit instances serve both
     // resident A without the fused producer: the promotion warps unpack the item's codes themselves
     const uint8_t* xcodes;
+    const uint8_t* wcodes;
     const float* xscale;
     int32_t row_bytes;         // I_pad / 2
     int32_t unpack_a;
@@ -104,8 +105,9 @@ struct Plan {
 // The g = 32 kernel (tdq_linear_g32.cu); the caller has run the operand expansion and built the plan and the map.
 // One accumulator per output element over the whole contraction (tdq_linear_one.cu).
 tdq_status launch_linear_one(LinArgs a, const CUtensorMap& ymap, int n_sm, int dev, bool i8, bool ybf, cudaStream_t stream);
-tdq_status launch_linear_pair(const LinArgs& a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, bool dbg,
-                                  cudaStream_t stream);   // tiles of 128 x 64, tdq_linear_pair.cu
+constexpr int kPairRing = 12;   // K-steps that its ring of operands holds
+tdq_status launch_linear_pair(const LinArgs& a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, bool dbg, bool direct,
+                              cudaStream_t stream);   // tiles of 128 x 64, tdq_linear_pair.cu
 tdq_status launch_linear_g32(const LinArgs& a, const CUtensorMap& ymap, uint32_t smem_bytes, unsigned grid, bool ybf,
                              bool dbg, cudaStream_t stream);
 
