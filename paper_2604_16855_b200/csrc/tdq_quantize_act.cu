@@ -456,6 +456,8 @@ cudaError_t launch_ragged(const ActArgs& a, cudaStream_t st) {
 // one image: the 32 channel rows are read with coalesced loads into a shared-memory tile, then
 // thread t gathers position t's 32 channels down the tile's columns and quantizes them like any
 // other group.  Codes and scales come out token-major, [B*H*W, C/2] and [B*H*W, C/32].
+// A programmatic dependent like the other quantizers: its blocks are in place when the kernel before it ends, and the linear
+// layer behind it sets up under its tail ([8, 256, 48, 48] bf16 6.36 -> 5.97 us, [1, 64, 56, 56] fp32 3.17 -> 2.76).
 
 struct NchwArgs {
     ActArgs a;          // x, K, k_zr, seven_tau, flags, codes, scale, offset
@@ -476,6 +478,8 @@ __global__ void __launch_bounds__(kFastThreads) act_g32_nchw_kernel(NchwArgs n) 
     const int64_t b = blockIdx.z;
     const uint8_t* img = reinterpret_cast<const uint8_t*>(a.x) + ((b * a.C + (int64_t)k * 32) * n.HW + s0) * esz;
     const int64_t left = n.HW - s0;                            // positions from s0 to the end of the image
+    pdl_wait();
+    pdl_trigger();
     if (n.vec_ok) {
 #pragma unroll
         for (int j = 0; j < 32 * kVecPerRow / kFastThreads; ++j) {
@@ -519,12 +523,11 @@ template <bool BF16>
 cudaError_t launch_nchw(const NchwArgs& n, int64_t B, cudaStream_t st) {
     dim3 grid((unsigned)((n.HW + kFastThreads - 1) / kFastThreads), (unsigned)n.a.K, (unsigned)B);
     switch (n.a.k_zr) {
-#define TDQ_CASE(KZ) case KZ: act_g32_nchw_kernel<BF16, KZ><<<grid, kFastThreads, 0, st>>>(n); break;
+#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_nchw_kernel<BF16, KZ>, grid, dim3(kFastThreads), 0, st, n);
         TDQ_CASE(4) TDQ_CASE(7) TDQ_CASE(10) TDQ_CASE(13) TDQ_CASE(16) TDQ_CASE(32)
 #undef TDQ_CASE
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------------------------
