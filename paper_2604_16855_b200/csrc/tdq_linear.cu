@@ -24,7 +24,11 @@
 //   The power of two is folded into the output-channel scale in the epilogue; both routes
 //   give bit-identical integer sums and the same float sequence.
 //
-// Two kernels per call:
+// This file prepares every call (linear_impl) and picks the kernel; the one below is the general form.  Others: g = 32, and
+// 64 and 128 where tiles are few or short, tdq_linear_pair.cu; g = 32 on long contractions tdq_linear_g32.cu; one accumulator
+// per output tdq_linear_one.cu.
+//
+// Two kernels per call (one for the small layers that tdq_linear_pair.cu expands itself):
 //   1. expand_kernel   rewrites the packed nibbles of both operands as operand bytes, in 128-row
 //      x 32-code blocks laid out in the tensor core's K-major core-matrix order (8 rows x 16
 //      bytes contiguous), and regroups the activation scales as [row block][group][128 rows].
@@ -1273,11 +1277,14 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
 
     if (use_pair) {
         a.tiles_n = (int32_t)((O + 63) / 64);
-        // Few groups and one tile per block: the kernel expands its own operands, and the call is one launch.  Quantizer and
+        // Few groups and few tiles: one block per tile, which expands its own operands, and the call is one launch.  Quantizer and
         // linear layer, us: 256 x 64 -> 64 fp32 9.1 -> 7.2, 9216 x 64 -> 128 10.6 -> 7.4, 18432 x 128 -> 128 13.3 -> 10.6,
         // 2000 x 192 -> 192 9.25 -> 7.6, 9217 x 147 -> 63 15.7 -> 13.4.  With more tiles than blocks a block would have to
-        // refill its ring with nothing under way (9216 x 320 -> 320, 360 tiles: 16.5 -> 18.5).
-        if (use_g32 && !dbg && p.n_steps <= kPairRing && p.tiles_m * a.tiles_n <= 2 * n_sm)
+        // refill its ring with nothing under way (9216 x 320 -> 320, 360 tiles: 16.5 -> 18.5), and each block column would
+        // expand the rows again.  A layer with one block column and few groups gains up to two rounds of blocks (73728 x 64
+        // -> 64 18.7 -> 17.0, 65536 x 160 -> 64 26.5 -> 23.8; 73728 x 256 -> 64 32.4 -> 33.1, 200000 x 128 -> 64 46.6 -> 50.7).
+        const int64_t tiles = p.tiles_m * a.tiles_n;
+        if (use_g32 && !dbg && p.n_steps <= kPairRing && (tiles <= 2 * n_sm || (a.tiles_n == 1 && p.n_steps <= 6 && tiles <= 4 * n_sm)))
             return launch_linear_pair(a, ymap, n_sm, dev, ybf, false, true, stream);
     }
     const unsigned pieces = (unsigned)((e.tiles_m + e.tiles_n) * p.n_chunks);

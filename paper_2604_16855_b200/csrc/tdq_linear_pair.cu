@@ -587,7 +587,7 @@ tdq_status launch_linear_pair(const LinArgs& a, const CUtensorMap& ymap, int n_s
     static std::atomic<uint64_t> smem_done[kInst];
     if (allow_smem(kernel, 113 * 1024, smem_done[inst], dev) != cudaSuccess) return TDQ_ERR_CUDA;
     const int64_t tiles = (int64_t)a.tiles_m * a.tiles_n;
-    const unsigned grid = (unsigned)(tiles < 2 * n_sm ? tiles : 2 * n_sm);
+    const unsigned grid = (unsigned)(direct || tiles < 2 * n_sm ? tiles : 2 * n_sm);
     if (launch_pdl(kernel, dim3(grid), dim3(kPairThreads), smem, stream, a, ymap) != cudaSuccess) return TDQ_ERR_CUDA;
     g_launch_count.fetch_add(1, std::memory_order_relaxed);
     return TDQ_OK;

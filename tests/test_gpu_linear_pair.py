@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("M,C,O", [(1, 32, 1), (127, 32, 64), (128, 64, 65), (129, 96, 63), (300, 128, 130), (257, 160, 4), (130, 192, 200),
                                    (200, 224, 64), (140, 256, 127), (20000, 64, 129), (6000, 288, 1028), (130, 1536, 72), (130, 1568, 72),
-                                   (40, 2048, 260), (3000, 2048, 1000), (12000, 768, 60), (9000, 512, 384), (30000, 384, 64), (140, 384, 65), (260, 416, 65)])
+                                   (40, 2048, 260), (3000, 2048, 1000), (12000, 768, 60), (9000, 512, 384), (30000, 384, 64), (140, 384, 65), (260, 416, 65), (50001, 192, 63)])
 @pytest.mark.parametrize("g", [32, 64, 128])
 def test_shapes(M, C, O, g):
     from paper_2604_16855_b200 import tdq
