@@ -82,8 +82,10 @@ void tdq_default_act_params(tdq_act_params* p /* HOST, out */);
  *              row_stride_elems % 8 == 0 and g == 32 takes the fast kernels, whatever the two
  *              ranks (the maximum as base radius with any zero-bin rank, and base ranks 29-31
  *              with zero-bin rank 7, have kernels of their own; any other pair runs a kernel
- *              that takes its ranks at run time, about a fifth slower); anything else takes a
- *              much slower general kernel with the same results.
+ *              that takes its ranks at run time, about a fifth slower).  Other rows and channel
+ *              counts at g = 32, and every g that is a multiple of 8, have one-pass kernels
+ *              too (loads are 16 bytes wide where the rows allow it); a g that is not a multiple
+ *              of 8 takes a much slower general kernel.  The results are the same.
  *   codes      [B*N, C_pad/2] bytes; byte j of a row holds channel 2j in its low nibble
  *              and channel 2j+1 in its high nibble, two's complement.
  *   scale      [B*N, K] float32, Delta_k.
