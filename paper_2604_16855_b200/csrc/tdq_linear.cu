@@ -1155,9 +1155,10 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     // then written in two passes of 16 columns; the ring gets the other 32 KB.  Both need the bulk tensor store.
     const int64_t y_esz = y_dtype == TDQ_BF16 ? 2 : 4;
     // (The copy engine clips at the edges of y in whole 16-byte pieces: a last column off that grid, in a y with a padded
-    // row pitch, would have zeros written behind it.)
-    const bool y_tma = reinterpret_cast<uintptr_t>(y) % 16 == 0 && (y_row_stride * y_esz) % 16 == 0 && (O * y_esz) % 16 == 0 &&
-                       O <= INT32_MAX && M <= INT32_MAX;
+    // row pitch, would have zeros written behind it.  A tensor map holds row pitches below 2^40 bytes; only a y of one row, whose
+    // pitch addresses nothing, can come with a larger one.)
+    const bool y_tma = reinterpret_cast<uintptr_t>(y) % 16 == 0 && y_row_stride < ((int64_t)1 << 40) / y_esz &&
+                       (y_row_stride * y_esz) % 16 == 0 && (O * y_esz) % 16 == 0 && O <= INT32_MAX && M <= INT32_MAX;
     const bool half_strips = y_tma && y_dtype == TDQ_F32 && !fx && !acc_debug && group_size >= 128;
     const bool narrow_strips = y_tma && (y_dtype == TDQ_BF16 || half_strips);
     // several instructions chain into one slot: keep the integer accumulator (the power-of-two variant
@@ -1302,7 +1303,8 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
 
     const int64_t items = p.tiles_m * p.n_parts;
     const unsigned grid = (unsigned)(items < n_sm ? items : n_sm);
-    if (use_one) return launch_linear_one(a, ymap, n_sm, dev, i8, ybf, stream);
+    // The cluster kernel and the one for long contractions at g = 32 can only write y through the map; the others also without.
+    if (use_one && a.tma_ok) return launch_linear_one(a, ymap, n_sm, dev, i8, ybf, stream);
     if (use_pair) return launch_linear_pair(a, ymap, n_sm, dev, ybf, dbg, false, stream);
     if (use_g32 && a.tma_ok) return launch_linear_g32(a, ymap, p.smem_bytes, grid, ybf, dbg, stream);
     if (launch_pdl(kernel, dim3(grid), dim3(kThreads), p.smem_bytes, stream, a, ymap) != cudaSuccess) return TDQ_ERR_CUDA;

@@ -53,3 +53,28 @@ def test_one_group(M, C, O):
                                      (4100, 4096, 1032, 1024), (3000, 480, 1032, 160)])
 def test_several_groups(M, C, O, g):
     _check(M, C, O, g, False)
+
+
+@pytest.mark.parametrize("C,g,pow2", [(32, 32, True), (64, 64, False), (96, 96, False), (96, 32, True), (256, 256, False), (64, 32, False)])
+def test_one_row_of_any_pitch(C, g, pow2):
+    """A y of one row may come with a pitch (2^40 bytes and more) that no tensor map holds: the same numbers, by a kernel that
+    writes without one.  (The contractions of fewer than 128 channels went to the cluster kernel with an empty map.)"""
+    from paper_2604_16855_b200 import tdq
+    O = 16384
+    rng = np.random.default_rng(C)
+    x = torch.from_numpy(rng.standard_normal((1, C)).astype(np.float32)).cuda()
+    xc, xs = tdq.quantize_act(x, tdq.act_params(g=g, flags=7 if pow2 else 3))
+    wc, ws = tdq.quantize_weight(torch.from_numpy(si.weights(rng, O, C)).cuda(), pad_to=g)
+    fn = tdq.w4a4_linear_pow2 if pow2 else tdq.w4a4_linear
+    wsp = tdq.linear_workspace(1, C, O, g, "cuda")
+    terms = C if pow2 else C // g                            # rounded additions per output
+    want = oracle.w4a4_linear(xc.cpu().numpy(), xs.cpu().numpy(), wc.cpu().numpy(), ws.cpu().numpy(), g=g)
+    for dt in (torch.float32, torch.bfloat16):
+        for pitch in (O, 1 << 40, 1 << 61):
+            buf = torch.full((O + 8,), 3.0, dtype=dt, device="cuda")
+            y = fn(xc, xs, wc, ws, g=g, y=buf[:O].as_strided((1, O), (pitch, 1)), workspace=wsp)
+            assert y.stride(0) == pitch and tdq.workspace_status(wsp) == (tdq.OK, 0)
+            assert bool((buf[O:] == 3.0).all())
+            err = np.abs(buf[:O].float().cpu().numpy()[None].astype(np.float64) - want["y_d"])
+            half_ulp = 0.0 if dt == torch.float32 else 2.0 ** -8 * np.abs(want["y_d"])
+            assert (err <= np.maximum(1e-5 * np.abs(want["y_d"]), (terms + 2) * 2.0 ** -24 * want["t_abs"]) + half_ulp).all()
