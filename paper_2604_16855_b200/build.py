@@ -1,5 +1,5 @@
 """Builds libtdq.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _tdq_host.so (the Python binding's host
-side, which reads torch tensors in C++) with g++.
+side, which reads torch tensors in C++) with g++, where there is a PyTorch and a C++ compiler for it.
 
     python -m paper_2604_16855_b200.build [--force] [--verbose]
 
@@ -9,6 +9,7 @@ travels with the source tree; nothing is installed into site-packages.
 from __future__ import annotations
 
 import os
+import shutil
 import subprocess
 import sys
 from concurrent.futures import ThreadPoolExecutor
@@ -25,14 +26,30 @@ FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std
          "-Xcompiler", "-fPIC", "--ftz=false", "--prec-div=true", "--prec-sqrt=true"]
 
 
-def _deps_mtime(headers_only: bool = False):
-    """When the newest source (or header, which every source may include) was written."""
-    newest = 0.0
+def _newest(keep) -> float:
+    """When the newest file of the two source folders that `keep` names, or this one, was written."""
+    newest = os.path.getmtime(os.path.abspath(__file__))
     for root in (CSRC, os.path.join(os.path.dirname(HERE), "include")):
         for name in os.listdir(root):
-            if not headers_only or not name.endswith((".cu", ".cpp")):
+            if keep(name):
                 newest = max(newest, os.path.getmtime(os.path.join(root, name)))
-    return max(newest, os.path.getmtime(os.path.abspath(__file__)))
+    return newest
+
+
+def _fresh(path: str, newest: float) -> bool:
+    return os.path.exists(path) and os.path.getmtime(path) >= newest
+
+
+def _host_missing() -> str:
+    """What the extension module needs and this machine has not got ("" when it has everything)."""
+    try:
+        import torch
+    except ImportError:
+        return "PyTorch"
+    if torch.version.cuda is None:
+        return "a PyTorch with CUDA"
+    cxx = os.environ.get("CXX", "g++")
+    return "" if shutil.which(cxx) else cxx
 
 
 def _compile_host():
@@ -56,17 +73,30 @@ def _compile_host():
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    newest = _deps_mtime()
-    if not force and all(os.path.exists(f) and os.path.getmtime(f) >= newest for f in (LIB, HOST)):
-        return LIB
+    """Builds what is older than its sources and returns the path of libtdq.so.  The library needs nvcc alone; where PyTorch
+    or a C++ compiler is missing, the binding's extension module is left out (and an older one removed, so that it
+    cannot be loaded against another library): callers of the C ABI do not need it."""
+    if force or not _fresh(LIB, _newest(lambda name: not name.endswith(".cpp"))):
+        _compile_lib(force, verbose)
+    if force or not _fresh(HOST, _newest(lambda name: not name.endswith((".cu", ".cuh", ".inc")))):
+        missing = _host_missing()
+        if not missing:
+            _compile_host()
+        else:
+            if os.path.exists(HOST):
+                os.remove(HOST)
+            sys.stderr.write("%s is missing: %s is not built, the C library is complete without it\n" % (missing, os.path.basename(HOST)))
+    return LIB
+
+
+def _compile_lib(force: bool, verbose: bool):
     os.makedirs(OBJ, exist_ok=True)
     extra = ["-Xptxas", "-v"] if verbose else []
-    headers = _deps_mtime(headers_only=True)
+    headers = _newest(lambda name: not name.endswith((".cu", ".cpp")))
 
     def compile_one(src):
         obj = os.path.join(OBJ, src.replace(".cu", ".o"))
-        if not (force or verbose) and os.path.exists(obj) and \
-                os.path.getmtime(obj) >= max(headers, os.path.getmtime(os.path.join(CSRC, src))):
+        if not (force or verbose) and _fresh(obj, max(headers, os.path.getmtime(os.path.join(CSRC, src)))):
             return obj
         cmd = [NVCC] + FLAGS + extra + ["-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
@@ -82,8 +112,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
     subprocess.check_call([NVCC, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp] + objs +
                           ["-cudart", "static"])
     os.replace(tmp, LIB)
-    _compile_host()
-    return LIB
 
 
 if __name__ == "__main__":
