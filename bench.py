@@ -77,7 +77,9 @@ def profiled_traffic(kernel, workload_name, files):
     return None
 
 
-LINEAR_G32_SOURCES = ["tdq_linear_g32.cu", "tdq_tc.cuh"]
+# the kernel that the default workload's linear layer runs, and the files its profile summary is bound to
+LINEAR_KERNEL = "w4a4_pair_kernel"
+LINEAR_KERNEL_SOURCES = ["tdq_linear_pair.cu", "tdq_tc.cuh"]
 
 
 def load_peaks():
@@ -693,7 +695,7 @@ def run_tdq(args):
             if l_kernel["bound"] == "hbm":
                 roof = dict(kernel="tdq_w4a4_linear", bound="hbm", achieved=l_gbs, peak=peaks["hbm_gbs"],
                             unit="GB/s", frac=l_gbs / peaks["hbm_gbs"],
-                            traffic=profiled_traffic("w4a4_g32_kernel", args.workload, LINEAR_G32_SOURCES))
+                            traffic=profiled_traffic(LINEAR_KERNEL, args.workload, LINEAR_KERNEL_SOURCES))
             else:
                 roof = dict(kernel="tdq_w4a4_linear", bound="tensor", achieved=l_tops, peak=int8_peak,
                             unit="TOP/s", frac=l_tops / int8_peak, traffic=None)
