@@ -1218,7 +1218,7 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     // SMs (1000 x 2048 -> 256 at 64 14.9 -> 12.0 us).  4616 x 768 -> 3072 at 128 is level, 18464 rows 87 -> 99 us.
     const bool use_pair_wide = !pow2_steps && !fx && !use_one && (group_size == 64 || group_size == 128) && p.tiles_m * p.tiles_n <= INT32_MAX / 4 &&
                                (p.n_steps <= 16 || O <= 64 || p.tiles_m * p.tiles_n <= n_sm);
-    const bool use_pair = use_pair_wide || (use_g32 && (!y_tma || p.n_steps <= 48 || p.tiles_m * p.tiles_n * 4 <= n_sm));
+    const bool use_pair = use_pair_wide || (use_g32 && (!y_tma || p.n_steps <= kPairMaxSteps || p.tiles_m * p.tiles_n * 4 <= n_sm));
     const bool unpack_a = !fx && !pow2_steps && !use_pair && !use_one && p.a_resident && steps_per_item >= 256;
     e.tiles_m = (fx || unpack_a) ? 0 : (int32_t)p.tiles_m;   // then only the weights are expanded here
     e.tiles_n = (int32_t)p.tiles_n;

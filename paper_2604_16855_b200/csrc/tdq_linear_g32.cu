@@ -1,6 +1,6 @@
 // The W4A4 linear layer at the paper's group size g = 32 (Algorithm S1 step 10 with Eq. 9 and Eq. 4
-// substituted) for long contractions, with y that bulk tensor stores can write (16-byte aligned base and row pitch); shorter
-// ones go to tdq_linear_pair.cu:
+// substituted) for long contractions (more than kPairMaxSteps groups), with y that bulk tensor stores can write (16-byte
+// aligned base and row pitch); the others go to tdq_linear_pair.cu:
 //
 //   acc[m,o,k] = sum_{i in group k} q_x[m,i] q_w[o,i]      one tcgen05.mma (E4M3 operands, exact) per group
 //   y[m,o]     = s_o * sum_k Delta[m,k] * acc[m,o,k] + b_o  fp32 in registers ("promotion")
@@ -22,10 +22,12 @@
 //   * a lone warp runs dependent scalar code at one instruction every several clocks, so the per-group
 //     bookkeeping of the tensor-core side is spread over four MMA-issuing warps, one per TMEM slot, and
 //     every wait in a hot loop is one barrier test with the bounded, sleeping wait out of line.
-//   Warps 0-1 stream the weight blocks (and A when it does not stay resident), warps 2-5 issue the
-//   MMAs (warp 2 + j owns TMEM slot j), warp 6 issues the stores; warp 7 only keeps the register
-//   partitions of the four schedulers even.  Operand blocks, the ring, the item buffers and the bounded
-//   waits are those of the general kernel (tdq_linear.cu).
+//   Warps 0-1 stream the operand blocks of A and B, warps 2-5 issue the MMAs (warp 2 + j owns TMEM
+//   slot j), warp 6 issues the stores; warp 7 only keeps the register partitions of the four
+//   schedulers even.  A work item is one 128-row block with a range of column tiles; its steps Delta
+//   (all groups) are in shared memory while it is worked on.  At this length A never fits beside them
+//   (the assertion below), so it streams with B.  Operand blocks, the ring and the bounded waits are
+//   those of the general kernel (tdq_linear.cu).
 #include "tdq_tc.cuh"
 
 namespace tdq {
@@ -42,6 +44,10 @@ constexpr int kRegsCtl = 40, kRegsP = 208;                  // 256 * 40 + 256 * 
 constexpr uint32_t kBoxF32 = 128 * 128, kBoxBF16 = 128 * 64;   // one 32-column box of 128 rows in the staging area
 static_assert(2 * kBN * 4 <= kWsbBytes, "the tile's channel scales and biases outgrew their reservation");
 static_assert(4 * kBoxF32 <= kStagingBytes, "the staged tile outgrew its reservation");
+// make_plan keeps A resident when three stages of B fit beside it; from kPairMaxSteps + 1 groups on they do not, with the
+// smallest staging area (16-bit output) either
+static_assert(kSmemLimit - (1024 + kCtrlBytes + (kPairMaxSteps + 1) * kScaleBlock + kStagingBytes / 2 + kWsbBytes) -
+                      (kPairMaxSteps + 1) * kBlock < 3 * kChunk * kBlock, "this kernel streams A");
 
 // Waits for this thread's outstanding TMEM loads.  The landing registers are passed through as operands so
 // that no use of them can be scheduled above the wait.
@@ -72,21 +78,16 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
     extern __shared__ __align__(128) uint8_t smem_raw[];
     Ctrl* c = reinterpret_cast<Ctrl*>(smem_raw);
     const uint32_t sm_s = smem_u32(smem_raw);
-    // item buffer b: [Kg][128] floats of the item's scales, then its [n_steps] operand blocks if resident
-    const uint32_t ibuf_s = sm_s + kCtrlBytes;
-    const uint32_t a_in_ibuf = (uint32_t)a.Kg * kScaleBlock;
+    const uint32_t scales_s = sm_s + kCtrlBytes;            // [Kg][128] floats: the steps of the work item's rows
     const uint32_t ring_s = sm_s + a.ring_off;
     const uint32_t stage_s = (sm_s + a.staging_off + 1023u) & ~1023u;   // the swizzle patterns repeat every 1024 bytes
     const int t = threadIdx.x, warp = uniform_warp(), lane = t & 31;
-    const bool resident = a.a_resident != 0;
 
     if (t == 0) {
         for (int i = 0; i < kMaxStages; ++i) { mbar_init(&c->full[i], 1); mbar_init(&c->empty[i], kMmaWarps); }
         for (int i = 0; i < kSlots; ++i) { mbar_init(&c->tfull[i], 1); mbar_init(&c->tempty[i], kPWarps); }
-        for (int i = 0; i < kMaxItemBufs; ++i) {
-            mbar_init(&c->a_full[i], a.unpack_a ? kPWarps : 1);
-            mbar_init(&c->a_empty[i], kMmaWarps + kPWarps);
-        }
+        mbar_init(&c->a_full[0], 1);
+        mbar_init(&c->a_empty[0], kMmaWarps + kPWarps);
         mbar_init(&c->sfull, kPWarps);
         mbar_init(&c->sfree, 1);
         c->abort_flag = 0;
@@ -115,31 +116,24 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
         if (warp < kProdWarps) {
             // ------------------------------------------------------------ producers: alternate ring stages
             uint32_t sc = 0, s = 0, ph = 0;   // stage counter, its ring slot and phase
-            uint32_t ib = 0, iu = 0;          // item buffer and its phase
+            uint32_t iu = 0;                  // phase of the item's scales
             bool ok = true;
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
                 const int mt = item / a.n_parts, part = item % a.n_parts;
                 const uint8_t* a_src = a.a_blocks + (int64_t)mt * a.n_steps * kBlock;
-                if (warp == 0 && !a.unpack_a) {
-                    wait_hot(smem_u32(&c->a_empty[ib]), iu ^ 1, c, a.status, 1u);
+                if (warp == 0) {
+                    wait_hot(smem_u32(&c->a_empty[0]), iu ^ 1, c, a.status, 1u);
                     if (c->abort_flag) break;
                     if (lane == 0) {
                         const uint32_t sbytes = (uint32_t)a.Kg * kScaleBlock;
-                        const uint32_t scales_s = ibuf_s + ib * a.ibuf_bytes, ares_s = scales_s + a_in_ibuf;
-                        mbar_expect_tx(&c->a_full[ib], sbytes + (resident ? (uint32_t)a.n_steps * kBlock : 0u));
+                        mbar_expect_tx(&c->a_full[0], sbytes);
                         const uint8_t* s_src = a.s_blocks + (int64_t)mt * a.Kg * kScaleBlock;
                         for (uint32_t off = 0; off < sbytes; off += 16384u)
-                            bulk_load(scales_s + off, s_src + off, min(16384u, sbytes - off), &c->a_full[ib]);
-                        if (resident)
-                            for (int kc = 0; kc < n_chunks; ++kc) {
-                                const int nk = min(kChunk, a.n_steps - kc * kChunk);
-                                bulk_load(ares_s + kc * kChunk * kBlock, a_src + (int64_t)kc * kChunk * kBlock,
-                                          (uint32_t)nk * kBlock, &c->a_full[ib]);
-                            }
+                            bulk_load(scales_s + off, s_src + off, min(16384u, sbytes - off), &c->a_full[0]);
                     }
                     __syncwarp();
                 }
-                if (++ib == (uint32_t)a.n_ibuf) { ib = 0; iu ^= 1; }
+                iu ^= 1;
                 for (int nt = part_begin(part); nt < part_begin(part + 1) && ok; ++nt) {
                     const uint8_t* b_src = a.b_blocks + (int64_t)nt * a.n_steps * kBlock;
                     for (int kc = 0; kc < n_chunks; ++kc, ++sc) {
@@ -149,11 +143,10 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
                             if (lane == 0) {
                                 const int nk = min(kChunk, a.n_steps - kc * kChunk);
                                 const uint32_t stage = ring_s + s * a.stage_bytes;
-                                mbar_expect_tx(&c->full[s], (uint32_t)nk * kBlock * (resident ? 1u : 2u));
+                                mbar_expect_tx(&c->full[s], (uint32_t)nk * kBlock * 2u);
                                 bulk_load(stage, b_src + (int64_t)kc * kChunk * kBlock, (uint32_t)nk * kBlock, &c->full[s]);
-                                if (!resident)
-                                    bulk_load(stage + kChunk * kBlock, a_src + (int64_t)kc * kChunk * kBlock,
-                                              (uint32_t)nk * kBlock, &c->full[s]);
+                                bulk_load(stage + kChunk * kBlock, a_src + (int64_t)kc * kChunk * kBlock, (uint32_t)nk * kBlock,
+                                          &c->full[s]);
                             }
                             __syncwarp();
                         }
@@ -169,21 +162,20 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
             const uint32_t lane0 = lane == 0 ? 1u : 0u;
             const uint32_t ring_lo = desc_lo(ring_s);
             const uint32_t stage_step = a.stage_bytes >> 4, n_stages = (uint32_t)a.n_stages;
-            const uint32_t a_in_stage = resident ? 0u : (uint32_t)(kChunk * (kBlock >> 4));
+            constexpr uint32_t a_in_stage = kChunk * (kBlock >> 4);
             const uint32_t full_s = smem_u32(&c->full[0]), empty_s = smem_u32(&c->empty[0]);
             const uint32_t tfull_me = smem_u32(&c->tfull[me]), tempty_me = smem_u32(&c->tempty[me]);
             const uint32_t tm_me = tmem_base + me * kBN, off_me = me * (kBlock >> 4);
             const int n_steps = a.n_steps;
-            uint32_t s = 0, ph = 0, ib = 0, iu = 0;
+            uint32_t s = 0, ph = 0, iu = 0;
             uint32_t q_me = 1;             // parity to wait for on tempty; a fresh barrier passes parity 1
             for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
                 const int part = item % a.n_parts;
                 const int n_tiles = part_begin(part + 1) - part_begin(part);
-                wait_hot(smem_u32(&c->a_full[ib]), iu, c, a.status, 6u);
+                wait_hot(smem_u32(&c->a_full[0]), iu, c, a.status, 6u);
                 if (c->abort_flag) break;
-                const uint32_t ares_lo = desc_lo(ibuf_s + ib * a.ibuf_bytes + a_in_ibuf);
+                iu ^= 1;
                 for (int tl = 0; tl < n_tiles; ++tl) {
-                    uint32_t a_lo = ares_lo + off_me;   // resident: walks through the item's A blocks
 #pragma unroll 1
                     for (int k0 = 0; k0 < n_steps; k0 += kChunk) {
                         wait_hot(full_s + s * 8, ph, c, a.status, 4u);
@@ -195,20 +187,18 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
                         tc_fence_after();
                         if (elect_one()) {
                             if (k0 + (int)me < n_steps) {
-                                mma_f8(tm_me, desc_of(resident ? a_lo : b_lo + a_in_stage), desc_of(b_lo), kIdescF8);
+                                mma_f8(tm_me, desc_of(b_lo + a_in_stage), desc_of(b_lo), kIdescF8);
                                 mma_commit(tfull_me);
                             }
                             mma_commit(empty_s + s * 8);
                         }
                         __syncwarp();
-                        a_lo += kChunk * (kBlock >> 4);
                         if (++s == n_stages) { s = 0; ph ^= 1; }
                     }
                     if (c->abort_flag) break;
                 }
                 if (c->abort_flag) break;
-                mma_commit_if(lane0, smem_u32(&c->a_empty[ib]));
-                if (++ib == (uint32_t)a.n_ibuf) { ib = 0; iu ^= 1; }
+                mma_commit_if(lane0, smem_u32(&c->a_empty[0]));
             }
         } else if (warp == kStoreWarp) {
             // ------------------------------------------------------------ output stores, channel scales
@@ -273,8 +263,8 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
         const int row = quarter * 32 + lane;
         const int col0 = half * kPCols;
         const uint32_t wsb_s = stage_s + a.staging_bytes;   // [128] channel scales, [128] biases of the current tile
-        uint32_t ib = 0, iu = 0;                      // item buffer and its phase
-        uint32_t my_scale_s = ibuf_s + (uint32_t)row * 4;   // this row's scales in the current item buffer
+        uint32_t iu = 0;                              // phase of the item's scales
+        const uint32_t my_scale_s = scales_s + (uint32_t)row * 4;   // this row's
 
         uint64_t yacc[kPCols / 2];     // 64 floats of one output row, packed in pairs
         uint32_t va[32], vb[32];       // landing buffers: columns 0-31 and 32-63 of this thread's share of a slot
@@ -291,44 +281,7 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
             const int part = item % a.n_parts;
             nt = part_begin(part);
             nt_end = part_begin(part + 1);
-            const uint32_t scales_s = ibuf_s + ib * a.ibuf_bytes, ares_s = scales_s + a_in_ibuf;
-            my_scale_s = scales_s + (uint32_t)row * 4;
-            if (a.unpack_a) {
-                // Packed codes -> operand bytes, straight into the item buffer: thread pt takes row pt / 2 and
-                // every second K-step from pt % 2 (a warp reads 32 contiguous bytes of each of 16 rows).
-                wait_hot(smem_u32(&c->a_empty[ib]), iu ^ 1, c, a.status, 1u);
-                {
-                    const int pt = pw * 32 + lane, r = pt >> 1;
-                    const int64_t mr = (int64_t)mt * kBM + r;
-                    const uint32_t off = (uint32_t)((r >> 3) * 256 + (r & 7) * 16);
-                    const uint8_t* src = a.xcodes + mr * a.row_bytes;
-#pragma unroll 2
-                    for (int ks = pt & 1; ks < a.n_steps; ks += 2) {
-                        uint4 p4 = make_uint4(0u, 0u, 0u, 0u);
-                        if (mr < a.M) p4 = __ldg(reinterpret_cast<const uint4*>(src + ks * 16));
-                        uint4 c0, c1;
-                        expand8<false>(p4.x, c0.x, c0.y);
-                        expand8<false>(p4.y, c0.z, c0.w);
-                        expand8<false>(p4.z, c1.x, c1.y);
-                        expand8<false>(p4.w, c1.z, c1.w);
-                        const uint32_t dst = ares_s + (uint32_t)ks * kBlock + off;
-                        sts128(dst, c0.x, c0.y, c0.z, c0.w);
-                        sts128(dst + 128, c1.x, c1.y, c1.z, c1.w);
-                    }
-                    // scales: [group][128 rows]; thread pt takes row pt % 128 and every second group
-                    const int rs = pt & (kBM - 1);
-                    const int64_t ms = (int64_t)mt * kBM + rs;
-#pragma unroll 1
-                    for (int k = pt >> 7; k < a.Kg; k += kPWarps * 32 / kBM)
-                        sts32(scales_s + (uint32_t)k * kScaleBlock + (uint32_t)rs * 4,
-                              ms < a.M ? __float_as_uint(__ldg(a.xscale + ms * a.Kg + k)) : 0u);
-                    // written through the generic proxy, read by the tensor core through the async proxy
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    __syncwarp();
-                    mbar_arrive_lane0(&c->a_full[ib], lane);
-                }
-            }
-            wait_hot(smem_u32(&c->a_full[ib]), iu, c, a.status, 7u);
+            wait_hot(smem_u32(&c->a_full[0]), iu, c, a.status, 7u);
         };
         auto begin_tile = [&]() {
             n0 = (int64_t)nt * kBN + col0;
@@ -392,8 +345,8 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
                 // overwrite them through the async proxy, which only a proxy fence orders after the reads
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
-                mbar_arrive_lane0(&c->a_empty[ib], lane);
-                if (++ib == (uint32_t)a.n_ibuf) { ib = 0; iu ^= 1; }
+                mbar_arrive_lane0(&c->a_empty[0], lane);
+                iu ^= 1;
                 item += gridDim.x;
                 if (item < n_items) begin_item();
             }
@@ -484,7 +437,7 @@ __global__ void __launch_bounds__(kThreadsG32, 1) w4a4_g32_kernel(const LinArgs 
                     }
                 }
                 // The next tile's first load runs under the epilogue when it belongs to the same work item; the
-                // first group of another item cannot start before this warp has handed the item's buffers back.
+                // first group of another item cannot start before this warp has handed the item's steps back.
                 const bool same_item = nt + 1 < nt_end;
                 if (same_item) first_load();
                 finish_tile();

@@ -105,7 +105,8 @@ struct Plan {
 // The g = 32 kernel (tdq_linear_g32.cu); the caller has run the operand expansion and built the plan and the map.
 // One accumulator per output element over the whole contraction (tdq_linear_one.cu).
 tdq_status launch_linear_one(LinArgs a, const CUtensorMap& ymap, int n_sm, int dev, bool i8, bool ybf, cudaStream_t stream);
-constexpr int kPairRing = 12;   // K-steps that its ring of operands holds
+constexpr int kPairRing = 12;       // K-steps that the ring of operands of tdq_linear_pair.cu holds
+constexpr int kPairMaxSteps = 48;   // longest contraction it takes at g = 32 where tdq_linear_g32.cu could
 tdq_status launch_linear_pair(const LinArgs& a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, bool dbg, bool direct,
                               cudaStream_t stream);   // tiles of 128 x 64, tdq_linear_pair.cu
 tdq_status launch_linear_g32(const LinArgs& a, const CUtensorMap& ymap, uint32_t smem_bytes, unsigned grid, bool ybf,
