@@ -59,10 +59,6 @@ __device__ __forceinline__ void arrive_cta0_lane0(uint32_t bar_s, int lane) {
         "@p mbarrier.arrive.shared::cluster.b64 _, [ra];\n\t}"
         ::"r"(bar_s), "r"(lane) : "memory");
 }
-__device__ __forceinline__ void wait_one(uint32_t bar_s, uint32_t parity, Ctrl* c, uint32_t* status, uint32_t code) {
-    if (!mbar_test_s(bar_s, parity))
-        mbar_wait_slow(reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(c) + (bar_s - smem_u32(c))), parity, c, status, code);
-}
 template <bool I8>
 __device__ __forceinline__ void mma_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
     if (I8)
@@ -78,16 +74,6 @@ __device__ __forceinline__ void commit_both(uint32_t bar_s) {
                  ::"r"(bar_s), "h"((uint16_t)3) : "memory");
 }
 __device__ __forceinline__ void bulk_wait_group_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
-
-__device__ __forceinline__ void ld_wait_on(uint32_t* v) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
-                   "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]),
-                   "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
-                   "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
-                 :
-                 : "memory");
-}
 
 template <bool I8, bool YBF16>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOneThreads, 1)
@@ -137,7 +123,7 @@ w4a4_one_kernel(const LinArgs a, const __grid_constant__ CUtensorMap ymap) {
 #pragma unroll 1
             for (int k0 = 0; k0 < a.n_steps; k0 += kOneSteps) {
                 const uint32_t bytes = (uint32_t)min(kOneSteps, a.n_steps - k0) * kBlock;
-                wait_one(empty_s + s * 8, ph, c, a.status, 5u);
+                wait_hot(empty_s + s * 8, ph, c, a.status, 5u);
                 if (c->abort_flag) break;
                 if (elect_one()) {
                     mbar_expect_tx(&g->full[s], bytes);
@@ -155,7 +141,7 @@ w4a4_one_kernel(const LinArgs a, const __grid_constant__ CUtensorMap ymap) {
         for (int tile = first; tile < n_tiles && !c->abort_flag; tile += n_clusters)
 #pragma unroll 1
             for (int kc = 0; kc < n_chunks; ++kc) {
-                wait_one(full_s + s * 8, ph, c, a.status, 4u);
+                wait_hot(full_s + s * 8, ph, c, a.status, 4u);
                 if (c->abort_flag) break;
                 __syncwarp();
                 arrive_cta0_lane0(peer_s + s * 8, lane);
@@ -169,11 +155,11 @@ w4a4_one_kernel(const LinArgs a, const __grid_constant__ CUtensorMap ymap) {
         uint32_t s = 0, ph = 0, n = 0;
         for (int tile = first; tile < n_tiles && !c->abort_flag; tile += n_clusters, ++n) {
             const uint32_t slot = n & 1u, d = tmem_base + slot * kOneN;
-            wait_one(tempty_s + slot * 8, ((n >> 1) & 1u) ^ 1u, c, a.status, 3u);
+            wait_hot(tempty_s + slot * 8, ((n >> 1) & 1u) ^ 1u, c, a.status, 3u);
 #pragma unroll 1
             for (int kc = 0; kc < n_chunks; ++kc) {
-                wait_one(full_s + s * 8, ph, c, a.status, 4u);
-                wait_one(peer_s + s * 8, ph, c, a.status, 6u);
+                wait_hot(full_s + s * 8, ph, c, a.status, 4u);
+                wait_hot(peer_s + s * 8, ph, c, a.status, 6u);
                 if (c->abort_flag) break;
                 tc_fence_after();
                 if (elect_one()) {
@@ -217,14 +203,14 @@ w4a4_one_kernel(const LinArgs a, const __grid_constant__ CUtensorMap ymap) {
             }
             __syncwarp();
             const uint32_t slot = n & 1u;
-            wait_one(tfull_s + slot * 8, (n >> 1) & 1u, c, a.status, 2u);
+            wait_hot(tfull_s + slot * 8, (n >> 1) & 1u, c, a.status, 2u);
             tc_fence_after();
             const uint32_t tm = tmem_base + ((uint32_t)(quarter * 32) << 16) + slot * kOneN + half * kOneCols;
             tmem_ld32(tm, va);
 #pragma unroll
             for (int i = 0; i < kOneCols / 32; ++i) {
                 uint32_t* const v = (i & 1) ? vb : va;
-                ld_wait_on(v);
+                tmem_ld_wait_on(v);
                 if (i < kOneCols / 32 - 1) {
                     tmem_ld32(tm + 32 * (i + 1), (i & 1) ? va : vb);
                 } else {

@@ -55,24 +55,6 @@ struct PairCtrl {
 };
 static_assert(sizeof(Ctrl) + sizeof(PairCtrl) <= kPairCtrl, "control block outgrew its reservation");
 
-__device__ __forceinline__ void tmem_ld_wait_on(uint32_t* v) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
-                   "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]),
-                   "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
-                   "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
-                 :
-                 : "memory");
-}
-
-__device__ __forceinline__ void wait_cold(uint32_t bar_s, uint32_t parity, Ctrl* c, uint32_t* status, uint32_t code) {
-    uint64_t* bar = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(c) + (bar_s - smem_u32(c)));
-    mbar_wait_slow(bar, parity, c, status, code);
-}
-__device__ __forceinline__ void wait_hot(uint32_t bar_s, uint32_t parity, Ctrl* c, uint32_t* status, uint32_t code) {
-    if (!mbar_test_s(bar_s, parity)) wait_cold(bar_s, parity, c, status, code);
-}
-
 // The operands of a block's only tile straight from the packed codes (DIRECT; contractions that the ring holds whole): 128 rows
 // of A, 64 of B and the rows' steps, stage by stage.  A lane takes a row, so that the 16-byte stores of a quarter warp fill a
 // core matrix; the loads of neighbouring K-steps share sectors.  STAGES: how many stages' loads are in flight together.

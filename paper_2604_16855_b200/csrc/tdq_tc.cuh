@@ -191,6 +191,17 @@ __device__ __forceinline__ bool mbar_test_s(uint32_t bar_s, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
+// Waits in the hot loops: one test of the barrier; if the phase is not complete yet, the bounded sleeping
+// wait, out of line.  Every lane asks about the same barrier in the same instruction, so the lanes agree
+// without a vote.  A wait that gives up raises the CTA's abort flag (and records its code); the loops look
+// at that flag once per tile, and every later wait returns at once.
+__device__ __forceinline__ void wait_cold(uint32_t bar_s, uint32_t parity, Ctrl* c, uint32_t* status, uint32_t code) {
+    uint64_t* bar = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(c) + (bar_s - smem_u32(c)));
+    mbar_wait_slow(bar, parity, c, status, code);
+}
+__device__ __forceinline__ void wait_hot(uint32_t bar_s, uint32_t parity, Ctrl* c, uint32_t* status, uint32_t code) {
+    if (!mbar_test_s(bar_s, parity)) wait_cold(bar_s, parity, c, status, code);
+}
 __device__ __forceinline__ void mbar_arrive_lane0_s(uint32_t bar_s, int lane) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -305,6 +316,17 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v) {
         : "memory");
 }
 
+// Waits for this thread's outstanding TMEM loads.  The landing registers are passed through as operands so
+// that no use of them can be scheduled above the wait.
+__device__ __forceinline__ void tmem_ld_wait_on(uint32_t* v) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                   "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]),
+                   "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
+                   "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
+                 :
+                 : "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
