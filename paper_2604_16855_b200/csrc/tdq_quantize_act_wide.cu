@@ -2,7 +2,7 @@
 // whole token of 4096 channels), channel counts that are not a multiple of the group, rows without 16-byte alignment.
 // (g = 32 on aligned rows has kernels of its own in tdq_quantize_act.cu.)
 //
-// L lanes of a warp (2 to 32), or all of two or four warps, own a group and hold it in registers: chunk n of 8
+// L lanes of a warp (1 to 32), or all of two or four warps, own a group and hold it in registers: chunk n of 8
 // channels belongs to lane n % (lanes), so a warp reads and writes contiguous pieces.  One pass over memory: 2 or 4 bytes in, 0.5 out per channel.
 //
 // What bounds it is instruction issue, and of that the rank selection.  It is a search for the k-th smallest magnitude
@@ -16,7 +16,9 @@
 // Lanes per group and chunks per lane (NC): as few lanes as keep a lane at four chunks (32 channels), because the
 // probe's bookkeeping and the reduction over the group are paid per lane.  Past 1024 channels two or four warps share a
 // group: a lane with more chunks has the same instruction count, but the straight-line code for 16 chunks ran at 0.47
-// instructions per clock with the instruction cache as its main stall.
+// instructions per clock with the instruction cache as its main stall.  Groups of up to 32 channels follow the same rule,
+// one lane each: 18464 x 768 bf16 at g = 8 143 -> 39 us against four lanes with one chunk each, at g = 16 81 -> 30, at
+// g = 24 56 -> 25, at g = 32 (codes off the 16-byte grid) 43 -> 24.
 //
 // Measured (B200, from a graph, input not in L2) against the bisection kernel with the group in shared memory that served
 // these cases before: 4616 x 768 bf16 at g = 128 65 -> 9 us; 18464 x 768 bf16 at g = 128 24 us (of which the rank
@@ -370,7 +372,10 @@ cudaError_t launch(const WideArgs& w, cudaStream_t st) {
 template <bool BF16>
 cudaError_t pick(const WideArgs& w, cudaStream_t st) {
     const int chunks = w.a.g / 8;
-    if (chunks <= 4) return launch<BF16, 1, 4>(w, st);
+    if (chunks <= 1) return launch<BF16, 1, 1>(w, st);
+    if (chunks <= 2) return launch<BF16, 2, 1>(w, st);
+    if (chunks <= 3) return launch<BF16, 3, 1>(w, st);
+    if (chunks <= 4) return launch<BF16, 4, 1>(w, st);
     if (chunks <= 6) return launch<BF16, 3, 2>(w, st);
     if (chunks <= 8) return launch<BF16, 4, 2>(w, st);
     if (chunks <= 12) return launch<BF16, 3, 4>(w, st);

@@ -50,3 +50,25 @@ def test_many_groups():
     codes, scale = tdq.quantize_act(to_cuda(x, bf16=True), tdq.act_params(g=64), offset=off)
     assert np.array_equal(codes.cpu().numpy(), ref["codes"]) and np.array_equal(scale.cpu().numpy(), ref["scale"])
     assert float(off.abs().max()) == 0.0
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("g", [8, 16, 24, 32])
+def test_one_lane_per_group(g, bf16):
+    """Groups that a single lane holds: a last warp with one group, cut chunks, every load width, codes that are only 4-byte
+    aligned (which at g = 32 is what brings a group here)."""
+    from paper_2604_16855_b200 import tdq
+    rng = np.random.default_rng(100 + g)
+    for M, C, pitch in ((97, g, g), (65, 5 * g, 5 * g + 8), (33, 3 * g - 3, 3 * g + 2), (129, 7 * g - 1, 7 * g + 1), (41, 2 * g + 4, 2 * g + 4)):
+        full = _rows(rng, M, pitch)
+        full = si.f32_to_bf16_bits(full) if bf16 else full
+        x = np.ascontiguousarray(full[:, :C])
+        K = (C + g - 1) // g
+        buf = torch.full((M * K * g // 2 + 20,), 0x55, dtype=torch.uint8, device="cuda")
+        for kw in (dict(), dict(p=0.8, zr=0.5), dict(tau=0.4, zr=1.0)):
+            ref = oracle.quantize_act(x, g=g, **kw)
+            params = tdq.act_params(g=g, tau=kw.get("tau", 1.0), zr=kw.get("zr", 0.2), p=kw.get("p", 1.0))
+            codes, scale = tdq.quantize_act(to_cuda(full, bf16=bf16)[:, :C], params, codes=buf[4:-16].view(M, K * g // 2))
+            rep = compare_quantizer(si.bf16_bits_to_f32(x) if bf16 else x, g, ref, codes.cpu().numpy(), scale.cpu().numpy())
+            assert rep["scale_max_rel"] <= 1e-6, (M, C, kw, rep)
+            assert bool((buf[:4] == 0x55).all()) and bool((buf[-16:] == 0x55).all())
