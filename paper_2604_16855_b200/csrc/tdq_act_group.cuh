@@ -1,6 +1,6 @@
 // The per-group arithmetic of the token-group quantizer's fast path (g = 32, one thread per group):
 // Algorithm S1 steps 2-7 on a group held in registers.  Shared by the stand-alone quantizer
-// kernels and by the linear layer's fused producer.
+// kernels and by the linear layer's fused producer; the kernel for wide groups uses the screen and the quotient.
 #pragma once
 #include <cmath>
 
@@ -29,8 +29,11 @@ namespace {
 
 // True when the binary32 moments prove that 7 tau sigma exceeds cmin by a safe margin, i.e.
 // the C1 bound cannot be the minimum.  s1 = sum x, s2 = sum x^2 over the g elements, inv_g = 1/g.
-// The estimate var = s2/g - mean^2 has relative error below 1e-4 once var >= s2/512, and
-// the test keeps a 1 % margin on the squared radius, so a true result is always right; a
+// A term passes through at most 40 additions whatever the group (32 in one thread at g = 32; in the wide kernel up to 32
+// in a lane, 5 levels of a warp, 3 warps), so with u = 2^-24 and E = E[x^2] the mean is off by at most 40 u sqrt(E), its
+// square by 80 u E, s2 / g by 41 u E, and with the few roundings of the estimate itself var is off by less than
+// 130 u E = 7.8e-6 E.  Asking for var >= E / 16 makes that a relative error below 1.3e-4, and the test keeps a 1 %
+// margin on the squared radius, so a true result is always right; a
 // false one only means the deviation is recomputed exactly.  When the other bounds already put the radius at or below
 // its floor, the floor decides whatever sigma is (the usual case of groups that are mostly zeros or padding).
 __device__ __forceinline__ bool c1_cannot_bind(float s1, float s2, float seven_tau, float cmin, float inv_g = 1.0f / 32.0f) {
@@ -42,7 +45,7 @@ __device__ __forceinline__ bool c1_cannot_bind(float s1, float s2, float seven_t
     return cmin <= kClipFloor || ((var >= ex2 * (1.0f / 16.0f)) && (lhs > rhs) && (rhs >= 1e-30f) && (s2 < 1e37f) && (lhs < 1e37f));
 }
 
-// sigma = Std(x_k) + 1e-12 in binary64, sequentially over the group, rounded to binary32.
+// sigma = Std(x_k) + 1e-12 in binary64, sequentially over the group as the definition's loop does, rounded to binary32.
 template <typename GetF>
 __device__ __forceinline__ float sigma_exact32(GetF get) {
     double s = 0.0;

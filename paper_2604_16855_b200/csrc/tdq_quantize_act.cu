@@ -27,8 +27,11 @@
 // is the correctly rounded quotient unless x / Delta lies within that distance of a midpoint
 // between two floats; a quotient that is exactly a multiple of 0.5 is reproduced exactly.
 // The group standard deviation only matters when the C1 bound can be the minimum; a cheap
-// binary32 test with a 0.5 % margin proves it cannot for almost every zero-mean group, and
-// the other groups recompute it in binary64 in the sequential order of the definition.
+// binary32 test with a 1 % margin on the squared radius (a bf16 one with a wider margin on bf16 input at g = 32) proves
+// it cannot for almost every zero-mean group, and the other groups recompute it in binary64: at g = 32, and for groups
+// that one lane holds, in the sequential order of the definition; where several lanes share a group (act_wide_kernel,
+// act_generic_kernel) lane by lane and then across the lanes.  The two orders differ by at most g 2^-53 relative, which
+// moves the binary32 deviation by one unit in its last place in fewer than one group in 2^29 / g.
 #include <cmath>
 
 #include "tdq_act_group.cuh"
@@ -366,7 +369,7 @@ cudaError_t launch_fast(const ActArgs& a, cudaStream_t st) {
 // 16-byte grid): the same per-group code behind a staging pass that reads element by element.  A warp stages whole
 // groups, lane = channel (or channel pair of bf16), so every load instruction still reads up to 128 contiguous bytes;
 // channels past the end of the row are zeros.  The staging costs about as many instructions as the groups themselves.
-// Measured, 9217 x 147 fp32: 89 us in the bisection kernel that served these rows before, 6.5 us here.
+// Measured, 9217 x 147 fp32: 89 us in the bisection kernel that served these rows before, 7.0 us here.
 
 template <bool BF16, int KZR, int KB>
 __global__ void __launch_bounds__(kFastThreads) act_g32_ragged_kernel(ActArgs a, int32_t pairs_ok) {

@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(W > 1 ? W * 32 : kWideThreads, wide_blocks(BF1
         const bool idle = c1_cannot_bind(s1, s2, a.seven_tau, cmin, 1.0f / (float)g);
         if (!__all_sync(0xffffffffu, idle)) {
             x.opaque();
-            // binary64; the absent chunks are left out of the second sum
+            // binary64, per lane and then across the lanes; the absent chunks are left out of the second sum
             double s = 0.0;
 #pragma unroll
             for (int j = 0; j < NC * 8; ++j) s = __dadd_rn(s, (double)x.get(j));

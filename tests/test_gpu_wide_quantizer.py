@@ -72,3 +72,28 @@ def test_one_lane_per_group(g, bf16):
             rep = compare_quantizer(si.bf16_bits_to_f32(x) if bf16 else x, g, ref, codes.cpu().numpy(), scale.cpu().numpy())
             assert rep["scale_max_rel"] <= 1e-6, (M, C, kw, rep)
             assert bool((buf[:4] == 0x55).all()) and bool((buf[-16:] == 0x55).all())
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("g", [32, 64, 320, 768, 1024, 2048, 4096])
+def test_dispersion_bound_beside_the_other_bounds(g, bf16):
+    """The binary32 screen may only say that the dispersion bound is idle when it is: groups whose 7 tau sigma lies within a
+    few 1e-6 to 2 % of the smaller of the other two bounds, on either side, with means up to where the screen gives up
+    (mean^2 = 15 var) and past it."""
+    from paper_2604_16855_b200 import tdq
+    rng = np.random.default_rng(g)
+    base = rng.standard_normal((8, g))
+    base = base - base.mean(1, keepdims=True)
+    base /= base.std(1, keepdims=True)
+    x = (base + np.array([0.0, 0.3, 1.0, 2.0, 3.0, 3.8, 4.2, 30.0])[:, None]).astype(np.float32)
+    full = si.f32_to_bf16_bits(x) if bf16 else x
+    xf = si.bf16_bits_to_f32(full) if bf16 else x
+    mags = np.sort(np.abs(xf), axis=1)
+    other = np.minimum(mags[:, -1], np.float32(14.0) * mags[:, int(np.ceil(0.2 * g)) - 1]).astype(np.float64)
+    ratio = other / (7.0 * xf.astype(np.float64).std(1))     # tau at which the two meet
+    for row in range(8):
+        for d in (-2e-2, -6e-3, -4e-3, -1e-3, -1e-4, -1e-5, -2e-6, 0.0, 2e-6, 1e-5, 1e-4, 1e-3, 4e-3, 6e-3, 2e-2):
+            tau = float(np.float32(ratio[row] * (1.0 + d)))
+            ref = oracle.quantize_act(full, g=g, tau=tau)
+            codes, scale = tdq.quantize_act(to_cuda(full, bf16=bf16), tdq.act_params(g=g, tau=tau))
+            compare_quantizer(xf, g, ref, codes.cpu().numpy(), scale.cpu().numpy())
