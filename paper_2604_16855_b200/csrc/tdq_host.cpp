@@ -2,8 +2,9 @@
 // makes the outputs the caller did not pass and enqueues the call.
 //
 // One pass of a small layer is a few microseconds of GPU work, so what the host does per call decides its time:
-// marshalled through ctypes a quantize_act + w4a4_linear pair took 27.5 us to issue (46 us with outputs and workspace
-// made by the calls), of which the two calls into the library were about 11.  Here the tensors are read in C++.
+// marshalled through ctypes a quantize_act + w4a4_linear pair took 27 us to issue (46 us with outputs and workspace
+// made by the calls), of which the two calls into the library were about 11.  Here the tensors are read in C++: 5 to 8 us
+// (8.5), two launches included.
 //
 // The functions take every argument by position (binding.py gives them names and defaults) and release the
 // interpreter lock while the library works, as ctypes does.

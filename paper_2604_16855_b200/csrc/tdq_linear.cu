@@ -26,7 +26,8 @@
 //
 // This file prepares every call (linear_impl) and picks the kernel; the one below is the general form.  Others: g = 32, and
 // 64 and 128 where tiles are few or short, tdq_linear_pair.cu; g = 32 on long contractions tdq_linear_g32.cu; one accumulator
-// per output tdq_linear_one.cu.
+// per output tdq_linear_one.cu.  The general kernel keeps groups of 64 and 128 on larger layers, other widths with several
+// groups per token, small layers with one, and the fused variant (the only one that runs it at g = 32).
 //
 // Two kernels per call (one for the small layers that tdq_linear_pair.cu expands itself):
 //   1. expand_kernel   rewrites the packed nibbles of both operands as operand bytes, in 128-row
@@ -1170,14 +1171,15 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     const bool i8 = group_size > 128 && !pow2_steps;
     int64_t staging_bytes = narrow_strips ? kStagingBytes / 2 : kStagingBytes;
     if (!make_plan(M, I_pad, O, group_size, n_sm, p, staging_bytes)) return TDQ_ERR_UNSUPPORTED;
+    // One group per token, or power-of-two steps: pairs of CTAs on 256 x 256 tiles (tdq_linear_one.cu), unless there are too
+    // few of those: with 24 (2000 x 768 -> 768) the two kernels are level, with 64 (2048 x 2048 -> 2048) it is 15.7 -> 13.0 us;
+    // 18464 x 768 -> 3072 at g = 768 61.4 -> 52.4 (bf16 out 49.3 -> 40.8), 16384 x 4096 -> 4096 at g = 4096 242 -> 157.
+    const int64_t tiles256 = ((p.tiles_m + 1) / 2) * ((p.tiles_n + 1) / 2);
+    const bool use_one = y_tma && !fx && !acc_debug && p.Kg == 1 && (group_size > 32 || pow2_steps) && tiles256 <= INT32_MAX / 4 && tiles256 * 4 >= n_sm;
     // Wide groups run with two MMA-issuing warps, each with half of the ring, and the ring is what bounds them: strips
     // with 32-byte rows (16 KB in all, written in passes) leave room for more stages.  Taken when that gives the smaller
     // half of the ring another stage without changing whether A stays resident; with several groups per tile only where
     // the operands stream (a long contraction), since the passes cost a short tile more than the stage gives.
-    // One group per token, or power-of-two steps: pairs of CTAs on 256 x 256 tiles (tdq_linear_one.cu), unless there are too
-    // few of those: with 24 (2000 x 768 -> 768) the two kernels are level, with 64 (2048 x 2048 -> 2048) it is 15.7 -> 13.0 us.
-    const int64_t tiles256 = ((p.tiles_m + 1) / 2) * ((p.tiles_n + 1) / 2);
-    const bool use_one = y_tma && !fx && !acc_debug && p.Kg == 1 && (group_size > 32 || pow2_steps) && tiles256 <= INT32_MAX / 4 && tiles256 * 4 >= n_sm;
     bool quarter_strips = !use_one && y_tma && !fx && !acc_debug && (wide || pow2_steps) && p.n_chunks >= 2 &&
                           ((p.Kg == 1 && p.n_steps % kChunk == 0) ||
                            (wide && (group_size / 32) % kChunk == 0 && p.Kg >= 2 && !p.a_resident));
@@ -1210,12 +1212,16 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     // so it only pays when an item carries much more work than its own unpacking.
     const int64_t steps_per_item = (p.tiles_n + p.n_parts - 1) / p.n_parts * (int64_t)p.n_steps;
     // g = 32 goes to the kernels built for it.  Two blocks per SM with narrow tiles (tdq_linear_pair.cu) win up to about
-    // 1536 channels (16384 x 1024 -> 2048 86.6 against 92.7 us, 2048 channels 158 against 156) and whenever wide tiles would
-    // leave most SMs idle (1152 x 2048 -> 512 13.9 against 16.0 us), and they also take a y that tensor stores cannot write.
+    // 1536 channels (16384 x 1024 -> 2048 86.6 against 92.7 us) and whenever wide tiles would leave most SMs idle
+    // (1152 x 2048 -> 512 13.9 against 16.0 us), and they also take a y that tensor stores cannot write.  Above, us, pair kernel
+    // and the one for long contractions: 16384 x 1568 -> 2048 bf16 130 and 127, 18464 x 1600 -> 768 fp32 67.7 and 61.8,
+    // 16384 x 2048 -> 2048 bf16 159 and 155, 18464 x 3072 -> 768 fp32 115.6 and 106.2, 16384 x 4096 -> 4096 bf16 577 and 519;
+    // 4096 x 2048 -> 4096 fp32 is the other way round, 82.8 and 88.3.
     const bool use_g32 = group_size == 32 && !pow2_steps && !fx && p.tiles_m * p.tiles_n <= INT32_MAX / 4;
     // Groups of 64 and 128 too where the general kernel's wide tiles are mostly overhead: contractions of up to 512 channels
-    // (9216 x 128 -> 512 at 64 10.1 -> 8.3 us), at most 64 outputs (30000 x 640 -> 64 at 128 17.7 -> 12.5 us), fewer tiles than
-    // SMs (1000 x 2048 -> 256 at 64 14.9 -> 12.0 us).  4616 x 768 -> 3072 at 128 is level, 18464 rows 87 -> 99 us.
+    // (9216 x 128 -> 512 at 64 11.1 -> 10.3 us), at most 64 outputs (30000 x 640 -> 64 at 128 18.4 -> 14.2 us), fewer tiles than
+    // SMs (1000 x 2048 -> 256 at 64 14.7 -> 12.4 us).  Otherwise the general kernel: 4616 x 768 -> 3072 at 128 fp16 23.7 us
+    // against 24.8 in the pair kernel, 18464 rows fp32 84 against 100, at 64 98 against 108.
     const bool use_pair_wide = !pow2_steps && !fx && !use_one && (group_size == 64 || group_size == 128) && p.tiles_m * p.tiles_n <= INT32_MAX / 4 &&
                                (p.n_steps <= 16 || O <= 64 || p.tiles_m * p.tiles_n <= n_sm);
     const bool use_pair = use_pair_wide || (use_g32 && (!y_tma || p.n_steps <= kPairMaxSteps || p.tiles_m * p.tiles_n * 4 <= n_sm));
@@ -1279,11 +1285,12 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     if (use_pair) {
         a.tiles_n = (int32_t)((O + 63) / 64);
         // Few groups and few tiles: one block per tile, which expands its own operands, and the call is one launch.  Quantizer and
-        // linear layer, us: 256 x 64 -> 64 fp32 9.1 -> 7.2, 9216 x 64 -> 128 10.6 -> 7.4, 18432 x 128 -> 128 13.3 -> 10.6,
-        // 2000 x 192 -> 192 9.25 -> 7.6, 9217 x 147 -> 63 15.7 -> 13.4.  With more tiles than blocks a block would have to
-        // refill its ring with nothing under way (9216 x 320 -> 320, 360 tiles: 16.5 -> 18.5), and each block column would
-        // expand the rows again.  A layer with one block column and few groups gains up to two rounds of blocks (73728 x 64
-        // -> 64 18.7 -> 17.0, 65536 x 160 -> 64 26.5 -> 23.8; 73728 x 256 -> 64 32.4 -> 33.1, 200000 x 128 -> 64 46.6 -> 50.7).
+        // linear layer, us: 256 x 64 -> 64 fp32 8.6 -> 6.9, 9216 x 64 -> 128 11.2 -> 8.2, 9216 x 64 -> 256 11.4 -> 9.2,
+        // 18432 x 128 -> 128 12.8 -> 10.8, 2000 x 192 -> 192 9.3 -> 8.0, 9217 x 147 -> 63 16.2 -> 14.3.  With more tiles than
+        // blocks a block would have to refill its ring with nothing under way (9216 x 320 -> 320, 360 tiles: 16.5 -> 18.5), and
+        // each block column would expand the rows again.  A layer with one block column and few groups gains up to two rounds of
+        // blocks (73728 x 64 -> 64 18.8 -> 17.2, 65536 x 160 -> 64 26.4 -> 24.0; 73728 x 256 -> 64 32.4 -> 33.1, 200000 x 128
+        // -> 64 46.6 -> 50.7).
         const int64_t tiles = p.tiles_m * a.tiles_n;
         if (use_g32 && !dbg && p.n_steps <= kPairRing && (tiles <= 2 * n_sm || (a.tiles_n == 1 && p.n_steps <= 6 && tiles <= 4 * n_sm)))
             return launch_linear_pair(a, ymap, n_sm, dev, ybf, false, true, stream);

@@ -17,8 +17,9 @@
 //   warp 2      allocates TMEM
 //   warps 4-11  epilogue: 32 rows x 128 columns each, 32 columns at a time (sixteen warps of half the width: 10 % slower)
 //
-// Measured, with the operand expansion in front (general kernel -> this one): 16384 x 4096 -> 4096 bf16 231 -> 156 us (134 of
-// them here, against 115 at the instruction's own rate), 18464 x 768 -> 3072 bf16 50.8 -> 40.6, fp32 63.8 -> 52.5, power-of-two steps bf16 54.0 -> 44.6, 9216 x 320 -> 320 12.4 -> 8.2.
+// Measured, with the operand expansion in front (general kernel -> this one): 16384 x 4096 -> 4096 bf16 242 -> 157 us (134 of
+// them here, against 115 at the instruction's own rate), 18464 x 768 -> 3072 bf16 49.3 -> 40.8, fp32 61.4 -> 52.4, power-of-two
+// steps bf16 54.0 -> 44.6, 9216 x 320 -> 320 12.4 -> 8.2.
 #include "tdq_tc.cuh"
 
 namespace tdq {

@@ -28,8 +28,8 @@
 //
 // Measured against the other kernel (us; with the operand expansion): 73728 x 64 -> 64 fp32 16.2 -> 11.0, 73728 x 64 -> 192
 // 25.0 -> 18.0, 9216 x 64 -> 256 8.4 -> 7.2, 16384 x 512 -> 2048 bf16 63.8 -> 51.4, 16384 x 1024 -> 2048 92.7 -> 86.6,
-// 18464 x 768 -> 3072 fp32 119.7 -> 115.4; from 2048 channels on the other one is 1-9 % faster (narrower tiles read A twice
-// as often and the older of an SM's two blocks runs an eighth faster than the other).
+// 18464 x 768 -> 3072 fp32 119.7 -> 115.4; above 48 groups the other one is 2-10 % faster (narrower tiles read A twice
+// as often and the older of an SM's two blocks runs an eighth faster than the other; both sides in tdq_linear.cu).
 #include "tdq_tc.cuh"
 
 namespace tdq {
@@ -106,8 +106,9 @@ __device__ __forceinline__ void fill_stages(const LinArgs& a, int mt, int nt, ui
 }
 
 // DIRECT: at most 12 groups (the ring holds them all) and one tile per block; the operands come from the packed codes
-// (fill_stages), and the call is one launch instead of an expansion and this.  SPG: K-steps per group (1, 2 or 4).  With one, a stage holds two pairs of groups and their steps; with more, a pair of
-// groups is one stage or two, one MMA warp takes them all, and the row's steps come from global memory a pair ahead.
+// (fill_stages), and the call is one launch instead of an expansion and this.  SPG: K-steps per group (1, 2 or 4).  With
+// one, a stage holds two pairs of groups and their steps; with more, a pair of groups is one stage or two, one MMA warp
+// takes them all, and the row's steps come from global memory a pair ahead.
 template <bool YBF16, bool DBG, int SPG, bool DIRECT = false>
 __global__ void __launch_bounds__(kPairThreads, 2) w4a4_pair_kernel(const LinArgs a, const __grid_constant__ CUtensorMap ymap) {
     extern __shared__ __align__(128) uint8_t smem_raw[];
@@ -482,7 +483,7 @@ __global__ void __launch_bounds__(kPairThreads, 2) w4a4_pair_kernel(const LinArg
                 } else {
                     // y off the 16-byte grid: the warp writes its own 32 rows, a row's columns side by side (two columns a
                     // lane where a pair of 16-bit values is one aligned word).  9217 x 160 -> 63 fp32 9.3 -> 8.6 us against
-                    // the general kernel.
+                    // the general kernel when both had the expansion in front.
                     __syncwarp();
                     const int64_t m0 = (int64_t)mt * kBM + quarter * 32, c0 = (int64_t)nt * kN;
                     const int rows = (int)min((int64_t)32, a.M - m0), cols = (int)min((int64_t)kN, a.O - c0);

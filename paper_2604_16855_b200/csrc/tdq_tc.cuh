@@ -1,7 +1,7 @@
 // Shared pieces of the W4A4 linear layer's kernels: tile constants, the argument block, mbarrier /
 // bulk-copy / tcgen05 wrappers (inline PTX), the nibble-to-operand-byte expansion, the tensor map
-// of y and the shared-memory plan.  Included by tdq_linear.cu (all group widths, the fused and the
-// power-of-two variants) and tdq_linear_g32.cu (the g = 32 kernel).
+// of y and the shared-memory plan.  Included by tdq_linear.cu (the choice of kernel, the general one, the
+// fused and the power-of-two variants), tdq_linear_pair.cu, tdq_linear_g32.cu and tdq_linear_one.cu.
 #pragma once
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -102,15 +102,16 @@ struct Plan {
     size_t a_bytes, b_bytes, s_bytes;   // operand and scale blocks in the workspace
 };
 
-// The g = 32 kernel (tdq_linear_g32.cu); the caller has run the operand expansion and built the plan and the map.
-// One accumulator per output element over the whole contraction (tdq_linear_one.cu).
-tdq_status launch_linear_one(LinArgs a, const CUtensorMap& ymap, int n_sm, int dev, bool i8, bool ybf, cudaStream_t stream);
+// The other kernels of the linear layer; the caller has built the plan, encoded y's map and, unless `direct`, run the
+// operand expansion.
 constexpr int kPairRing = 12;       // K-steps that the ring of operands of tdq_linear_pair.cu holds
 constexpr int kPairMaxSteps = 48;   // longest contraction it takes at g = 32 where tdq_linear_g32.cu could
 tdq_status launch_linear_pair(const LinArgs& a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, bool dbg, bool direct,
-                              cudaStream_t stream);   // tiles of 128 x 64, tdq_linear_pair.cu
+                              cudaStream_t stream);   // two blocks per SM, tiles of 128 x 64 (tdq_linear_pair.cu)
 tdq_status launch_linear_g32(const LinArgs& a, const CUtensorMap& ymap, uint32_t smem_bytes, unsigned grid, bool ybf,
-                             bool dbg, cudaStream_t stream);
+                             bool dbg, cudaStream_t stream);   // g = 32, long contractions (tdq_linear_g32.cu)
+// one accumulator per output element over the whole contraction (tdq_linear_one.cu)
+tdq_status launch_linear_one(LinArgs a, const CUtensorMap& ymap, int n_sm, int dev, bool i8, bool ybf, cudaStream_t stream);
 
 namespace {
 
@@ -194,7 +195,7 @@ __device__ __forceinline__ bool mbar_test_s(uint32_t bar_s, uint32_t parity) {
 // Waits in the hot loops: one test of the barrier; if the phase is not complete yet, the bounded sleeping
 // wait, out of line.  Every lane asks about the same barrier in the same instruction, so the lanes agree
 // without a vote.  A wait that gives up raises the CTA's abort flag (and records its code); the loops look
-// at that flag once per tile, and every later wait returns at once.
+// at that flag once per tile or stage, and every later wait gives up after one burst of sleeps.
 __device__ __forceinline__ void wait_cold(uint32_t bar_s, uint32_t parity, Ctrl* c, uint32_t* status, uint32_t code) {
     uint64_t* bar = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(c) + (bar_s - smem_u32(c)));
     mbar_wait_slow(bar, parity, c, status, code);
