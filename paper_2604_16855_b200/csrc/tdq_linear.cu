@@ -189,9 +189,10 @@ constexpr int kPow2Tables = 14 - kPow2MinShift + 1;        // one table per s in
 constexpr int kPow2Chunks = 2;                             // chunks of K-steps per CTA of the expansion
 
 // A step that is not a positive power of two is reported as the status word 11 | epoch << 8, stored by
-// whichever thread meets one.  The epoch is the workspace's third status word: the GEMM kernel of every call
+// whichever thread meets one.  The epoch is the workspace's third status word: the GEMM kernel of every such call
 // adds one to it, after this kernel has finished, so it is fixed while this kernel runs and differs from the
-// epoch of the call before (also when the calls are replays of one captured graph).  The CTA that clears the
+// epoch of the call before (also when the calls are replays of one captured graph; a call of the exact layer in between
+// clears it, and the status word with it).  The CTA that clears the
 // status word for this call leaves exactly the value 11 | epoch << 8 alone, so the order of the clear and the
 // reports does not matter, and a report left by an earlier call is cleared like any other stale word.
 __global__ void __launch_bounds__(kExpandThreads) expand_pow2_kernel(ExpandArgs a, int32_t act_steps_per_grp, int32_t act_Kg) {
