@@ -78,8 +78,8 @@ def profiled_traffic(kernel, workload_name, files):
 
 
 # the kernel that the default workload's linear layer runs, and the files its profile summary is bound to
-LINEAR_KERNEL = "w4a4_pair_kernel"
-LINEAR_KERNEL_SOURCES = ["tdq_linear_pair.cu", "tdq_tc.cuh"]
+LINEAR_KERNEL = "w4a4_defer_kernel"
+LINEAR_KERNEL_SOURCES = ["tdq_linear_defer.cu", "tdq_tc.cuh"]
 
 
 def load_peaks():

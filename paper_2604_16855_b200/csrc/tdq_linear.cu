@@ -1225,8 +1225,23 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     // against 24.8 in the pair kernel, 18464 rows fp32 84 against 100, at 64 98 against 108.
     const bool use_pair_wide = !pow2_steps && !fx && !use_one && (group_size == 64 || group_size == 128) && p.tiles_m * p.tiles_n <= INT32_MAX / 4 &&
                                (p.n_steps <= 16 || O <= 64 || p.tiles_m * p.tiles_n <= n_sm);
-    const bool use_pair = use_pair_wide || (use_g32 && (!y_tma || p.n_steps <= kPairMaxSteps || p.tiles_m * p.tiles_n * 4 <= n_sm));
-    const bool unpack_a = !fx && !pow2_steps && !use_pair && !use_one && p.a_resident && steps_per_item >= 256;
+    const bool pair_ok = use_pair_wide || (use_g32 && (!y_tma || p.n_steps <= kPairMaxSteps || p.tiles_m * p.tiles_n * 4 <= n_sm));
+    // Several 128 x 128 tiles per SM: one block per SM that does a tile's epilogue during the next tile (tdq_linear_defer.cu).
+    // Against the pair kernel it wins from about four tiles an SM on, three for longer contractions, and not where the last
+    // column tile is mostly empty; us, pair kernel and this one, at g = 32 fp32: 18432 x 320 -> 1280 (1440 tiles) 36.6 and 34.8,
+    // 9216 x 768 -> 960 (576) 25.7 and 24.2, 4608 x 768 -> 1280 (360) 20.0 and 19.3, 9216 x 256 -> 960 14.8 and 17.0, 4608 x 768 ->
+    // 320 (108) 11.0 and 11.4.  Above kPairMaxSteps the steps of a tile leave the ring too little room.  At g = 64 and 128 it takes
+    // over from the general kernel wherever there is more than a tile per SM (4616 x 768 -> 3072 at 128 fp16 23.8 and 20.8,
+    // 2304 x 768 -> 1280 (180 tiles) at 64 fp32 14.7 and 12.7).
+    const int64_t tiles128 = p.tiles_m * p.tiles_n;
+    const bool full_tiles = (O + 63) / 64 * 4 >= p.tiles_n * 7;           // at least 7/8 of the column tiles' halves have outputs
+    const bool use_defer = y_tma && !acc_debug && !pow2_steps && !fx && !use_one && tiles128 <= INT32_MAX / 64 && p.Kg > 1 &&
+                           linear_defer_fits(y_dtype == TDQ_BF16, p.Kg) &&
+                           (group_size == 32 ? p.n_steps <= kPairMaxSteps && full_tiles && (p.n_steps >= 24 ? tiles128 > 3 * n_sm : p.n_steps >= 10 && tiles128 > 4 * n_sm)
+                                             : (group_size == 64 || group_size == 128) &&
+                                               (use_pair_wide ? p.n_steps >= 16 && full_tiles && tiles128 > 3 * n_sm : tiles128 > n_sm));
+    const bool use_pair = pair_ok && !use_defer;
+    const bool unpack_a = !fx && !pow2_steps && !use_pair && !use_one && !use_defer && p.a_resident && steps_per_item >= 256;
     e.tiles_m = (fx || unpack_a) ? 0 : (int32_t)p.tiles_m;   // then only the weights are expanded here
     e.tiles_n = (int32_t)p.tiles_n;
     e.b_rows = use_pair ? 64 : 128;
@@ -1250,8 +1265,8 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     memset(&ymap, 0, sizeof(ymap));
     a.tma_ok = 0;
     if (y_tma && encode_y_map(&ymap, y, y_dtype == TDQ_BF16, M, O, y_row_stride,
-                              (use_one || use_pair) ? kCols : quarter_strips ? (y_dtype == TDQ_BF16 ? kCols / 2 : kCols / 4) : half_strips ? kCols / 2 : kCols,
-                              (use_g32 || use_pair) ? kBM : 32, y_f16))
+                              (use_one || use_pair || use_defer) ? kCols : quarter_strips ? (y_dtype == TDQ_BF16 ? kCols / 2 : kCols / 4) : half_strips ? kCols / 2 : kCols,
+                              (use_g32 || use_pair || use_defer) ? kBM : 32, y_f16))
         a.tma_ok = 1;
     else if (narrow_strips || quarter_strips)
         return TDQ_ERR_CUDA;   // the plan counted on the tensor store
@@ -1313,6 +1328,7 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     const unsigned grid = (unsigned)(items < n_sm ? items : n_sm);
     // The cluster kernel and the one for long contractions at g = 32 can only write y through the map; the others also without.
     if (use_one && a.tma_ok) return launch_linear_one(a, ymap, n_sm, dev, i8, ybf, stream);
+    if (use_defer && a.tma_ok) return launch_linear_defer(a, ymap, n_sm, dev, ybf, stream);
     if (use_pair) return launch_linear_pair(a, ymap, n_sm, dev, ybf, dbg, false, stream);
     if (use_g32 && a.tma_ok) return launch_linear_g32(a, ymap, p.smem_bytes, grid, ybf, dbg, stream);
     if (launch_pdl(kernel, dim3(grid), dim3(kThreads), p.smem_bytes, stream, a, ymap) != cudaSuccess) return TDQ_ERR_CUDA;

@@ -1,7 +1,7 @@
 // Shared pieces of the W4A4 linear layer's kernels: tile constants, the argument block, mbarrier /
 // bulk-copy / tcgen05 wrappers (inline PTX), the nibble-to-operand-byte expansion, the tensor map
 // of y and the shared-memory plan.  Included by tdq_linear.cu (the choice of kernel, the general one, the
-// fused and the power-of-two variants), tdq_linear_pair.cu, tdq_linear_g32.cu and tdq_linear_one.cu.
+// fused and the power-of-two variants), tdq_linear_pair.cu, tdq_linear_defer.cu, tdq_linear_g32.cu and tdq_linear_one.cu.
 #pragma once
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -108,6 +108,8 @@ constexpr int kPairRing = 12;       // K-steps that the ring of operands of tdq_
 constexpr int kPairMaxSteps = 48;   // longest contraction it takes at g = 32 where tdq_linear_g32.cu could
 tdq_status launch_linear_pair(const LinArgs& a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, bool dbg, bool direct,
                               cudaStream_t stream);   // two blocks per SM, tiles of 128 x 64 (tdq_linear_pair.cu)
+bool linear_defer_fits(bool y16, int32_t Kg);   // g = 32, 64, 128 with several tiles per SM (tdq_linear_defer.cu)
+tdq_status launch_linear_defer(LinArgs a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, cudaStream_t stream);
 tdq_status launch_linear_g32(const LinArgs& a, const CUtensorMap& ymap, uint32_t smem_bytes, unsigned grid, bool ybf,
                              bool dbg, cudaStream_t stream);   // g = 32, long contractions (tdq_linear_g32.cu)
 // one accumulator per output element over the whole contraction (tdq_linear_one.cu)
@@ -381,6 +383,9 @@ __device__ __forceinline__ uint32_t lds32(uint32_t addr) {
     uint32_t v;
     asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
+}
+__device__ __forceinline__ void lds128(uint32_t addr, uint64_t& x, uint64_t& y) {
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "r"(addr) : "memory");
 }
 __device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
     asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
