@@ -76,9 +76,9 @@ __device__ __forceinline__ uint32_t nibble_fast(float x, float c, float delta, f
 // half): s2 is within 4 % and the mean within 0.032 rms, so the variance estimate is off by at
 // most 0.105 E[x^2].  Requiring var >= E[x^2] / 2 turns that into var_true >= 0.78 var, and the
 // factor 0.7 then leaves 7 tau sigma_true >= 1.05 cmin.  Anything else goes to the exact path.
-__device__ __forceinline__ bool c1_cannot_bind_rough(float s1, float s2, float seven_tau, float cmin) {
-    const float mean = s1 * (1.0f / 32.0f);
-    const float ex2 = s2 * (1.0f / 32.0f);
+__device__ __forceinline__ bool c1_cannot_bind_rough(float s1, float s2, float seven_tau, float cmin, float inv_g = 1.0f / 32.0f) {
+    const float mean = s1 * inv_g;
+    const float ex2 = s2 * inv_g;
     const float var = fmaf(-mean, mean, ex2);
     const float lhs = seven_tau * seven_tau * var * 0.7f;
     const float rhs = cmin * cmin;

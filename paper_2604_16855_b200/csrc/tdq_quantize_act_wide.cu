@@ -7,11 +7,18 @@
 //
 // What bounds it is instruction issue, and of that the rank selection.  It is a search for the k-th smallest magnitude
 // over the ordered bit patterns of |x|: count the elements <= a probe (bf16: two per packed compare and add), narrow the
-// bracket, repeat.  A plain bisection needs 15 (bf16) or 31 (fp32) counting passes.  The distribution of |x| is nearly
-// flat near zero, where the zero-bin rank lies, so the search starts at the Gaussian quantile of the group's rms and
-// then follows straight lines of the counting function, with a bisection step every fourth probe as the guarantee; it
-// ends when the bracket's upper end has exactly k elements at or below it or its lower end k - 1.  Three to five probes
-// on average, five to six for the slowest of the eight groups of a warp.
+// bracket, repeat.  A plain bisection needs 15 (bf16) or 31 (fp32) counting passes.  Three things keep their number down:
+//   * the zero-bin rank only matters where 14 thr < c_base, so the search ends once the bracket lies above c_base / 14, and
+//     the first probe is that or the Gaussian quantile of the group's rms, whichever is less (for a Gaussian group of 128 the
+//     20 % quantile is 3.5 sigma / 14 and the maximum 2.8 sigma: one probe);
+//   * the probes then follow straight lines of the counting function (it is nearly flat near zero, where the rank lies), and
+//     an end of the bracket that stays while the other moves twice counts for half (the Illinois rule), which is what a steep or
+//     curved piece needs: the percentile radius, heavy tails;
+//   * the third probe asks for the zeros, of which padding and rectified inputs have more than the rank: the lines approach
+//     that jump from above a bit at a time (36 probes for bf16, 70 for fp32, for every group of such a warp).
+// A bisection step every sixth probe is the guarantee; the search ends when the bracket's upper end has exactly k elements
+// at or below it or its lower end k - 1.  1.5 probes on average at g = 128 and zr = 0.2, three for the slowest of the eight
+// groups of a warp, 4.5 and 6.6 for a 0.9 percentile.
 //
 // Lanes per group and chunks per lane (NC): as few lanes as keep a lane at four chunks (32 channels), because the
 // probe's bookkeeping and the reduction over the group are paid per lane.  Past 1024 channels two or four warps share a
@@ -20,10 +27,11 @@
 // one lane each: 18464 x 768 bf16 at g = 8 143 -> 39 us against four lanes with one chunk each, at g = 16 81 -> 30, at
 // g = 24 56 -> 25, at g = 32 (codes off the 16-byte grid) 43 -> 24.
 //
-// Measured (B200, from a graph, input not in L2) against the bisection kernel with the group in shared memory that served
-// these cases before: 4616 x 768 bf16 at g = 128 65 -> 9 us; 18464 x 768 bf16 at g = 128 24 us (of which the rank
-// search 12), at g = 64 24 us, at g = 768 20 us; 16384 x 4096 bf16 at g = 4096 978 -> 76 us (2.2 TB/s, 46 us without
-// the rank search).
+// Measured (B200, from a graph), us, before the search had the last two rules, the first one and rough moments, and now:
+// bf16 18464 x 768 at g = 128 24.8 -> 19.5 (zr = 0.3 24.8 -> 16.8, rectified 47.2 -> 17.6, p = 0.9 48.7 -> 33.2, with a mean
+// of 30 39.3 -> 22.9), at g = 64 25.0 -> 20.7; 46005 x 608 at g = 128 (a quarter of a row's last group is padding) 129.4 ->
+// 36.9, with p = 0.9 175.0 -> 69.1; 16384 x 4096 at g = 4096 76.8 -> 64.6 (of it eight chunks a lane 8.4); fp32 18464 x 768 at
+// g = 128 26.2 -> 22.8, rectified 76.1 -> 18.6.  The bisection kernel that served these cases at first: 978 us on the long groups.
 #include "tdq_act_group.cuh"
 #include "tdq_common.cuh"
 
@@ -112,22 +120,37 @@ struct Share {
         }
         return n0 + n1;
     }
-    // largest magnitude of this share that is at most that
-    __device__ __forceinline__ uint32_t max_le(uint32_t key) const {
+    // largest magnitude of this share that is at most that (bf16: packed, two masks and maxima at a time)
+    __device__ __forceinline__ uint32_t max_le(const uint32_t (&mag)[NC * kWords], uint32_t key) const {
         uint32_t r = 0;
+        if (BF16) {
+            const uint32_t m = __byte_perm(key, 0u, 0x3232u);
+            const __nv_bfloat162 m2 = *reinterpret_cast<const __nv_bfloat162*>(&m);
+#pragma unroll
+            for (int i = 0; i < NC * kWords; ++i) r = __vmaxu2(r, mag[i] & __hle2_mask(*reinterpret_cast<const __nv_bfloat162*>(&mag[i]), m2));
+            return max(r & 0xffffu, r >> 16) << 16;
+        }
 #pragma unroll
         for (int i = 0; i < NC * 8; ++i) {
-            const uint32_t u = __float_as_uint(get(i)) & 0x7fffffffu;
+            const uint32_t u = w[i] & 0x7fffffffu;
             r = max(r, u <= key ? u : 0u);
         }
         return r;
     }
-    // smallest magnitude of this share above it
-    __device__ __forceinline__ uint32_t min_gt(int key) const {
+    // smallest magnitude of this share above it (any, if it is negative)
+    __device__ __forceinline__ uint32_t min_gt(const uint32_t (&mag)[NC * kWords], int key) const {
+        if (BF16) {
+            uint32_t r = 0x7fff7fffu;
+            const uint32_t m = key < 0 ? 0x80008000u + 0x3f803f80u : __byte_perm((uint32_t)key, 0u, 0x3232u);   // -1 for "none"
+            const __nv_bfloat162 m2 = *reinterpret_cast<const __nv_bfloat162*>(&m);
+#pragma unroll
+            for (int i = 0; i < NC * kWords; ++i) r = __vminu2(r, mag[i] | __hle2_mask(*reinterpret_cast<const __nv_bfloat162*>(&mag[i]), m2));
+            return min(r & 0xffffu, r >> 16) << 16;
+        }
         uint32_t r = 0x7fffffffu;
 #pragma unroll
         for (int i = 0; i < NC * 8; ++i) {
-            const uint32_t u = __float_as_uint(get(i)) & 0x7fffffffu;
+            const uint32_t u = w[i] & 0x7fffffffu;
             r = min(r, (int)u > key ? u : 0x7fffffffu);
         }
         return r;
@@ -135,9 +158,10 @@ struct Share {
 };
 
 // The k-th smallest magnitude (bit pattern) of the group; k counts the zeros that stand for absent elements too.
-// kmax is the group's largest magnitude, n its number of elements with the absent ones, guess the first probe.
+// kmax is the group's largest magnitude, guess the first probe.  limit: a magnitude above which the caller does not need to
+// know the result; what is returned then is some magnitude above it.
 template <bool BF16, int NC, int L, int W>
-__device__ __forceinline__ uint32_t group_kth(const Share<BF16, NC>& x, int k, int absent, uint32_t kmax, float guess, uint32_t& turn) {
+__device__ __forceinline__ uint32_t group_kth(const Share<BF16, NC>& x, int k, int absent, uint32_t kmax, float guess, float limit, uint32_t& turn) {
     constexpr int kStep = BF16 ? 16 : 0;             // keys are compared as key >> kStep
     constexpr float n = (float)(L * W * NC * 8);
     constexpr int kWords = Share<BF16, NC>::kWords;
@@ -147,40 +171,48 @@ __device__ __forceinline__ uint32_t group_kth(const Share<BF16, NC>& x, int k, i
     auto umax = [](uint32_t p, uint32_t q) { return max(p, q); };
     if (BF16) kmax >>= kStep;
     int lo = -1, hi = (int)kmax;                     // count(lo) < k <= count(hi)
+    const int enough = (int)(__float_as_uint(limit) >> kStep);
     // counts without the absent elements' zeros (a count below them stands for none)
     const float kf = (float)k, af = (float)absent;
     float c_lo = 0.0f, c_hi = n;
-    float probe_v = guess;
+    float probe_v = fminf(guess, limit);
     const float aim = kf - af - 0.5f;                // between the k-th element and the one before it
+    float w_lo = 1.0f, w_hi = 1.0f;                  // an end that stays while the other moves twice counts for half (Illinois rule)
+    int last = 0;
     int round = 0;
 #pragma unroll 1
     for (;;) {
-        const bool done = hi - lo <= 1 || c_hi == kf || c_lo + 1.0f == kf;
+        const bool done = hi - lo <= 1 || c_hi == kf || c_lo + 1.0f == kf || lo >= enough;
         if (L == 32 ? done : __all_sync(0xffffffffu, done)) break;
         int p = (int)(__float_as_uint(probe_v) >> kStep);
-        if ((++round & 3) == 0) p = lo + ((hi - lo) >> 1);   // the guarantee
+        ++round;
+        if (round == 3 && lo < 0) p = 0;             // as many zeros as that: padding, rectified inputs
+        if (round == 6) { p = lo + ((hi - lo) >> 1); round = 0; }   // the guarantee
         p = max(lo + 1, min(hi - 1, p));
         const float c = group_sum_count<L, W>(x.count_le(mag, (uint32_t)p << kStep), turn);
         if (!done) {
-            if (c >= kf) { hi = p; c_hi = c; } else { lo = p; c_lo = c; }
+            const bool up = c >= kf;
+            if (up) { hi = p; c_hi = c; w_lo = last > 0 ? 0.5f * w_lo : 1.0f; w_hi = 1.0f; last = 1; }
+            else { lo = p; c_lo = c; w_hi = last < 0 ? 0.5f * w_hi : 1.0f; w_lo = 1.0f; last = -1; }
             const float v_lo = __uint_as_float((uint32_t)max(lo, 0) << kStep), v_hi = __uint_as_float((uint32_t)hi << kStep);
             const float n_lo = fmaxf(c_lo - af, 0.0f);
             // no upper end but the maximum yet: the line through the origin; else the line between the ends
             const bool open = c_hi == n && n_lo > 0.0f;
-            const float slope = __fdividef(open ? v_lo : v_hi - v_lo, open ? n_lo : c_hi - af - n_lo);
-            probe_v = open ? slope * aim : fmaf(slope, aim - n_lo, v_lo);
+            const float below = (aim - n_lo) * w_lo, above = (c_hi - af - aim) * w_hi;
+            const float slope = __fdividef(open ? v_lo : v_hi - v_lo, open ? n_lo : below + above);
+            probe_v = open ? slope * aim : fmaf(slope, below, v_lo);
         }
     }
     // exactly k elements at or below hi: the largest of them; exactly k - 1 at or below lo: the smallest of the rest
     // (all lanes of the warp take part in the reductions)
-    const bool wide = hi - lo > 1, below = wide && c_hi == kf, above = wide && !below;
+    const bool wide = hi - lo > 1 && lo < enough, below = wide && c_hi == kf, above = wide && !below;
     uint32_t r = (uint32_t)hi << kStep;
     if (__any_sync(0xffffffffu, below)) {
-        const uint32_t m = group_reduce<L, W>(x.max_le(r), umax, turn);
+        const uint32_t m = group_reduce<L, W>(x.max_le(mag, r), umax, turn);
         if (below) r = m;
     }
     if (__any_sync(0xffffffffu, above)) {
-        const uint32_t m = group_reduce<L, W>(x.min_gt((int)((uint32_t)lo << kStep)), [](uint32_t p, uint32_t q) { return min(p, q); }, turn);
+        const uint32_t m = group_reduce<L, W>(x.min_gt(mag, lo < 0 ? -1 : (int)((uint32_t)lo << kStep)), [](uint32_t p, uint32_t q) { return min(p, q); }, turn);
         if (above) r = m;
     }
     return r;
@@ -272,11 +304,28 @@ __global__ void __launch_bounds__(W > 1 ? W * 32 : kWideThreads, wide_blocks(BF1
 #pragma unroll
         for (int j = 0; j < NC * kW; ++j) kmax = max(kmax, x.w[j] & 0x7fffffffu);
     }
+    // Moments: for bf16 rough ones, two channels per instruction, at most 16 additions in a sum (see c1_cannot_bind_rough)
+    if (BF16) {
 #pragma unroll
-    for (int j = 0; j < NC * 8; ++j) {
-        const float v = x.get(j);
-        s1 += v;
-        s2 = fmaf(v, v, s2);
+        for (int h = 0; h < NC * kW; h += 16) {
+            __nv_bfloat162 s1b = *reinterpret_cast<const __nv_bfloat162*>(&x.w[h]);
+            __nv_bfloat162 s2b = __hmul2(s1b, s1b);
+#pragma unroll
+            for (int j = h + 1; j < (h + 16 < NC * kW ? h + 16 : NC * kW); ++j) {
+                const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(&x.w[j]);
+                s1b = __hadd2(s1b, v);
+                s2b = __hfma2(v, v, s2b);
+            }
+            s1 += __low2float(s1b) + __high2float(s1b);
+            s2 += __low2float(s2b) + __high2float(s2b);
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < NC * 8; ++j) {
+            const float v = x.get(j);
+            s1 += v;
+            s2 = fmaf(v, v, s2);
+        }
     }
     x.opaque();
     kmax = group_reduce<L, W>(kmax, [](uint32_t p, uint32_t q) { return max(p, q); }, turn);
@@ -286,13 +335,29 @@ __global__ void __launch_bounds__(W > 1 ? W * 32 : kWideThreads, wide_blocks(BF1
     const int absent = kLanes * NC * 8 - g;
     const float rms = sqrtf(s2 / (float)g);
     float c_base = __uint_as_float(kmax), thr = 0.0f;
-    if (a.k_base < g) c_base = __uint_as_float(group_kth<BF16, NC, L, W>(x, a.k_base + absent, absent, kmax, rms * wa.guess_base, turn));
-    if (a.flags & TDQ_ENABLE_C2) thr = __uint_as_float(group_kth<BF16, NC, L, W>(x, a.k_zr + absent, absent, kmax, rms * wa.guess_zr, turn));
+    if (a.k_base < g) c_base = __uint_as_float(group_kth<BF16, NC, L, W>(x, a.k_base + absent, absent, kmax, rms * wa.guess_base, INFINITY, turn));
+    // C2 only acts if 14 thr < c_base: a threshold above c_base / 14 (rounded up a little) need not be known
+    if (a.flags & TDQ_ENABLE_C2)
+        thr = __uint_as_float(group_kth<BF16, NC, L, W>(x, a.k_zr + absent, absent, kmax, rms * wa.guess_zr, c_base * (1.000001f / 14.0f), turn));
     float sigma = INFINITY;                           // an idle C1 bound
     if (a.flags & TDQ_ENABLE_C1) {
         float cmin = c_base;
         if (a.flags & TDQ_ENABLE_C2) cmin = fminf(cmin, __fmul_rn(14.0f, thr));
-        const bool idle = c1_cannot_bind(s1, s2, a.seven_tau, cmin, 1.0f / (float)g);
+        bool idle = BF16 ? c1_cannot_bind_rough(s1, s2, a.seven_tau, cmin, 1.0f / (float)g) : c1_cannot_bind(s1, s2, a.seven_tau, cmin, 1.0f / (float)g);
+        if (BF16 && !__all_sync(0xffffffffu, idle)) {     // the rough moments do not decide: binary32 ones
+            x.opaque();
+            s1 = 0.0f;
+            s2 = 0.0f;
+#pragma unroll
+            for (int j = 0; j < NC * 8; ++j) {
+                const float v = x.get(j);
+                s1 += v;
+                s2 = fmaf(v, v, s2);
+            }
+            s1 = group_reduce<L, W>(s1, [](float p, float q) { return p + q; }, turn);
+            s2 = group_reduce<L, W>(s2, [](float p, float q) { return p + q; }, turn);
+            idle = c1_cannot_bind(s1, s2, a.seven_tau, cmin, 1.0f / (float)g);
+        }
         if (!__all_sync(0xffffffffu, idle)) {
             x.opaque();
             // binary64, per lane and then across the lanes; the absent chunks are left out of the second sum
@@ -386,6 +451,18 @@ cudaError_t pick(const WideArgs& w, cudaStream_t st) {
     if (chunks <= 64) return launch<BF16, 4, 16>(w, st);
     if (chunks <= 96) return launch<BF16, 3, 32>(w, st);
     if (chunks <= 128) return launch<BF16, 4, 32>(w, st);
+    if constexpr (BF16) {
+        // From 8 M channels on, long groups of bf16 take half the lanes: what a lane does besides its channels (reductions,
+        // barriers, the probes' bookkeeping) weighs as much as they do.  us, four chunks a lane and eight: 16384 x 4096 73.0 and
+        // 64.6, 16384 x 3072 64.2 and 48.8, 4096 x 2048 11.7 and 10.7, 2048 x 4096 12.0 and 11.1; 2048 x 2048 7.7 and 8.4, 1024 x
+        // 4096 7.8 and 8.8 (too few warps); groups of up to 1024 gain nothing (18464 x 768 at 128 19.5 and 20.9, at 768 17.8 and 17.5).
+        if (chunks > 128 && w.a.total_groups * w.a.g >= ((int64_t)1 << 23)) {
+            if (chunks <= 192) return launch<BF16, 6, 32>(w, st);
+            if (chunks <= 256) return launch<BF16, 8, 32>(w, st);
+            if (chunks <= 384) return launch<BF16, 6, 32, 2>(w, st);
+            return launch<BF16, 8, 32, 2>(w, st);
+        }
+    }
     if (chunks <= 192) return launch<BF16, 3, 32, 2>(w, st);
     if (chunks <= 256) return launch<BF16, 4, 32, 2>(w, st);
     if (chunks <= 384) return launch<BF16, 3, 32, 4>(w, st);

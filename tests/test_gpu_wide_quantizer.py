@@ -97,3 +97,61 @@ def test_dispersion_bound_beside_the_other_bounds(g, bf16):
             ref = oracle.quantize_act(full, g=g, tau=tau)
             codes, scale = tdq.quantize_act(to_cuda(full, bf16=bf16), tdq.act_params(g=g, tau=tau))
             compare_quantizer(xf, g, ref, codes.cpu().numpy(), scale.cpu().numpy())
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("g", [64, 96, 128, 1024, 2048, 4096])
+def test_rank_search_edges(g, bf16):
+    """Groups at the edges of the rank search: as many zeros as the zero-bin rank and one more or less, padding, few distinct
+    values, magnitudes over the whole range, and a rank-k magnitude at, just above and just below a fourteenth of the base
+    radius, above which the search may stop."""
+    from paper_2604_16855_b200 import tdq
+    rng = np.random.default_rng(200 + g)
+    k = int(np.ceil(0.2 * g - 1e-6))
+    rows = []
+    for z in (k - 1, k, k + 1, g // 2, g - 1):
+        x = rng.standard_normal(g)
+        x[:z] = 0.0
+        rows.append(x)
+    rows.append(np.full(g, -0.3))
+    rows.append(np.where(np.arange(g) % 3 == 0, 1.0, -14.0))
+    rows.append(rng.choice([0.5, -1.0, 2.0, 6.0], g))
+    rows.append(np.clip(rng.standard_normal(g) * 4.0, 0.0, 6.0))
+    rows.append(10.0 ** rng.uniform(-30, 30, g))
+    rows.append(10.0 ** rng.uniform(-44, -36, g))
+    rows.append(1.0 + 1e-3 * np.arange(g))
+    for top in (14.0, 13.9, 7.0 * 1.5, 1.234567e-3, 3e33):
+        edge = np.float32(top) / np.float32(14.0)
+        for ulps in (-66000, -65536, -2, -1, 0, 1, 2, 65536, 66000):
+            v = (np.float32(edge).view(np.int32) + np.int32(ulps)).view(np.float32)
+            x = rng.uniform(1.5, 13.0, g) * float(v)
+            x[:k - 1] = rng.uniform(0.1, 0.9, k - 1) * float(v)
+            x[k - 1] = v
+            x[-1] = top
+            rows.append(x)
+    x = np.stack([rng.permutation(r) for r in rows]).astype(np.float32)
+    x *= rng.choice([-1.0, 1.0], x.shape).astype(np.float32)
+    for C in (g, g - g // 4 - 3):                            # the second: a quarter of the group is padding
+        full = si.f32_to_bf16_bits(x[:, :C]) if bf16 else np.ascontiguousarray(x[:, :C])
+        for kw in (dict(), dict(p=0.9), dict(zr=0.5, p=0.3)):
+            ref = oracle.quantize_act(full, g=g, **kw)
+            codes, scale = tdq.quantize_act(to_cuda(full, bf16=bf16), tdq.act_params(g=g, zr=kw.get("zr", 0.2), p=kw.get("p", 1.0)))
+            compare_quantizer(si.bf16_bits_to_f32(full) if bf16 else full, g, ref, codes.cpu().numpy(), scale.cpu().numpy())
+
+
+@pytest.mark.parametrize("M,C,g", [(5462, 1536, 1536), (6100, 1030, 1152), (4097, 2048, 2048), (3500, 2056, 2056), (2731, 3072, 3072), (2049, 4090, 4096), (1400, 6144, 3072)])
+def test_eight_chunks_a_lane(M, C, g):
+    """Long groups of bf16 in tensors of 8 M channels and more; rows off the 16-byte grid as well."""
+    from paper_2604_16855_b200 import tdq
+    rng = np.random.default_rng(M)
+    some = _rows(rng, 97, C)
+    pick = np.sort(rng.choice(M, 97, replace=False))
+    for pad in (0, 1, 8):
+        gen = torch.Generator("cuda").manual_seed(M)
+        x = torch.randn((M, C + pad), device="cuda", generator=gen).to(torch.bfloat16)
+        bits = si.f32_to_bf16_bits(some)
+        x[torch.from_numpy(pick).cuda(), :C] = to_cuda(bits, bf16=True)
+        for kw in (dict(), dict(p=0.9, zr=0.5), dict(tau=0.4, flags=7)):
+            ref = oracle.quantize_act(bits, g=g, **kw)
+            codes, scale = tdq.quantize_act(x[:, :C], tdq.act_params(g=g, tau=kw.get("tau", 1.0), zr=kw.get("zr", 0.2), p=kw.get("p", 1.0), flags=kw.get("flags", 3)))
+            compare_quantizer(si.bf16_bits_to_f32(bits), g, ref, codes.cpu().numpy()[pick], scale.cpu().numpy()[pick])
