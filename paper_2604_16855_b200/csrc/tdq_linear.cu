@@ -1240,6 +1240,15 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
                            (group_size == 32 ? p.n_steps <= kPairMaxSteps && full_tiles && (p.n_steps >= 24 ? tiles128 > 3 * n_sm : p.n_steps >= 10 && tiles128 > 4 * n_sm)
                                              : (group_size == 64 || group_size == 128) &&
                                                (use_pair_wide ? p.n_steps >= 16 && full_tiles && tiles128 > 3 * n_sm : tiles128 > n_sm));
+    // No more 128 x 64 tiles than SMs: one launch, with all of an SM for a tile (tdq_linear_solo.cu).  us, the kernels that took
+    // these layers before (with the expansion in front from 13 groups, or beyond 32 codes a group, on) and this one, 1152 rows -> 512 fp32:
+    // g = 32, 128 channels 4.9 and 4.8, 256 6.6 and 5.7, 512 8.1 and 7.6, 896 9.8 and 9.1, 1280 11.7 and 11.3 (one tile: 10.3 and 11.0); g = 64,
+    // 512 channels 8.0 and 5.9, 1024 9.9 and 7.9, 2048 12.8 and 13.5; g = 128, 512 7.4 and 5.4, 2048 11.2 and 10.1, 4096 15.8 and 18.0; one step
+    // per token, 768 8.1 and 6.1, 1312 12.9 and 7.8, 4096 13.1 and 13.8.  Up to 128 channels the two-blocks-per-SM kernel's single launch is
+    // level (256 x 64 -> 64 4.3 and 4.2) unless y is off the 16-byte grid (97 x 64 -> 2047 6.1 and 4.7).  With more tiles than
+    // SMs the second round costs as much as the first (1200 x 320 -> 960 at g = 32, 150 tiles, 8.0 and 11.0).
+    const bool use_solo = !acc_debug && !pow2_steps && !fx && !use_one && p.tiles_m * ((O + 63) / 64) <= n_sm &&
+                          (group_size == 32 ? p.n_steps <= 28 && (p.n_steps > 4 || !y_tma) : p.n_steps <= (group_size == 64 ? 32 : 64));
     const bool use_pair = pair_ok && !use_defer;
     const bool unpack_a = !fx && !pow2_steps && !use_pair && !use_one && !use_defer && p.a_resident && steps_per_item >= 256;
     e.tiles_m = (fx || unpack_a) ? 0 : (int32_t)p.tiles_m;   // then only the weights are expanded here
@@ -1298,6 +1307,12 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     const int inst = fx ? 8 + (fx->bf16 ? 2 : 0) + (ybf ? 1 : 0) : (i8 ? 4 : 0) + (ybf ? 2 : 0) + (dbg ? 1 : 0);
     if (allow_smem(kernel, kSmemLimit, smem_done[inst], dev) != cudaSuccess) return TDQ_ERR_CUDA;
 
+    if (use_solo) {
+        a.tiles_n = (int32_t)((O + 63) / 64);
+        a.tma_ok = 0;
+        if (y_tma && encode_y_map(&ymap, y, y_dtype == TDQ_BF16, M, O, y_row_stride, kCols, kBM, y_f16)) a.tma_ok = 1;
+        return launch_linear_solo(a, ymap, dev, ybf, stream);
+    }
     if (use_pair) {
         a.tiles_n = (int32_t)((O + 63) / 64);
         // Few groups and few tiles: one block per tile, which expands its own operands, and the call is one launch.  Quantizer and

@@ -110,6 +110,8 @@ tdq_status launch_linear_pair(const LinArgs& a, const CUtensorMap& ymap, int n_s
                               cudaStream_t stream);   // two blocks per SM, tiles of 128 x 64 (tdq_linear_pair.cu)
 bool linear_defer_fits(bool y16, int32_t Kg);   // g = 32, 64, 128 with several tiles per SM (tdq_linear_defer.cu)
 tdq_status launch_linear_defer(LinArgs a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, cudaStream_t stream);
+// no more 128 x 64 tiles than SMs, one launch (tdq_linear_solo.cu)
+tdq_status launch_linear_solo(LinArgs a, const CUtensorMap& ymap, int dev, bool ybf, cudaStream_t stream);
 tdq_status launch_linear_g32(const LinArgs& a, const CUtensorMap& ymap, uint32_t smem_bytes, unsigned grid, bool ybf,
                              bool dbg, cudaStream_t stream);   // g = 32, long contractions (tdq_linear_g32.cu)
 // one accumulator per output element over the whole contraction (tdq_linear_one.cu)
