@@ -369,7 +369,8 @@ cudaError_t launch_fast(const ActArgs& a, cudaStream_t st) {
 // 16-byte grid): the same per-group code behind a staging pass that reads element by element.  A warp stages whole
 // groups, lane = channel (or channel pair of bf16), so every load instruction still reads up to 128 contiguous bytes;
 // channels past the end of the row are zeros.  The staging costs about as many instructions as the groups themselves.
-// Measured, 9217 x 147 fp32: 89 us in the bisection kernel that served these rows before, 7.0 us here.
+// Measured, 9217 x 147 fp32: 89 us in the bisection kernel that served these rows before, 7.0 us with batches of eight loads, 6.3
+// with all 32 of a warp in flight (20000 x 1000 fp32 47.8 -> 38.9; bf16, 16 at a time, 20689 x 161 12.6 -> 12.0).
 
 template <bool BF16, int KZR, int KB>
 __global__ void __launch_bounds__(kFastThreads) act_g32_ragged_kernel(ActArgs a, int32_t pairs_ok) {
@@ -409,7 +410,8 @@ __global__ void __launch_bounds__(kFastThreads) act_g32_ragged_kernel(ActArgs a,
         if (++k == a.K) { k = 0; row += pitch; }
     };
     if (pairs && lane >= 16) step();
-    constexpr int kBatch = 8;
+    constexpr int kBatch = BF16 ? 16 : 32;                // with pairs a batch is 32 groups, all that a warp stages
+    static_assert((BF16 ? 2 : 1) * kBatch <= 32, "a warp's groups");
 #pragma unroll 1
     for (int j0 = 0; j0 < 32; j0 += kBatch * per) {
         uint32_t v[kBatch];
@@ -448,8 +450,14 @@ template <bool BF16>
 cudaError_t launch_ragged(const ActArgs& a, cudaStream_t st) {
     const dim3 grid((unsigned)((a.total_groups + kFastThreads - 1) / kFastThreads)), block(kFastThreads);
     const int32_t pairs_ok = reinterpret_cast<uintptr_t>(a.x) % 4 == 0 && a.row_stride % 2 == 0;
-    // the paper's ranks have an instance of their own, every other pair shares the one with run-time ranks
-    if (a.k_base == 32 && a.k_zr == 7) return launch_pdl(act_g32_ragged_kernel<BF16, 7, 32>, grid, block, 0, st, a, pairs_ok);
+    // the zero-bin ranks of the paper's sweep have an instance of their own, every other pair shares the one with run-time ranks
+    if (a.k_base == 32) {
+        switch (a.k_zr) {
+#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_ragged_kernel<BF16, KZ, 32>, grid, block, 0, st, a, pairs_ok);
+            TDQ_CASE(4) TDQ_CASE(7) TDQ_CASE(10) TDQ_CASE(13) TDQ_CASE(16) TDQ_CASE(32)
+#undef TDQ_CASE
+        }
+    }
     return launch_pdl(act_g32_ragged_kernel<BF16, 0, 0>, grid, block, 0, st, a, pairs_ok);
 }
 
