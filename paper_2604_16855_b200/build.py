@@ -20,7 +20,7 @@ OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libtdq.so")
 HOST = os.path.join(HERE, "_tdq_host.so")
 HOST_SOURCE = "tdq_host.cpp"
-SOURCES = ["tdq_quantize_act.cu", "tdq_quantize_act_wide.cu", "tdq_quantize_weight.cu", "tdq_linear.cu", "tdq_linear_g32.cu", "tdq_linear_pair.cu", "tdq_linear_defer.cu", "tdq_linear_solo.cu", "tdq_linear_one.cu", "tdq_fused.cu", "tdq_api.cu", "tdq_peak.cu"]
+SOURCES = ["tdq_quantize_act.cu", "tdq_quantize_act_wide.cu", "tdq_quantize_weight.cu", "tdq_linear.cu", "tdq_linear_g32.cu", "tdq_linear_pair.cu", "tdq_linear_defer.cu", "tdq_linear_solo.cu", "tdq_linear_strip.cu", "tdq_linear_one.cu", "tdq_fused.cu", "tdq_api.cu", "tdq_peak.cu"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC", "--ftz=false", "--prec-div=true", "--prec-sqrt=true"]

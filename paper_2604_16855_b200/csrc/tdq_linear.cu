@@ -1249,6 +1249,31 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     // SMs the second round costs as much as the first (1200 x 320 -> 960 at g = 32, 150 tiles, 8.0 and 11.0).
     const bool use_solo = !acc_debug && !pow2_steps && !fx && !use_one && p.tiles_m * ((O + 63) / 64) <= n_sm &&
                           (group_size == 32 ? p.n_steps <= 28 && (p.n_steps > 4 || !y_tma) : p.n_steps <= (group_size == 64 ? 32 : 64));
+    // The two-blocks-per-SM kernel in one launch (see below): a block per tile, at most two rounds of them for a single column tile.
+    const int64_t tiles64 = p.tiles_m * ((O + 63) / 64);
+    const bool one_shot = use_g32 && !acc_debug && p.n_steps <= kPairRing && (tiles64 <= 2 * n_sm || (O <= 64 && p.n_steps <= 6 && tiles64 <= 4 * n_sm));
+    // g = 32 with a few 128 x 128 tiles per SM: one launch that expands a row block once for all its column tiles
+    // (tdq_linear_strip.cu).  us, quantizer and layer, the kernels that took these layers before and this one, called in turn / from a
+    // graph.  Up to 192 channels: 73728 x 64 -> 256 fp32 (1152 tiles) 32.5 and 28.0 / 29.4 and 27.7, 18432 x 128 -> 384 20.5 and 16.9 /
+    // 17.6 and 16.4, 18432 x 192 -> 768 29.6 and 27.7 / 26.5 and 27.0, but 60000 x 64 -> 500 (1876) 41.4 and 44.4 and 20000 x 192 ->
+    // 2048 (2512) 51.2 and 51.6.  From 224 to 288: 18432 x 224 -> 512 (576) 26.2 and 23.0 / 21.8 and 22.4, 18432 x 288 -> 640 bf16 (720)
+    // 30.1 and 27.1 / 27.1 and 26.4, but 18432 x 256 -> 1024 (1152) 35.5 and 34.4 / 31.6 and 33.7.  A single column tile: 18432 x 768 -> 128
+    // 30.6 and 26.2 / 27.4 and 25.8; 73728 x 256 -> 64, half of each tile empty, 34.9 and 33.5 / 32.3 and 33.1.  Up to a tile per SM: 1152 x
+    // 384 -> 1536 14.5 and 12.1 / 14.0 and 11.6, 1152 x 512 -> 2048 15.8 and 13.9 / 13.1 and 13.3, but 1152 x 640 -> 2000 16.4 and 15.6 / 13.7 and 15.0.
+    // From 320 to 512 channels and up to four tiles per SM the expansion's launch decides, which costs two microseconds in a stream
+    // and one in a graph: 9216 x 320 -> 960 bf16 (576) 24.6 and 22.9 / 21.6 and 22.3, 4608 x 320 -> 960 18.4 and 16.7 / 15.3 and 16.3, 4608 x
+    // 512 -> 1536 (432) 24.6 and 23.3 / 21.8 and 22.8.  One launch for a block per tile stays up to 192 channels (18432 x 192 -> 128 bf16 13.0
+    // and 13.4, 9216 x 64 -> 256 9.5 and 10.6); above, a row block is expanded too often there (2304 x 320 -> 960 13.4 and 12.8).
+    bool use_strip = use_g32 && y_tma && !acc_debug && !use_solo && O > 64 && linear_strip_fits(y_dtype == TDQ_BF16, p.n_steps) &&
+                     (p.n_steps <= 6    ? !one_shot && tiles128 <= 12 * n_sm
+                      : p.n_steps <= 9  ? tiles128 <= 5 * n_sm
+                      : p.n_steps <= 16 ? tiles128 <= 4 * n_sm
+                                        : p.n_steps <= 24 && O <= 128 && tiles128 <= 4 * n_sm);
+    if (use_strip && p.n_steps >= 10 && O > 128 && tiles128 > n_sm) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        use_strip = cudaStreamIsCapturing(stream, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone;
+        if (!use_strip) (void)cudaGetLastError();
+    }
     const bool use_pair = pair_ok && !use_defer;
     const bool unpack_a = !fx && !pow2_steps && !use_pair && !use_one && !use_defer && p.a_resident && steps_per_item >= 256;
     e.tiles_m = (fx || unpack_a) ? 0 : (int32_t)p.tiles_m;   // then only the weights are expanded here
@@ -1307,6 +1332,7 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     const int inst = fx ? 8 + (fx->bf16 ? 2 : 0) + (ybf ? 1 : 0) : (i8 ? 4 : 0) + (ybf ? 2 : 0) + (dbg ? 1 : 0);
     if (allow_smem(kernel, kSmemLimit, smem_done[inst], dev) != cudaSuccess) return TDQ_ERR_CUDA;
 
+    if (use_strip && a.tma_ok) return launch_linear_strip(a, ymap, n_sm, dev, ybf, stream);
     if (use_solo) {
         a.tiles_n = (int32_t)((O + 63) / 64);
         a.tma_ok = 0;
@@ -1322,9 +1348,7 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
         // each block column would expand the rows again.  A layer with one block column and few groups gains up to two rounds of
         // blocks (73728 x 64 -> 64 18.8 -> 17.2, 65536 x 160 -> 64 26.4 -> 24.0; 73728 x 256 -> 64 32.4 -> 33.1, 200000 x 128
         // -> 64 46.6 -> 50.7).
-        const int64_t tiles = p.tiles_m * a.tiles_n;
-        if (use_g32 && !dbg && p.n_steps <= kPairRing && (tiles <= 2 * n_sm || (a.tiles_n == 1 && p.n_steps <= 6 && tiles <= 4 * n_sm)))
-            return launch_linear_pair(a, ymap, n_sm, dev, ybf, false, true, stream);
+        if (one_shot) return launch_linear_pair(a, ymap, n_sm, dev, ybf, false, true, stream);
     }
     const unsigned pieces = (unsigned)((e.tiles_m + e.tiles_n) * p.n_chunks);
     if (pow2_steps) {

@@ -1,7 +1,8 @@
 // Shared pieces of the W4A4 linear layer's kernels: tile constants, the argument block, mbarrier /
 // bulk-copy / tcgen05 wrappers (inline PTX), the nibble-to-operand-byte expansion, the tensor map
 // of y and the shared-memory plan.  Included by tdq_linear.cu (the choice of kernel, the general one, the
-// fused and the power-of-two variants), tdq_linear_pair.cu, tdq_linear_defer.cu, tdq_linear_g32.cu and tdq_linear_one.cu.
+// fused and the power-of-two variants), tdq_linear_pair.cu, tdq_linear_defer.cu, tdq_linear_solo.cu, tdq_linear_strip.cu,
+// tdq_linear_g32.cu and tdq_linear_one.cu.
 #pragma once
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -112,6 +113,9 @@ bool linear_defer_fits(bool y16, int32_t Kg);   // g = 32, 64, 128 with several 
 tdq_status launch_linear_defer(LinArgs a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, cudaStream_t stream);
 // no more 128 x 64 tiles than SMs, one launch (tdq_linear_solo.cu)
 tdq_status launch_linear_solo(LinArgs a, const CUtensorMap& ymap, int dev, bool ybf, cudaStream_t stream);
+// g = 32, a few 128 x 128 tiles per SM, one launch (tdq_linear_strip.cu)
+bool linear_strip_fits(bool y16, int32_t n_steps);
+tdq_status launch_linear_strip(LinArgs a, const CUtensorMap& ymap, int n_sm, int dev, bool ybf, cudaStream_t stream);
 tdq_status launch_linear_g32(const LinArgs& a, const CUtensorMap& ymap, uint32_t smem_bytes, unsigned grid, bool ybf,
                              bool dbg, cudaStream_t stream);   // g = 32, long contractions (tdq_linear_g32.cu)
 // one accumulator per output element over the whole contraction (tdq_linear_one.cu)
