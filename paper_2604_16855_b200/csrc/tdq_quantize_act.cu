@@ -13,8 +13,8 @@
 //     projection, an exact quotient, round-half-even, and one 128-bit store of 32 nibbles.
 //     One pass over HBM: 2 (bf16) or 4 (fp32) bytes in, 0.5 + 0.125 bytes out per element.
 //   * act_g32_ragged_kernel   g = 32 on any other rows: staged element by element.
-//   * act_g32_nchw_kernel   channel-major input [B, C, H*W]: a tile of 32 channel rows is staged in
-//     shared memory and each thread gathers one position's 32 channels (tdq_quantize_act_nchw).
+//   * act_g32_nchw_kernel   channel-major input [B, C, H*W]: each thread loads one position's 32
+//     channels (tdq_quantize_act_nchw).
 //   * act_fixed_kernel   the fixed-radius control: no reductions, 8 channels per thread
 //     (tdq_quantize_act_fixed).
 //   * act_wide_kernel   (tdq_quantize_act_wide.cu) groups of a multiple of 8, any C, any alignment.
@@ -463,78 +463,57 @@ cudaError_t launch_ragged(const ActArgs& a, cudaStream_t st) {
 
 // ------------------------------------------------------------------------------------------
 // channel-major input: x is [B][C][H*W] (a convolutional feature map) and is quantized along C
-// without a permuted copy.  A CTA takes one group of 32 channels and 256 consecutive positions of
-// one image: the 32 channel rows are read with coalesced loads into a shared-memory tile, then
-// thread t gathers position t's 32 channels down the tile's columns and quantizes them like any
-// other group.  Codes and scales come out token-major, [B*H*W, C/2] and [B*H*W, C/32].
+// without a permuted copy.  A thread takes one group: it loads its position's 32 channels, all in flight together and next to
+// its neighbours', and quantizes them like any other group.  Codes and scales come out token-major, [B*H*W, C/2] and
+// [B*H*W, C/32].
 // A programmatic dependent like the other quantizers: its blocks are in place when the kernel before it ends, and the linear
 // layer behind it sets up under its tail ([8, 256, 48, 48] bf16 6.36 -> 5.97 us, [1, 64, 56, 56] fp32 3.17 -> 2.76).
+// Bound by the instructions of the groups.  64 positions a block: ten blocks fill an SM's registers without the remainder that two
+// of 256 threads leave, and a row's last block wastes less.  us, before (blocks of 256 positions behind a tile in shared memory,
+// element-wise loads four at a time where rows are off the 16-byte grid) and now, bf16: [16, 320, 24, 24] 6.4 -> 5.0, [16, 768, 24, 24]
+// 12.2 -> 8.0, [16, 512, 60, 60] 39.1 -> 25.2, [16, 512, 33, 35] 33.5 -> 10.1, [2, 320, 7, 7] 3.1 -> 1.75; fp32: [16, 320, 24, 24] 7.2 -> 5.7,
+// [16, 256, 31, 31] 15.3 -> 7.0, [16, 768, 12, 12] 4.9 -> 5.4.  A tile in shared memory on 16-byte loads is level or up to 4 %
+// slower at 64 positions, 128 positions up to 11 %, 32 up to 5 %.
+constexpr int kNchwThreads = 64;
 
 struct NchwArgs {
     ActArgs a;          // x, K, k_zr, seven_tau, flags, codes, scale, offset
     int64_t HW;         // positions per image
-    int32_t vec_ok;     // channel rows can be read with 16-byte loads
 };
 
 template <bool BF16, int KZR>
-__global__ void __launch_bounds__(kFastThreads) act_g32_nchw_kernel(NchwArgs n) {
+__global__ void __launch_bounds__(kNchwThreads) act_g32_nchw_kernel(NchwArgs n) {
     constexpr int esz = BF16 ? 2 : 4;
-    constexpr int kRowBytes = kFastThreads * esz + 16;        // 16 bytes of padding per channel row
-    constexpr int kVecPerRow = kFastThreads * esz / 16;       // 16-byte pieces of a channel row
-    __shared__ __align__(16) uint8_t tile[32 * kRowBytes];
     const ActArgs& a = n.a;
     const int t = threadIdx.x;
-    const int64_t s0 = (int64_t)blockIdx.x * kFastThreads;    // first position of the tile
+    const int64_t s0 = (int64_t)blockIdx.x * kNchwThreads;    // first position of the block
     const int k = blockIdx.y;                                  // channel group
     const int64_t b = blockIdx.z;
-    const uint8_t* img = reinterpret_cast<const uint8_t*>(a.x) + ((b * a.C + (int64_t)k * 32) * n.HW + s0) * esz;
-    const int64_t left = n.HW - s0;                            // positions from s0 to the end of the image
     pdl_wait();
     pdl_trigger();
-    if (n.vec_ok) {
-#pragma unroll
-        for (int j = 0; j < 32 * kVecPerRow / kFastThreads; ++j) {
-            const int idx = t + j * kFastThreads;
-            const int c = idx / kVecPerRow, piece = idx % kVecPerRow;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if ((int64_t)(piece + 1) * (16 / esz) <= left)     // HW is a multiple of 16 bytes here: pieces are whole
-                v = __ldg(reinterpret_cast<const uint4*>(img + (int64_t)c * n.HW * esz) + piece);
-            *reinterpret_cast<uint4*>(tile + c * kRowBytes + piece * 16) = v;
-        }
-    } else {
-#pragma unroll 4
-        for (int c = 0; c < 32; ++c) {
-            const uint8_t* src = img + ((int64_t)c * n.HW + t) * esz;
-            if (BF16)
-                *reinterpret_cast<uint16_t*>(tile + c * kRowBytes + t * 2) =
-                    t < left ? __ldg(reinterpret_cast<const uint16_t*>(src)) : (uint16_t)0;
-            else
-                *reinterpret_cast<uint32_t*>(tile + c * kRowBytes + t * 4) =
-                    t < left ? __ldg(reinterpret_cast<const uint32_t*>(src)) : 0u;
-        }
-    }
-    __syncthreads();
-    if (t >= left) return;
+    if (t >= n.HW - s0) return;
+    const int64_t row = n.HW * esz;
+    const uint8_t* src = reinterpret_cast<const uint8_t*>(a.x) + (b * a.C + (int64_t)k * 32) * row + (s0 + t) * esz;
     uint32_t w[BF16 ? 16 : 32];
     if (BF16) {
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-            const uint32_t lo = *reinterpret_cast<const uint16_t*>(tile + (2 * i) * kRowBytes + t * 2);
-            const uint32_t hi = *reinterpret_cast<const uint16_t*>(tile + (2 * i + 1) * kRowBytes + t * 2);
+            const uint32_t lo = __ldg(reinterpret_cast<const uint16_t*>(src + (2 * i) * row));
+            const uint32_t hi = __ldg(reinterpret_cast<const uint16_t*>(src + (2 * i + 1) * row));
             w[i] = lo | (hi << 16);
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) w[i] = *reinterpret_cast<const uint32_t*>(tile + i * kRowBytes + t * 4);
+        for (int i = 0; i < 32; ++i) w[i] = __ldg(reinterpret_cast<const uint32_t*>(src + i * row));
     }
     process_group<BF16, KZR>(w, a, ((b * n.HW + s0 + t) * a.K) + k);
 }
 
 template <bool BF16>
 cudaError_t launch_nchw(const NchwArgs& n, int64_t B, cudaStream_t st) {
-    dim3 grid((unsigned)((n.HW + kFastThreads - 1) / kFastThreads), (unsigned)n.a.K, (unsigned)B);
+    dim3 grid((unsigned)((n.HW + kNchwThreads - 1) / kNchwThreads), (unsigned)n.a.K, (unsigned)B);
     switch (n.a.k_zr) {
-#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_nchw_kernel<BF16, KZ>, grid, dim3(kFastThreads), 0, st, n);
+#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_nchw_kernel<BF16, KZ>, grid, dim3(kNchwThreads), 0, st, n);
         TDQ_CASE(4) TDQ_CASE(7) TDQ_CASE(10) TDQ_CASE(13) TDQ_CASE(16) TDQ_CASE(32)
 #undef TDQ_CASE
         default: return cudaErrorInvalidValue;
@@ -719,7 +698,7 @@ extern "C" tdq_status tdq_quantize_act_nchw(const void* x, tdq_dtype x_dtype, in
     if (g != 32 || C % 32 != 0 || rank_of(p->base_percentile, g) != g || reinterpret_cast<uintptr_t>(codes) % 16 ||
         ((p->flags & TDQ_ENABLE_C2) && !fast_rank(rank_of(p->zr, g))))
         return TDQ_ERR_UNSUPPORTED;
-    if (C / 32 > 65535 || B > 65535 || (HW + kFastThreads - 1) / kFastThreads > INT32_MAX) return TDQ_ERR_UNSUPPORTED;
+    if (C / 32 > 65535 || B > 65535 || (HW + kNchwThreads - 1) / kNchwThreads > INT32_MAX) return TDQ_ERR_UNSUPPORTED;
     NchwArgs n;
     n.a.x = x;
     n.a.M = B * HW;
@@ -736,8 +715,6 @@ extern "C" tdq_status tdq_quantize_act_nchw(const void* x, tdq_dtype x_dtype, in
     n.a.scale = scale;
     n.a.offset = offset;
     n.HW = HW;
-    const int64_t esz = x_dtype == TDQ_BF16 ? 2 : 4;
-    n.vec_ok = (reinterpret_cast<uintptr_t>(x) % 16 == 0 && (HW * esz) % 16 == 0) ? 1 : 0;
     cudaStream_t stream = reinterpret_cast<cudaStream_t>(cuda_stream);
     const cudaError_t e = (x_dtype == TDQ_BF16) ? launch_nchw<true>(n, B, stream) : launch_nchw<false>(n, B, stream);
     if (e != cudaSuccess) return TDQ_ERR_CUDA;

@@ -1,0 +1,21 @@
+"""The channel-major quantizer at the edges of its 64-position blocks, with channel rows on and off the 16-byte grid, against the
+row-major kernel on the permuted tensor (itself pinned to the oracle): the same bits."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("H,W", [(1, 1), (1, 8), (3, 7), (1, 63), (8, 8), (1, 65), (9, 8), (12, 12), (1, 127), (16, 8), (11, 12), (17, 19), (24, 24)])
+@pytest.mark.parametrize("B,C,first", [(1, 32, 0), (3, 96, 0), (2, 64, 1)])
+def test_shapes(B, C, H, W, first, dtype):
+    from paper_2604_16855_b200 import tdq
+    gen = torch.Generator("cuda").manual_seed(B + C + H * W)
+    store = torch.randn((first + B * C * H * W,), device="cuda", generator=gen).to(dtype)
+    x = store[first:].view(B, C, H, W)          # first = 1: no row of x is on the 16-byte grid
+    for zr in (0.1, 0.2, 0.3):
+        p = tdq.act_params(zr=zr)
+        codes, scale = tdq.quantize_act_nchw(x, p)
+        want_codes, want_scale = tdq.quantize_act(x.permute(0, 2, 3, 1).reshape(-1, C).contiguous(), p)
+        assert torch.equal(codes.view(want_codes.shape), want_codes) and torch.equal(scale.view(want_scale.shape), want_scale)
