@@ -284,7 +284,7 @@ tdq_status tdq_workspace_status(const void* workspace, void* cuda_stream, uint32
  * (tdq_quantize_act and its variants, which have no workspace) record a bounded wait that ran out:
  * TDQ_OK, or TDQ_ERR_DEVICE_TIMEOUT when one did since the last query (codes and scales of that
  * call are then incomplete).  detail (HOST, nullable) receives the raw word: bits 0-7 name the wait
- * (12 the tile producer, 13 a consumer warp, 14 the self-test), bits 8-31 the thread block.  A
+ * (14 the self-test; no quantizer kernel waits at present), bits 8-31 the thread block.  A
  * non-zero word is cleared by the query.  The word is shared by all streams of the device.
  */
 tdq_status tdq_quantize_status(void* cuda_stream, uint32_t* detail /* HOST */);

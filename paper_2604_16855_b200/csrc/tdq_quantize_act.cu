@@ -1,16 +1,10 @@
 // tdq_quantize_act: token-group dual-constraint activation quantizer (Algorithm S1 steps 1-7).
 //
-// Seven kernels:
-//   * act_g32_ring_kernel   the fast path on dense rows (row stride == C): persistent, two CTAs per
-//     SM; one producer lane streams 16 KB tiles of 256 groups into a shared-memory ring with 1-D
-//     bulk copies and mbarrier transaction counts, eight consumer warps take one group per thread
-//     (the per-group arithmetic is in tdq_act_group.cuh).
-//   * act_g32_kernel   the same per-group code for strided rows: g = 32, C % 32 == 0, 16-byte
-//     aligned rows.  A CTA stages a tile of
-//     consecutive token-groups in shared memory with coalesced 128-bit loads (XOR-swizzled
-//     so the read-back is conflict free); then every thread owns one whole group in
-//     registers: max, sums, a pruned sorting network for the rank-k magnitude, the DCRP
-//     projection, an exact quotient, round-half-even, and one 128-bit store of 32 nibbles.
+// Six kernels:
+//   * act_g32_kernel   the fast path: g = 32, C % 32 == 0, 16-byte aligned rows.  A thread owns one
+//     whole group in registers: max, sums, a pruned sorting network for the rank-k magnitude, the DCRP
+//     projection, an exact quotient, round-half-even, and one 128-bit store of 32 nibbles (the
+//     per-group arithmetic is in tdq_act_group.cuh).
 //     One pass over HBM: 2 (bf16) or 4 (fp32) bytes in, 0.5 + 0.125 bytes out per element.
 //   * act_g32_ragged_kernel   g = 32 on any other rows: staged element by element.
 //   * act_g32_nchw_kernel   channel-major input [B, C, H*W]: each thread loads one position's 32
@@ -124,7 +118,9 @@ __global__ void __launch_bounds__(kGenericWarps * 32) act_generic_kernel(ActArgs
 // ------------------------------------------------------------------------------------------
 // fast kernel: g = 32, one thread per group
 
-constexpr int kFastThreads = 256;   // groups per CTA tile
+// Threads, and so groups, of a block of the fast kernels.  Small blocks: ten of them fill an SM's registers without the remainder
+// that two of 256 threads leave, and no warp waits for more than one other.
+constexpr int kFastThreads = 64;
 
 // One group: quantize it in registers, write its 16 code bytes and its scale.
 template <bool BF16, int KZR, int KB = 32>
@@ -137,191 +133,75 @@ __device__ __forceinline__ void process_group(const uint32_t (&w)[BF16 ? 16 : 32
     if (a.offset) a.offset[gi] = 0.0f;
 }
 
+// Bound by the instructions of the groups (about 490 a thread, of which the ALU pipe takes most).  Warps that depend on
+// nothing but their own loads keep the pipes fed better than a persistent block with a ring of bulk copies, whose first and last
+// tiles cost a latency each and whose number of tiles is rarely a multiple of the blocks; us, that ring (two blocks of eight working
+// warps per SM) and this: bf16 18464 x 768 13.7 and 11.8, 73728 x 256 17.0 and 14.9, 9216 x 320 5.9 and 3.8, 1152 x 512 2.4 and 1.75, 16384 x
+// 4096 50.4 and 46.3; fp32 18464 x 768 22.6 and 16.2, 9216 x 320 8.8 and 4.9, 256 x 64 3.3 and 1.7.
+// A bf16 group is four 16-byte loads of its own thread, whose sectors the neighbours share.  An fp32 group is eight, too far apart
+// for that, so a warp loads its 32 groups in order and passes them on through its own part of shared memory (18464 x 768 17.2
+// against 16.2 us, 9216 x 320 6.2 and 4.9; bf16 11.8 against 12.0); rows with a pitch, which cost a division a group, are loaded
+// directly in either type.  Blocks of 128 threads: level, long bf16 inputs 1 to 2 % slower.
 template <bool BF16, int KZR, int KB = 32>
 __global__ void __launch_bounds__(kFastThreads) act_g32_kernel(ActArgs a) {
     constexpr int kGroupBytes = BF16 ? 64 : 128;
     constexpr int kChunks = kGroupBytes / 16;          // 16-byte chunks per group
-    constexpr int kSwzMask = kChunks - 1;
-    __shared__ __align__(16) uint4 tile[kFastThreads * kChunks];
-
+    const int t = threadIdx.x;
+    const int64_t gi = (int64_t)blockIdx.x * kFastThreads + t;
+    const char* xb = reinterpret_cast<const char*>(a.x);
+    const bool flat = a.row_stride == a.C;
+    uint32_t w[kChunks * 4];                           // this thread's group: 16 packed bf16 pairs or 32 floats
     pdl_wait();
     pdl_trigger();
-    const int t = threadIdx.x;
-    const int64_t g0 = (int64_t)blockIdx.x * kFastThreads;
-    const char* xb = reinterpret_cast<const char*>(a.x);
-    const int64_t esize = BF16 ? 2 : 4;
-    const bool flat = (a.row_stride == a.C);
-
-    // stage: coalesced 16-byte loads; chunk p of local group l lands at l*kChunks + (p ^ swz(l))
-#pragma unroll
-    for (int j = 0; j < kChunks; ++j) {
-        const int ch = t + j * kFastThreads;
-        const int l = ch / kChunks, p = ch % kChunks;
-        const int64_t gi = g0 + l;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (gi < a.total_groups) {
-            int64_t off;
-            if (flat) {
-                off = gi * kGroupBytes + p * 16;
+    if (BF16 || !flat) {
+        if (gi >= a.total_groups) return;
+        int64_t off = gi * kGroupBytes;
+        if (!flat) {
+            int64_t m, k;
+            if (a.total_groups <= 0x7fffffff) {
+                m = (uint32_t)gi / (uint32_t)a.K;
+                k = (uint32_t)gi - (uint32_t)m * (uint32_t)a.K;
             } else {
-                const int64_t m = gi / a.K;
-                const int64_t k = gi - m * a.K;
-                off = (m * a.row_stride + k * 32) * esize + p * 16;
+                m = gi / a.K;
+                k = gi - m * a.K;
             }
-            v = __ldg(reinterpret_cast<const uint4*>(xb + off));
+            off = m * a.row_stride * (BF16 ? 2 : 4) + k * kGroupBytes;
         }
-        const int swz = BF16 ? ((l >> 1) & kSwzMask) : (l & kSwzMask);
-        tile[l * kChunks + (p ^ swz)] = v;
-    }
-    __syncthreads();
-
-    const int64_t gi = g0 + t;
-    if (gi >= a.total_groups) return;
-
-    // this thread's group: words w[], 16 packed bf16 pairs or 32 floats
-    uint32_t w[kChunks * 4];
-    {
-        const int swz = BF16 ? ((t >> 1) & kSwzMask) : (t & kSwzMask);
+        const uint4* src = reinterpret_cast<const uint4*>(xb + off);
 #pragma unroll
         for (int p = 0; p < kChunks; ++p) {
-            uint4 v = tile[t * kChunks + (p ^ swz)];
+            const uint4 v = __ldg(src + p);
             w[4 * p + 0] = v.x; w[4 * p + 1] = v.y; w[4 * p + 2] = v.z; w[4 * p + 3] = v.w;
+        }
+    } else {
+        // chunk p of the warp's group l lands at l * kChunks + (p ^ l % kChunks): conflict-free both ways
+        __shared__ __align__(16) uint4 tile[BF16 ? 1 : kFastThreads * kChunks];
+        const int lane = t & 31, w0 = t & ~31;
+        const int64_t g0 = gi - lane;
+        const uint4* src = reinterpret_cast<const uint4*>(xb + g0 * kGroupBytes) + lane;
+        uint4 v[kChunks];
+#pragma unroll
+        for (int j = 0; j < kChunks; ++j) {
+            v[j] = make_uint4(0u, 0u, 0u, 0u);
+            if (g0 + (lane + 32 * j) / kChunks < a.total_groups) v[j] = __ldg(src + 32 * j);
+        }
+#pragma unroll
+        for (int j = 0; j < kChunks; ++j) {
+            const int ch = lane + 32 * j, l = ch / kChunks, p = ch % kChunks;
+            tile[(w0 + l) * kChunks + (p ^ (l % kChunks))] = v[j];
+        }
+        __syncwarp();
+        if (gi >= a.total_groups) return;
+#pragma unroll
+        for (int p = 0; p < kChunks; ++p) {
+            const uint4 u = tile[t * kChunks + (p ^ (t % kChunks))];
+            w[4 * p + 0] = u.x; w[4 * p + 1] = u.y; w[4 * p + 2] = u.z; w[4 * p + 3] = u.w;
         }
     }
     process_group<BF16, KZR, KB>(w, a, gi);
 }
 
-// ------------------------------------------------------------------------------------------
-// fast kernel for dense rows (row stride == C): persistent CTAs, bulk-copy ring
-//
-// Consecutive groups are consecutive in memory, so a tile of 256 groups is one contiguous
-// piece (16 KB of bf16, 32 KB of fp32).  A producer lane streams tiles into a ring of
-// shared-memory stages with cp.async.bulk; the 256 consumer threads take one group each out of
-// a stage, hand the stage back, and then spend their time on the selection network while the
-// next tiles are already landing.  Waits are bounded (see kRingTimeout).
-
-constexpr int kRingStagesBf16 = 4, kRingStagesF32 = 3;
-constexpr int kRingThreads = kFastThreads + 32;
-constexpr long long kRingTimeout = 2000000000LL;
-// A ring wait that ran out leaves its code here (first writer wins): bits 0-7 name the wait (12 producer, 13 consumer,
-// 14 the self-test), bits 8-31 the CTA.  One word per device, read and cleared by tdq_quantize_status().
-__device__ uint32_t g_act_wait_status = 0u;
-
-__device__ __forceinline__ uint32_t ring_smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ bool ring_test(uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(ring_smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// false when the phase did not complete in about a second (the caller then stops working)
-__device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, uint32_t code,
-                                          long long limit = kRingTimeout) {
-    if (ring_test(bar, parity)) return true;
-    long long t0 = 0;
-    uint32_t polls = 0;
-#pragma unroll 1
-    while (!ring_test(bar, parity)) {
-        if ((++polls & 63u) == 0u) {
-            if (*abort_flag) return false;
-            const long long now = clock64();
-            if (t0 == 0) t0 = now;
-            if (now - t0 > limit) {
-                atomicCAS(&g_act_wait_status, 0u, code | ((uint32_t)blockIdx.x << 8));
-                *abort_flag = 1;
-                return false;
-            }
-        }
-    }
-    return true;
-}
-
-template <bool BF16, int KZR, int KB = 32>
-__global__ void __launch_bounds__(kRingThreads) act_g32_ring_kernel(ActArgs a, int64_t n_tiles) {
-    constexpr int kGroupBytes = BF16 ? 64 : 128;
-    constexpr int kChunks = kGroupBytes / 16;
-    constexpr int kStages = BF16 ? kRingStagesBf16 : kRingStagesF32;
-    constexpr int kStageBytes = kFastThreads * kGroupBytes;
-    extern __shared__ __align__(128) uint8_t ring_smem[];
-    __shared__ uint64_t full[kStages], empty[kStages];
-    __shared__ volatile int abort_flag;
-    const int t = threadIdx.x;
-    if (t == 0) {
-        for (int i = 0; i < kStages; ++i) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(ring_smem_u32(&full[i])), "r"(1) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(ring_smem_u32(&empty[i])), "r"(kFastThreads / 32) : "memory");
-        }
-        abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-    pdl_wait();          // everything above overlaps the tail of the kernel before this one
-    pdl_trigger();
-    const char* xb = reinterpret_cast<const char*>(a.x);
-    if (t >= kFastThreads) {
-        if (t == kFastThreads) {   // producer lane
-            uint32_t s = 0, ph = 0;
-            for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-                if (!ring_wait(&empty[s], ph ^ 1, &abort_flag, 12u)) break;
-                const int64_t g0 = tile * kFastThreads;
-                const int64_t ng = min((int64_t)kFastThreads, a.total_groups - g0);
-                const uint32_t bytes = (uint32_t)(ng * kGroupBytes);
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(ring_smem_u32(&full[s])), "r"(bytes) : "memory");
-                asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                             ::"r"(ring_smem_u32(ring_smem + (size_t)s * kStageBytes)), "l"(xb + g0 * kGroupBytes), "r"(bytes),
-                               "r"(ring_smem_u32(&full[s]))
-                             : "memory");
-                if (++s == kStages) { s = 0; ph ^= 1; }
-            }
-        }
-        return;
-    }
-    uint32_t s = 0, ph = 0;
-    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        if (!__all_sync(0xffffffffu, ring_wait(&full[s], ph, &abort_flag, 13u))) break;
-        const int64_t gi = tile * kFastThreads + t;
-        uint32_t w[kChunks * 4];
-        // volatile loads: the stage is handed back right below, so these must be the only reads of it
-        const uint32_t src = ring_smem_u32(ring_smem + (size_t)s * kStageBytes + (size_t)t * kGroupBytes);
-#pragma unroll
-        for (int p = 0; p < kChunks; ++p)
-            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(w[4 * p + 0]), "=r"(w[4 * p + 1]), "=r"(w[4 * p + 2]), "=r"(w[4 * p + 3])
-                         : "r"(src + p * 16)
-                         : "memory");
-        // The producer refills the stage through the async proxy as soon as the eighth warp has
-        // arrived.  Reads made through the generic proxy are only ordered before such writes by a
-        // proxy fence; without it the refill was observed to overtake these loads.
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if ((t & 31) == 0)
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ring_smem_u32(&empty[s])) : "memory");
-        if (++s == kStages) { s = 0; ph ^= 1; }
-        if (gi < a.total_groups) process_group<BF16, KZR, KB>(w, a, gi);
-    }
-}
-
-template <bool BF16, int KZR, int KB = 32>
-cudaError_t launch_ring(const ActArgs& a, cudaStream_t st) {
-    constexpr int kStages = BF16 ? kRingStagesBf16 : kRingStagesF32;
-    constexpr int smem = kStages * kFastThreads * (BF16 ? 64 : 128);
-    static std::atomic<uint64_t> attr_done{0};      // per template instance, one bit per device
-    int dev = 0;
-    const int n_sm = current_device_sm_count(&dev);
-    if (n_sm <= 0) return cudaErrorUnknown;
-    const cudaError_t e = allow_smem(act_g32_ring_kernel<BF16, KZR, KB>, smem, attr_done, dev);
-    if (e != cudaSuccess) return e;
-    const int64_t n_tiles = (a.total_groups + kFastThreads - 1) / kFastThreads;
-    const int64_t grid = n_tiles < 2 * n_sm ? n_tiles : 2 * n_sm;
-    return launch_pdl(act_g32_ring_kernel<BF16, KZR, KB>, dim3((unsigned)grid), dim3(kRingThreads), smem, st, a, n_tiles);
-}
-
-// every zero-bin rank of a group of 32 has its instance of the two row-major kernels
+// every zero-bin rank of a group of 32 has its instance of the row-major kernel
 #define TDQ_ALL_RANKS \
     TDQ_CASE(1) TDQ_CASE(2) TDQ_CASE(3) TDQ_CASE(4) TDQ_CASE(5) TDQ_CASE(6) TDQ_CASE(7) TDQ_CASE(8) \
     TDQ_CASE(9) TDQ_CASE(10) TDQ_CASE(11) TDQ_CASE(12) TDQ_CASE(13) TDQ_CASE(14) TDQ_CASE(15) TDQ_CASE(16) \
@@ -333,24 +213,12 @@ cudaError_t launch_fast(const ActArgs& a, cudaStream_t st) {
     dim3 grid((unsigned)blocks), block(kFastThreads);
     if (a.k_base != 32 && (a.k_base < 29 || a.k_zr != 7)) {
         // any other pair of ranks: the instance that takes both at run time
-        if (a.row_stride == a.C) return launch_ring<BF16, 0, 0>(a, st);
         return launch_pdl(act_g32_kernel<BF16, 0, 0>, grid, block, 0, st, a);
     }
     if (a.k_base != 32) {        // percentile base radius: ranks 29..31 beside the default zero-bin rank
         switch (a.k_base) {
-#define TDQ_CASE(KB_)                                                                  \
-            case KB_:                                                                  \
-                if (a.row_stride == a.C) return launch_ring<BF16, 7, KB_>(a, st);      \
-                return launch_pdl(act_g32_kernel<BF16, 7, KB_>, grid, block, 0, st, a);
+#define TDQ_CASE(KB_) case KB_: return launch_pdl(act_g32_kernel<BF16, 7, KB_>, grid, block, 0, st, a);
             TDQ_CASE(29) TDQ_CASE(30) TDQ_CASE(31)
-#undef TDQ_CASE
-            default: return cudaErrorInvalidValue;
-        }
-    }
-    if (a.row_stride == a.C) {   // dense rows: the persistent ring kernel
-        switch (a.k_zr) {
-#define TDQ_CASE(KZ) case KZ: return launch_ring<BF16, KZ>(a, st);
-            TDQ_ALL_RANKS
 #undef TDQ_CASE
             default: return cudaErrorInvalidValue;
         }
@@ -361,7 +229,6 @@ cudaError_t launch_fast(const ActArgs& a, cudaStream_t st) {
 #undef TDQ_CASE
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------------------------
@@ -372,16 +239,19 @@ cudaError_t launch_fast(const ActArgs& a, cudaStream_t st) {
 // Measured, 9217 x 147 fp32: 89 us in the bisection kernel that served these rows before, 7.0 us with batches of eight loads, 6.3
 // with all 32 of a warp in flight (20000 x 1000 fp32 47.8 -> 38.9; bf16, 16 at a time, 20689 x 161 12.6 -> 12.0).
 
+// Blocks of 256 threads: with 64 the kernel alone is up to a microsecond faster (9217 x 147 fp32 5.9 -> 4.8), but all SMs then finish
+// together and the layer behind it has none to set itself up on: 9217 x 147 -> 63 as a pair 11.9 -> 12.6.
+constexpr int kRaggedThreads = 256;
 template <bool BF16, int KZR, int KB>
-__global__ void __launch_bounds__(kFastThreads) act_g32_ragged_kernel(ActArgs a, int32_t pairs_ok) {
+__global__ void __launch_bounds__(kRaggedThreads) act_g32_ragged_kernel(ActArgs a, int32_t pairs_ok) {
     constexpr int kGroupBytes = BF16 ? 64 : 128;
     constexpr int kChunks = kGroupBytes / 16;
     constexpr int kSwzMask = kChunks - 1;
-    __shared__ __align__(16) uint4 tile[kFastThreads * kChunks];
+    __shared__ __align__(16) uint4 tile[kRaggedThreads * kChunks];
     pdl_wait();
     pdl_trigger();
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int64_t g0 = (int64_t)blockIdx.x * kFastThreads;
+    const int64_t g0 = (int64_t)blockIdx.x * kRaggedThreads;
     uint8_t* tb = reinterpret_cast<uint8_t*>(tile);
     // channel `e` of local group `l` lands where act_g32_kernel's 16-byte pieces put it
     auto slot = [&](int l, int e) -> uint8_t* {
@@ -448,7 +318,7 @@ __global__ void __launch_bounds__(kFastThreads) act_g32_ragged_kernel(ActArgs a,
 
 template <bool BF16>
 cudaError_t launch_ragged(const ActArgs& a, cudaStream_t st) {
-    const dim3 grid((unsigned)((a.total_groups + kFastThreads - 1) / kFastThreads)), block(kFastThreads);
+    const dim3 grid((unsigned)((a.total_groups + kRaggedThreads - 1) / kRaggedThreads)), block(kRaggedThreads);
     const int32_t pairs_ok = reinterpret_cast<uintptr_t>(a.x) % 4 == 0 && a.row_stride % 2 == 0;
     // the zero-bin ranks of the paper's sweep have an instance of their own, every other pair shares the one with run-time ranks
     if (a.k_base == 32) {
@@ -754,21 +624,60 @@ extern "C" tdq_status tdq_quantize_act_fixed(const void* x, tdq_dtype x_dtype, i
 }
 
 // ------------------------------------------------------------------------------------------
-// bounded waits of the quantizer: the status word and the self-test
+// bounded waits of the quantizer: the status word, the routine and the self-test
 
 namespace tdq {
 namespace {
-// One warp: a fresh barrier with one expected arrival that never comes, waited on with the ring kernel's own
+// A wait of a quantizer kernel that ran out leaves its code here (first writer wins): bits 0-7 name the wait (14 the
+// self-test; no quantizer kernel waits on a barrier at present), bits 8-31 the CTA.  One word per device, read and cleared by
+// tdq_quantize_status().
+__device__ uint32_t g_act_wait_status = 0u;
+
+__device__ __forceinline__ uint32_t act_smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ bool act_wait_test(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(act_smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// false when the phase did not complete in about a second (the caller then stops working)
+__device__ __forceinline__ bool act_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, uint32_t code,
+                                          long long limit) {
+    if (act_wait_test(bar, parity)) return true;
+    long long t0 = 0;
+    uint32_t polls = 0;
+#pragma unroll 1
+    while (!act_wait_test(bar, parity)) {
+        if ((++polls & 63u) == 0u) {
+            if (*abort_flag) return false;
+            const long long now = clock64();
+            if (t0 == 0) t0 = now;
+            if (now - t0 > limit) {
+                atomicCAS(&g_act_wait_status, 0u, code | ((uint32_t)blockIdx.x << 8));
+                *abort_flag = 1;
+                return false;
+            }
+        }
+    }
+    return true;
+}
+
+// One warp: a fresh barrier with one expected arrival that never comes, waited on with that
 // routine and a short limit.  Nothing is in flight when the warp leaves.
 __global__ void __launch_bounds__(32) act_wait_selftest_kernel(long long limit) {
     __shared__ uint64_t bar;
     __shared__ volatile int abort_flag;
     if (threadIdx.x == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(ring_smem_u32(&bar)) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(act_smem_u32(&bar)) : "memory");
         abort_flag = 0;
     }
     __syncwarp();
-    ring_wait(&bar, 0u, &abort_flag, 14u, limit);
+    act_wait(&bar, 0u, &abort_flag, 14u, limit);
 }
 }  // namespace
 

@@ -1,0 +1,28 @@
+"""The row-major quantizer at g = 32 at the edges of its 64-group blocks and 32-group warps: dense rows and rows with a pitch, both
+input types, every block boundary, against the oracle; nothing written past the last group."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth_inputs as si
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("pad", [0, 8])
+@pytest.mark.parametrize("M,K", [(1, 1), (1, 3), (31, 1), (32, 1), (33, 1), (1, 63), (64, 1), (13, 5), (9, 7), (19, 5), (96, 1), (1, 127), (64, 2), (43, 3), (5, 64)])
+def test_block_edges(M, K, pad, dtype):
+    from paper_2604_16855_b200 import tdq
+    rng = np.random.default_rng(100 * M + K)
+    x = si.token_mixture(rng, 1, M, 32 * K, sigma_log_std=0.5, bg_frac=0.1, bg_nu=3.0, bg_amp=20.0).reshape(M, 32 * K)
+    store = torch.zeros((M, 32 * K + pad), dtype=dtype, device="cuda")
+    store[:, :32 * K] = torch.from_numpy(x).to(dtype)
+    xt = store[:, :32 * K]
+    want = oracle.quantize_act(xt.float().cpu().numpy())
+    codes = torch.full((M + 1, 16 * K), 77, dtype=torch.uint8, device="cuda")
+    scale = torch.full((M + 1, K), -1.0, device="cuda")
+    tdq.quantize_act(xt, codes=codes[:M], scale=scale[:M])
+    assert np.array_equal(codes[:M].cpu().numpy(), want["codes"]) and np.array_equal(scale[:M].cpu().numpy(), want["scale"])
+    assert bool((codes[M] == 77).all()) and bool((scale[M] == -1.0).all())
