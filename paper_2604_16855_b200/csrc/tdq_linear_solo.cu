@@ -22,7 +22,8 @@
 // code takes one bit operation as q + 8, and a second instruction with a constant block of -8 takes 8 sum q_w off again
 // (exact: everything is below 2^12 in units of 2^-18); the sign-and-magnitude bytes that the weights get cost five times
 // as much.  Wider groups go as int8: 16 q is a mask or a shift away from the codes, and a group's conversion to float is
-// spread over several K-steps.
+// spread over several K-steps.  The promotion works in the units of the kernels that take these groups elsewhere (E4M3's 2^-18 up
+// to 128 codes a group), so a sum is finite here exactly where it is finite there.
 //
 // Measured (B200, from a graph), us, against the expansion and the kernels behind it: 1152 x 512 -> 512 fp32 at g = 32 8.1 -> 7.6,
 // at g = 64 8.0 -> 5.9; 576 x 320 -> 960 at g = 32 6.8 -> 6.0; 200 x 768 -> 768 bf16 at g = 768 7.8 -> 5.7; 128 x 1312 -> 56 fp16 at
@@ -309,6 +310,11 @@ __global__ void __launch_bounds__(kSoloThreads, 1) w4a4_solo_kernel(const LinArg
         asm volatile("" : "+r"(tfull_s), "+r"(tempty_s), "+r"(tmem_row));
         const int64_t m_row = (int64_t)mt * kBM + row;
         const float* gx = a.xscale + (m_row < a.M ? m_row : 0) * a.Kg;   // otherwise the steps come from memory, a group ahead
+        // int8 sums are 256 times the group's.  Up to 128 codes a group the other kernels add sums in units of 2^-18 (E4M3), beyond
+        // that 256 times the sums; the same units here, or a product near the ends of binary32's range would be rounded or
+        // overflow in one kernel and not in the other.  (Exact: a power of two, and the sums are whole numbers below 2^26.)
+        const uint32_t unit = a.steps_per_grp <= 4 ? 0x32800000u : 0x3F800000u;   // 2^-26 or 1
+        const uint64_t unit2 = pack2(unit, unit);
         uint32_t par = 0u;                            // parity of the slots' completions in this turn of eight groups
         uint32_t dnext = 0u;
         bool ready = true;                            // the barrier of the group after the one whose load is in flight
@@ -353,7 +359,11 @@ __global__ void __launch_bounds__(kSoloThreads, 1) w4a4_solo_kernel(const LinArg
                 for (int q = 0; q < 32; ++q) v[q] = __float_as_uint((float)(int32_t)v[q]);
             }
 #pragma unroll
-            for (int q = 0; q < 16; ++q) fma2(yacc[q], pack2(v[2 * q], v[2 * q + 1]), d2);
+            for (int q = 0; q < 16; ++q) {
+                uint64_t f = pack2(v[2 * q], v[2 * q + 1]);
+                if (I8) asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(f) : "l"(unit2));
+                fma2(yacc[q], f, d2);
+            }
         };
         const std::integral_constant<int, 0> u0{};
         const std::integral_constant<int, 1> u1{};
@@ -477,7 +487,7 @@ tdq_status launch_linear_solo(LinArgs a, const CUtensorMap& ymap, int dev, bool 
     void (*const kernels[kInst])(LinArgs, CUtensorMap) = {
         w4a4_solo_kernel<false, true>, w4a4_solo_kernel<true, true>, w4a4_solo_kernel<false, false>, w4a4_solo_kernel<true, false>};
     const int inst = (ybf ? 1 : 0) + (a.steps_per_grp > 1 ? 2 : 0);
-    a.out_scale = a.steps_per_grp > 1 ? 0.00390625f : 262144.0f;     // operands 16 q and 16 q, or q 2^-9 and q 2^-9
+    a.out_scale = a.steps_per_grp > 4 ? 0.00390625f : 262144.0f;     // the units of the sums that the promotion adds: 2^8 or 2^-18
     static std::atomic<uint64_t> smem_done[kInst];
     if (allow_smem(kernels[inst], (int)kSoloSmem, smem_done[inst], dev) != cudaSuccess) return TDQ_ERR_CUDA;
     if (launch_pdl(kernels[inst], dim3((unsigned)(a.tiles_m * a.tiles_n)), dim3(kSoloThreads), kSoloSmem, stream, a, ymap) != cudaSuccess) return TDQ_ERR_CUDA;

@@ -62,3 +62,26 @@ def test_extreme_codes(g, K, x, w):
     xs = torch.from_numpy(rng.uniform(0.1, 2.0, (M, K)).astype(np.float32)).cuda()
     ws = torch.from_numpy(rng.uniform(0.1, 2.0, O).astype(np.float32)).cuda()
     _check(xc, xs, wc, ws, g, O)
+
+
+@pytest.mark.parametrize("g,K", [(32, 9), (64, 5), (96, 3), (128, 4), (160, 3), (256, 4), (768, 1)])
+@pytest.mark.parametrize("step,channel", [(1e-8, 1e-30), (2e34, 1e-30), (1e-37, 1e37), (1e-30, 1.0), (0.0, 1.0), (float("inf"), 1.0), (1.0, float("inf")), (float("nan"), 1.0)])
+def test_ends_of_the_range(g, K, step, channel):
+    """Steps and channel scales at which a product or a sum nears the ends of binary32: the same bits, infinities and NaNs as the
+    kernel that writes the group sums, which takes every layer."""
+    from paper_2604_16855_b200 import tdq
+    M, O = 131, 72
+    rng = np.random.default_rng(g + K)
+    xc = torch.from_numpy(rng.integers(0, 256, (M, K * g // 2), dtype=np.uint8)).cuda()
+    wc = torch.from_numpy(rng.integers(0, 256, (O, K * g // 2), dtype=np.uint8)).cuda()
+    xs = torch.from_numpy(rng.uniform(0.1, 2.0, (M, K)).astype(np.float32)).cuda() * step
+    ws = torch.from_numpy(rng.uniform(0.1, 2.0, O).astype(np.float32)).cuda() * channel
+    bias = torch.from_numpy(rng.standard_normal(O).astype(np.float32)).cuda()
+    wsp = tdq.linear_workspace(M, K * g, O, g, "cuda")
+    acc = torch.zeros((M, O, K), dtype=torch.int32, device="cuda")
+    want = tdq.w4a4_linear(xc, xs, wc, ws, bias, g=g, workspace=wsp, acc_debug=acc)
+    n0 = tdq.kernel_launch_count()
+    got = tdq.w4a4_linear(xc, xs, wc, ws, bias, g=g, workspace=wsp)
+    assert tdq.kernel_launch_count() - n0 == 1                # this kernel, not the expansion and another one
+    assert torch.equal(torch.isnan(got), torch.isnan(want))
+    assert torch.equal(torch.nan_to_num(got, nan=0.0, posinf=3e38, neginf=-3e38), torch.nan_to_num(want, nan=0.0, posinf=3e38, neginf=-3e38))
