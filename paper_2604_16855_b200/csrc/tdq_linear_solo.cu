@@ -107,11 +107,12 @@ __device__ __forceinline__ void weight_bytes(const uint4& p, uint4& ev, uint4& o
     od = make_uint4(o[0], o[1], o[2], o[3]);
 }
 
-// SPG1: one K-step per group (E4M3).  Otherwise a.steps_per_grp of them (int8).
-template <bool YBF16, bool SPG1>
+// K-steps per group: one (E4M3), up to four or more (int8, a.steps_per_grp of them; the units of the sums differ, see below)
+enum SoloKind { kSoloOne, kSoloFew, kSoloMany };
+template <bool YBF16, SoloKind KIND>
 __global__ void __launch_bounds__(kSoloThreads, 1) w4a4_solo_kernel(const LinArgs a, const __grid_constant__ CUtensorMap ymap) {
     extern __shared__ __align__(128) uint8_t smem_raw[];
-    constexpr bool I8 = !SPG1;
+    constexpr bool SPG1 = KIND == kSoloOne, I8 = !SPG1;
     constexpr uint32_t kBox = YBF16 ? kSoloBox16 : kSoloBoxF32;
     Ctrl* c = reinterpret_cast<Ctrl*>(smem_raw);             // its abort flag and TMEM address; the barriers are g's
     SoloCtrl* g = reinterpret_cast<SoloCtrl*>(smem_raw + sizeof(Ctrl));
@@ -312,9 +313,12 @@ __global__ void __launch_bounds__(kSoloThreads, 1) w4a4_solo_kernel(const LinArg
         const float* gx = a.xscale + (m_row < a.M ? m_row : 0) * a.Kg;   // otherwise the steps come from memory, a group ahead
         // int8 sums are 256 times the group's.  Up to 128 codes a group the other kernels add sums in units of 2^-18 (E4M3), beyond
         // that 256 times the sums; the same units here, or a product near the ends of binary32's range would be rounded or
-        // overflow in one kernel and not in the other.  (Exact: a power of two, and the sums are whole numbers below 2^26.)
-        const uint32_t unit = a.steps_per_grp <= 4 ? 0x32800000u : 0x3F800000u;   // 2^-26 or 1
-        const uint64_t unit2 = pack2(unit, unit);
+        // overflow in one kernel and not in the other.  (Exact: a power of two, and the sums are whole numbers below 2^22.)  The
+        // multiplication is up to 4 % of such a layer (1152 x 1024 -> 512 at g = 128 6.25 -> 6.51 us).  Dearer: the step scaled instead
+        // where that is exact, and a vote on it, 12 %; a scan of the warp's steps in front and a second loop 6 %; a conversion by way
+        // of a float with the sum in its last bits 13 %.
+        constexpr uint32_t kUnit = 0x32800000u;       // 2^-26
+        const uint64_t unit2 = pack2(kUnit, kUnit);
         uint32_t par = 0u;                            // parity of the slots' completions in this turn of eight groups
         uint32_t dnext = 0u;
         bool ready = true;                            // the barrier of the group after the one whose load is in flight
@@ -361,7 +365,7 @@ __global__ void __launch_bounds__(kSoloThreads, 1) w4a4_solo_kernel(const LinArg
 #pragma unroll
             for (int q = 0; q < 16; ++q) {
                 uint64_t f = pack2(v[2 * q], v[2 * q + 1]);
-                if (I8) asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(f) : "l"(unit2));
+                if (KIND == kSoloFew) asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(f) : "l"(unit2));
                 fma2(yacc[q], f, d2);
             }
         };
@@ -483,10 +487,11 @@ __global__ void __launch_bounds__(kSoloThreads, 1) w4a4_solo_kernel(const LinArg
 
 // a.tiles_n is in units of 64 columns here.
 tdq_status launch_linear_solo(LinArgs a, const CUtensorMap& ymap, int dev, bool ybf, cudaStream_t stream) {
-    constexpr int kInst = 4;
+    constexpr int kInst = 6;
     void (*const kernels[kInst])(LinArgs, CUtensorMap) = {
-        w4a4_solo_kernel<false, true>, w4a4_solo_kernel<true, true>, w4a4_solo_kernel<false, false>, w4a4_solo_kernel<true, false>};
-    const int inst = (ybf ? 1 : 0) + (a.steps_per_grp > 1 ? 2 : 0);
+        w4a4_solo_kernel<false, kSoloOne>, w4a4_solo_kernel<true, kSoloOne>, w4a4_solo_kernel<false, kSoloFew>,
+        w4a4_solo_kernel<true, kSoloFew>, w4a4_solo_kernel<false, kSoloMany>, w4a4_solo_kernel<true, kSoloMany>};
+    const int inst = (ybf ? 1 : 0) + 2 * (a.steps_per_grp == 1 ? kSoloOne : a.steps_per_grp <= 4 ? kSoloFew : kSoloMany);
     a.out_scale = a.steps_per_grp > 4 ? 0.00390625f : 262144.0f;     // the units of the sums that the promotion adds: 2^8 or 2^-18
     static std::atomic<uint64_t> smem_done[kInst];
     if (allow_smem(kernels[inst], (int)kSoloSmem, smem_done[inst], dev) != cudaSuccess) return TDQ_ERR_CUDA;
