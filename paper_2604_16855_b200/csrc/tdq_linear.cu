@@ -1269,10 +1269,24 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
                       : p.n_steps <= 9  ? tiles128 <= 5 * n_sm
                       : p.n_steps <= 16 ? tiles128 <= 4 * n_sm
                                         : p.n_steps <= 24 && O <= 128 && tiles128 <= 4 * n_sm);
-    if (use_strip && p.n_steps >= 10 && O > 128 && tiles128 > n_sm) {
+    // In a stream the expansion in front costs two microseconds of launch, in a graph one, so there are layers where this kernel
+    // wins in the one and loses in the other, and a call that is being captured takes the faster one for a replay.  In a graph it loses
+    // from 320 channels on with several column tiles and more than a tile per SM; from 224 on where a last round of tiles is less than
+    // 0.4 full of the others; from 128 on where half of the last column tile is empty, with more than three tiles per SM.  Layer alone
+    // from a graph, us, expansion and the kernel behind it, and this one: 4608 x 512 -> 768 bf16 12.4 and 14.1, 9216 x 320 -> 640 13.6 and
+    // 14.1; 2304 x 288 -> 1280 fp32 (180 tiles) 11.1 and 11.6 (with the quantizer 13.2 and 14.6), 2304 x 256 -> 1280 bf16 9.1 and 9.4;
+    // 36864 x 256 -> 192 bf16 14.2 and 15.3, 73728 x 192 -> 192 21.9 and 23.1, 73728 x 128 -> 192 17.2 and 17.9.  In a stream, with
+    // the quantizer, the same: 18.5 and 17.7, 19.4 and 18.1, 15.3 and 15.2, 14.4 and 12.9, 24.7 and 23.5, 35.0 and 34.6, 27.9 and 26.8.
+    // Over 454 sizes the rule is within 0.2 % of the better kernel of each in a graph; never this kernel 5.8 %, always 0.9 %.
+    const int64_t rounds = (tiles128 + n_sm - 1) / n_sm;
+    const bool graph_loses = O > 128 && tiles128 > n_sm &&
+                             (p.n_steps >= 10 || (p.n_steps >= 7 && rounds * n_sm * 5 >= tiles128 * 7) ||
+                              (p.n_steps >= 4 && !full_tiles && tiles128 > 3 * n_sm));
+    if (use_strip && graph_loses) {
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-        use_strip = cudaStreamIsCapturing(stream, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone;
-        if (!use_strip) (void)cudaGetLastError();
+        const bool known = cudaStreamIsCapturing(stream, &capture) == cudaSuccess;
+        if (!known) (void)cudaGetLastError();     // the query's own error (a legacy stream while another one is being captured)
+        use_strip = known && capture == cudaStreamCaptureStatusNone;
     }
     const bool use_pair = pair_ok && !use_defer;
     const bool unpack_a = !fx && !pow2_steps && !use_pair && !use_one && !use_defer && p.a_resident && steps_per_item >= 256;

@@ -2,6 +2,10 @@
 SM), at the edges of its dispatch: every number of groups modulo four, one to six chunks, row blocks that end inside a block's
 run and reuse another's place, ragged rows and columns, an empty second half, each output type, nothing written past the
 last column, codes at the ends of their range, and the same bits under capture."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -10,6 +14,7 @@ import oracle
 import synth_inputs as si
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def _check(xc, xs, wc, ws, O):
@@ -90,3 +95,45 @@ def test_under_capture():
     graph.replay()
     assert tdq.workspace_status(wsp) == (tdq.OK, 0)
     assert torch.equal(y, want)
+
+
+FIRST_USE = """
+import sys
+import torch
+from paper_2604_16855_b200 import tdq
+warm, M, C, O = [int(v) for v in sys.argv[1:]]
+gen = torch.Generator("cuda").manual_seed(M)
+xc, xs = tdq.quantize_act(torch.randn((M, C), device="cuda", generator=gen))
+wc, ws = tdq.quantize_weight(torch.randn((O, C), device="cuda", generator=gen))
+wsp = tdq.linear_workspace(M, C, O, 32, "cuda")
+y = torch.empty((M, O), device="cuda")
+counts = []
+if warm:
+    n = tdq.kernel_launch_count()
+    tdq.w4a4_linear(xc, xs, wc, ws, y=y, workspace=wsp)
+    counts.append(tdq.kernel_launch_count() - n)
+    y.zero_()
+torch.cuda.synchronize()
+graph = torch.cuda.CUDAGraph()
+with torch.cuda.graph(graph):
+    n = tdq.kernel_launch_count()
+    tdq.w4a4_linear(xc, xs, wc, ws, y=y, workspace=wsp)
+    counts.append(tdq.kernel_launch_count() - n)
+graph.replay()
+assert tdq.workspace_status(wsp) == (tdq.OK, 0)
+z = tdq.w4a4_linear(xc, xs, wc, ws, workspace=wsp)
+assert torch.equal(y, z), "the replay's bits differ"
+print("launches", counts)
+"""
+
+
+# launches of the eager and of the captured call: one where this kernel wins in a graph too; expansion and another kernel where it
+# does not (many groups; a last round of tiles that is mostly empty; half of the last column tile empty)
+@pytest.mark.parametrize("M,C,O,captured", [(9216, 320, 320, 2), (2304, 288, 1280, 2), (64000, 128, 192, 2), (18432, 192, 768, 1), (1152, 512, 2048, 1)])
+@pytest.mark.parametrize("warm", [0, 1])
+def test_first_use_in_a_capture(M, C, O, captured, warm):
+    """A process whose first launch of the layer's kernels is inside a capture, and one that has only called the layer eagerly
+    before: the captured call takes the kernel that is the faster one in a graph, and its replay gives the eager call's bits."""
+    r = subprocess.run([sys.executable, "-c", FIRST_USE, str(warm), str(M), str(C), str(O)], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    assert "launches %s" % ([1, captured] if warm else [captured]) in r.stdout
