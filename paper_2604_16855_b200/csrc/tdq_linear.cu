@@ -1271,8 +1271,9 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
                                         : p.n_steps <= 24 && O <= 128 && tiles128 <= 4 * n_sm);
     // In a stream the expansion in front costs two microseconds of launch, in a graph one, so there are layers where this kernel
     // wins in the one and loses in the other, and a call that is being captured takes the faster one for a replay.  In a graph it loses
-    // from 320 channels on with several column tiles and more than a tile per SM; from 224 on where a last round of tiles is less than
-    // 0.4 full of the others; from 128 on where half of the last column tile is empty, with more than three tiles per SM.  Layer alone
+    // from 320 channels on with several column tiles and more than a tile per SM; from 256 on where the rounds of tiles are less than
+    // 5/7 full; where half of the last column tile is empty, from 192 channels on with more than three tiles per SM and from 128 on
+    // with more than six (36864 x 160 -> 192 fp32, four tiles, with the quantizer 20.4 and 20.5).  Layer alone
     // from a graph, us, expansion and the kernel behind it, and this one: 4608 x 512 -> 768 bf16 12.4 and 14.1, 9216 x 320 -> 640 13.6 and
     // 14.1; 2304 x 288 -> 1280 fp32 (180 tiles) 11.1 and 11.6 (with the quantizer 13.2 and 14.6), 2304 x 256 -> 1280 bf16 9.1 and 9.4;
     // 36864 x 256 -> 192 bf16 14.2 and 15.3, 73728 x 192 -> 192 21.9 and 23.1, 73728 x 128 -> 192 17.2 and 17.9.  In a stream, with
@@ -1280,8 +1281,8 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     // Over 454 sizes the rule is within 0.2 % of the better kernel of each in a graph; never this kernel 5.8 %, always 0.9 %.
     const int64_t rounds = (tiles128 + n_sm - 1) / n_sm;
     const bool graph_loses = O > 128 && tiles128 > n_sm &&
-                             (p.n_steps >= 10 || (p.n_steps >= 7 && rounds * n_sm * 5 >= tiles128 * 7) ||
-                              (p.n_steps >= 4 && !full_tiles && tiles128 > 3 * n_sm));
+                             (p.n_steps >= 10 || (p.n_steps >= 8 && rounds * n_sm * 5 >= tiles128 * 7) ||
+                              (p.n_steps >= 4 && !full_tiles && tiles128 > (p.n_steps >= 6 ? 3 : 6) * n_sm));
     if (use_strip && graph_loses) {
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
         const bool known = cudaStreamIsCapturing(stream, &capture) == cudaSuccess;
