@@ -346,24 +346,34 @@ cudaError_t launch_ragged(const ActArgs& a, cudaStream_t st) {
 // slower at 64 positions, 128 positions up to 11 %, 32 up to 5 %.
 constexpr int kNchwThreads = 64;
 
+// ACROSS: the positions of all images in one row, a division a thread, instead of blocks of their own for each image, whose last one
+// is a quarter full at 144 positions and a sixth at 72.  The time goes in steps of about five blocks per SM (2.5 warps per scheduler), so
+// this is taken where it saves one; us, blocks per image and across, the 256-position blocks before them in brackets: bf16 [16, 512,
+// 12, 12] (5.2 and 3.9 blocks per SM) 3.42 and 2.63 (2.86), [32, 256, 12, 12] 3.37 and 2.54 (2.83), fp32 [16, 768, 10, 10] (5.2 and 4.05)
+// 3.91 and 3.01 (3.47), [64, 512, 12, 12] (20.8 and 15.6) 8.58 and 7.84 (9.79); without a step saved [16, 768, 12, 12] (7.8 and 5.8) 4.43 and 4.69
+// (4.55), bf16 [16, 64, 18, 18] 1.91 and 2.03.
 struct NchwArgs {
-    ActArgs a;          // x, K, k_zr, seven_tau, flags, codes, scale, offset
+    ActArgs a;          // x, M (positions of all images), K, k_zr, seven_tau, flags, codes, scale, offset
     int64_t HW;         // positions per image
 };
 
-template <bool BF16, int KZR>
+template <bool BF16, int KZR, bool ACROSS>
 __global__ void __launch_bounds__(kNchwThreads) act_g32_nchw_kernel(NchwArgs n) {
     constexpr int esz = BF16 ? 2 : 4;
     const ActArgs& a = n.a;
     const int t = threadIdx.x;
     const int64_t s0 = (int64_t)blockIdx.x * kNchwThreads;    // first position of the block
     const int k = blockIdx.y;                                  // channel group
-    const int64_t b = blockIdx.z;
+    int64_t b = blockIdx.z, s = s0 + t;                        // image and position in it
     pdl_wait();
     pdl_trigger();
-    if (t >= n.HW - s0) return;
+    if (t >= (ACROSS ? a.M : n.HW) - s0) return;
+    if (ACROSS) {
+        b = (uint32_t)s / (uint32_t)n.HW;
+        s -= b * n.HW;
+    }
     const int64_t row = n.HW * esz;
-    const uint8_t* src = reinterpret_cast<const uint8_t*>(a.x) + (b * a.C + (int64_t)k * 32) * row + (s0 + t) * esz;
+    const uint8_t* src = reinterpret_cast<const uint8_t*>(a.x) + (b * a.C + (int64_t)k * 32) * row + s * esz;
     uint32_t w[BF16 ? 16 : 32];
     if (BF16) {
 #pragma unroll
@@ -376,14 +386,15 @@ __global__ void __launch_bounds__(kNchwThreads) act_g32_nchw_kernel(NchwArgs n) 
 #pragma unroll
         for (int i = 0; i < 32; ++i) w[i] = __ldg(reinterpret_cast<const uint32_t*>(src + i * row));
     }
-    process_group<BF16, KZR>(w, a, ((b * n.HW + s0 + t) * a.K) + k);
+    process_group<BF16, KZR>(w, a, ((b * n.HW + s) * a.K) + k);
 }
 
-template <bool BF16>
+template <bool BF16, bool ACROSS>
 cudaError_t launch_nchw(const NchwArgs& n, int64_t B, cudaStream_t st) {
-    dim3 grid((unsigned)((n.HW + kNchwThreads - 1) / kNchwThreads), (unsigned)n.a.K, (unsigned)B);
+    const int64_t blocks = ((ACROSS ? n.a.M : n.HW) + kNchwThreads - 1) / kNchwThreads;
+    const dim3 grid((unsigned)blocks, (unsigned)n.a.K, ACROSS ? 1u : (unsigned)B);
     switch (n.a.k_zr) {
-#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_nchw_kernel<BF16, KZ>, grid, dim3(kNchwThreads), 0, st, n);
+#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_nchw_kernel<BF16, KZ, ACROSS>, grid, dim3(kNchwThreads), 0, st, n);
         TDQ_CASE(4) TDQ_CASE(7) TDQ_CASE(10) TDQ_CASE(13) TDQ_CASE(16) TDQ_CASE(32)
 #undef TDQ_CASE
         default: return cudaErrorInvalidValue;
@@ -585,8 +596,17 @@ extern "C" tdq_status tdq_quantize_act_nchw(const void* x, tdq_dtype x_dtype, in
     n.a.scale = scale;
     n.a.offset = offset;
     n.HW = HW;
+    const int64_t apart = B * ((HW + kNchwThreads - 1) / kNchwThreads) * n.a.K, together = (n.a.M + kNchwThreads - 1) / kNchwThreads * n.a.K;
+    bool across = false;
+    if (together < apart && n.a.M <= INT32_MAX) {
+        const int n_sm = current_device_sm_count();
+        const int64_t step = 5 * (int64_t)(n_sm > 0 ? n_sm : 148);
+        across = (together + step - 1) / step < (apart + step - 1) / step;
+    }
     cudaStream_t stream = reinterpret_cast<cudaStream_t>(cuda_stream);
-    const cudaError_t e = (x_dtype == TDQ_BF16) ? launch_nchw<true>(n, B, stream) : launch_nchw<false>(n, B, stream);
+    const bool bf16 = x_dtype == TDQ_BF16;
+    const cudaError_t e = across ? (bf16 ? launch_nchw<true, true>(n, B, stream) : launch_nchw<false, true>(n, B, stream))
+                                 : (bf16 ? launch_nchw<true, false>(n, B, stream) : launch_nchw<false, false>(n, B, stream));
     if (e != cudaSuccess) return TDQ_ERR_CUDA;
     g_launch_count.fetch_add(1, std::memory_order_relaxed);
     return TDQ_OK;

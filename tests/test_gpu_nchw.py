@@ -19,3 +19,17 @@ def test_shapes(B, C, H, W, first, dtype):
         codes, scale = tdq.quantize_act_nchw(x, p)
         want_codes, want_scale = tdq.quantize_act(x.permute(0, 2, 3, 1).reshape(-1, C).contiguous(), p)
         assert torch.equal(codes.view(want_codes.shape), want_codes) and torch.equal(scale.view(want_scale.shape), want_scale)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("B,C,H,W", [(16, 512, 12, 12), (70, 768, 9, 9), (700, 160, 1, 3), (1500, 32, 13, 5), (900, 32, 1, 1)])
+def test_blocks_across_images(B, C, H, W, dtype):
+    """Maps whose blocks of positions run on from one image to the next."""
+    from paper_2604_16855_b200 import tdq
+    x = torch.randn((B, C, H, W), device="cuda", generator=torch.Generator("cuda").manual_seed(B)).to(dtype)
+    codes = torch.full((B * H * W + 1, C // 2), 77, dtype=torch.uint8, device="cuda")
+    scale = torch.full((B * H * W + 1, C // 32), -1.0, device="cuda")
+    tdq.quantize_act_nchw(x, codes=codes[:-1], scale=scale[:-1])
+    want_codes, want_scale = tdq.quantize_act(x.permute(0, 2, 3, 1).reshape(-1, C).contiguous())
+    assert torch.equal(codes[:-1], want_codes.view(-1, C // 2)) and torch.equal(scale[:-1], want_scale.view(-1, C // 32))
+    assert bool((codes[-1] == 77).all()) and bool((scale[-1] == -1.0).all())
