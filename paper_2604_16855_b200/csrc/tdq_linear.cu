@@ -1313,11 +1313,12 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     CUtensorMap ymap;
     memset(&ymap, 0, sizeof(ymap));
     a.tma_ok = 0;
+    const bool whole_rows = use_solo || use_pair || use_defer;   // these stage boxes of 32 columns x 128 rows
     if (y_tma && encode_y_map(&ymap, y, y_dtype == TDQ_BF16, M, O, y_row_stride,
-                              (use_one || use_pair || use_defer) ? kCols : quarter_strips ? (y_dtype == TDQ_BF16 ? kCols / 2 : kCols / 4) : half_strips ? kCols / 2 : kCols,
-                              (use_g32 || use_pair || use_defer) ? kBM : 32, y_f16))
+                              (use_one || whole_rows) ? kCols : quarter_strips ? (y_dtype == TDQ_BF16 ? kCols / 2 : kCols / 4) : half_strips ? kCols / 2 : kCols,
+                              (use_g32 || whole_rows) ? kBM : 32, y_f16))
         a.tma_ok = 1;
-    else if (narrow_strips || quarter_strips)
+    else if (!use_solo && (narrow_strips || quarter_strips))
         return TDQ_ERR_CUDA;   // the plan counted on the tensor store
     a.y_words = reinterpret_cast<uintptr_t>(y) % 4 == 0 && y_row_stride % 2 == 0 ? 1 : 0;
     a.staging_bytes = (uint32_t)staging_bytes;
@@ -1350,8 +1351,6 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     if (use_strip && a.tma_ok) return launch_linear_strip(a, ymap, n_sm, dev, ybf, stream);
     if (use_solo) {
         a.tiles_n = (int32_t)((O + 63) / 64);
-        a.tma_ok = 0;
-        if (y_tma && encode_y_map(&ymap, y, y_dtype == TDQ_BF16, M, O, y_row_stride, kCols, kBM, y_f16)) a.tma_ok = 1;
         return launch_linear_solo(a, ymap, dev, ybf, stream);
     }
     if (use_pair) {
