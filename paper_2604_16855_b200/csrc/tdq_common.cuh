@@ -46,7 +46,7 @@ tdq_status check_act_args(const void* x, tdq_dtype dt, int64_t B, int64_t N, int
                           const tdq_act_params* p);
 bool act_fast_path_ok(const void* x, tdq_dtype dt, int64_t C, int64_t stride, const tdq_act_params* p);
 
-// One warp waits, with the quantizer's wait routine and the given cycle limit, on a barrier nobody arrives on
+// One warp waits, with the bounded-wait routine of the kernels and the given cycle limit, on a barrier nobody arrives on
 // (tdq_selftest_wait_timeout; tdq_quantize_act.cu).
 tdq_status act_wait_selftest(long long limit_cycles, cudaStream_t stream);
 

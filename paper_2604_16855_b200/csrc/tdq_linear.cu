@@ -660,7 +660,6 @@ __global__ void __launch_bounds__(kThreads, 1) w4a4_gemm_kernel(const LinArgs a,
         uint32_t v[kLand];
 #pragma unroll
         for (int q = 0; q < kLand; ++q) v[q] = 0u;
-        uint32_t ic = 0;                 // items so far
         uint32_t p_full[kSlots] = {0u, 0u, 0u, 0u};   // parity of the completion of tfull[s] to wait for next
         int item = blockIdx.x, mt = 0, nt = 0, nt_end = 0;
         int64_t n0 = 0;
@@ -1308,7 +1307,6 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     a.staging_off = p.staging_off;
     a.y = y; a.y_stride = y_row_stride; a.acc_debug = acc_debug;
     a.status = reinterpret_cast<uint32_t*>(workspace);
-    const int64_t esz = y_dtype == TDQ_BF16 ? 2 : 4;
     // bulk tensor stores want a 16-byte aligned base and row pitch; anything else goes element by element
     CUtensorMap ymap;
     memset(&ymap, 0, sizeof(ymap));

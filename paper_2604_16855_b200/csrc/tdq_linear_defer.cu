@@ -96,7 +96,6 @@ __global__ void __launch_bounds__(kDeferThreads, 1) w4a4_defer_kernel(const LinA
     const uint32_t tmem_base = c->tmem_base;
     const uint32_t buf_mask = (uint32_t)a.n_ibuf - 1u, buf_shift = buf_mask;   // tile n's steps are in buffer n & mask, phase n >> shift
     const int n_tiles = a.tiles_m * a.tiles_n, n_steps = a.n_steps;
-    const int chunks = (n_steps + kChunk - 1) / kChunk;
 
     if (warp < kDeferCtlWarps) {
         setmaxnreg_dec<kRegsDeferCtl>();

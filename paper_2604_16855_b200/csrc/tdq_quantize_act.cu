@@ -30,6 +30,7 @@
 
 #include "tdq_act_group.cuh"
 #include "tdq_common.cuh"
+#include "tdq_tc.cuh"
 
 namespace tdq {
 
@@ -253,7 +254,7 @@ __global__ void __launch_bounds__(kRaggedThreads) act_g32_ragged_kernel(ActArgs 
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const int64_t g0 = (int64_t)blockIdx.x * kRaggedThreads;
     uint8_t* tb = reinterpret_cast<uint8_t*>(tile);
-    // channel `e` of local group `l` lands where act_g32_kernel's 16-byte pieces put it
+    // channel `e` of local group `l`: the group's 16-byte pieces are swizzled so that a warp reads its groups without bank conflicts
     auto slot = [&](int l, int e) -> uint8_t* {
         const int byte = e * (BF16 ? 2 : 4), swz = BF16 ? ((l >> 1) & kSwzMask) : (l & kSwzMask);
         return tb + (l * kChunks + ((byte >> 4) ^ swz)) * 16 + (byte & 15);
@@ -644,60 +645,24 @@ extern "C" tdq_status tdq_quantize_act_fixed(const void* x, tdq_dtype x_dtype, i
 }
 
 // ------------------------------------------------------------------------------------------
-// bounded waits of the quantizer: the status word, the routine and the self-test
+// tdq_quantize_status and its self-test.  No quantizer kernel waits on a barrier at present, so only the self-test writes the word.
 
 namespace tdq {
 namespace {
-// A wait of a quantizer kernel that ran out leaves its code here (first writer wins): bits 0-7 name the wait (14 the
-// self-test; no quantizer kernel waits on a barrier at present), bits 8-31 the CTA.  One word per device, read and cleared by
+// Bits 0-7 name the wait that ran out (14 the self-test), bits 8-31 the CTA.  One word per device, read and cleared by
 // tdq_quantize_status().
 __device__ uint32_t g_act_wait_status = 0u;
 
-__device__ __forceinline__ uint32_t act_smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ bool act_wait_test(uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(act_smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// false when the phase did not complete in about a second (the caller then stops working)
-__device__ __forceinline__ bool act_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, uint32_t code,
-                                          long long limit) {
-    if (act_wait_test(bar, parity)) return true;
-    long long t0 = 0;
-    uint32_t polls = 0;
-#pragma unroll 1
-    while (!act_wait_test(bar, parity)) {
-        if ((++polls & 63u) == 0u) {
-            if (*abort_flag) return false;
-            const long long now = clock64();
-            if (t0 == 0) t0 = now;
-            if (now - t0 > limit) {
-                atomicCAS(&g_act_wait_status, 0u, code | ((uint32_t)blockIdx.x << 8));
-                *abort_flag = 1;
-                return false;
-            }
-        }
-    }
-    return true;
-}
-
-// One warp: a fresh barrier with one expected arrival that never comes, waited on with that
+// One warp: a fresh barrier with one expected arrival that never comes, waited on with the linear layer's
 // routine and a short limit.  Nothing is in flight when the warp leaves.
 __global__ void __launch_bounds__(32) act_wait_selftest_kernel(long long limit) {
-    __shared__ uint64_t bar;
-    __shared__ volatile int abort_flag;
+    __shared__ Ctrl c;
     if (threadIdx.x == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(act_smem_u32(&bar)) : "memory");
-        abort_flag = 0;
+        mbar_init(&c.full[0], 1);
+        c.abort_flag = 0;
     }
     __syncwarp();
-    act_wait(&bar, 0u, &abort_flag, 14u, limit);
+    mbar_wait_warp(&c.full[0], 0u, &c, &g_act_wait_status, 14u, limit);
 }
 }  // namespace
 

@@ -124,37 +124,39 @@ struct Share {
     // largest magnitude of this share that is at most that (bf16: packed, two masks and maxima at a time)
     __device__ __forceinline__ uint32_t max_le(const uint32_t (&mag)[NC * kWords], uint32_t key) const {
         uint32_t r = 0;
-        if (BF16) {
+        if constexpr (BF16) {
             const uint32_t m = __byte_perm(key, 0u, 0x3232u);
             const __nv_bfloat162 m2 = *reinterpret_cast<const __nv_bfloat162*>(&m);
 #pragma unroll
             for (int i = 0; i < NC * kWords; ++i) r = __vmaxu2(r, mag[i] & __hle2_mask(*reinterpret_cast<const __nv_bfloat162*>(&mag[i]), m2));
             return max(r & 0xffffu, r >> 16) << 16;
-        }
+        } else {
 #pragma unroll
-        for (int i = 0; i < NC * 8; ++i) {
-            const uint32_t u = w[i] & 0x7fffffffu;
-            r = max(r, u <= key ? u : 0u);
+            for (int i = 0; i < NC * 8; ++i) {
+                const uint32_t u = w[i] & 0x7fffffffu;
+                r = max(r, u <= key ? u : 0u);
+            }
+            return r;
         }
-        return r;
     }
     // smallest magnitude of this share above it (any, if it is negative)
     __device__ __forceinline__ uint32_t min_gt(const uint32_t (&mag)[NC * kWords], int key) const {
-        if (BF16) {
+        if constexpr (BF16) {
             uint32_t r = 0x7fff7fffu;
             const uint32_t m = key < 0 ? 0x80008000u + 0x3f803f80u : __byte_perm((uint32_t)key, 0u, 0x3232u);   // -1 for "none"
             const __nv_bfloat162 m2 = *reinterpret_cast<const __nv_bfloat162*>(&m);
 #pragma unroll
             for (int i = 0; i < NC * kWords; ++i) r = __vminu2(r, mag[i] | __hle2_mask(*reinterpret_cast<const __nv_bfloat162*>(&mag[i]), m2));
             return min(r & 0xffffu, r >> 16) << 16;
-        }
-        uint32_t r = 0x7fffffffu;
+        } else {
+            uint32_t r = 0x7fffffffu;
 #pragma unroll
-        for (int i = 0; i < NC * 8; ++i) {
-            const uint32_t u = w[i] & 0x7fffffffu;
-            r = min(r, (int)u > key ? u : 0x7fffffffu);
+            for (int i = 0; i < NC * 8; ++i) {
+                const uint32_t u = w[i] & 0x7fffffffu;
+                r = min(r, (int)u > key ? u : 0x7fffffffu);
+            }
+            return r;
         }
-        return r;
     }
 };
 
@@ -219,7 +221,9 @@ __device__ __forceinline__ uint32_t group_kth(const Share<BF16, NC>& x, int k, i
     return r;
 }
 
-// Resident blocks the registers are allocated for: the share (4 or 8 words a chunk) and about fifty more.
+// Resident blocks the registers are allocated for: the share (4 or 8 words a chunk) and about fifty more.  The bf16 instances with
+// four and six chunks a lane on eight lanes and more spill a word or two there.  A block less, which holds them, is faster on a few
+// hundred groups (1024 x 4096 at 1024 and 4096 8 %) and slower on many: 16384 x 1536 at 256 2.3 %, at 512 2.9 %, at 1536 4.5 %.
 constexpr int wide_blocks(bool bf16, int nc) {
     const int regs = bf16 ? 4 * nc + 48 : 8 * nc + 64;
     return 512 / (regs < 64 ? 64 : regs);
@@ -457,7 +461,7 @@ cudaError_t pick(const WideArgs& w, cudaStream_t st) {
         // barriers, the probes' bookkeeping) weighs as much as they do.  us, four chunks a lane and eight: 16384 x 4096 73.0 and
         // 64.6, 16384 x 3072 64.2 and 48.8, 4096 x 2048 11.7 and 10.7, 2048 x 4096 12.0 and 11.1; 2048 x 2048 7.7 and 8.4, 1024 x
         // 4096 7.8 and 8.8 (too few warps); groups of up to 1024 gain nothing (18464 x 768 at 128 19.5 and 20.9, at 768 17.8 and 17.5).
-        if (chunks > 128 && w.a.total_groups * w.a.g >= ((int64_t)1 << 23)) {
+        if (w.a.total_groups * w.a.g >= ((int64_t)1 << 23)) {
             if (chunks <= 192) return launch<BF16, 6, 32>(w, st);
             if (chunks <= 256) return launch<BF16, 8, 32>(w, st);
             if (chunks <= 384) return launch<BF16, 6, 32, 2>(w, st);
