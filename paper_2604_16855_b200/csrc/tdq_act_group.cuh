@@ -29,10 +29,10 @@ namespace {
 
 // True when the binary32 moments prove that 7 tau sigma exceeds cmin by a safe margin, i.e.
 // the C1 bound cannot be the minimum.  s1 = sum x, s2 = sum x^2 over the g elements, inv_g = 1/g.
-// A term passes through at most 40 additions whatever the group (32 in one thread at g = 32; in the wide kernel up to 32
-// in a lane, 5 levels of a warp, 3 warps), so with u = 2^-24 and E = E[x^2] the mean is off by at most 40 u sqrt(E), its
-// square by 80 u E, s2 / g by 41 u E, and with the few roundings of the estimate itself var is off by less than
-// 130 u E = 7.8e-6 E.  Asking for var >= E / 16 makes that a relative error below 1.3e-4, and the test keeps a 1 %
+// A term passes through at most 70 additions whatever the group (32 in one thread at g = 32; in the wide kernel up to 64
+// in a lane, 5 levels of a warp, one more warp, or 32, 5 and 3), so with u = 2^-24 and E = E[x^2] the mean is off by at most 70 u
+// sqrt(E), its square by 140 u E, s2 / g by 72 u E, and with the few roundings of the estimate itself var is off by less than
+// 220 u E = 1.4e-5 E.  Asking for var >= E / 16 makes that a relative error below 2.2e-4, and the test keeps a 1 %
 // margin on the squared radius, so a true result is always right; a
 // false one only means the deviation is recomputed exactly.  When the other bounds already put the radius at or below
 // its floor, the floor decides whatever sigma is (the usual case of groups that are mostly zeros or padding).
@@ -72,10 +72,13 @@ __device__ __forceinline__ uint32_t nibble_fast(float x, float c, float delta, f
     return __float_as_uint(__fadd_rn(q1, kRoundMagic)) & 0xFu;
 }
 
-// The same test on moments accumulated in bf16 pairs (2^-9 unit roundoff, 16 sequential adds per
-// half): s2 is within 4 % and the mean within 0.032 rms, so the variance estimate is off by at
-// most 0.105 E[x^2].  Requiring var >= E[x^2] / 2 turns that into var_true >= 0.78 var, and the
-// factor 0.7 then leaves 7 tau sigma_true >= 1.05 cmin.  Anything else goes to the exact path.
+// The same test on moments accumulated in bf16 pairs, at most 16 terms to a sum (u = 2^-8; binary32 adds those sums).  The i-th
+// term of such a sum passes through k_i = 16, 16, 15, ... 2 roundings for s2 and 15, 15, 14, ... 1 for s1, so with s_i the mean square
+// of the i-th terms (their sum is 16 E) E[x^2] is off by at most sum ((1 + u)^k_i - 1) s_i / 16 and, as the mean of |x| is at most the
+// root of the mean square, the mean by sum ((1 + u)^k_i - 1) sqrt(s_i) / 16.  Requiring var >= E[x^2] / 2 bounds the mean by 0.77 sqrt(E),
+// and over all s_i the error of the variance is then largest at 0.114 E (0.057 E from E[x^2]; the mean is off by 0.037 sqrt(E)).  E[x^2]
+// itself is never more than 6.5 % too small, so var >= 0.467 E and var_true >= 0.75 var, and the factor 0.7 leaves 7 tau
+// sigma_true >= 1.03 cmin.  Anything else goes to the exact path.
 __device__ __forceinline__ bool c1_cannot_bind_rough(float s1, float s2, float seven_tau, float cmin, float inv_g = 1.0f / 32.0f) {
     const float mean = s1 * inv_g;
     const float ex2 = s2 * inv_g;

@@ -155,3 +155,31 @@ def test_eight_chunks_a_lane(M, C, g):
             ref = oracle.quantize_act(bits, g=g, **kw)
             codes, scale = tdq.quantize_act(x[:, :C], tdq.act_params(g=g, tau=kw.get("tau", 1.0), zr=kw.get("zr", 0.2), p=kw.get("p", 1.0), flags=kw.get("flags", 3)))
             compare_quantizer(si.bf16_bits_to_f32(bits), g, ref, codes.cpu().numpy()[pick], scale.cpu().numpy()[pick])
+
+
+@pytest.mark.parametrize("g", [32, 128, 256, 2048, 4096])
+def test_dispersion_screen_on_bf16_sums(g):
+    """Groups whose bf16 partial sums round one way (a dominant first term, equal terms, terms about a mean) with 7 tau sigma just
+    above and below the maximum, where only the exact deviation may decide."""
+    from paper_2604_16855_b200 import tdq
+    rng = np.random.default_rng(300 + g)
+    rows = []
+    for first, rest in ((1.0, 0.06298828125), (1.0, 0.0629), (3.0, 0.19), (1.0, 0.3)):
+        x = np.full(g, rest)
+        x[::32] = first                                   # the first two terms of every sum of sixteen pairs
+        x[1::32] = -first
+        rows.append(x)
+    for mean, spread in ((1.0, 1.0), (1.004, 0.97), (0.73, 0.69), (0.0, 1.0)):
+        rows.append(mean + spread * np.where(np.arange(g) // 2 % 2 == 0, 1.0, -1.0))
+        rows.append(mean + spread * rng.standard_normal(g))
+    x = np.stack(rows).astype(np.float32)
+    bits = si.f32_to_bf16_bits(x)
+    v = si.bf16_bits_to_f32(bits).astype(np.float64)
+    edge = np.abs(v).max(1) / (7.0 * v.std(1))             # tau at which the two bounds meet
+    fill = 7 * 32 * 32 // g + 1                           # whole blocks of the kernels take part
+    for e in edge:
+        for off in (-0.05, -1e-3, -1e-6, 1e-6, 1e-3, 0.02, 0.04, 0.08, 0.2):
+            tau = float(np.float32(e * (1.0 + off)))
+            ref = oracle.quantize_act(np.tile(bits, (fill, 1)), g=g, tau=tau, flags=1)
+            codes, scale = tdq.quantize_act(to_cuda(np.tile(bits, (fill, 1)), bf16=True), tdq.act_params(g=g, tau=tau, flags=1))
+            compare_quantizer(si.bf16_bits_to_f32(np.tile(bits, (fill, 1))), g, ref, codes.cpu().numpy(), scale.cpu().numpy())
