@@ -17,7 +17,9 @@ def _check(xc, xs, wc, ws, g, O):
     bias = torch.randn((O,), device="cuda", generator=torch.Generator("cuda").manual_seed(O))
     want = oracle.w4a4_linear(xc.cpu().numpy(), xs.cpu().numpy(), wc.cpu().numpy(), ws.cpu().numpy(), bias=bias.cpu().numpy(), g=g)
     wsp = tdq.linear_workspace(M, K * g, O, g, "cuda")
+    n0 = tdq.kernel_launch_count()
     y = tdq.w4a4_linear(xc, xs, wc, ws, bias, g=g, workspace=wsp)
+    assert tdq.kernel_launch_count() - n0 == (2 if g == 32 and K > 28 else 1)   # no expansion but beyond the rule's end
     assert tdq.workspace_status(wsp) == (tdq.OK, 0)
     # K products, K sums, the scaling and the bias, each rounded once (2^-24 of a partial sum)
     t = want["t_abs"] + np.abs(bias.cpu().numpy())[None, :]

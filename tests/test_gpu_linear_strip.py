@@ -27,7 +27,9 @@ def _check(xc, xs, wc, ws, O):
     ref = tdq.w4a4_linear(xc, xs, wc, ws, bias, y=odd, workspace=wsp)
     for dt in (torch.float32, torch.bfloat16, torch.float16):
         buf = torch.full((M, O + 8), 3.0, dtype=dt, device="cuda")
+        n0 = tdq.kernel_launch_count()
         y = tdq.w4a4_linear(xc, xs, wc, ws, bias, y=buf[:, :O], workspace=wsp)
+        assert tdq.kernel_launch_count() - n0 == 1            # this kernel: the others expand the operands first at these sizes
         assert tdq.workspace_status(wsp) == (tdq.OK, 0)
         assert torch.equal(y, ref.to(dt))
         assert bool((buf[:, O:] == 3.0).all())
