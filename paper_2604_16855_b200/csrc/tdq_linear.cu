@@ -1277,11 +1277,14 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     // 14.1; 2304 x 288 -> 1280 fp32 (180 tiles) 11.1 and 11.6 (with the quantizer 13.2 and 14.6), 2304 x 256 -> 1280 bf16 9.1 and 9.4;
     // 36864 x 256 -> 192 bf16 14.2 and 15.3, 73728 x 192 -> 192 21.9 and 23.1, 73728 x 128 -> 192 17.2 and 17.9.  In a stream, with
     // the quantizer, the same: 18.5 and 17.7, 19.4 and 18.1, 15.3 and 15.2, 14.4 and 12.9, 24.7 and 23.5, 35.0 and 34.6, 27.9 and 26.8.
-    // Over 454 sizes the rule is within 0.2 % of the better kernel of each in a graph; never this kernel 5.8 %, always 0.9 %.
+    // And with binary32 y from 192 to 256 channels, eight column tiles or more and more than four tiles per SM: 9216 x 256 -> 1280 17.5 and
+    // 18.4 (with the quantizer 20.9 and 22.8, in a stream 25.1 and 23.4), 18432 x 192 -> 960 22.4 and 24.1.
+    // Over 711 sizes the rule is 0.3 % from the better kernel of each in a graph on average; never this kernel would be 6 %, always 1 %.
     const int64_t rounds = (tiles128 + n_sm - 1) / n_sm;
     const bool graph_loses = O > 128 && tiles128 > n_sm &&
                              (p.n_steps >= 10 || (p.n_steps >= 8 && rounds * n_sm * 5 >= tiles128 * 7) ||
-                              (p.n_steps >= 4 && !full_tiles && tiles128 > (p.n_steps >= 6 ? 3 : 6) * n_sm));
+                              (p.n_steps >= 4 && !full_tiles && tiles128 > (p.n_steps >= 6 ? 3 : 6) * n_sm) ||
+                              (y_dtype == TDQ_F32 && p.n_steps >= 6 && p.n_steps <= 8 && p.tiles_n >= 8 && tiles128 > 4 * n_sm));
     if (use_strip && graph_loses) {
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
         const bool known = cudaStreamIsCapturing(stream, &capture) == cudaSuccess;
