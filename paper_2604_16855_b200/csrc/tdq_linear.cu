@@ -11,7 +11,7 @@
 // 128 x 128 x 32 instruction takes 64 clocks, while 16384 fp32 FMAs take 128 clocks of the SM's
 // FMA pipes.  The operand encoding is chosen so that nothing else is added to that:
 //
-//   * g <= 128: kind::f8f6f4, E4M3 operands, fp32 accumulator.  A code q in [-8, 8] is stored as
+//   * g <= 128: kind::f8f6f4, E4M3 operands, fp32 accumulator (but for tdq_linear_solo.cu, which takes 64 to 128 as int8).  A code q in [-8, 8] is stored as
 //     the byte sign(q) << 7 | |q|, which E4M3 reads as q * 2^-9 (the values are subnormal, or
 //     2^-6 for |q| = 8).  g / 32 instructions contract one group into a fresh slot; the products
 //     (|p| <= 64) and their sum (<= 8192) are exact in the fp32 accumulator, so TMEM holds
@@ -24,12 +24,18 @@
 //   The power of two is folded into the output-channel scale in the epilogue; both routes
 //   give bit-identical integer sums and the same float sequence.
 //
-// This file prepares every call (linear_impl) and picks the kernel; the one below is the general form.  Others: g = 32, and
-// 64 and 128 where tiles are few or short, tdq_linear_pair.cu; g = 32 on long contractions tdq_linear_g32.cu; one accumulator
-// per output tdq_linear_one.cu.  The general kernel keeps groups of 64 and 128 on larger layers, other widths with several
-// groups per token, small layers with one, and the fused variant (the only one that runs it at g = 32).
+// This file prepares every call (linear_impl) and picks the kernel; the one below is the general form.  Others:
+//   tdq_linear_solo.cu    no more 128 x 64 tiles than SMs, any group size, from the packed codes
+//   tdq_linear_strip.cu   g = 32, a few 128 x 128 tiles per SM, from the packed codes
+//   tdq_linear_pair.cu    g = 32 otherwise up to 1536 channels, or a y that tensor stores cannot write; 64 and 128 where contractions are
+//                         short or outputs few; small layers of few groups from the packed codes
+//   tdq_linear_defer.cu   g = 32, 64, 128 with several 128 x 128 tiles per SM
+//   tdq_linear_g32.cu     g = 32, long contractions
+//   tdq_linear_one.cu     one accumulator per output: one step per token, power-of-two steps
+// The general kernel keeps other widths with several groups per token, wide groups whose y tensor stores cannot write or whose
+// group sums are asked for (acc_debug), and the fused variant (the only one that runs it at g = 32).
 //
-// Two kernels per call (one for the small layers that tdq_linear_pair.cu expands itself):
+// Two kernels per call (one where the kernel makes its operands from the packed codes):
 //   1. expand_kernel   rewrites the packed nibbles of both operands as operand bytes, in 128-row
 //      x 32-code blocks laid out in the tensor core's K-major core-matrix order (8 rows x 16
 //      bytes contiguous), and regroups the activation scales as [row block][group][128 rows].
@@ -1220,8 +1226,7 @@ tdq_status linear_impl(const FusedSrc* fx, const uint8_t* xcodes, const float* x
     const bool use_g32 = group_size == 32 && !pow2_steps && !fx && p.tiles_m * p.tiles_n <= INT32_MAX / 4;
     // Groups of 64 and 128 too where the general kernel's wide tiles are mostly overhead: contractions of up to 512 channels
     // (9216 x 128 -> 512 at 64 11.1 -> 10.3 us), at most 64 outputs (30000 x 640 -> 64 at 128 18.4 -> 14.2 us), fewer tiles than
-    // SMs (1000 x 2048 -> 256 at 64 14.7 -> 12.4 us).  Otherwise the general kernel: 4616 x 768 -> 3072 at 128 fp16 23.7 us
-    // against 24.8 in the pair kernel, 18464 rows fp32 84 against 100, at 64 98 against 108.
+    // SMs (1000 x 2048 -> 256 at 64 14.7 -> 12.4 us); of these, few tiles go to tdq_linear_solo.cu and many to tdq_linear_defer.cu below.
     const bool use_pair_wide = !pow2_steps && !fx && !use_one && (group_size == 64 || group_size == 128) && p.tiles_m * p.tiles_n <= INT32_MAX / 4 &&
                                (p.n_steps <= 16 || O <= 64 || p.tiles_m * p.tiles_n <= n_sm);
     const bool pair_ok = use_pair_wide || (use_g32 && (!y_tma || p.n_steps <= kPairMaxSteps || p.tiles_m * p.tiles_n * 4 <= n_sm));

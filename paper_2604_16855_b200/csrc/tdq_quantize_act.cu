@@ -142,7 +142,8 @@ __device__ __forceinline__ void process_group(const uint32_t (&w)[BF16 ? 16 : 32
 // A bf16 group is four 16-byte loads of its own thread, whose sectors the neighbours share.  An fp32 group is eight, too far apart
 // for that, so a warp loads its 32 groups in order and passes them on through its own part of shared memory (18464 x 768 17.2
 // against 16.2 us, 9216 x 320 6.2 and 4.9; bf16 11.8 against 12.0); rows with a pitch, which cost a division a group, are loaded
-// directly in either type.  Blocks of 128 threads: level, long bf16 inputs 1 to 2 % slower.
+// directly in either type (the staging kernel that had them before and this, pitch 8 longer: 18464 x 768 bf16 21.6 and 12.8, 9216 x
+// 320 6.0 and 3.75; fp32 2304 x 768 8.4 and 5.25, 1152 x 512 4.8 and 2.4).  Blocks of 128 threads: level, long bf16 inputs 1 to 2 % slower.
 template <bool BF16, int KZR, int KB = 32>
 __global__ void __launch_bounds__(kFastThreads) act_g32_kernel(ActArgs a) {
     constexpr int kGroupBytes = BF16 ? 64 : 128;
