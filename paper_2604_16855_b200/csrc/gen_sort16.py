@@ -1,6 +1,10 @@
 """Writes sort16_network.inc: Batcher's odd-even merge sort for 16 inputs as a list of
 compare-exchange steps TDQ_CE(i, j) (i < j; the smaller value ends in slot i).
 
+The eight steps on neighbours (2 i, 2 i + 1) come first, with the line TDQ_PAIRS behind them: the larger of each pair then
+stands in the odd slots, and the includer takes the maximum of all sixteen from there (no step before them touches a slot
+of theirs, so the order changes nothing).
+
 The network is checked here with the 0-1 principle (all 65536 binary inputs) before it
 is written.  The CUDA quantizer includes the file twice-unrolled in registers and uses
 only the lowest few outputs, so the compiler drops the comparators that cannot reach them.
@@ -31,7 +35,8 @@ def batcher(n):
             merge(lo, hi, 1)
 
     sort(0, n - 1)
-    return steps
+    pairs = [(i, i + 1) for i in range(0, n, 2)]
+    return pairs + [s for s in steps if s not in pairs]
 
 
 def sorts_all_binary_inputs(steps, n):
@@ -51,6 +56,6 @@ if __name__ == "__main__":
     path = os.path.join(os.path.dirname(os.path.abspath(__file__)), "sort16_network.inc")
     with open(path, "w") as f:
         f.write("// Generated by gen_sort16.py: Batcher odd-even merge sort, 16 inputs, 63 steps.\n")
-        for a, b in net:
-            f.write("TDQ_CE(%d, %d)\n" % (a, b))
+        for n, (a, b) in enumerate(net):
+            f.write("TDQ_CE(%d, %d)\n" % (a, b) + ("TDQ_PAIRS\n" if n == 7 else ""))
     print("wrote", path)

@@ -88,6 +88,31 @@ __device__ __forceinline__ bool c1_cannot_bind_rough(float s1, float s2, float s
     return cmin <= kClipFloor || ((var >= ex2 * 0.5f) && (lhs > rhs) && (rhs >= 1e-30f) && (s2 < 1e37f) && (lhs < 1e37f));
 }
 
+// x clipped to [-c, c], c >= 0, in one instruction: the smaller magnitude with x's sign.  (On a NaN it gives c or -c.)
+__device__ __forceinline__ float clip_f32(float x, float c) {
+    float r;
+    asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(r) : "f"(x), "f"(c));
+    return r;
+}
+// Two bf16 at a time: the smaller and the larger magnitude of each pair of halves, with the product of their signs.  So a network of
+// them orders magnitudes without a pass that takes the signs off (which comes at the end, on what is left), and against a c >= 0
+// the smaller one is the clip.
+__device__ __forceinline__ uint32_t min_mag2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("min.xorsign.abs.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+__device__ __forceinline__ uint32_t max_mag2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("max.xorsign.abs.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+// the larger magnitude of the two halves, as a float
+__device__ __forceinline__ float larger_half(uint32_t p) {
+    p &= 0x7fff7fffu;
+    return __uint_as_float(max(p & 0xffffu, p >> 16) << 16);
+}
+
 // two binary32 lanes in one 64-bit register; each lane rounds exactly like the scalar .rn instruction
 __device__ __forceinline__ uint64_t f2_pack(float lo, float hi) {
     uint64_t r;
@@ -137,19 +162,19 @@ __device__ __forceinline__ uint32_t nibble_ieee(float x, float c, float delta) {
     return (uint32_t)quantize_ieee(x, c, delta) & 0xFu;
 }
 
-// K-th smallest of 32 magnitudes given as two sorted halves (even and odd channels of a bf16 group in
-// the low and high 16 bits of s[0..15]; s[0..15] and s[16..31] of an fp32 group): the maximum over
+// K-th smallest of 32 magnitudes given as two halves sorted by magnitude (even and odd channels of a bf16 group in
+// the low and high 16 bits of s[0..15], signs at random; s[0..15] and s[16..31] of an fp32 group): the maximum over
 // i + j = K - 1 of min(E[i], O[j]), an index past the end counting as +inf.
 template <int K>
-__device__ __forceinline__ uint32_t kth_of_sorted_halves_u16(const uint32_t (&s)[16]) {
+__device__ __forceinline__ float kth_of_sorted_halves_bf16(const uint32_t (&s)[16]) {
     constexpr int lo_i = (K > 16) ? K - 16 : 0;
     constexpr int hi_i = (K - 1 < 15) ? K - 1 : 15;
-    constexpr int mid_i = (lo_i + hi_i) / 2;
+    constexpr int mid_i = (lo_i + hi_i) / 2;      // a packed minimum with the partner's halves swapped covers index i and its mirror
     uint32_t r = (K > 16) ? s[(K > 16) ? K - 17 : 0] : 0u;
 #pragma unroll
     for (int i = lo_i; i <= mid_i && i <= hi_i; ++i)
-        r = __vmaxu2(r, __vminu2(s[i], __byte_perm(s[K - 1 - i], 0u, 0x1032u)));
-    return max(r & 0xffffu, r >> 16);
+        r = max_mag2(r, min_mag2(s[i], __byte_perm(s[K - 1 - i], 0u, 0x1032u)));
+    return larger_half(r);
 }
 template <int K>
 __device__ __forceinline__ float kth_of_sorted_halves_f32(const float (&s)[32]) {
@@ -167,13 +192,13 @@ __device__ __forceinline__ float kth_of_sorted_halves_f32(const float (&s)[32]) 
     TDQ_RC(1) TDQ_RC(2) TDQ_RC(3) TDQ_RC(4) TDQ_RC(5) TDQ_RC(6) TDQ_RC(7) TDQ_RC(8) TDQ_RC(9) TDQ_RC(10) TDQ_RC(11) \
     TDQ_RC(12) TDQ_RC(13) TDQ_RC(14) TDQ_RC(15) TDQ_RC(16) TDQ_RC(17) TDQ_RC(18) TDQ_RC(19) TDQ_RC(20) TDQ_RC(21) \
     TDQ_RC(22) TDQ_RC(23) TDQ_RC(24) TDQ_RC(25) TDQ_RC(26) TDQ_RC(27) TDQ_RC(28) TDQ_RC(29) TDQ_RC(30) TDQ_RC(31) TDQ_RC(32)
-__device__ __forceinline__ uint32_t kth_of_sorted_halves_u16_rt(const uint32_t (&s)[16], int k) {
+__device__ __forceinline__ float kth_of_sorted_halves_bf16_rt(const uint32_t (&s)[16], int k) {
     switch (k) {
-#define TDQ_RC(K_) case K_: return kth_of_sorted_halves_u16<K_>(s);
+#define TDQ_RC(K_) case K_: return kth_of_sorted_halves_bf16<K_>(s);
         TDQ_RANK_CASES
 #undef TDQ_RC
     }
-    return 0u;
+    return 0.0f;
 }
 __device__ __forceinline__ float kth_of_sorted_halves_f32_rt(const float (&s)[32], int k) {
     switch (k) {
@@ -184,17 +209,51 @@ __device__ __forceinline__ float kth_of_sorted_halves_f32_rt(const float (&s)[32
     return 0.0f;
 }
 
+// The rare paths of a group (the deviation in binary64, 32 IEEE divisions), out of line for kernels that want few registers: inline they take
+// registers from the instructions that every group needs.
+template <bool BF16>
+struct GroupWords {
+    uint32_t w[BF16 ? 16 : 32];
+    __device__ __forceinline__ float get(int i) const {
+        if (BF16) return (i & 1) ? __uint_as_float(w[i >> 1] & 0xffff0000u) : __uint_as_float(w[i >> 1] << 16);
+        return __uint_as_float(w[i]);
+    }
+};
+template <bool BF16>
+__device__ __noinline__ float sigma_exact_group(GroupWords<BF16> g) {
+    return sigma_exact32([&](int i) -> float { return g.get(i); });
+}
+template <bool BF16>
+__device__ __forceinline__ uint4 codes_ieee(const GroupWords<BF16>& g, float c, float delta) {
+    uint32_t out[4];
+#pragma unroll
+    for (int wd = 0; wd < 4; ++wd) {
+        out[wd] = 0u;
+#pragma unroll
+        for (int n = 0; n < 8; ++n) out[wd] |= nibble_ieee(g.get(wd * 8 + n), c, delta) << (4 * n);
+    }
+    return make_uint4(out[0], out[1], out[2], out[3]);
+}
+template <bool BF16>
+__device__ __noinline__ uint4 codes_ieee_group(GroupWords<BF16> g, float c, float delta) { return codes_ieee(g, c, delta); }
+
 // One group held in registers (w: 16 packed bf16 pairs or 32 floats, in channel order): statistics,
 // projection, quantization.  out: the group's 32 two's complement nibbles, channel 8 w + n in
 // nibble n of word w; delta: its step.  KB: rank of the base radius among the magnitudes (32: the maximum,
 // Eq. 5; less: the percentile option of Supp. S4.8, which takes the group's KB-th smallest magnitude).
 // KB == 0: both ranks are run-time values (rt_kzr, rt_kb in 1..32), for the settings that have no instance of their own.
-template <bool BF16, int KZR, int KB = 32>
+template <bool BF16, int KZR, int KB = 32, bool OUT_OF_LINE = false>
 __device__ __forceinline__ void quantize_group32(const uint32_t (&w)[BF16 ? 16 : 32], float seven_tau, uint32_t flags,
                                                  uint32_t (&out)[4], float& delta, int rt_kzr = 0, int rt_kb = 0) {
     auto get = [&](int i) -> float {
         if (BF16) return (i & 1) ? __uint_as_float(w[i >> 1] & 0xffff0000u) : __uint_as_float(w[i >> 1] << 16);
         return __uint_as_float(w[i]);
+    };
+    auto all = [&]() {
+        GroupWords<BF16> g;
+#pragma unroll
+        for (int i = 0; i < (BF16 ? 16 : 32); ++i) g.w[i] = w[i];
+        return g;
     };
 
     // base radius, rank-KZR magnitude, moments
@@ -204,27 +263,31 @@ __device__ __forceinline__ void quantize_group32(const uint32_t (&w)[BF16 ? 16 :
         if (BF16) {
             uint32_t s[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) s[i] = w[i] & 0x7fff7fffu;
-#define TDQ_CE(i, j) { uint32_t lo_ = __vminu2(s[i], s[j]); s[j] = __vmaxu2(s[i], s[j]); s[i] = lo_; }
+            for (int i = 0; i < 16; ++i) s[i] = w[i];
+#define TDQ_CE(i, j) { const uint32_t lo_ = min_mag2(s[i], s[j]); s[j] = max_mag2(s[i], s[j]); s[i] = lo_; }
+#define TDQ_PAIRS
 #include "sort16_network.inc"
+#undef TDQ_PAIRS
 #undef TDQ_CE
             if (KB == 0) {
-                c_base = __uint_as_float(kth_of_sorted_halves_u16_rt(s, rt_kb) << 16);
-                if (flags & TDQ_ENABLE_C2) thr = __uint_as_float(kth_of_sorted_halves_u16_rt(s, rt_kzr) << 16);
+                c_base = kth_of_sorted_halves_bf16_rt(s, rt_kb);
+                if (flags & TDQ_ENABLE_C2) thr = kth_of_sorted_halves_bf16_rt(s, rt_kzr);
             } else {
-                c_base = __uint_as_float(kth_of_sorted_halves_u16<(KB ? KB : 1)>(s) << 16);
-                if (flags & TDQ_ENABLE_C2) thr = __uint_as_float(kth_of_sorted_halves_u16<(KZR ? KZR : 1)>(s) << 16);
+                c_base = kth_of_sorted_halves_bf16<(KB ? KB : 1)>(s);
+                if (flags & TDQ_ENABLE_C2) thr = kth_of_sorted_halves_bf16<(KZR ? KZR : 1)>(s);
             }
         } else {
             float s[32];
 #pragma unroll
             for (int i = 0; i < 32; ++i) s[i] = fabsf(__uint_as_float(w[i]));
+#define TDQ_PAIRS
 #define TDQ_CE(i, j) { float lo_ = fminf(s[i], s[j]); s[j] = fmaxf(s[i], s[j]); s[i] = lo_; }
 #include "sort16_network.inc"
 #undef TDQ_CE
 #define TDQ_CE(i, j) { float lo_ = fminf(s[16 + i], s[16 + j]); s[16 + j] = fmaxf(s[16 + i], s[16 + j]); s[16 + i] = lo_; }
 #include "sort16_network.inc"
 #undef TDQ_CE
+#undef TDQ_PAIRS
             if (KB == 0) {
                 c_base = kth_of_sorted_halves_f32_rt(s, rt_kb);
                 if (flags & TDQ_ENABLE_C2) thr = kth_of_sorted_halves_f32_rt(s, rt_kzr);
@@ -234,57 +297,45 @@ __device__ __forceinline__ void quantize_group32(const uint32_t (&w)[BF16 ? 16 :
             }
         }
     } else if (BF16) {
-        // |x| of a bf16 is a 15-bit key whose unsigned order is the numeric order, so the network
-        // runs on packed 16-bit integer min/max (two channels per instruction, integer pipe)
         uint32_t s[16];
-        uint32_t mx = 0;
+        uint32_t mx = 0u;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            s[i] = w[i] & 0x7fff7fffu;
-            mx = __vmaxu2(mx, s[i]);
-        }
-        c_base = __uint_as_float(max(mx & 0xffffu, mx >> 16) << 16);
+        for (int i = 0; i < 16; ++i) s[i] = w[i];
         if (flags & TDQ_ENABLE_C2) {
-#define TDQ_CE(i, j) { uint32_t lo_ = __vminu2(s[i], s[j]); s[j] = __vmaxu2(s[i], s[j]); s[i] = lo_; }
+            // the larger ones of the network's first eight pairs hold the maximum
+#define TDQ_CE(i, j) { const uint32_t lo_ = min_mag2(s[i], s[j]); s[j] = max_mag2(s[i], s[j]); s[i] = lo_; }
+#define TDQ_PAIRS mx = max_mag2(max_mag2(max_mag2(s[1], s[3]), max_mag2(s[5], s[7])), max_mag2(max_mag2(s[9], s[11]), max_mag2(s[13], s[15])));
 #include "sort16_network.inc"
+#undef TDQ_PAIRS
 #undef TDQ_CE
-            // low halves: sorted even channels E, high halves: sorted odd channels O.  The KZR-th
-            // smallest of the union is max over i + j = KZR - 1 of min(E[i], O[j]), where an
-            // index past the end counts as +inf (so for KZR > 16 the terms E[KZR-17] and
-            // O[KZR-17] stand alone).  One packed min with the partner's halves swapped covers
-            // index i and its mirror at once.
-            constexpr int lo_i = (KZR > 16) ? KZR - 16 : 0;
-            constexpr int hi_i = (KZR - 1 < 15) ? KZR - 1 : 15;
-            constexpr int mid_i = (lo_i + hi_i) / 2;
-            uint32_t r = (KZR > 16) ? s[(KZR > 16) ? KZR - 17 : 0] : 0u;
+            thr = kth_of_sorted_halves_bf16<KZR>(s);
+        } else {
 #pragma unroll
-            for (int i = lo_i; i <= mid_i && i <= hi_i; ++i)
-                r = __vmaxu2(r, __vminu2(s[i], __byte_perm(s[KZR - 1 - i], 0u, 0x1032u)));
-            thr = __uint_as_float(max(r & 0xffffu, r >> 16) << 16);
+            for (int i = 0; i < 16; ++i) mx = max_mag2(mx, s[i]);
         }
+        c_base = larger_half(mx);
     } else {
         float s[32];
         float mx = 0.0f;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            s[i] = fabsf(__uint_as_float(w[i]));
-            mx = fmaxf(mx, s[i]);
-        }
-        c_base = mx;
+        for (int i = 0; i < 32; ++i) s[i] = fabsf(__uint_as_float(w[i]));
         if (flags & TDQ_ENABLE_C2) {
 #define TDQ_CE(i, j) { float lo_ = fminf(s[i], s[j]); s[j] = fmaxf(s[i], s[j]); s[i] = lo_; }
+#define TDQ_PAIRS mx = fmaxf(fmaxf(fmaxf(s[1], s[3]), fmaxf(s[5], s[7])), fmaxf(fmaxf(s[9], s[11]), fmaxf(s[13], s[15])));
 #include "sort16_network.inc"
+#undef TDQ_PAIRS
 #undef TDQ_CE
 #define TDQ_CE(i, j) { float lo_ = fminf(s[16 + i], s[16 + j]); s[16 + j] = fmaxf(s[16 + i], s[16 + j]); s[16 + i] = lo_; }
+#define TDQ_PAIRS mx = fmaxf(mx, fmaxf(fmaxf(fmaxf(s[17], s[19]), fmaxf(s[21], s[23])), fmaxf(fmaxf(s[25], s[27]), fmaxf(s[29], s[31]))));
 #include "sort16_network.inc"
+#undef TDQ_PAIRS
 #undef TDQ_CE
-            constexpr int lo_i = (KZR > 16) ? KZR - 16 : 0;
-            constexpr int hi_i = (KZR - 1 < 15) ? KZR - 1 : 15;
-            float r = (KZR > 16) ? fmaxf(s[(KZR > 16) ? KZR - 17 : 0], s[(KZR > 16) ? KZR - 1 : 16]) : 0.0f;
+            thr = kth_of_sorted_halves_f32<KZR>(s);
+        } else {
 #pragma unroll
-            for (int i = lo_i; i <= hi_i; ++i) r = fmaxf(r, fminf(s[i], s[16 + KZR - 1 - i]));
-            thr = r;
+            for (int i = 0; i < 32; ++i) mx = fmaxf(mx, s[i]);
         }
+        c_base = mx;
     }
 
     float sigma = INFINITY;   // an idle C1 bound
@@ -313,7 +364,7 @@ __device__ __forceinline__ void quantize_group32(const uint32_t (&w)[BF16 ? 16 :
             }
             idle = c1_cannot_bind(s1, s2, seven_tau, cmin);
         }
-        if (!idle) sigma = sigma_exact32(get);
+        if (!idle) sigma = OUT_OF_LINE ? sigma_exact_group<BF16>(all()) : sigma_exact32(get);
     }
 
     float c;
@@ -327,7 +378,7 @@ __device__ __forceinline__ void quantize_group32(const uint32_t (&w)[BF16 ? 16 :
         // between c and that bound still divides to less than 7.5 (or 1.5 under the step floor),
         // so it rounds to the same code as c itself
         const uint32_t cup = (__float_as_uint(c) + 0xffffu) >> 16;
-        const uint32_t cpos = cup | (cup << 16), cneg = cpos | 0x80008000u;
+        const uint32_t c2 = cup | (cup << 16);
 #pragma unroll
         for (int wd = 0; wd < 4; ++wd) {
             uint32_t acc = 0;
@@ -335,26 +386,19 @@ __device__ __forceinline__ void quantize_group32(const uint32_t (&w)[BF16 ? 16 :
             for (int n = 6; n >= 0; n -= 2) {
                 uint64_t xt;
                 if (BF16) {
-                    const __nv_bfloat162 lim_hi = *reinterpret_cast<const __nv_bfloat162*>(&cpos);
-                    const __nv_bfloat162 lim_lo = *reinterpret_cast<const __nv_bfloat162*>(&cneg);
-                    const __nv_bfloat162 xp = __hmin2(__hmax2(*reinterpret_cast<const __nv_bfloat162*>(&w[wd * 4 + n / 2]), lim_lo), lim_hi);
-                    const uint32_t u = *reinterpret_cast<const uint32_t*>(&xp);
+                    const uint32_t u = min_mag2(w[wd * 4 + n / 2], c2);
                     xt = f2_pack(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
                 } else {
-                    xt = f2_pack(fminf(fmaxf(get(wd * 8 + n), -c), c), fminf(fmaxf(get(wd * 8 + n + 1), -c), c));
+                    xt = f2_pack(clip_f32(get(wd * 8 + n), c), clip_f32(get(wd * 8 + n + 1), c));
                 }
                 nibbles_fast2(xt, neg_delta2, rcp2, magic2, acc);
             }
             out[wd] = pack_word(acc);
         }
     } else {   // 1 / Delta would be subnormal: take the IEEE division
-#pragma unroll
-        for (int wd = 0; wd < 4; ++wd) {
-            uint32_t acc = 0;
-#pragma unroll
-            for (int n = 0; n < 8; ++n) acc |= nibble_ieee(get(wd * 8 + n), c, delta) << (4 * n);
-            out[wd] = acc;
-        }
+        const GroupWords<BF16> g = all();
+        const uint4 o = OUT_OF_LINE ? codes_ieee_group<BF16>(g, c, delta) : codes_ieee(g, c, delta);
+        out[0] = o.x; out[1] = o.y; out[2] = o.z; out[3] = o.w;
     }
 }
 

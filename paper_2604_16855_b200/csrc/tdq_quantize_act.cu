@@ -120,21 +120,35 @@ __global__ void __launch_bounds__(kGenericWarps * 32) act_generic_kernel(ActArgs
 // fast kernel: g = 32, one thread per group
 
 // Threads, and so groups, of a block of the fast kernels.  Small blocks: ten of them fill an SM's registers without the remainder
-// that two of 256 threads leave, and no warp waits for more than one other.
-constexpr int kFastThreads = 64;
+// that two of 256 threads leave, and no warp waits for more than one other.  The instances for long inputs hold sixteen.
+constexpr int kFastThreads = 64, kFastBlocks = 16;
+
+// Whether an input is long: more than 24 blocks per SM.  Its instances are held to 64 registers (72 channel-major), with the rare paths out
+// of line, so that 32 warps instead of 20 hide each other's latencies: issue slots 0.54 -> 0.68 busy.  us from a graph, the other instances
+// (ten blocks per SM) and these: bf16 16384 x 4096 44.4 and 38.6, 73728 x 256 14.3 and 13.1, 18464 x 768 9.9 and 9.4, 18432 x 512 8.6 and 7.95,
+// fp32 73728 x 256 19.7 and 19.4, bf16 map [16, 512, 60, 60] 28.5 and 26.4.  Short inputs lose: where all blocks are resident at once the
+// SMs get uneven shares of them, and the kernel behind finds no room to set itself up in; quantizer and layer behind it, 9216 x 320 -> 960
+// (9.7 blocks per SM) 22.4 and 23.9, 18432 x 128 -> 128 (7.8) 10.1 and 11.5, 73728 x 64 -> 64 (15.6) 15.6 and 16.4, 4608 x 1280 -> 320 (19.5) 20.1 and
+// 20.8, but 18432 x 512 -> 128 (31) 18.7 and 17.9, 73728 x 256 -> 64 (62) 30.3 and 29.5.  Twenty blocks (48 registers): fp32 spills, up to 14 %
+// slower; two or four groups a thread, the next one's loads in flight: bf16 level, fp32 8 % slower.
+bool many_blocks(int64_t blocks) {
+    const int n_sm = current_device_sm_count();
+    return blocks > 24 * (int64_t)(n_sm > 0 ? n_sm : 148);
+}
 
 // One group: quantize it in registers, write its 16 code bytes and its scale.
-template <bool BF16, int KZR, int KB = 32>
+template <bool BF16, int KZR, int KB = 32, bool LONG = false>
 __device__ __forceinline__ void process_group(const uint32_t (&w)[BF16 ? 16 : 32], const ActArgs& a, int64_t gi) {
     uint32_t out[4];
     float delta;
-    quantize_group32<BF16, KZR, KB>(w, a.seven_tau, a.flags, out, delta, a.k_zr, a.k_base);
+    quantize_group32<BF16, KZR, KB, LONG>(w, a.seven_tau, a.flags, out, delta, a.k_zr, a.k_base);
     reinterpret_cast<uint4*>(a.codes)[gi] = make_uint4(out[0], out[1], out[2], out[3]);
     a.scale[gi] = delta;
     if (a.offset) a.offset[gi] = 0.0f;
 }
 
-// Bound by the instructions of the groups (about 490 a thread, of which the ALU pipe takes most).  Warps that depend on
+// Bound by the instructions of the groups (about 435 a thread, of which the ALU pipe takes 205 at two clocks each; 456 and 235 before
+// the clip was one instruction, the maximum came from the network's first layer and the network took signed numbers).  Warps that depend on
 // nothing but their own loads keep the pipes fed better than a persistent block with a ring of bulk copies, whose first and last
 // tiles cost a latency each and whose number of tiles is rarely a multiple of the blocks; us, that ring (two blocks of eight working
 // warps per SM) and this: bf16 18464 x 768 13.7 and 11.8, 73728 x 256 17.0 and 14.9, 9216 x 320 5.9 and 3.8, 1152 x 512 2.4 and 1.75, 16384 x
@@ -144,8 +158,8 @@ __device__ __forceinline__ void process_group(const uint32_t (&w)[BF16 ? 16 : 32
 // against 16.2 us, 9216 x 320 6.2 and 4.9; bf16 11.8 against 12.0); rows with a pitch, which cost a division a group, are loaded
 // directly in either type (the staging kernel that had them before and this, pitch 8 longer: 18464 x 768 bf16 21.6 and 12.8, 9216 x
 // 320 6.0 and 3.75; fp32 2304 x 768 8.4 and 5.25, 1152 x 512 4.8 and 2.4).  Blocks of 128 threads: level, long bf16 inputs 1 to 2 % slower.
-template <bool BF16, int KZR, int KB = 32>
-__global__ void __launch_bounds__(kFastThreads) act_g32_kernel(ActArgs a) {
+template <bool BF16, int KZR, int KB = 32, bool LONG = false>
+__global__ void __launch_bounds__(kFastThreads, LONG ? kFastBlocks : 1) act_g32_kernel(ActArgs a) {
     constexpr int kGroupBytes = BF16 ? 64 : 128;
     constexpr int kChunks = kGroupBytes / 16;          // 16-byte chunks per group
     const int t = threadIdx.x;
@@ -200,7 +214,7 @@ __global__ void __launch_bounds__(kFastThreads) act_g32_kernel(ActArgs a) {
             w[4 * p + 0] = u.x; w[4 * p + 1] = u.y; w[4 * p + 2] = u.z; w[4 * p + 3] = u.w;
         }
     }
-    process_group<BF16, KZR, KB>(w, a, gi);
+    process_group<BF16, KZR, KB, LONG>(w, a, gi);
 }
 
 // every zero-bin rank of a group of 32 has its instance of the row-major kernel
@@ -223,6 +237,14 @@ cudaError_t launch_fast(const ActArgs& a, cudaStream_t st) {
             TDQ_CASE(29) TDQ_CASE(30) TDQ_CASE(31)
 #undef TDQ_CASE
             default: return cudaErrorInvalidValue;
+        }
+    }
+    if (many_blocks(blocks)) {
+        switch (a.k_zr) {
+#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_kernel<BF16, KZ, 32, true>, grid, block, 0, st, a);
+            TDQ_CASE(4) TDQ_CASE(7) TDQ_CASE(10) TDQ_CASE(13) TDQ_CASE(16) TDQ_CASE(32)
+#undef TDQ_CASE
+            default: break;
         }
     }
     switch (a.k_zr) {
@@ -346,7 +368,7 @@ cudaError_t launch_ragged(const ActArgs& a, cudaStream_t st) {
 // 12.2 -> 8.0, [16, 512, 60, 60] 39.1 -> 25.2, [16, 512, 33, 35] 33.5 -> 10.1, [2, 320, 7, 7] 3.1 -> 1.75; fp32: [16, 320, 24, 24] 7.2 -> 5.7,
 // [16, 256, 31, 31] 15.3 -> 7.0, [16, 768, 12, 12] 4.9 -> 5.4.  A tile in shared memory on 16-byte loads is level or up to 4 %
 // slower at 64 positions, 128 positions up to 11 %, 32 up to 5 %.
-constexpr int kNchwThreads = 64;
+constexpr int kNchwThreads = 64, kNchwBlocks = 14;
 
 // ACROSS: the positions of all images in one row, a division a thread, instead of blocks of their own for each image, whose last one
 // is a quarter full at 144 positions and a sixth at 72.  The time goes in steps of about five blocks per SM (2.5 warps per scheduler), so
@@ -359,8 +381,8 @@ struct NchwArgs {
     int64_t HW;         // positions per image
 };
 
-template <bool BF16, int KZR, bool ACROSS>
-__global__ void __launch_bounds__(kNchwThreads) act_g32_nchw_kernel(NchwArgs n) {
+template <bool BF16, int KZR, bool ACROSS, bool LONG = false>
+__global__ void __launch_bounds__(kNchwThreads, LONG ? kNchwBlocks : 1) act_g32_nchw_kernel(NchwArgs n) {
     constexpr int esz = BF16 ? 2 : 4;
     const ActArgs& a = n.a;
     const int t = threadIdx.x;
@@ -388,13 +410,21 @@ __global__ void __launch_bounds__(kNchwThreads) act_g32_nchw_kernel(NchwArgs n) 
 #pragma unroll
         for (int i = 0; i < 32; ++i) w[i] = __ldg(reinterpret_cast<const uint32_t*>(src + i * row));
     }
-    process_group<BF16, KZR>(w, a, ((b * n.HW + s) * a.K) + k);
+    process_group<BF16, KZR, 32, LONG>(w, a, ((b * n.HW + s) * a.K) + k);
 }
 
 template <bool BF16, bool ACROSS>
 cudaError_t launch_nchw(const NchwArgs& n, int64_t B, cudaStream_t st) {
     const int64_t blocks = ((ACROSS ? n.a.M : n.HW) + kNchwThreads - 1) / kNchwThreads;
     const dim3 grid((unsigned)blocks, (unsigned)n.a.K, ACROSS ? 1u : (unsigned)B);
+    if (!ACROSS && many_blocks(blocks * n.a.K * B)) {
+        switch (n.a.k_zr) {
+#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_nchw_kernel<BF16, KZ, false, true>, grid, dim3(kNchwThreads), 0, st, n);
+            TDQ_CASE(4) TDQ_CASE(7) TDQ_CASE(10) TDQ_CASE(13) TDQ_CASE(16) TDQ_CASE(32)
+#undef TDQ_CASE
+            default: return cudaErrorInvalidValue;
+        }
+    }
     switch (n.a.k_zr) {
 #define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_nchw_kernel<BF16, KZ, ACROSS>, grid, dim3(kNchwThreads), 0, st, n);
         TDQ_CASE(4) TDQ_CASE(7) TDQ_CASE(10) TDQ_CASE(13) TDQ_CASE(16) TDQ_CASE(32)
@@ -454,7 +484,7 @@ __global__ void __launch_bounds__(256) act_fixed_kernel(FixedArgs f) {
         uint32_t acc = 0u;
 #pragma unroll
         for (int n = 6; n >= 0; n -= 2)
-            nibbles_fast2(f2_pack(fminf(fmaxf(v[n], -f.c), f.c), fminf(fmaxf(v[n + 1], -f.c), f.c)), neg_delta2, rcp2, magic2, acc);
+            nibbles_fast2(f2_pack(clip_f32(v[n], f.c), clip_f32(v[n + 1], f.c)), neg_delta2, rcp2, magic2, acc);
         word = pack_word(acc);
     } else {                  // 1 / Delta would be subnormal: take the IEEE division
 #pragma unroll

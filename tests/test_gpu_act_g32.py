@@ -26,3 +26,32 @@ def test_block_edges(M, K, pad, dtype):
     tdq.quantize_act(xt, codes=codes[:M], scale=scale[:M])
     assert np.array_equal(codes[:M].cpu().numpy(), want["codes"]) and np.array_equal(scale[:M].cpu().numpy(), want["scale"])
     assert bool((codes[M] == 77).all()) and bool((scale[M] == -1.0).all())
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("zr", [0.1, 0.2, 1.0])
+@pytest.mark.parametrize("M,K,pad", [(7301, 32, 0), (3701, 63, 8)])
+def test_long_inputs(M, K, pad, zr, dtype):
+    """Inputs of more than 24 blocks per SM have an instance of their own, whose rare paths are calls: groups with a large mean (the
+    deviation in binary64) and of huge numbers (IEEE division) among the others.  The same bits as row by row block, and the oracle's."""
+    from paper_2604_16855_b200 import tdq
+    assert M * K > 24 * 64 * torch.cuda.get_device_properties(0).multi_processor_count and M * K % 64
+    gen = torch.Generator("cuda").manual_seed(M + K)
+    x = torch.randn((M, 32 * K), device="cuda", generator=gen) * torch.exp(0.5 * torch.randn((M, 1), device="cuda", generator=gen))
+    x[5::50] += 30.0
+    x[7::50] *= 1e32
+    x[9::50] = 0.0
+    store = torch.zeros((M, 32 * K + pad), dtype=dtype, device="cuda")
+    store[:, :32 * K] = x.to(dtype)
+    xt = store[:, :32 * K]
+    p = tdq.act_params(zr=zr)
+    codes = torch.full((M + 1, 16 * K), 77, dtype=torch.uint8, device="cuda")
+    scale = torch.full((M + 1, K), -1.0, device="cuda")
+    tdq.quantize_act(xt, p, codes=codes[:M], scale=scale[:M])
+    assert bool((codes[M] == 77).all()) and bool((scale[M] == -1.0).all())
+    for r in range(0, M, 1000):
+        c, s = tdq.quantize_act(xt[r:r + 1000], p)
+        assert torch.equal(c, codes[r:min(r + 1000, M)]) and torch.equal(s, scale[r:min(r + 1000, M)])
+    some = list(range(0, M, 61)) + [5, 7, 9, M - 1]
+    want = oracle.quantize_act(xt[some].float().cpu().numpy(), zr=zr)
+    assert np.array_equal(codes[some].cpu().numpy(), want["codes"]) and np.array_equal(scale[some].cpu().numpy(), want["scale"])

@@ -33,3 +33,20 @@ def test_blocks_across_images(B, C, H, W, dtype):
     want_codes, want_scale = tdq.quantize_act(x.permute(0, 2, 3, 1).reshape(-1, C).contiguous())
     assert torch.equal(codes[:-1], want_codes.view(-1, C // 2)) and torch.equal(scale[:-1], want_scale.view(-1, C // 32))
     assert bool((codes[-1] == 77).all()) and bool((scale[-1] == -1.0).all())
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("B,C,H,W", [(16, 512, 33, 35), (17, 768, 24, 24)])
+def test_long_maps(B, C, H, W, dtype):
+    """Maps of more than 24 blocks per SM have an instance of their own, whose rare paths (a large mean, huge numbers) are calls."""
+    from paper_2604_16855_b200 import tdq
+    assert B * (C // 32) * ((H * W + 63) // 64) > 24 * torch.cuda.get_device_properties(0).multi_processor_count
+    x = torch.randn((B, C, H, W), device="cuda", generator=torch.Generator("cuda").manual_seed(C))
+    x[:, :, 1::7] += 30.0
+    x[:, :, 3::7] *= 1e32
+    x = x.to(dtype)
+    for zr in (0.1, 0.2, 1.0):
+        p = tdq.act_params(zr=zr)
+        codes, scale = tdq.quantize_act_nchw(x, p)
+        want_codes, want_scale = tdq.quantize_act(x.permute(0, 2, 3, 1).reshape(-1, C).contiguous(), p)
+        assert torch.equal(codes.view(want_codes.shape), want_codes) and torch.equal(scale.view(want_scale.shape), want_scale)
