@@ -34,6 +34,10 @@
 // of 30 39.3 -> 22.9), at g = 64 25.0 -> 20.7; 46005 x 608 at g = 128 (a quarter of a row's last group is padding) 129.4 ->
 // 36.9, with p = 0.9 175.0 -> 69.1; 16384 x 4096 at g = 4096 76.8 -> 64.6 (of it eight chunks a lane 8.4); fp32 18464 x 768 at
 // g = 128 26.2 -> 22.8, rectified 76.1 -> 18.6.  The bisection kernel that served these cases at first: 978 us on the long groups.
+// Since then the maximum and both moments take one exchange, the element next to the last probe is found in one pass for either side of it,
+// and the clip is one instruction: 16384 x 4096 at g = 4096 64.1 -> 55.9, with the layer behind it 242 -> 226 (from a graph).
+#include <climits>
+
 #include "tdq_act_group.cuh"
 #include "tdq_common.cuh"
 
@@ -68,6 +72,46 @@ __device__ __forceinline__ T group_reduce(T v, F f, uint32_t& turn) {
     return v;
 }
 
+// Largest bit pattern of the group: over a full warp one instruction instead of five shuffles.
+template <int L, int W>
+__device__ __forceinline__ uint32_t group_max(uint32_t v, uint32_t& turn) {
+    auto f = [](uint32_t p, uint32_t q) { return max(p, q); };
+    if constexpr (L < 32) return group_reduce<L, W>(v, f, turn);
+    v = __reduce_max_sync(0xffffffffu, v);
+    return W > 1 ? group_reduce<1, W>(v, f, turn) : v;
+}
+// The group's largest magnitude and its two moments, with one exchange between the warps.  The lanes of a group halve the moments between
+// them first, so that a shuffle after the first carries one of the two for each half.
+template <int L, int W>
+__device__ __forceinline__ void group_stats(uint32_t& kmax, float& s1, float& s2, uint32_t& turn) {
+    kmax = group_max<L, 1>(kmax, turn);
+    if constexpr (L > 1) {
+        const bool up = (threadIdx.x & (L / 2)) != 0;
+        float v = (up ? s2 : s1) + __shfl_xor_sync(0xffffffffu, up ? s1 : s2, L / 2);
+#pragma unroll
+        for (int o = L / 4; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        const float w = __shfl_xor_sync(0xffffffffu, v, L / 2);
+        s1 = up ? w : v;
+        s2 = up ? v : w;
+    }
+    if constexpr (W > 1) {
+        __shared__ float4 slots[W];
+        if ((threadIdx.x & 31) == 0) slots[threadIdx.x >> 5] = make_float4(__uint_as_float(kmax), s1, s2, 0.0f);
+        __syncthreads();
+        const float4 v = slots[0];
+        kmax = __float_as_uint(v.x);
+        s1 = v.y;
+        s2 = v.z;
+#pragma unroll
+        for (int w = 1; w < W; ++w) {
+            const float4 u = slots[w];
+            kmax = max(kmax, __float_as_uint(u.x));
+            s1 += u.y;
+            s2 += u.z;
+        }
+    }
+}
+
 // The same for a sum of small whole numbers held in floats.  Over a full warp it is one integer reduction of the floats'
 // bits above 2^23 (whose low bits are the number) instead of five shuffles and adds.
 template <int L, int W>
@@ -99,7 +143,8 @@ struct Share {
         for (int i = 0; i < NC * kWords; ++i) asm volatile("" : "+r"(w[i]));
     }
     // Elements of this share whose magnitude is at most the float with bit pattern `key`, as a float: counts stay exact
-    // and never pass through the conversion unit.  bf16: `mag` holds |x| packed, probes are whole bf16 keys, the packed
+    // and never pass through the conversion unit.  bf16: `mag` holds |x| packed (taking the
+    // signs off in every compare is slower), probes are whole bf16 keys, the packed
     // compare yields 1.0 or 0.0 and a bf16 holds counts up to 256.
     __device__ __forceinline__ float count_le(const uint32_t (&mag)[NC * kWords], uint32_t key) const {
         if (BF16) {
@@ -122,42 +167,37 @@ struct Share {
         }
         return n0 + n1;
     }
-    // largest magnitude of this share that is at most that (bf16: packed, two masks and maxima at a time)
-    __device__ __forceinline__ uint32_t max_le(const uint32_t (&mag)[NC * kWords], uint32_t key) const {
-        uint32_t r = 0;
+    // The magnitude of this share that is nearest to `key` from below (at most it) or from above, as a number that is larger the nearer it is;
+    // magnitude() takes the group's largest such number back.  Setting the sign bit and taking key + 1 off leaves 0x8000 + |x| - key - 1,
+    // which as a signed number is largest for the one and smallest for the other, with those on the wrong side beyond zero.
+    __device__ __forceinline__ uint32_t nearest(int key, bool below) const {
         if constexpr (BF16) {
-            const uint32_t m = __byte_perm(key, 0u, 0x3232u);
-            const __nv_bfloat162 m2 = *reinterpret_cast<const __nv_bfloat162*>(&m);
+            const uint32_t m = ((uint32_t)key + 1u) * 0x00010001u;
+            uint32_t hi = 0x80008000u, lo = 0x7fff7fffu;
 #pragma unroll
-            for (int i = 0; i < NC * kWords; ++i) r = __vmaxu2(r, mag[i] & __hle2_mask(*reinterpret_cast<const __nv_bfloat162*>(&mag[i]), m2));
-            return max(r & 0xffffu, r >> 16) << 16;
-        } else {
-#pragma unroll
-            for (int i = 0; i < NC * 8; ++i) {
-                const uint32_t u = w[i] & 0x7fffffffu;
-                r = max(r, u <= key ? u : 0u);
+            for (int i = 0; i < NC * kWords; i += 2) {
+                const uint32_t t0 = (w[i] | 0x80008000u) - m, t1 = (w[i + 1] | 0x80008000u) - m;   // no borrow: key + 1 <= 0x8000
+                hi = __vimax3_s16x2(hi, t0, t1);
+                lo = __vimin3_s16x2(lo, t0, t1);
             }
-            return r;
+            const int a = max((int)(int16_t)hi, (int)hi >> 16), b = min((int)(int16_t)lo, (int)lo >> 16);
+            return (uint32_t)(below ? a : ~b) ^ 0x80000000u;
+        } else {
+            const uint32_t m = (uint32_t)key + 1u;
+            int hi = INT_MIN, lo = INT_MAX;
+#pragma unroll
+            for (int i = 0; i < NC * kWords; i += 2) {
+                const int t0 = (int)((w[i] | 0x80000000u) - m), t1 = (int)((w[i + 1] | 0x80000000u) - m);
+                hi = __vimax3_s32(hi, t0, t1);
+                lo = __vimin3_s32(lo, t0, t1);
+            }
+            return (uint32_t)(below ? hi : ~lo) ^ 0x80000000u;
         }
     }
-    // smallest magnitude of this share above it (any, if it is negative)
-    __device__ __forceinline__ uint32_t min_gt(const uint32_t (&mag)[NC * kWords], int key) const {
-        if constexpr (BF16) {
-            uint32_t r = 0x7fff7fffu;
-            const uint32_t m = key < 0 ? 0x80008000u + 0x3f803f80u : __byte_perm((uint32_t)key, 0u, 0x3232u);   // -1 for "none"
-            const __nv_bfloat162 m2 = *reinterpret_cast<const __nv_bfloat162*>(&m);
-#pragma unroll
-            for (int i = 0; i < NC * kWords; ++i) r = __vminu2(r, mag[i] | __hle2_mask(*reinterpret_cast<const __nv_bfloat162*>(&mag[i]), m2));
-            return min(r & 0xffffu, r >> 16) << 16;
-        } else {
-            uint32_t r = 0x7fffffffu;
-#pragma unroll
-            for (int i = 0; i < NC * 8; ++i) {
-                const uint32_t u = w[i] & 0x7fffffffu;
-                r = min(r, (int)u > key ? u : 0x7fffffffu);
-            }
-            return r;
-        }
+    static __device__ __forceinline__ uint32_t magnitude(uint32_t n, int key, bool below) {   // bit pattern
+        n ^= 0x80000000u;
+        const uint32_t t = (below ? n : ~n) + (uint32_t)key + 1u;
+        return BF16 ? (t & 0x7fffu) << 16 : t & 0x7fffffffu;
     }
 };
 
@@ -168,12 +208,10 @@ template <bool BF16, int NC, int L, int W>
 __device__ __forceinline__ uint32_t group_kth(const Share<BF16, NC>& x, int k, int absent, uint32_t kmax, float guess, float limit, uint32_t& turn) {
     constexpr int kStep = BF16 ? 16 : 0;             // keys are compared as key >> kStep
     constexpr float n = (float)(L * W * NC * 8);
-    constexpr int kWords = Share<BF16, NC>::kWords;
-    uint32_t mag[NC * kWords];
-#pragma unroll
-    for (int i = 0; i < NC * kWords; ++i) mag[i] = BF16 ? x.w[i] & 0x7fff7fffu : 0u;
-    auto umax = [](uint32_t p, uint32_t q) { return max(p, q); };
     if (BF16) kmax >>= kStep;
+    uint32_t mag[NC * Share<BF16, NC>::kWords];
+#pragma unroll
+    for (int i = 0; i < NC * Share<BF16, NC>::kWords; ++i) mag[i] = BF16 ? x.w[i] & 0x7fff7fffu : 0u;
     int lo = -1, hi = (int)kmax;                     // count(lo) < k <= count(hi)
     const int enough = (int)(__float_as_uint(limit) >> kStep);
     // counts without the absent elements' zeros (a count below them stands for none)
@@ -209,15 +247,12 @@ __device__ __forceinline__ uint32_t group_kth(const Share<BF16, NC>& x, int k, i
     }
     // exactly k elements at or below hi: the largest of them; exactly k - 1 at or below lo: the smallest of the rest
     // (all lanes of the warp take part in the reductions)
-    const bool wide = hi - lo > 1 && lo < enough, below = wide && c_hi == kf, above = wide && !below;
+    const bool wide = hi - lo > 1 && lo < enough, below = wide && c_hi == kf;
     uint32_t r = (uint32_t)hi << kStep;
-    if (__any_sync(0xffffffffu, below)) {
-        const uint32_t m = group_reduce<L, W>(x.max_le(mag, r), umax, turn);
-        if (below) r = m;
-    }
-    if (__any_sync(0xffffffffu, above)) {
-        const uint32_t m = group_reduce<L, W>(x.min_gt(mag, lo < 0 ? -1 : (int)((uint32_t)lo << kStep)), [](uint32_t p, uint32_t q) { return min(p, q); }, turn);
-        if (above) r = m;
+    if (__any_sync(0xffffffffu, wide)) {
+        const int key = below ? hi : lo;
+        const uint32_t n = group_max<L, W>(x.nearest(key, below), turn);
+        if (wide) r = x.magnitude(n, key, below);
     }
     return r;
 }
@@ -228,6 +263,12 @@ __device__ __forceinline__ uint32_t group_kth(const Share<BF16, NC>& x, int k, i
 constexpr int wide_blocks(bool bf16, int nc) {
     const int regs = bf16 ? 4 * nc + 48 : 8 * nc + 64;
     return 512 / (regs < 64 ? 64 : regs);
+}
+
+// Eight codes by IEEE division, out of line: 1 / Delta is subnormal in hardly any group.
+__device__ __noinline__ uint32_t word_ieee(float4 a, float4 b, float c, float delta) {
+    return nibble_ieee(a.x, c, delta) | nibble_ieee(a.y, c, delta) << 4 | nibble_ieee(a.z, c, delta) << 8 | nibble_ieee(a.w, c, delta) << 12 |
+           nibble_ieee(b.x, c, delta) << 16 | nibble_ieee(b.y, c, delta) << 20 | nibble_ieee(b.z, c, delta) << 24 | nibble_ieee(b.w, c, delta) << 28;
 }
 
 template <bool BF16, int NC, int L, int W>
@@ -304,8 +345,8 @@ __global__ void __launch_bounds__(W > 1 ? W * 32 : kWideThreads, wide_blocks(BF1
     float s1 = 0.0f, s2 = 0.0f;
     if (BF16) {
 #pragma unroll
-        for (int j = 0; j < NC * kW; ++j) kmax = __vmaxu2(kmax, x.w[j] & 0x7fff7fffu);
-        kmax = max(kmax & 0xffffu, kmax >> 16) << 16;
+        for (int j = 0; j < NC * kW; ++j) kmax = max_mag2(kmax, x.w[j]);
+        kmax = __float_as_uint(larger_half(kmax));
     } else {
 #pragma unroll
         for (int j = 0; j < NC * kW; ++j) kmax = max(kmax, x.w[j] & 0x7fffffffu);
@@ -334,9 +375,7 @@ __global__ void __launch_bounds__(W > 1 ? W * 32 : kWideThreads, wide_blocks(BF1
         }
     }
     x.opaque();
-    kmax = group_reduce<L, W>(kmax, [](uint32_t p, uint32_t q) { return max(p, q); }, turn);
-    s1 = group_reduce<L, W>(s1, [](float p, float q) { return p + q; }, turn);
-    s2 = group_reduce<L, W>(s2, [](float p, float q) { return p + q; }, turn);
+    group_stats<L, W>(kmax, s1, s2, turn);
 
     const int absent = kLanes * NC * 8 - g;
     const float rms = sqrtf(s2 / (float)g);
@@ -396,7 +435,7 @@ __global__ void __launch_bounds__(W > 1 ? W * 32 : kWideThreads, wide_blocks(BF1
         uint32_t* codes = reinterpret_cast<uint32_t*>(a.codes) + gi * (g / 8);
         const bool fast = delta <= 1e30f;             // otherwise 1 / Delta would be subnormal: take the IEEE division
         const float rcp = fast ? __frcp_rn(delta) : 0.0f;
-        const uint32_t cup = (__float_as_uint(c) + 0xffffu) >> 16, cpos = cup | (cup << 16), cneg = cpos | 0x80008000u;
+        const uint32_t cup = (__float_as_uint(c) + 0xffffu) >> 16, c2 = cup | (cup << 16);
         const uint64_t rcp2 = f2_pack(rcp, rcp), neg_delta2 = f2_pack(-delta, -delta), magic2 = f2_pack(kRoundMagic8, kRoundMagic8);
 #pragma unroll
         for (int ch = 0; ch < NC; ++ch) {
@@ -408,21 +447,18 @@ __global__ void __launch_bounds__(W > 1 ? W * 32 : kWideThreads, wide_blocks(BF1
                 for (int j = 6; j >= 0; j -= 2) {
                     uint64_t xt;
                     if (BF16) {                       // two channels at a time against c rounded up to a bf16 (see quantize_group32)
-                        const __nv_bfloat162 v = __hmin2(__hmax2(*reinterpret_cast<const __nv_bfloat162*>(&x.w[ch * 4 + j / 2]),
-                                                                *reinterpret_cast<const __nv_bfloat162*>(&cneg)),
-                                                        *reinterpret_cast<const __nv_bfloat162*>(&cpos));
-                        const uint32_t u = *reinterpret_cast<const uint32_t*>(&v);
+                        const uint32_t u = min_mag2(x.w[ch * 4 + j / 2], c2);
                         xt = f2_pack(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
                     } else {
                         const float v0 = x.get(ch * 8 + j), v1 = x.get(ch * 8 + j + 1);
-                        xt = f2_pack(fminf(fmaxf(v0, -c), c), fminf(fmaxf(v1, -c), c));
+                        xt = f2_pack(clip_f32(v0, c), clip_f32(v1, c));
                     }
                     nibbles_fast2(xt, neg_delta2, rcp2, magic2, acc);
                 }
                 acc = pack_word(acc);
             } else {
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc |= nibble_ieee(x.get(ch * 8 + j), c, delta) << (4 * j);
+                acc = word_ieee(make_float4(x.get(ch * 8), x.get(ch * 8 + 1), x.get(ch * 8 + 2), x.get(ch * 8 + 3)),
+                                make_float4(x.get(ch * 8 + 4), x.get(ch * 8 + 5), x.get(ch * 8 + 6), x.get(ch * 8 + 7)), c, delta);
             }
             codes[n] = acc;
         }
