@@ -120,7 +120,10 @@ __global__ void __launch_bounds__(kGenericWarps * 32) act_generic_kernel(ActArgs
 // fast kernel: g = 32, one thread per group
 
 // Threads, and so groups, of a block of the fast kernels.  Small blocks: ten of them fill an SM's registers without the remainder
-// that two of 256 threads leave, and no warp waits for more than one other.  The instances for long inputs hold sixteen.
+// that two of 256 threads leave, and no warp waits for more than one other.  The instances for long inputs hold sixteen; the others have
+// no bound (0), which gives 88 to 96 registers, ten or eleven blocks.  A bound of 1 is not the same: it lets fp32 take 108 registers, nine blocks,
+// and the 9.7 blocks per SM of 9216 x 320 no longer run at once (fp32 from a graph 5.10 and 5.59 us; channel-major [16, 320, 24, 24] bf16 4.47
+// and 5.19, with its layer 15.31 and 16.12).
 constexpr int kFastThreads = 64, kFastBlocks = 16;
 
 // Whether an input is long: more than 24 blocks per SM.  Its instances are held to 64 registers (72 channel-major), with the rare paths out
@@ -159,7 +162,7 @@ __device__ __forceinline__ void process_group(const uint32_t (&w)[BF16 ? 16 : 32
 // directly in either type (the staging kernel that had them before and this, pitch 8 longer: 18464 x 768 bf16 21.6 and 12.8, 9216 x
 // 320 6.0 and 3.75; fp32 2304 x 768 8.4 and 5.25, 1152 x 512 4.8 and 2.4).  Blocks of 128 threads: level, long bf16 inputs 1 to 2 % slower.
 template <bool BF16, int KZR, int KB = 32, bool LONG = false>
-__global__ void __launch_bounds__(kFastThreads, LONG ? kFastBlocks : 1) act_g32_kernel(ActArgs a) {
+__global__ void __launch_bounds__(kFastThreads, LONG ? kFastBlocks : 0) act_g32_kernel(ActArgs a) {
     constexpr int kGroupBytes = BF16 ? 64 : 128;
     constexpr int kChunks = kGroupBytes / 16;          // 16-byte chunks per group
     const int t = threadIdx.x;
@@ -382,7 +385,7 @@ struct NchwArgs {
 };
 
 template <bool BF16, int KZR, bool ACROSS, bool LONG = false>
-__global__ void __launch_bounds__(kNchwThreads, LONG ? kNchwBlocks : 1) act_g32_nchw_kernel(NchwArgs n) {
+__global__ void __launch_bounds__(kNchwThreads, LONG ? kNchwBlocks : 0) act_g32_nchw_kernel(NchwArgs n) {
     constexpr int esz = BF16 ? 2 : 4;
     const ActArgs& a = n.a;
     const int t = threadIdx.x;

@@ -1,5 +1,10 @@
 """The row-major quantizer at g = 32 at the edges of its 64-group blocks and 32-group warps: dense rows and rows with a pitch, both
 input types, every block boundary, against the oracle; nothing written past the last group."""
+import json
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -8,6 +13,7 @@ import oracle
 import synth_inputs as si
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
@@ -55,3 +61,37 @@ def test_long_inputs(M, K, pad, zr, dtype):
     some = list(range(0, M, 61)) + [5, 7, 9, M - 1]
     want = oracle.quantize_act(xt[some].float().cpu().numpy(), zr=zr)
     assert np.array_equal(codes[some].cpu().numpy(), want["codes"]) and np.array_equal(scale[some].cpu().numpy(), want["scale"])
+
+
+SHORT = """
+import json, os, tempfile
+import torch
+from torch.profiler import ProfilerActivity, profile
+from paper_2604_16855_b200 import tdq
+x = torch.randn((256, 64), device="cuda")
+maps = torch.randn((2, 64, 24, 24), device="cuda"), torch.randn((70, 64, 9, 9), device="cuda")       # blocks per image, and across the images
+with profile(activities=[ProfilerActivity.CUDA]) as prof:
+    for dtype in (torch.bfloat16, torch.float32):
+        for zr, p in [(0.1, 1.0), (0.2, 1.0), (0.35, 1.0), (1.0, 1.0), (0.2, 0.9), (0.3, 0.5)]:
+            tdq.quantize_act(x.to(dtype), tdq.act_params(zr=zr, p=p))
+        for zr in (0.1, 0.2, 1.0):
+            for m in maps:
+                tdq.quantize_act_nchw(m.to(dtype), tdq.act_params(zr=zr))
+    torch.cuda.synchronize()
+with tempfile.TemporaryDirectory() as d:
+    prof.export_chrome_trace(os.path.join(d, "t.json"))
+    for e in json.load(open(os.path.join(d, "t.json")))["traceEvents"]:
+        if e.get("cat") == "kernel" and "act_g32" in e["name"]:
+            print(json.dumps([e["name"], e["args"]["registers per thread"], e["args"]["block"][0]]))
+"""
+
+
+def test_ten_blocks_of_a_short_input_per_sm():
+    """Inputs of up to ten blocks per SM run at once: the registers of the instances that they take leave room for as many."""
+    r = subprocess.run([sys.executable, "-c", SHORT], cwd=ROOT, capture_output=True, text=True, timeout=300)   # the profiler stays out of this process
+    assert r.returncode == 0, r.stderr
+    kernels = [json.loads(line) for line in r.stdout.splitlines()]
+    assert len(kernels) == 2 * (6 + 3 * 2) and {n.split("<")[0].split("::")[-1] for n, _, _ in kernels} == {"act_g32_kernel", "act_g32_nchw_kernel"}
+    for name, registers, threads in kernels:
+        warp = -(-registers * 32 // 256) * 256            # a warp's registers come in pieces of 256, an SM has 65536
+        assert 65536 // (warp * threads // 32) >= 10, (name, registers)
