@@ -126,14 +126,17 @@ __global__ void __launch_bounds__(kGenericWarps * 32) act_generic_kernel(ActArgs
 // and 5.19, with its layer 15.31 and 16.12).
 constexpr int kFastThreads = 64, kFastBlocks = 16;
 
-// Whether an input is long: more than 24 blocks per SM.  Its instances are held to 64 registers (72 channel-major), with the rare paths out
-// of line, so that 32 warps instead of 20 hide each other's latencies: issue slots 0.54 -> 0.68 busy.  us from a graph, the other instances
-// (ten blocks per SM) and these: bf16 16384 x 4096 44.4 and 38.6, 73728 x 256 14.3 and 13.1, 18464 x 768 9.9 and 9.4, 18432 x 512 8.6 and 7.95,
-// fp32 73728 x 256 19.7 and 19.4, bf16 map [16, 512, 60, 60] 28.5 and 26.4.  Short inputs lose: where all blocks are resident at once the
-// SMs get uneven shares of them, and the kernel behind finds no room to set itself up in; quantizer and layer behind it, 9216 x 320 -> 960
-// (9.7 blocks per SM) 22.4 and 23.9, 18432 x 128 -> 128 (7.8) 10.1 and 11.5, 73728 x 64 -> 64 (15.6) 15.6 and 16.4, 4608 x 1280 -> 320 (19.5) 20.1 and
-// 20.8, but 18432 x 512 -> 128 (31) 18.7 and 17.9, 73728 x 256 -> 64 (62) 30.3 and 29.5.  Twenty blocks (48 registers): fp32 spills, up to 14 %
-// slower; two or four groups a thread, the next one's loads in flight: bf16 level, fp32 8 % slower.
+// Whether a bf16 input is long: more than 24 blocks per SM.  Its instances are held to 64 registers (72 channel-major; they spill 8 and 12
+// bytes), with the rare paths out of line, so that 32 warps instead of 20 hide each other's latencies: issue slots 0.54 -> 0.68 busy.  us from a
+// graph, the other instances (ten blocks per SM) and these: 16384 x 4096 44.3 and 38.6, 73728 x 256 14.6 and 13.2, 18464 x 768 11.4 and 10.4, the
+// same with a mean of 30 (every group takes a rare path) 14.3 and 13.4, map [16, 512, 60, 60] 28.3 and 26.3.  Short inputs lose: where all blocks
+// are resident at once the SMs get uneven shares of them, and the kernel behind finds no room to set itself up in; quantizer and layer behind it,
+// 9216 x 320 -> 960 (9.7 blocks per SM) 22.4 and 23.9, 18432 x 128 -> 128 (7.8) 10.1 and 11.5, 73728 x 64 -> 64 (15.6) 15.6 and 16.4, 4608 x 1280 ->
+// 320 (19.5) 20.1 and 20.8, but 18432 x 512 -> 128 (31) 18.3 and 17.7, 73728 x 256 -> 64 (62) 30.4 and 29.6.  Twenty blocks (48 registers)
+// are 2 % faster alone (not timed with a layer); two or four groups a thread, the next one's loads in flight: level.
+// fp32 has no such instances: with 64 registers it is up to 6 % faster alone (18464 x 768 15.4 and 15.3, 16384 x 4096 62.2 and 58.7), but slower
+// with the layer behind it (36864 x 320 -> 320 39.6 and 42.9, 73728 x 256 -> 64 38.8 and 41.9, 18464 x 768 -> 768 52.9 and 55.8, map
+// [16, 512, 33, 35] -> 512 34.1 and 35.4), on rows with a pitch (18464 x 768 16.8 and 18.0) and with a mean of 30 (17.8 and 19.8).
 bool many_blocks(int64_t blocks) {
     const int n_sm = current_device_sm_count();
     return blocks > 24 * (int64_t)(n_sm > 0 ? n_sm : 148);
@@ -242,12 +245,14 @@ cudaError_t launch_fast(const ActArgs& a, cudaStream_t st) {
             default: return cudaErrorInvalidValue;
         }
     }
-    if (many_blocks(blocks)) {
-        switch (a.k_zr) {
-#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_kernel<BF16, KZ, 32, true>, grid, block, 0, st, a);
-            TDQ_CASE(4) TDQ_CASE(7) TDQ_CASE(10) TDQ_CASE(13) TDQ_CASE(16) TDQ_CASE(32)
+    if constexpr (BF16) {
+        if (many_blocks(blocks)) {
+            switch (a.k_zr) {
+#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_kernel<true, KZ, 32, true>, grid, block, 0, st, a);
+                TDQ_CASE(4) TDQ_CASE(7) TDQ_CASE(10) TDQ_CASE(13) TDQ_CASE(16) TDQ_CASE(32)
 #undef TDQ_CASE
-            default: break;
+                default: break;
+            }
         }
     }
     switch (a.k_zr) {
@@ -420,12 +425,14 @@ template <bool BF16, bool ACROSS>
 cudaError_t launch_nchw(const NchwArgs& n, int64_t B, cudaStream_t st) {
     const int64_t blocks = ((ACROSS ? n.a.M : n.HW) + kNchwThreads - 1) / kNchwThreads;
     const dim3 grid((unsigned)blocks, (unsigned)n.a.K, ACROSS ? 1u : (unsigned)B);
-    if (!ACROSS && many_blocks(blocks * n.a.K * B)) {
-        switch (n.a.k_zr) {
-#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_nchw_kernel<BF16, KZ, false, true>, grid, dim3(kNchwThreads), 0, st, n);
-            TDQ_CASE(4) TDQ_CASE(7) TDQ_CASE(10) TDQ_CASE(13) TDQ_CASE(16) TDQ_CASE(32)
+    if constexpr (BF16 && !ACROSS) {
+        if (many_blocks(blocks * n.a.K * B)) {
+            switch (n.a.k_zr) {
+#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_nchw_kernel<true, KZ, false, true>, grid, dim3(kNchwThreads), 0, st, n);
+                TDQ_CASE(4) TDQ_CASE(7) TDQ_CASE(10) TDQ_CASE(13) TDQ_CASE(16) TDQ_CASE(32)
 #undef TDQ_CASE
-            default: return cudaErrorInvalidValue;
+                default: return cudaErrorInvalidValue;
+            }
         }
     }
     switch (n.a.k_zr) {

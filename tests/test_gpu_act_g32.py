@@ -63,20 +63,26 @@ def test_long_inputs(M, K, pad, zr, dtype):
     assert np.array_equal(codes[some].cpu().numpy(), want["codes"]) and np.array_equal(scale[some].cpu().numpy(), want["scale"])
 
 
-SHORT = """
-import json, os, tempfile
+RESIDENCY = """
+import json, os, sys, tempfile
 import torch
 from torch.profiler import ProfilerActivity, profile
 from paper_2604_16855_b200 import tdq
-x = torch.randn((256, 64), device="cuda")
-maps = torch.randn((2, 64, 24, 24), device="cuda"), torch.randn((70, 64, 9, 9), device="cuda")       # blocks per image, and across the images
+dtype = getattr(torch, sys.argv[1])
+if sys.argv[2] == "short":
+    x = torch.randn((256, 64), device="cuda")
+    maps = torch.randn((2, 64, 24, 24), device="cuda"), torch.randn((70, 64, 9, 9), device="cuda")       # blocks per image, and across the images
+    settings = [(0.1, 1.0), (0.2, 1.0), (0.35, 1.0), (1.0, 1.0), (0.2, 0.9), (0.3, 0.5)]
+else:
+    x = torch.randn((18464, 768), device="cuda")
+    maps = torch.randn((16, 512, 60, 60), device="cuda"),
+    settings = [(0.1, 1.0), (0.2, 1.0), (1.0, 1.0)]
 with profile(activities=[ProfilerActivity.CUDA]) as prof:
-    for dtype in (torch.bfloat16, torch.float32):
-        for zr, p in [(0.1, 1.0), (0.2, 1.0), (0.35, 1.0), (1.0, 1.0), (0.2, 0.9), (0.3, 0.5)]:
-            tdq.quantize_act(x.to(dtype), tdq.act_params(zr=zr, p=p))
-        for zr in (0.1, 0.2, 1.0):
-            for m in maps:
-                tdq.quantize_act_nchw(m.to(dtype), tdq.act_params(zr=zr))
+    for zr, p in settings:
+        tdq.quantize_act(x.to(dtype), tdq.act_params(zr=zr, p=p))
+    for zr in (0.1, 0.2, 1.0):
+        for m in maps:
+            tdq.quantize_act_nchw(m.to(dtype), tdq.act_params(zr=zr))
     torch.cuda.synchronize()
 with tempfile.TemporaryDirectory() as d:
     prof.export_chrome_trace(os.path.join(d, "t.json"))
@@ -86,12 +92,16 @@ with tempfile.TemporaryDirectory() as d:
 """
 
 
-def test_ten_blocks_of_a_short_input_per_sm():
-    """Inputs of up to ten blocks per SM run at once: the registers of the instances that they take leave room for as many."""
-    r = subprocess.run([sys.executable, "-c", SHORT], cwd=ROOT, capture_output=True, text=True, timeout=300)   # the profiler stays out of this process
+@pytest.mark.parametrize("dtype", ["bfloat16", "float32"])
+@pytest.mark.parametrize("length,launches", [("short", 6 + 3 * 2), ("long", 3 + 3)])
+def test_resident_blocks(length, launches, dtype):
+    """Inputs of up to ten blocks per SM run at once: the registers of the instances that they take leave room for as many.  Long bf16 inputs have
+    instances of which more fit; long fp32 inputs keep those of the short ones (more blocks per SM take the room in which the layer behind starts)."""
+    r = subprocess.run([sys.executable, "-c", RESIDENCY, dtype, length], cwd=ROOT, capture_output=True, text=True, timeout=300)   # the profiler stays out of this process
     assert r.returncode == 0, r.stderr
     kernels = [json.loads(line) for line in r.stdout.splitlines()]
-    assert len(kernels) == 2 * (6 + 3 * 2) and {n.split("<")[0].split("::")[-1] for n, _, _ in kernels} == {"act_g32_kernel", "act_g32_nchw_kernel"}
+    assert len(kernels) == launches and {n.split("<")[0].split("::")[-1] for n, _, _ in kernels} == {"act_g32_kernel", "act_g32_nchw_kernel"}
     for name, registers, threads in kernels:
         warp = -(-registers * 32 // 256) * 256            # a warp's registers come in pieces of 256, an SM has 65536
-        assert 65536 // (warp * threads // 32) >= 10, (name, registers)
+        blocks = 65536 // (warp * threads // 32)
+        assert blocks >= 14 if (length, dtype) == ("long", "bfloat16") else 10 <= blocks <= 12, (name, registers)
