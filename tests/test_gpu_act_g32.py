@@ -73,9 +73,10 @@ if sys.argv[2] == "short":
     x = torch.randn((256, 64), device="cuda")
     maps = torch.randn((2, 64, 24, 24), device="cuda"), torch.randn((70, 64, 9, 9), device="cuda")       # blocks per image, and across the images
     settings = [(0.1, 1.0), (0.2, 1.0), (0.35, 1.0), (1.0, 1.0), (0.2, 0.9), (0.3, 0.5)]
-else:
-    x = torch.randn((18464, 768), device="cuda")
-    maps = torch.randn((16, 512, 60, 60), device="cuda"),
+else:                                                                    # 28 and 27.7 blocks per SM, or 47 and 99
+    below = sys.argv[2] == "below"
+    x = torch.randn((11050 if below else 18464, 768), device="cuda")
+    maps = torch.randn((16, 512, 32, 32) if below else (16, 512, 60, 60), device="cuda"),
     settings = [(0.1, 1.0), (0.2, 1.0), (1.0, 1.0)]
 with profile(activities=[ProfilerActivity.CUDA]) as prof:
     for zr, p in settings:
@@ -93,10 +94,11 @@ with tempfile.TemporaryDirectory() as d:
 
 
 @pytest.mark.parametrize("dtype", ["bfloat16", "float32"])
-@pytest.mark.parametrize("length,launches", [("short", 6 + 3 * 2), ("long", 3 + 3)])
+@pytest.mark.parametrize("length,launches", [("short", 6 + 3 * 2), ("below", 3 + 3), ("long", 3 + 3)])
 def test_resident_blocks(length, launches, dtype):
-    """Inputs of up to ten blocks per SM run at once: the registers of the instances that they take leave room for as many.  Long bf16 inputs have
-    instances of which more fit; long fp32 inputs keep those of the short ones (more blocks per SM take the room in which the layer behind starts)."""
+    """Inputs of up to ten blocks per SM run at once: the registers of the instances that they take leave room for as many.  bf16 inputs of
+    more than 30 blocks per SM have instances of which more fit; long fp32 inputs keep those of the short ones (more blocks per SM take the
+    room in which the layer behind starts)."""
     r = subprocess.run([sys.executable, "-c", RESIDENCY, dtype, length], cwd=ROOT, capture_output=True, text=True, timeout=300)   # the profiler stays out of this process
     assert r.returncode == 0, r.stderr
     kernels = [json.loads(line) for line in r.stdout.splitlines()]
