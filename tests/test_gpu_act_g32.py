@@ -34,33 +34,53 @@ def test_block_edges(M, K, pad, dtype):
     assert bool((codes[M] == 77).all()) and bool((scale[M] == -1.0).all())
 
 
-@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
-@pytest.mark.parametrize("zr", [0.1, 0.2, 1.0])
-@pytest.mark.parametrize("M,K,pad", [(7301, 32, 0), (3701, 63, 8)])
-def test_long_inputs(M, K, pad, zr, dtype):
-    """Inputs of more than 24 blocks per SM have an instance of their own, whose rare paths are calls: groups with a large mean (the
-    deviation in binary64) and of huge numbers (IEEE division) among the others.  The same bits as row by row block, and the oracle's."""
-    from paper_2604_16855_b200 import tdq
-    assert M * K > 24 * 64 * torch.cuda.get_device_properties(0).multi_processor_count and M * K % 64
-    gen = torch.Generator("cuda").manual_seed(M + K)
-    x = torch.randn((M, 32 * K), device="cuda", generator=gen) * torch.exp(0.5 * torch.randn((M, 1), device="cuda", generator=gen))
+def _rows_with_rare_ones(M, C, seed):
+    """Rows among which some have a large mean (the deviation in binary64), some huge numbers (IEEE division) and some nothing but zeros."""
+    gen = torch.Generator("cuda").manual_seed(seed)
+    x = torch.randn((M, C), device="cuda", generator=gen) * torch.exp(0.5 * torch.randn((M, 1), device="cuda", generator=gen))
     x[5::50] += 30.0
     x[7::50] *= 1e32
     x[9::50] = 0.0
-    store = torch.zeros((M, 32 * K + pad), dtype=dtype, device="cuda")
-    store[:, :32 * K] = x.to(dtype)
-    xt = store[:, :32 * K]
-    p = tdq.act_params(zr=zr)
-    codes = torch.full((M + 1, 16 * K), 77, dtype=torch.uint8, device="cuda")
-    scale = torch.full((M + 1, K), -1.0, device="cuda")
-    tdq.quantize_act(xt, p, codes=codes[:M], scale=scale[:M])
+    return x
+
+
+def _check_long(xt, p, **oracle_args):
+    """Codes and steps of a long input: nothing written past them, the same bits as block by block of rows (too short for the instances
+    of long inputs), and the oracle's on some rows."""
+    from paper_2604_16855_b200 import tdq
+    M, C = xt.shape
+    codes = torch.full((M + 1, C // 2), 77, dtype=torch.uint8, device="cuda")
+    scale = torch.full((M + 1, C // 32), -1.0, device="cuda")
+    offset = torch.full((M + 1, C // 32), -1.0, device="cuda")
+    tdq.quantize_act(xt, p, codes=codes[:M], scale=scale[:M], offset=offset[:M])
     assert bool((codes[M] == 77).all()) and bool((scale[M] == -1.0).all())
+    assert bool((offset[:M] == 0.0).all()) and bool((offset[M] == -1.0).all())
     for r in range(0, M, 1000):
         c, s = tdq.quantize_act(xt[r:r + 1000], p)
         assert torch.equal(c, codes[r:min(r + 1000, M)]) and torch.equal(s, scale[r:min(r + 1000, M)])
     some = list(range(0, M, 61)) + [5, 7, 9, M - 1]
-    want = oracle.quantize_act(xt[some].float().cpu().numpy(), zr=zr)
+    want = oracle.quantize_act(xt[some].float().cpu().numpy(), **oracle_args)
     assert np.array_equal(codes[some].cpu().numpy(), want["codes"]) and np.array_equal(scale[some].cpu().numpy(), want["scale"])
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("zr", [0.1, 0.2, 0.3, 0.4, 0.5, 1.0])
+@pytest.mark.parametrize("M,K,pad,long", [(7301, 32, 0, False), (3701, 63, 8, False), (9001, 32, 0, True), (4701, 63, 8, True)])
+def test_long_inputs(M, K, pad, long, zr, dtype):
+    """bf16 inputs of more than 30 blocks per SM have an instance of their own for each of these zero-bin ranks, whose rare paths are
+    calls; both sides of that line."""
+    from paper_2604_16855_b200 import tdq
+    assert (M * K > 30 * 64 * torch.cuda.get_device_properties(0).multi_processor_count) == long and M * K % 64
+    store = torch.zeros((M, 32 * K + pad), dtype=dtype, device="cuda")
+    store[:, :32 * K] = _rows_with_rare_ones(M, 32 * K, M + K).to(dtype)
+    _check_long(store[:, :32 * K], tdq.act_params(zr=zr), zr=zr)
+
+
+@pytest.mark.parametrize("flags", [0, oracle.ENABLE_C1, oracle.ENABLE_C2, oracle.ENABLE_C1 | oracle.ENABLE_C2 | oracle.POW2_STEP])
+def test_long_inputs_by_setting(flags):
+    """The same with the bounds off, with one of them, and with power-of-two steps."""
+    from paper_2604_16855_b200 import tdq
+    _check_long(_rows_with_rare_ones(9001, 1024, 11).to(torch.bfloat16), tdq.act_params(flags=flags), flags=flags)
 
 
 RESIDENCY = """
