@@ -126,16 +126,17 @@ __global__ void __launch_bounds__(kGenericWarps * 32) act_generic_kernel(ActArgs
 // and 5.19, with its layer 15.31 and 16.12).
 constexpr int kFastThreads = 64, kFastBlocks = 16;
 
-// Whether a bf16 input is long: more than 30 blocks per SM.  Its instances are held to 64 registers (72 channel-major; they spill 8 and 12
-// bytes), with the rare paths out of line, so that 32 warps instead of 20 hide each other's latencies: issue slots 0.54 -> 0.68 busy.  us from a
+// Whether a bf16 input is long: at least 40 blocks per SM.  Its instances are held to 64 registers (72 channel-major; they spill 8 and 12
+// bytes), with the rare paths out of line, so that 32 warps instead of 20 hide each other's latencies: issue slots 0.54 -> 0.59 busy.  us from a
 // graph, the other instances (ten blocks per SM) and these: 16384 x 4096 44.3 and 38.6, 73728 x 256 14.6 and 13.2, 18464 x 768 11.4 and 10.4, the
 // same with a mean of 30 (every group takes a rare path) 14.3 and 13.4, map [16, 512, 60, 60] 28.3 and 26.3.  Short inputs lose: where all blocks
 // are resident at once the SMs get uneven shares of them, and the kernel behind finds no room to set itself up in; quantizer and layer behind it,
 // 9216 x 320 -> 960 (9.7 blocks per SM) 22.4 and 23.9, 18432 x 128 -> 128 (7.8) 10.1 and 11.5, 73728 x 64 -> 64 (15.6) 15.6 and 16.4, 4608 x 1280 ->
-// 320 (19.5) 20.1 and 20.8, but 18432 x 512 -> 128 (31) 18.3 and 17.7, 73728 x 256 -> 64 (62) 30.4 and 29.6.  At 30 the others have three full
-// rounds and these nearly two.  The ratio of the two with a layer behind, over 16 layers of 64 to 768 channels in a graph and in a stream, worst and
-// best: at 25 blocks per SM 1.028 and 0.97 (most with a binary32 output lose), 28 1.015 and 0.976, 32 1.013 and 0.96, 40 1.005 and 0.94, 64
-// 0.997 and 0.95; maps, 8 layers: at 26 1.013 and 0.988, 30 1.008 and 0.987, 34 1.002 and 0.964, 50 1.000 and 0.95.  Twenty blocks (48 registers)
+// 320 (19.5) 20.1 and 20.8, but 18432 x 512 -> 128 (31) 18.3 and 17.7, 73728 x 256 -> 64 (62) 30.4 and 29.6.  The ratio of the two with a
+// layer behind, over 16 layers of 64 to 768 channels in a graph and in a stream, worst and best: at 25 blocks per SM 1.028 and 0.97, 28 1.015 and
+// 0.976, 32 1.013 and 0.96, 40 1.005 and 0.94, 64 0.997 and 0.95; maps, 8 layers: at 26 1.013 and 0.988, 34 1.002 and 0.964, 50 1.000 and 0.95.
+// Behind a layer with a large output they gain less: of two layers C -> 4 C -> C with their quantizers, C 64 to 768, at 31 blocks per SM 1.023 and
+// 0.975, 42 1.012 and 0.98, 64 1.005 and 0.97, 100 0.996 and 0.97 (worst at C = 64 with a binary32 output, which loses up to 80).  Twenty blocks (48 registers)
 // are 2 % faster alone (not timed with a layer); two or four groups a thread, the next one's loads in flight: level.
 // The ranks of the paper's sweep with the maximum as base radius have them; percentile radii, other ranks and maps taken across the images keep
 // the other instances at every length (not timed).
@@ -144,7 +145,7 @@ constexpr int kFastThreads = 64, kFastBlocks = 16;
 // [16, 512, 33, 35] -> 512 34.1 and 35.4), on rows with a pitch (18464 x 768 16.8 and 18.0) and with a mean of 30 (17.8 and 19.8).
 bool many_blocks(int64_t blocks) {
     const int n_sm = current_device_sm_count();
-    return blocks > 30 * (int64_t)(n_sm > 0 ? n_sm : 148);
+    return blocks >= 40 * (int64_t)(n_sm > 0 ? n_sm : 148);
 }
 
 // One group: quantize it in registers, write its 16 code bytes and its scale.

@@ -35,7 +35,8 @@
 // 36.9, with p = 0.9 175.0 -> 69.1; 16384 x 4096 at g = 4096 76.8 -> 64.6 (of it eight chunks a lane 8.4); fp32 18464 x 768 at
 // g = 128 26.2 -> 22.8, rectified 76.1 -> 18.6.  The bisection kernel that served these cases at first: 978 us on the long groups.
 // Since then the maximum and both moments take one exchange, the element next to the last probe is found in one pass for either side of it,
-// and the clip is one instruction: 16384 x 4096 at g = 4096 64.1 -> 55.9, with the layer behind it 242 -> 226 (from a graph).
+// and the clip is one instruction: 16384 x 4096 at g = 4096 64.2 -> 56.0; with the layer behind it 222.5 -> 213.1 from a graph, 245.8 -> 238.5 in a
+// stream (3 %).
 #include <climits>
 
 #include "tdq_act_group.cuh"
@@ -257,9 +258,10 @@ __device__ __forceinline__ uint32_t group_kth(const Share<BF16, NC>& x, int k, i
     return r;
 }
 
-// Resident blocks the registers are allocated for: the share (4 or 8 words a chunk) and about fifty more.  The bf16 instances with
-// four and six chunks a lane on eight lanes and more spill a word or two there.  A block less, which holds them, is faster on a few
-// hundred groups (1024 x 4096 at 1024 and 4096 8 %) and slower on many: 16384 x 1536 at 256 2.3 %, at 512 2.9 %, at 1536 4.5 %.
+// Resident blocks the registers are allocated for: the share (4 or 8 words a chunk) and about fifty more.  No instance spills.  us from a
+// graph, bf16, with a block less, so many and one more: 16384 x 4096 at g = 4096 59.6, 56.0 and 55.8 (with p = 0.9 96.2, 96.7 and 100.0), 16384 x
+// 1536 at 512 29.1, 28.1 and 28.0, 18464 x 768 at 128 19.1, 18.6 and 18.9 (p = 0.9 30.5, 30.3 and 31.4); inputs of one round or less like fewer:
+// 1024 x 4096 at 4096 7.4, 8.0 and 8.7, 4616 x 768 at 128 7.5, 8.1 and 8.8.  fp32 takes the same registers either way.
 constexpr int wide_blocks(bool bf16, int nc) {
     const int regs = bf16 ? 4 * nc + 48 : 8 * nc + 64;
     return 512 / (regs < 64 ? 64 : regs);
