@@ -120,11 +120,28 @@ __global__ void __launch_bounds__(kGenericWarps * 32) act_generic_kernel(ActArgs
 // fast kernel: g = 32, one thread per group
 
 // Threads, and so groups, of a block of the fast kernels.  Small blocks: ten of them fill an SM's registers without the remainder
-// that two of 256 threads leave, and no warp waits for more than one other.  The instances for long inputs hold sixteen; the others have
-// no bound (0), which gives 88 to 96 registers, ten or eleven blocks.  A bound of 1 is not the same: it lets fp32 take 108 registers, nine blocks,
-// and the 9.7 blocks per SM of 9216 x 320 no longer run at once (fp32 from a graph 5.10 and 5.59 us; channel-major [16, 320, 24, 24] bf16 4.47
-// and 5.19, with its layer 15.31 and 16.12).
+// that two of 256 threads leave, and no warp waits for more than one other.
 constexpr int kFastThreads = 64, kFastBlocks = 16;
+
+// The instances of the fast kernels differ in the registers that they may take, by the blocks per SM of the launch.
+enum Length { kFew, kShort, kLong };
+
+// The launch bound of an instance (0: none).
+constexpr int resident_blocks(Length len, int long_blocks) { return len == kLong ? long_blocks : len == kFew ? 1 : 0; }
+
+// Blocks per SM up to which fp32 inputs and maps are few.  A bound of one block lets the compiler take 106 to 108 registers (without a bound 87 to
+// 96), and the group is done sooner: all its loads are in flight first.  Four such warps fit a scheduler, eight blocks an SM, so beyond
+// eight a second round would start that ten or eleven blocks of the other instances do not need.  Quantizer and layer behind it, bound of one
+// over none at 1, 3, 5, 7, 8, 8.4 and 9 blocks per SM: fp32 rows of 320 -> 320 1.02, 0.95, 0.97, 0.97, 0.98, 1.01, 1.02, rows of 64 -> 64 1.0, 0.94,
+// 0.95, 0.95, 0.96, 1.02, 1.03; maps of 64 -> 64 bf16 0.98, 0.96, 0.95, 0.96, 0.96, 1.04, 1.05, of 768 -> 768 fp32 1.0, 1.0, 0.97, 0.96, 0.98, 0.98,
+// 1.04; images of 10 x 10 positions, 256 -> 256 bf16, as launched: 2.6 1.0, 3.8 0.96, 7.7 0.97, 9 1.05.  (Quantizers alone, one behind the
+// other, overlap less with it at four to five: 320 channels fp32 3.3 and 3.8 us at 4.9, 4.4 and 4.1 at 5.8.)  bf16 rows take 90 or 92 registers either way.
+constexpr int kFewBlocks = 8;
+
+bool few_blocks(int64_t blocks) {
+    const int n_sm = current_device_sm_count();
+    return blocks <= kFewBlocks * (int64_t)(n_sm > 0 ? n_sm : 148);
+}
 
 // Whether a bf16 input is long: at least 40 blocks per SM.  Its instances are held to 64 registers (72 channel-major; they spill 8 and 12
 // bytes), with the rare paths out of line, so that 32 warps instead of 20 hide each other's latencies: issue slots 0.54 -> 0.59 busy.  us from a
@@ -149,11 +166,11 @@ bool many_blocks(int64_t blocks) {
 }
 
 // One group: quantize it in registers, write its 16 code bytes and its scale.
-template <bool BF16, int KZR, int KB = 32, bool LONG = false>
+template <bool BF16, int KZR, int KB = 32, Length LEN = kShort>
 __device__ __forceinline__ void process_group(const uint32_t (&w)[BF16 ? 16 : 32], const ActArgs& a, int64_t gi) {
     uint32_t out[4];
     float delta;
-    quantize_group32<BF16, KZR, KB, LONG>(w, a.seven_tau, a.flags, out, delta, a.k_zr, a.k_base);
+    quantize_group32<BF16, KZR, KB, LEN == kLong>(w, a.seven_tau, a.flags, out, delta, a.k_zr, a.k_base);
     reinterpret_cast<uint4*>(a.codes)[gi] = make_uint4(out[0], out[1], out[2], out[3]);
     a.scale[gi] = delta;
     if (a.offset) a.offset[gi] = 0.0f;
@@ -170,8 +187,8 @@ __device__ __forceinline__ void process_group(const uint32_t (&w)[BF16 ? 16 : 32
 // against 16.2 us, 9216 x 320 6.2 and 4.9; bf16 11.8 against 12.0); rows with a pitch, which cost a division a group, are loaded
 // directly in either type (the staging kernel that had them before and this, pitch 8 longer: 18464 x 768 bf16 21.6 and 12.8, 9216 x
 // 320 6.0 and 3.75; fp32 2304 x 768 8.4 and 5.25, 1152 x 512 4.8 and 2.4).  Blocks of 128 threads: level, long bf16 inputs 1 to 2 % slower.
-template <bool BF16, int KZR, int KB = 32, bool LONG = false>
-__global__ void __launch_bounds__(kFastThreads, LONG ? kFastBlocks : 0) act_g32_kernel(ActArgs a) {
+template <bool BF16, int KZR, int KB, Length LEN>
+__global__ void __launch_bounds__(kFastThreads, resident_blocks(LEN, kFastBlocks)) act_g32_kernel(ActArgs a) {
     constexpr int kGroupBytes = BF16 ? 64 : 128;
     constexpr int kChunks = kGroupBytes / 16;          // 16-byte chunks per group
     const int t = threadIdx.x;
@@ -226,7 +243,7 @@ __global__ void __launch_bounds__(kFastThreads, LONG ? kFastBlocks : 0) act_g32_
             w[4 * p + 0] = u.x; w[4 * p + 1] = u.y; w[4 * p + 2] = u.z; w[4 * p + 3] = u.w;
         }
     }
-    process_group<BF16, KZR, KB, LONG>(w, a, gi);
+    process_group<BF16, KZR, KB, LEN>(w, a, gi);
 }
 
 // every zero-bin rank of a group of 32 has its instance of the row-major kernel
@@ -235,38 +252,45 @@ __global__ void __launch_bounds__(kFastThreads, LONG ? kFastBlocks : 0) act_g32_
     TDQ_CASE(9) TDQ_CASE(10) TDQ_CASE(11) TDQ_CASE(12) TDQ_CASE(13) TDQ_CASE(14) TDQ_CASE(15) TDQ_CASE(16) \
     TDQ_CASE(17) TDQ_CASE(18) TDQ_CASE(19) TDQ_CASE(20) TDQ_CASE(21) TDQ_CASE(22) TDQ_CASE(23) TDQ_CASE(24) \
     TDQ_CASE(25) TDQ_CASE(26) TDQ_CASE(27) TDQ_CASE(28) TDQ_CASE(29) TDQ_CASE(30) TDQ_CASE(31) TDQ_CASE(32)
-template <bool BF16>
-cudaError_t launch_fast(const ActArgs& a, cudaStream_t st) {
-    const int64_t blocks = (a.total_groups + kFastThreads - 1) / kFastThreads;
-    dim3 grid((unsigned)blocks), block(kFastThreads);
+template <bool BF16, Length LEN>
+cudaError_t launch_ranks(const ActArgs& a, dim3 grid, cudaStream_t st) {
+    const dim3 block(kFastThreads);
     if (a.k_base != 32 && (a.k_base < 29 || a.k_zr != 7)) {
         // any other pair of ranks: the instance that takes both at run time
-        return launch_pdl(act_g32_kernel<BF16, 0, 0>, grid, block, 0, st, a);
+        return launch_pdl(act_g32_kernel<BF16, 0, 0, LEN>, grid, block, 0, st, a);
     }
     if (a.k_base != 32) {        // percentile base radius: ranks 29..31 beside the default zero-bin rank
         switch (a.k_base) {
-#define TDQ_CASE(KB_) case KB_: return launch_pdl(act_g32_kernel<BF16, 7, KB_>, grid, block, 0, st, a);
+#define TDQ_CASE(KB_) case KB_: return launch_pdl(act_g32_kernel<BF16, 7, KB_, LEN>, grid, block, 0, st, a);
             TDQ_CASE(29) TDQ_CASE(30) TDQ_CASE(31)
 #undef TDQ_CASE
             default: return cudaErrorInvalidValue;
         }
     }
+    switch (a.k_zr) {
+#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_kernel<BF16, KZ, 32, LEN>, grid, block, 0, st, a);
+        TDQ_ALL_RANKS
+#undef TDQ_CASE
+        default: return cudaErrorInvalidValue;
+    }
+}
+template <bool BF16>
+cudaError_t launch_fast(const ActArgs& a, cudaStream_t st) {
+    const int64_t blocks = (a.total_groups + kFastThreads - 1) / kFastThreads;
+    const dim3 grid((unsigned)blocks);
     if constexpr (BF16) {
-        if (many_blocks(blocks)) {
+        if (a.k_base == 32 && many_blocks(blocks)) {
             switch (a.k_zr) {
-#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_kernel<true, KZ, 32, true>, grid, block, 0, st, a);
+#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_kernel<true, KZ, 32, kLong>, grid, dim3(kFastThreads), 0, st, a);
                 TDQ_CASE(4) TDQ_CASE(7) TDQ_CASE(10) TDQ_CASE(13) TDQ_CASE(16) TDQ_CASE(32)
 #undef TDQ_CASE
                 default: break;
             }
         }
+    } else if (few_blocks(blocks)) {
+        return launch_ranks<false, kFew>(a, grid, st);
     }
-    switch (a.k_zr) {
-#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_kernel<BF16, KZ>, grid, block, 0, st, a);
-        TDQ_ALL_RANKS
-#undef TDQ_CASE
-        default: return cudaErrorInvalidValue;
-    }
+    return launch_ranks<BF16, kShort>(a, grid, st);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -395,8 +419,8 @@ struct NchwArgs {
     int64_t HW;         // positions per image
 };
 
-template <bool BF16, int KZR, bool ACROSS, bool LONG = false>
-__global__ void __launch_bounds__(kNchwThreads, LONG ? kNchwBlocks : 0) act_g32_nchw_kernel(NchwArgs n) {
+template <bool BF16, int KZR, bool ACROSS, Length LEN>
+__global__ void __launch_bounds__(kNchwThreads, resident_blocks(LEN, kNchwBlocks)) act_g32_nchw_kernel(NchwArgs n) {
     constexpr int esz = BF16 ? 2 : 4;
     const ActArgs& a = n.a;
     const int t = threadIdx.x;
@@ -424,29 +448,27 @@ __global__ void __launch_bounds__(kNchwThreads, LONG ? kNchwBlocks : 0) act_g32_
 #pragma unroll
         for (int i = 0; i < 32; ++i) w[i] = __ldg(reinterpret_cast<const uint32_t*>(src + i * row));
     }
-    process_group<BF16, KZR, 32, LONG>(w, a, ((b * n.HW + s) * a.K) + k);
+    process_group<BF16, KZR, 32, LEN>(w, a, ((b * n.HW + s) * a.K) + k);
 }
 
-template <bool BF16, bool ACROSS>
-cudaError_t launch_nchw(const NchwArgs& n, int64_t B, cudaStream_t st) {
-    const int64_t blocks = ((ACROSS ? n.a.M : n.HW) + kNchwThreads - 1) / kNchwThreads;
-    const dim3 grid((unsigned)blocks, (unsigned)n.a.K, ACROSS ? 1u : (unsigned)B);
-    if constexpr (BF16 && !ACROSS) {
-        if (many_blocks(blocks * n.a.K * B)) {
-            switch (n.a.k_zr) {
-#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_nchw_kernel<true, KZ, false, true>, grid, dim3(kNchwThreads), 0, st, n);
-                TDQ_CASE(4) TDQ_CASE(7) TDQ_CASE(10) TDQ_CASE(13) TDQ_CASE(16) TDQ_CASE(32)
-#undef TDQ_CASE
-                default: return cudaErrorInvalidValue;
-            }
-        }
-    }
+template <bool BF16, bool ACROSS, Length LEN>
+cudaError_t launch_nchw_ranks(const NchwArgs& n, dim3 grid, cudaStream_t st) {
     switch (n.a.k_zr) {
-#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_nchw_kernel<BF16, KZ, ACROSS>, grid, dim3(kNchwThreads), 0, st, n);
+#define TDQ_CASE(KZ) case KZ: return launch_pdl(act_g32_nchw_kernel<BF16, KZ, ACROSS, LEN>, grid, dim3(kNchwThreads), 0, st, n);
         TDQ_CASE(4) TDQ_CASE(7) TDQ_CASE(10) TDQ_CASE(13) TDQ_CASE(16) TDQ_CASE(32)
 #undef TDQ_CASE
         default: return cudaErrorInvalidValue;
     }
+}
+template <bool BF16, bool ACROSS>
+cudaError_t launch_nchw(const NchwArgs& n, int64_t B, cudaStream_t st) {
+    const int64_t per_row = ((ACROSS ? n.a.M : n.HW) + kNchwThreads - 1) / kNchwThreads, blocks = per_row * n.a.K * (ACROSS ? 1 : B);
+    const dim3 grid((unsigned)per_row, (unsigned)n.a.K, ACROSS ? 1u : (unsigned)B);
+    if (few_blocks(blocks)) return launch_nchw_ranks<BF16, ACROSS, kFew>(n, grid, st);
+    if constexpr (BF16 && !ACROSS) {
+        if (many_blocks(blocks)) return launch_nchw_ranks<true, false, kLong>(n, grid, st);
+    }
+    return launch_nchw_ranks<BF16, ACROSS, kShort>(n, grid, st);
 }
 
 // ------------------------------------------------------------------------------------------
