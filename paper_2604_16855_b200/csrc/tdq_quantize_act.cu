@@ -130,7 +130,7 @@ enum Length { kFew, kShort, kLong };
 constexpr int resident_blocks(Length len, int long_blocks) { return len == kLong ? long_blocks : len == kFew ? 1 : 0; }
 
 // Blocks per SM up to which fp32 inputs and maps are few.  A bound of one block lets the compiler take 106 to 108 registers (without a bound 87 to
-// 96), and the group is done sooner: all its loads are in flight first.  Four such warps fit a scheduler, eight blocks an SM, so beyond
+// 96), and the group is done sooner (it may keep more of a group's loads in flight; not shown).  Four such warps fit a scheduler, eight blocks an SM, so beyond
 // eight a second round would start that ten or eleven blocks of the other instances do not need.  Quantizer and layer behind it, bound of one
 // over none at 1, 3, 5, 7, 8, 8.4 and 9 blocks per SM: fp32 rows of 320 -> 320 1.02, 0.95, 0.97, 0.97, 0.98, 1.01, 1.02, rows of 64 -> 64 1.0, 0.94,
 // 0.95, 0.95, 0.96, 1.02, 1.03; maps of 64 -> 64 bf16 0.98, 0.96, 0.95, 0.96, 0.96, 1.04, 1.05, of 768 -> 768 fp32 1.0, 1.0, 0.97, 0.96, 0.98, 0.98,
